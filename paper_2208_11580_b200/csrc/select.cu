@@ -7,20 +7,31 @@
 // lexicographic order (key, r, t).  Within a row keys are non-decreasing, so the popped entries of a row
 // are a prefix and counts[r] = #{key < T} + (share of the entries with key == T, handed out by row).
 //
-// Kernels: prefix-max keys -> 4-pass 8-bit radix select of the k-th key T -> per-row counts -> tie
-// distribution over rows -> mask scatter.  Keys are non-negative floats compared as unsigned integers.
+// One cooperative launch does all of it (a barrier over the grid per 9 + 11 + 11 bits of the key would be two launches and
+// their gaps otherwise: twelve kernels took 96 us a call, nearly all of it launch latency).  A block owns consecutive rows and keeps
+// their keys in shared memory.  Keys of a row do not decrease, so a digit histogram needs only the places where the
+// digit changes: key t with another digit than key t + 1 adds t + 1 to its own bin and takes t + 1 from the next one; and
+// once a digit is decided, a binary search per row narrows the row to the keys that share it, so only the first digit
+// (few bits: few changes) scans whole rows.
+// Keys are non-negative floats compared as unsigned integers.
 #include "common.cuh"
+#include "grid_barrier.cuh"
 #include <mutex>
 
 namespace obc {
 
-constexpr int SEL_THREADS = 256;
+constexpr int SEL_THREADS = 1024;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int SEL_MAX_BLOCKS = 512;
+constexpr int SEL_MAX_UNITS = 128;                // row segments of a block, when rows are cut into segments
+constexpr int SEL_BINS = 2048;
+constexpr int SEL_SMEM = 200 * 1024;              // keys of a block's rows, if they fit
 
-struct SelectState {            // lives in the workspace
-    unsigned int hist[256];
-    unsigned int prefix;        // bits of T decided so far
-    unsigned int pad;
-    unsigned long long remaining;   // rank still to resolve inside the current prefix bucket (1-based)
+struct SelectState {            // in the workspace, zero before the launch
+    unsigned int hist[3][SEL_BINS];
+    unsigned int arrived;       // blocks at the grid barriers
+    unsigned int pad[63];
+    unsigned long long ties[SEL_MAX_BLOCKS];      // keys equal to the k-th one, per block
 };
 
 __device__ __forceinline__ unsigned int loss_key(float x) {
@@ -30,128 +41,281 @@ __device__ __forceinline__ unsigned int loss_key(float x) {
     return __float_as_uint(x);
 }
 
-// keys[r][t] = max_{t' <= t} key(L[r][t'])       one block per row
-__global__ void __launch_bounds__(SEL_THREADS) prefix_max_kernel(const float* __restrict__ loss, int d,
-                                                                 unsigned int* __restrict__ keys) {
-    __shared__ unsigned int part[SEL_THREADS];
-    const int r = blockIdx.x, tid = threadIdx.x;
-    const int chunk = (d + SEL_THREADS - 1) / SEL_THREADS;
-    const int b = tid * chunk, e = min(d, b + chunk);
-    const float* L = loss + (size_t)r * d;
-    unsigned int* K = keys + (size_t)r * d;
-    unsigned int mx = 0;
-    for (int t = b; t < e; ++t) mx = max(mx, loss_key(L[t]));
-    part[tid] = mx;
-    __syncthreads();
-    for (int off = 1; off < SEL_THREADS; off <<= 1) {           // inclusive max-scan of the chunk maxima
-        unsigned int o = tid >= off ? part[tid - off] : 0u;
-        __syncthreads();
-        part[tid] = max(part[tid], o);
-        __syncthreads();
+template <typename Count> struct SelectShared {
+    unsigned int hist[SEL_BINS];
+    unsigned int segmax[SEL_MAX_UNITS];
+    Count scan[SEL_WARPS];
+    Count rem, before;
+    unsigned int digit, digit_count;
+};
+
+// Inclusive scan over the block of one value per thread; sh.scan[w] = total of warps 0 .. w afterwards.
+template <typename Count>
+__device__ __forceinline__ Count block_scan(Count v, SelectShared<Count>& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const Count o = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v += o;
     }
-    unsigned int run = tid ? part[tid - 1] : 0u;
-    for (int t = b; t < e; ++t) { run = max(run, loss_key(L[t])); K[t] = run; }
-}
-
-__global__ void select_init_kernel(SelectState* s, long long k) {
-    if (threadIdx.x < 256) s->hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) { s->prefix = 0; s->remaining = (unsigned long long)k; }
-}
-
-// histogram of the digit at `shift` over keys whose higher bits equal the decided prefix
-__global__ void __launch_bounds__(SEL_THREADS) select_hist_kernel(const unsigned int* __restrict__ keys, long long n,
-                                                                  int shift, SelectState* s) {
-    __shared__ unsigned int h[256];
-    h[threadIdx.x] = 0;
+    __syncthreads();                                      // the previous scan's totals have been read
+    if (lane == 31) sh.scan[warp] = v;
     __syncthreads();
-    const unsigned int prefix = s->prefix;
-    const unsigned int himask = shift == 24 ? 0u : (0xffffffffu << (shift + 8));
-    for (long long i = blockIdx.x * (long long)SEL_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * SEL_THREADS) {
-        const unsigned int key = keys[i];
-        if ((key & himask) == prefix) atomicAdd(&h[(key >> shift) & 255u], 1u);
+    Count w = sh.scan[lane];                              // (every warp scans the 32 totals for itself)
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const Count o = __shfl_up_sync(0xffffffffu, w, off);
+        if (lane >= off) w += o;
+    }
+    const Count below = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    return warp > 0 ? v + below : v;
+}
+
+// Thread t owns bins 2t, 2t + 1 (counts a, b): the bin that holds rank sh.rem becomes sh.digit, sh.rem the rank inside it.
+template <typename Count>
+__device__ __forceinline__ void pick_digit(unsigned int a, unsigned int b, SelectShared<Count>& sh) {
+    const Count incl = block_scan((Count)a + b, sh);
+    const Count rem = sh.rem, before = incl - a - b;
+    __syncthreads();
+    if (before < rem && rem <= incl) {
+        const bool second = rem > before + a;
+        sh.digit = 2 * threadIdx.x + (second ? 1 : 0);
+        sh.digit_count = second ? b : a;
+        sh.rem = rem - before - (second ? a : 0);
     }
     __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(&s->hist[threadIdx.x], h[threadIdx.x]);
 }
 
-// pick the digit that contains rank `remaining`, update prefix / remaining, clear the histogram
-__global__ void select_pick_kernel(SelectState* s, int shift) {
-    if (threadIdx.x == 0) {
-        unsigned long long rem = s->remaining, acc = 0;
-        int dgt = 255;
-        if (rem == 0) { dgt = 0; }      // k == 0: T = 0 with nothing to take
-        else {
-            for (int b = 0; b < 256; ++b) {
-                const unsigned long long c = s->hist[b];
-                if (acc + c >= rem) { dgt = b; break; }
-                acc += c;
+// keys: the block's rows in shared memory (IN_SMEM) or this call's rows in the workspace.  A block takes rows
+// [rpb * blockIdx.x, + rpb), cut into `segs` segments each for the scans (one warp per segment).
+template <bool IN_SMEM, typename Count>
+__global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ loss, const int32_t* __restrict__ order, int rows, int d,
+                                                             unsigned long long k, int rpb, int segs, unsigned int* __restrict__ gkeys,
+                                                             int* __restrict__ glt, int* __restrict__ gle, SelectState* __restrict__ st,
+                                                             int* __restrict__ counts, uint8_t* __restrict__ mask) {
+    extern __shared__ __align__(16) unsigned int skeys[];
+    __shared__ SelectShared<Count> sh;
+    __shared__ int slt[SEL_THREADS], sle[SEL_THREADS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int r0 = blockIdx.x * rpb, nr = min(rpb, rows - r0);           // >= 1
+    const unsigned int G = gridDim.x;
+    const int ldk = IN_SMEM ? (d + 3) & ~3 : d;          // stride of the keys
+    const int seg_len = ((d + segs - 1) / segs + 3) & ~3;
+    const int units = nr * segs;
+    unsigned int* keys = IN_SMEM ? skeys : gkeys + (size_t)r0 * ldk;
+    const float* L = loss + (size_t)r0 * d;
+    int* row_lt = rpb <= SEL_THREADS ? slt : glt + r0;
+    int* row_le = rpb <= SEL_THREADS ? sle : gle + r0;
+    unsigned int barrier_no = 0;
+
+    for (int b = tid; b < SEL_BINS; b += SEL_THREADS) sh.hist[b] = 0u;
+    if (tid == 0) sh.rem = (Count)k;
+    // keys [row_lt, row_le) of a row share the digits decided so far (in the end: are equal to the k-th key)
+    for (int r = tid; r < nr; r += SEL_THREADS) { row_lt[r] = 0; row_le[r] = k > 0 ? d : 0; }
+    // ---- prefix maxima within segments
+    for (int u = warp; u < units; u += SEL_WARPS) {
+        const int r = u / segs, g = u - r * segs;
+        const int b = g * seg_len, e = min(d, b + seg_len);
+        const float* Lr = L + (size_t)r * d;
+        unsigned int carry = 0u;
+        float nx[8];                                      // the next 256 losses are on their way while these are scanned
+#pragma unroll
+        for (int q = 0; q < 8; ++q) nx[q] = b + 32 * q + lane < e ? __ldg(Lr + b + 32 * q + lane) : 0.f;
+        for (int t0 = b; t0 < e; t0 += 256) {
+            unsigned int v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = loss_key(nx[q]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) nx[q] = t0 + 256 + 32 * q + lane < e ? __ldg(Lr + t0 + 256 + 32 * q + lane) : 0.f;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {             // eight independent scans
+                    const unsigned int o = __shfl_up_sync(0xffffffffu, v[q], off);
+                    if (lane >= off) v[q] = max(v[q], o);
+                }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const unsigned int top = __shfl_sync(0xffffffffu, v[q], 31);
+                if (t0 + 32 * q + lane < e) keys[(size_t)r * ldk + t0 + 32 * q + lane] = max(v[q], carry);
+                carry = max(carry, top);
             }
-            rem -= acc;
         }
-        s->prefix |= ((unsigned int)dgt) << shift;
-        s->remaining = rem;
+        if (segs > 1 && lane == 0) sh.segmax[u] = carry;
     }
     __syncthreads();
-    if (threadIdx.x < 256) s->hist[threadIdx.x] = 0;
-}
-
-// per row: how many keys are below T, how many equal T          one block per row
-__global__ void __launch_bounds__(SEL_THREADS) select_count_kernel(const unsigned int* __restrict__ keys, int d,
-                                                                   const SelectState* s, int* __restrict__ lt,
-                                                                   int* __restrict__ eq) {
-    __shared__ int sl[SEL_THREADS], se[SEL_THREADS];
-    const unsigned int T = s->prefix;
-    const unsigned int* K = keys + (size_t)blockIdx.x * d;
-    int l = 0, e = 0;
-    for (int t = threadIdx.x; t < d; t += SEL_THREADS) { const unsigned int k = K[t]; l += k < T; e += k == T; }
-    sl[threadIdx.x] = l; se[threadIdx.x] = e;
+    // ---- the key of rank k, 9 + 11 + 11 bits
+    unsigned int prefix = 0u;
+    if (k > 0) {
+#pragma unroll 1
+        for (int pass = 0; pass < 3; ++pass) {
+            const int shift = pass == 0 ? 22 : (pass == 1 ? 11 : 0);
+            constexpr unsigned int dmask = 2047u;
+            if (pass == 0) {
+                // whole rows; segments also receive the maximum of what is before them
+                for (int u = warp; u < units; u += SEL_WARPS) {
+                    const int r = u / segs, g = u - r * segs;
+                    unsigned int* K = keys + (size_t)r * ldk;
+                    unsigned int carry = 0u;
+                    for (int q = 0; q < g; ++q) carry = max(carry, sh.segmax[r * segs + q]);
+                    const int e = min(d, (g + 1) * seg_len);
+                    auto change = [&](unsigned int key, unsigned int next, int t) {      // t < d
+                        const unsigned int f = key >> 22, fn = next >> 22;
+                        if (t + 1 == d) atomicAdd(&sh.hist[f], (unsigned int)d);
+                        else if (f != fn) {
+                            atomicAdd(&sh.hist[f], (unsigned int)(t + 1));
+                            atomicAdd(&sh.hist[fn], 0u - (unsigned int)(t + 1));
+                        }
+                    };
+                    if (IN_SMEM) {
+                        for (int t = g * seg_len + 4 * lane; t < e; t += 128) {
+                            uint4 x = *reinterpret_cast<uint4*>(K + t);
+                            unsigned int y = t + 4 < d ? K[t + 4] : 0u;
+                            if (g > 0) {
+                                x.x = max(x.x, carry); x.y = max(x.y, carry); x.z = max(x.z, carry); x.w = max(x.w, carry);
+                                *reinterpret_cast<uint4*>(K + t) = x;
+                            }
+                            const int left = min(4, d - t);
+                            // (y may be another segment's: at least this segment's last key)
+                            y = max(y, left == 4 ? x.w : 0u);
+                            if ((left == 4 && t + 4 < d) && ((x.x ^ y) >> 22) == 0u) continue;      // no change: the usual case
+                            change(x.x, x.y, t);
+                            if (left > 1) change(x.y, x.z, t + 1);
+                            if (left > 2) change(x.z, x.w, t + 2);
+                            if (left > 3) change(x.w, y, t + 3);
+                        }
+                    } else {
+                        for (int t = g * seg_len + lane; t < e; t += 32) {
+                            const unsigned int x = max(K[t], carry);
+                            const unsigned int y = t + 1 < d ? max(K[t + 1], x) : 0u;
+                            if (g > 0) K[t] = x;
+                            change(x, y, t);
+                        }
+                    }
+                }
+            } else {
+                for (int u = warp; u < nr; u += SEL_WARPS) {      // what is left of a row is short: one warp per row
+                    const unsigned int* K = keys + (size_t)u * ldk;
+                    const int b = row_lt[u], e = row_le[u];
+                    for (int t = b + lane; t < e; t += 32) {
+                        const int f = (int)((K[t] >> shift) & dmask);
+                        const int fn = t + 1 < e ? (int)((K[t + 1] >> shift) & dmask) : -1;
+                        if (t == b && b > 0) atomicAdd(&sh.hist[f], 0u - (unsigned int)b);
+                        if (f != fn) {
+                            atomicAdd(&sh.hist[f], (unsigned int)(t + 1));
+                            if (fn >= 0) atomicAdd(&sh.hist[fn], 0u - (unsigned int)(t + 1));
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            unsigned int a = sh.hist[2 * tid], b = sh.hist[2 * tid + 1];
+            if (G > 1) {
+                if (a) atomicAdd(&st->hist[pass][2 * tid], a);
+                if (b) atomicAdd(&st->hist[pass][2 * tid + 1], b);
+                if (!grid_barrier(&st->arrived, G * ++barrier_no)) {      // cannot happen in a cooperative launch; reported, not hidden
+                    for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = -1;
+                    return;
+                }
+                const uint2 v = __ldcg(reinterpret_cast<const uint2*>(st->hist[pass]) + tid);
+                a = v.x; b = v.y;
+            }
+            sh.hist[2 * tid] = 0u; sh.hist[2 * tid + 1] = 0u;
+            pick_digit(a, b, sh);
+            prefix |= sh.digit << shift;
+            // narrow every row to the keys that share the prefix: one thread per row, both ends in one loop
+            for (int r = tid; r < nr; r += SEL_THREADS) {
+                const unsigned int* K = keys + (size_t)r * ldk;
+                const unsigned int want = prefix >> shift;
+                int lo0 = row_lt[r], hi0 = row_le[r], lo1 = lo0, hi1 = hi0;
+                while (lo0 < hi0 || lo1 < hi1) {
+                    if (lo0 < hi0) { const int m = (lo0 + hi0) >> 1; if ((K[m] >> shift) < want) lo0 = m + 1; else hi0 = m; }
+                    if (lo1 < hi1) { const int m = (lo1 + hi1) >> 1; if ((K[m] >> shift) <= want) lo1 = m + 1; else hi1 = m; }
+                }
+                row_lt[r] = lo0; row_le[r] = lo1;
+            }
+            __syncthreads();
+        }
+    }
+    const Count rem = sh.rem;                             // of the keys equal to the k-th, this many are taken, in row order
+    const bool all_ties = k == 0 || rem == (Count)sh.digit_count;
+    // ---- counts; ties are handed out by row (only when not all of them are taken)
+    if (tid == 0) sh.before = 0;
+    if (!all_ties && G > 1) {
+        Count mine = 0;
+        for (int r = tid; r < nr; r += SEL_THREADS) mine += (Count)(row_le[r] - row_lt[r]);
+        const Count total = block_scan(mine, sh);
+        if (tid == SEL_THREADS - 1) st->ties[blockIdx.x] = total;
+        if (!grid_barrier(&st->arrived, G * ++barrier_no)) {
+            for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = -1;
+            return;
+        }
+        Count b = 0;
+        for (int q = tid; q < (int)blockIdx.x; q += SEL_THREADS) b += (Count)__ldcg(st->ties + q);
+        const Count lower = block_scan(b, sh);
+        if (tid == SEL_THREADS - 1) sh.before = lower;
+    }
     __syncthreads();
-    for (int off = SEL_THREADS / 2; off; off >>= 1) {
-        if (threadIdx.x < off) { sl[threadIdx.x] += sl[threadIdx.x + off]; se[threadIdx.x] += se[threadIdx.x + off]; }
+    for (int q = 0; q < nr; q += SEL_THREADS) {
+        const int r = q + tid;
+        int take = r < nr ? row_le[r] - row_lt[r] : 0;
+        if (!all_ties) {
+            const Count incl = block_scan((Count)take, sh), before = sh.before;
+            const Count first = before + incl - (Count)take;      // equal keys in rows before this one
+            const Count left = rem > first ? rem - first : 0;
+            if (left < (Count)take) take = (int)left;
+            __syncthreads();
+            if (tid == SEL_THREADS - 1) sh.before = before + incl;
+            __syncthreads();
+        }
+        if (r < nr) {
+            const int n = row_lt[r] + take;
+            row_lt[r] = n;
+            counts[r0 + r] = n;
+        }
+    }
+    __syncthreads();
+    // ---- mask: 1, then 0 at the first counts[r] entries of the row's order
+    const size_t bytes = (size_t)nr * d;
+    uint8_t* M = mask + (size_t)r0 * d;
+    if (IN_SMEM) {                                        // built where the keys were, written out in 16-byte pieces
+        const int skew = (int)(reinterpret_cast<uintptr_t>(M) & 15u);
+        uint8_t* S = reinterpret_cast<uint8_t*>(skeys) + skew;
+        uint4* S4 = reinterpret_cast<uint4*>(skeys);
+        const int n16 = (int)((bytes + skew + 15) >> 4);
+        for (int q = tid; q < n16; q += SEL_THREADS) S4[q] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
         __syncthreads();
-    }
-    if (threadIdx.x == 0) { lt[blockIdx.x] = sl[0]; eq[blockIdx.x] = se[0]; }
-}
-
-// hand the `remaining` entries with key == T to the rows in row order      single block
-__global__ void __launch_bounds__(SEL_THREADS) select_ties_kernel(const SelectState* s, const int* __restrict__ lt,
-                                                                  const int* __restrict__ eq, int rows,
-                                                                  int* __restrict__ counts) {
-    __shared__ unsigned long long part[SEL_THREADS];
-    const int tid = threadIdx.x;
-    const int chunk = (rows + SEL_THREADS - 1) / SEL_THREADS;
-    const int b = tid * chunk, e = min(rows, b + chunk);
-    unsigned long long sum = 0;
-    for (int r = b; r < e; ++r) sum += (unsigned long long)eq[r];
-    part[tid] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        unsigned long long acc = 0;
-        for (int i = 0; i < SEL_THREADS; ++i) { const unsigned long long c = part[i]; part[i] = acc; acc += c; }
-    }
-    __syncthreads();
-    unsigned long long before = part[tid];
-    const unsigned long long rem = s->remaining;
-    for (int r = b; r < e; ++r) {
-        const unsigned long long c = (unsigned long long)eq[r];
-        unsigned long long take = rem > before ? rem - before : 0ull;
-        if (take > c) take = c;
-        counts[r] = lt[r] + (int)take;
-        before += c;
-    }
-}
-
-// mask[r][:] = 1, then 0 at the first counts[r] entries of the row's order     one block per row
-__global__ void __launch_bounds__(SEL_THREADS) mask_kernel(const int32_t* __restrict__ order, const int* __restrict__ counts,
-                                                           int d, uint8_t* __restrict__ mask) {
-    const int r = blockIdx.x;
-    uint8_t* M = mask + (size_t)r * d;
-    for (int j = threadIdx.x; j < d; j += SEL_THREADS) M[j] = 1;
-    __syncthreads();
-    const int c = min(counts[r], d);
-    for (int t = threadIdx.x; t < c; t += SEL_THREADS) {
-        const int j = order[(size_t)r * d + t];
-        if (j >= 0 && j < d) M[j] = 0;
+        for (int u = warp; u < units; u += SEL_WARPS) {
+            const int r = u / segs, g = u - r * segs;
+            const int e = min(row_lt[r], (g + 1) * seg_len);
+            const int32_t* P = order + (size_t)(r0 + r) * d;
+            for (int t = g * seg_len + lane; t < e; t += 256) {      // eight loads in flight per lane
+                int j[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) j[q] = t + 32 * q < e ? __ldg(P + t + 32 * q) : -1;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) if (j[q] >= 0 && j[q] < d) S[(size_t)r * d + j[q]] = 0;
+            }
+        }
+        __syncthreads();
+        uint8_t* base = M - skew;
+        for (int q = tid; q < n16; q += SEL_THREADS) {
+            const int lo = 16 * q, hi = lo + 16;
+            if (lo >= skew && (size_t)hi <= bytes + skew) *reinterpret_cast<uint4*>(base + lo) = S4[q];
+            else
+                for (int x = max(lo, skew); x < hi && (size_t)x < bytes + skew; ++x) base[x] = reinterpret_cast<uint8_t*>(skeys)[x];
+        }
+    } else {
+        for (size_t x = tid; x < bytes; x += SEL_THREADS) M[x] = 1;
+        __syncthreads();
+        for (int u = warp; u < units; u += SEL_WARPS) {
+            const int r = u / segs, g = u - r * segs;
+            const int e = min(row_lt[r], (g + 1) * seg_len);
+            for (int t = g * seg_len + lane; t < e; t += 32) {
+                const int j = order[(size_t)(r0 + r) * d + t];
+                if (j >= 0 && j < d) M[(size_t)r * d + j] = 0;
+            }
+        }
     }
 }
 
@@ -161,35 +325,40 @@ size_t select_workspace_bytes(int rows, int d) {
 
 obc_status select_launch(const float* loss, const int32_t* order, int rows, int d, int64_t k, int32_t* counts,
                          uint8_t* mask, void* ws, cudaStream_t stream) {
+    DeviceInfo di;
+    const obc_status ds = device_info(&di);
+    if (ds != OBC_OK) return ds;
     char* p = reinterpret_cast<char*>(ws);
-    unsigned int* keys = reinterpret_cast<unsigned int*>(p); p += round_up((size_t)rows * d * 4, 256);
+    unsigned int* gkeys = reinterpret_cast<unsigned int*>(p); p += round_up((size_t)rows * d * 4, 256);
     SelectState* st = reinterpret_cast<SelectState*>(p); p += round_up(sizeof(SelectState), 256);
-    int* lt = reinterpret_cast<int*>(p); p += round_up((size_t)rows * 4, 256);
-    int* eq = reinterpret_cast<int*>(p);
-    const long long n = (long long)rows * d;
-    prefix_max_kernel<<<rows, SEL_THREADS, 0, stream>>>(loss, d, keys);
+    int* glt = reinterpret_cast<int*>(p); p += round_up((size_t)rows * 4, 256);
+    int* gle = reinterpret_cast<int*>(p);
+    // Blocks: one SM each, at least SEL_BLOCK_KEYS keys a block -- below that the barriers of a further block cost more than
+    // its share of the scans saves -- and a single block (no barriers at all) up to SEL_ONE_BLOCK_KEYS.
+    constexpr int64_t SEL_BLOCK_KEYS = 4096, SEL_ONE_BLOCK_KEYS = 12288;
+    const int64_t n = (int64_t)rows * d;
+    int64_t blocks = n <= SEL_ONE_BLOCK_KEYS ? 1 : (n + SEL_BLOCK_KEYS - 1) / SEL_BLOCK_KEYS;
+    const int most = di.sm_count < SEL_MAX_BLOCKS ? di.sm_count : SEL_MAX_BLOCKS;
+    if (blocks > most) blocks = most;
+    if (blocks > rows) blocks = rows;
+    int rpb = (int)((rows + blocks - 1) / blocks);
+    const int grid = (rows + rpb - 1) / rpb;
+    int segs = rpb >= 2 * SEL_WARPS ? 1 : 2 * SEL_WARPS / rpb;       // about two segments per warp, of 256 keys or more
+    while (segs > 1 && d / segs < 256) --segs;
+    const size_t key_bytes = (size_t)rpb * ((d + 3) & ~3) * 4 + 32;        // (the mask is built in the same space, shifted by up to 15 bytes)
+    const bool in_smem = key_bytes <= (size_t)SEL_SMEM && n < (1ll << 32);
+    unsigned long long kk = (unsigned long long)k;
+    if (grid > 1) OBC_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(SelectState), stream));
+    void* args[] = {&loss, &order, &rows, &d, &kk, &rpb, &segs, &gkeys, &glt, &gle, &st, &counts, &mask};
+    const void* kernel = in_smem ? (const void*)select_kernel<true, unsigned int>
+                                 : (n < (1ll << 32) ? (const void*)select_kernel<false, unsigned int> : (const void*)select_kernel<false, unsigned long long>);
+    const size_t smem = in_smem ? key_bytes : 0;
+    if (in_smem) OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
+    if (grid > 1) OBC_CUDA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(SEL_THREADS), args, smem, stream));
+    else OBC_CUDA_TRY(cudaLaunchKernel(kernel, dim3(1), dim3(SEL_THREADS), args, smem, stream));
     count_launch();
-    select_init_kernel<<<1, 256, 0, stream>>>(st, (long long)k);
-    count_launch();
-    int hb = (int)((n + SEL_THREADS * 8 - 1) / (SEL_THREADS * 8));
-    if (hb > 1184) hb = 1184;
-    if (hb < 1) hb = 1;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        select_hist_kernel<<<hb, SEL_THREADS, 0, stream>>>(keys, n, shift, st);
-        count_launch();
-        select_pick_kernel<<<1, 256, 0, stream>>>(st, shift);
-        count_launch();
-    }
-    select_count_kernel<<<rows, SEL_THREADS, 0, stream>>>(keys, d, st, lt, eq);
-    count_launch();
-    select_ties_kernel<<<1, SEL_THREADS, 0, stream>>>(st, lt, eq, rows, counts);
-    count_launch();
-    mask_kernel<<<rows, SEL_THREADS, 0, stream>>>(order, counts, d, mask);
-    count_launch();
-    OBC_CUDA_TRY(cudaGetLastError());
     return OBC_OK;
 }
-
 // ---- allocation-free variant ----------------------------------------------------------------------------------
 // Scratch for obc_select_global_mask_static: a fixed array in device memory that every GPU loading this library
 // holds until the process exits.  Sized for OBC_SELECT_STATIC_MAX_KEYS loss entries and
