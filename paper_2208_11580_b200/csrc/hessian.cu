@@ -8,15 +8,12 @@
 //
 // This file holds the FP32 CUDA-core path (OBC_PREC_FP32), the slice/finalize machinery, and the dispatch
 // to the tensor-core paths.
-#include "common.cuh"
+#include "gemm_fp32.cuh"
 
 namespace obc {
 
-constexpr int HT = 128;           // output tile
-constexpr int HK = 16;            // k chunk
-
 int hessian_splits(int d, int64_t n) {
-    const int T = (d + HT - 1) / HT;
+    const int T = (d + 127) / 128;
     const int ntiles = T * (T + 1) / 2;
     int64_t s = (444 + ntiles - 1) / ntiles;
     const int64_t by_len = (n + 2047) / 2048;      // short accumulation chains: partial sums are combined in FP32 RN
@@ -27,77 +24,44 @@ int hessian_splits(int d, int64_t n) {
     return (int)s;
 }
 
+// FP32 path: tile and slices.  64 x 64 tiles (four blocks per SM) waste less on the diagonal and on ragged edges;
+// 128 x 128 tiles (two blocks per SM) halve the traffic from L2, which matters once the padding no longer does.
+static bool fp32_small_tile(int d) { return d <= 640; }
+static int fp32_splits(int d, int64_t n) {
+    const int tile = fp32_small_tile(d) ? 64 : 128;
+    const int64_t T = (d + tile - 1) / tile, ntiles = T * (T + 1) / 2;
+    const int64_t resident = 148 * (tile == 64 ? F32<64>::BLOCKS : F32<128>::BLOCKS);
+    int64_t s = resident / ntiles;                                      // one full wave ...
+    const int64_t by_len = (n + 2047) / 2048;                           // ... or chains of at most 2048 products
+    if (by_len > s) s = (by_len * ntiles + resident - 1) / resident * resident / ntiles;      // (whole waves)
+    if (s * 128 > n) s = n / 128;                                       // slices of 128 or more
+    if (s > 512) s = 512;
+    return s < 1 ? 1 : (int)s;
+}
+
 size_t hessian_tc_extra_bytes(int d, int64_t n);
 
 size_t hessian_workspace_bytes(int d, int64_t n) {      // partial sums + what the tensor-core paths add
-    return round_up((size_t)hessian_splits(d, n) * d * d * sizeof(float), 256) + hessian_tc_extra_bytes(d, n);
+    const size_t tc = round_up((size_t)hessian_splits(d, n) * d * d * sizeof(float), 256) + hessian_tc_extra_bytes(d, n);
+    const size_t fp32 = round_up((size_t)fp32_splits(d, n) * d * d * sizeof(float), 256);
+    return tc > fp32 ? tc : fp32;
 }
 
 // partial[z][i][j] = sum_{k in slice z} X[i][k] X[j][k]   for tiles with bj <= bi
-__global__ void __launch_bounds__(256) syrk_fp32_kernel(const float* __restrict__ X, int d, int64_t n, int64_t ldx,
-                                                        int64_t slice, float* __restrict__ partial) {
-    // blockIdx.x enumerates lower-triangular tile pairs
-    int bi = 0, t = blockIdx.x;
+template <int TILE>
+__global__ void __launch_bounds__(F32<TILE>::THREADS, F32<TILE>::BLOCKS) syrk_fp32_kernel(const float* __restrict__ X, int d, int64_t n,
+                                                                                            int64_t ldx, int64_t slice, float* __restrict__ partial) {
+    extern __shared__ __align__(16) float fsm[];
+    int bi = 0, t = blockIdx.x;                            // lower-triangular tile pairs
     while (t > bi) { t -= bi + 1; ++bi; }
     const int bj = t;
     const int64_t kb = (int64_t)blockIdx.y * slice;
     const int64_t ke = kb + slice < n ? kb + slice : n;
-    __shared__ __align__(16) float As[HK][HT + 4];
-    __shared__ __align__(16) float Bs[HK][HT + 4];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    float acc[8][8] = {};
-    const bool vec_ok = (ldx % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0) && (kb % 4 == 0);
-    for (int64_t k0 = kb; k0 < ke; k0 += HK) {
-#pragma unroll
-        for (int rep = 0; rep < 2; ++rep) {
-            const int q = tid + rep * 256;
-            const int row = q >> 2, kq = (q & 3) * 4;
-            const int64_t k = k0 + kq;
-#pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                const int gi = (which ? bj : bi) * HT + row;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (gi < d) {
-                    const float* src = X + (size_t)gi * ldx + k;
-                    if (vec_ok && k + 3 < ke) v = *reinterpret_cast<const float4*>(src);
-                    else {
-                        if (k + 0 < ke) v.x = src[0];
-                        if (k + 1 < ke) v.y = src[1];
-                        if (k + 2 < ke) v.z = src[2];
-                        if (k + 3 < ke) v.w = src[3];
-                    }
-                }
-                float(*S)[HT + 4] = which ? Bs : As;
-                S[kq + 0][row] = v.x; S[kq + 1][row] = v.y; S[kq + 2][row] = v.z; S[kq + 3][row] = v.w;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < HK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
     float* P = partial + (size_t)blockIdx.y * d * d;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int gi = bi * HT + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
-        if (gi >= d) continue;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int gj = bj * HT + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
-            if (gj < d) P[(size_t)gi * d + gj] = acc[i][j];
-        }
-    }
+    f32_tile_product<TILE, true>(fsm, X, ldx, d, bi * TILE, X, ldx, d, bj * TILE, kb, ke, [&](int i, int j, float v) {
+        const int gi = bi * TILE + i, gj = bj * TILE + j;
+        if (gi < d && gj <= gi) P[(size_t)gi * d + gj] = v;
+    });
 }
 
 // H[i][j] = H[j][i] = (accumulate ? H[i][j] : 0) + 2 * sum_z partial[z][i][j]     for j <= i
@@ -111,7 +75,14 @@ __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __re
     if (info && i == 0 && j == 0) info[0] = (err && *err != 0) ? (int32_t)OBC_ERR_TIMEOUT : 0;
     if (j > i || j >= d) return;
     float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += partial[(size_t)z * d * d + (size_t)i * d + j];
+    const float* P = partial + (size_t)i * d + j;
+    for (int z0 = 0; z0 < splits; z0 += 16) {             // sixteen loads in flight, added in order
+        float v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = z0 + q < splits ? P[(size_t)(z0 + q) * d * d] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) s += v[q];
+    }
     float v = 2.f * s;
     if (accumulate) v += H[(size_t)i * ldh + j];
     if (err && *err != 0) v = __int_as_float(0x7fc00000);
@@ -130,13 +101,20 @@ obc_status hessian_finalize_launch(const float* partial, int splits, int d, floa
 
 obc_status hessian_fp32_launch(const float* X, int d, int64_t n, int64_t ldx, float* H, int ldh, int accumulate,
                                int32_t* info, void* ws, cudaStream_t stream) {
-    const int splits = hessian_splits(d, n);
+    const int splits = fp32_splits(d, n);
     int64_t slice = (n + splits - 1) / splits;
-    slice = (slice + HK - 1) / HK * HK;
-    const int T = (d + HT - 1) / HT;
+    slice = (slice + 31) / 32 * 32;
+    const int tile = fp32_small_tile(d) ? 64 : 128;
+    const int T = (d + tile - 1) / tile;
     dim3 grid(T * (T + 1) / 2, splits);
     float* partial = reinterpret_cast<float*>(ws);
-    syrk_fp32_kernel<<<grid, 256, 0, stream>>>(X, d, n, ldx, slice, partial);
+    if (tile == 64) {
+        OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_fp32_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32<64>::SMEM));
+        syrk_fp32_kernel<64><<<grid, F32<64>::THREADS, F32<64>::SMEM, stream>>>(X, d, n, ldx, slice, partial);
+    } else {
+        OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_fp32_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32<128>::SMEM));
+        syrk_fp32_kernel<128><<<grid, F32<128>::THREADS, F32<128>::SMEM, stream>>>(X, d, n, ldx, slice, partial);
+    }
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
     return hessian_finalize_launch(partial, splits, d, H, ldh, accumulate, nullptr, info, stream);
