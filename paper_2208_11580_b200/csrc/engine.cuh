@@ -4,6 +4,7 @@
 // row_engine_blocked.cu the engine that defers the Lemma-1 updates and applies them several at a time.
 #pragma once
 #include "common.cuh"
+#include <cuda_fp16.h>
 #include <math_constants.h>
 
 namespace obc {
@@ -30,6 +31,8 @@ struct EngineArgs {
                                           // 2^nm_lg consecutive columns (nm_prune = 0: no pattern)
     uint8_t* mask;                        // blocked engine, nullable: d_row x d mask, 0 at eliminated columns
     int block_c;                          // blocked engine: 4 = block pruning in blocks of 4 columns (Eq. 5), 0 = off
+    __half* Zws; int zld;                 // blocked engine: FP16 planes of the pending vectors, 128 rows of zld per block
+    signed char* zexp;                    // blocked engine: powers of two of the slots (cap per block; wide diagonals)
     float* Gpan; int g_vectors; int g_ld; // blocked engine: overflow pending vectors in global memory (per block
                                           // g_vectors rows of g_ld floats), nullptr = none
     int split;                            // blocked engine: rows are shared out in equal work per block, a row may be
@@ -73,6 +76,7 @@ __device__ __forceinline__ double grid_q_fast(double x, double sc, double isc, d
 // Launchers of the two engines (same arguments; each checks its own workspace need).
 size_t streaming_engine_workspace_bytes(int row_count, int d, const DeviceInfo& di);
 size_t blocked_engine_workspace_bytes(int row_count, int d, const DeviceInfo& di);
+size_t blk_plane_bytes(int blocks, int cap);       // blocked engine: operand planes of the pending vectors
 obc_status streaming_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaStream_t stream);
 obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaStream_t stream);
 

@@ -16,7 +16,7 @@
 // products it has issued, frees its tensor memory and returns; the finalize kernel then fills H with NaN and writes
 // OBC_ERR_TIMEOUT to the caller's info word, so that the failure cannot go unnoticed downstream.
 #include "common.cuh"
-#include <cuda.h>
+#include "tensor_map.cuh"
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <mutex>
@@ -307,6 +307,18 @@ static bool make_map(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes,
     cuuint32_t box[2] = {(cuuint32_t)(TC_KBYTES / elem_bytes), (cuuint32_t)TC_TILE};
     cuuint32_t estr[2] = {1, 1};
     return fn(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, int64_t inner, int64_t rows,
+                        int64_t planes, int box_inner, int box_rows, int box_planes) {
+    PFN_cuTensorMapEncodeTiled fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)planes};
+    cuuint64_t strides[2] = {(cuuint64_t)inner * elem_bytes, (cuuint64_t)inner * rows * elem_bytes};
+    cuuint32_t box[3] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, type, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
