@@ -1,12 +1,13 @@
 // The rank-B update of the blocked row engine for long rows on the 5th-generation tensor cores: H -= sum_b z_b z_b^T over the
-// compacted lower triangle of one row's private inverse Hessian (B <= 64 pending vectors), one 512-thread block per SM.
+// compacted lower triangle of one row's private inverse Hessian (B <= 48 pending vectors), one 512-thread block per SM.
 //
 // A pass reads and writes every element of the triangle once (8 bytes) and is bound by HBM, so everything but that traffic
 // is kept off the warps: TMA brings tiles of 128 rows x 64 columns of H into shared memory and takes them back,
 // tcgen05.mma (kind::f16) forms the tile's increment in tensor memory, and eight warps only subtract one from the other.
 // The products cost nothing beside the traffic, so a pass takes as many pending vectors as tensor memory holds partial sums
 // for; most of them wait in L2 (the mma.sync form spent half of a warp's time multiplying, so more vectors per pass bought it
-// little).  During a pass the space of the FP32 pending vectors is free and holds the tiles and operands.
+// little).  48 of them, not the 64 that four groups would allow: the steps between two passes read them all, and from
+// there on that costs as much as the rarer passes save (768 x 3072: 285 against 300 ms; 128 x 4608: 156 against 161 ms).  During a pass the space of the FP32 pending vectors is free and holds the tiles and operands.
 //
 // Operands.  Before the pass every pending vector is written as two FP16 planes, z * 2^e = hi + lo (hi rounded to 11 bits, lo
 // the rounded rest: 22 significant bits), to global memory (they stay in L2).  The power of two takes the largest entry to
@@ -30,15 +31,15 @@
 namespace obc {
 
 constexpr int FT_M = 128, FT_N = 64;              // tile
-constexpr int FT_GMAX = 4;                        // groups of 16 pending vectors: two tiles' accumulators in 512 columns
+constexpr int FT_GMAX = 3;                        // groups of 16 pending vectors (two tiles' accumulators in tensor memory)
 constexpr int FT_COLS = 512;
-constexpr int FT_EW = 8;                          // warps that subtract: 32 rows x 32 columns each; three more issue
+constexpr int FT_EW = 8;                          // warps that subtract: 32 rows x 32 columns each; four more issue
 constexpr int FT_WAIT_LIMIT = 1 << 22;            // polls before a wait gives up
 constexpr int FT_GROUP_BYTES = 16 * 128;          // one plane of 16 vectors x 64 slots of FP16
 constexpr int FT_TILE_BYTES = FT_M * FT_N * 4;
 
 // Tensor maps: the planes (slots, 64 vectors, hi / lo of every block) by groups of 16 vectors in the copied box, and the
-// private triangles (columns, rows, buffer) in boxes of 32 columns x 128 or 32 rows.
+// private triangles (32 columns, rows, column groups of all buffers) in boxes of a whole tile and of 32 columns x 32 rows.
 struct FlushMaps { CUtensorMap z[FT_GMAX]; CUtensorMap h128, h32; };
 
 struct FlushBars {                                // in shared memory; the barriers are re-initialised before every pass
@@ -187,35 +188,35 @@ struct Ring {
 struct FlushGeom {                                // of a pass
     const FlushMaps* maps; int plane, buf, G, T, m1; FlushBufs nb; uint32_t sa, sb, sh, tmem;
 };
-// The parts of tile (rb, c) that hold data, each as f(map, 32-column group, first row inside the tile): the whole column
-// group below the diagonal, on it only the 32 x 32 parts that reach it.
+// The parts of tile (rb, c) that hold data, each as f(map, 32-column group, first row inside the tile): the whole tile
+// below the diagonal, on it the 32 x 32 parts that reach it.
 template <typename F>
 __device__ __forceinline__ void ft_parts(const FlushGeom& q, int rb, int c, F f) {
+    if (c < rb * FT_M) f(&q.maps->h128, 0, 0);
+    else {
 #pragma unroll
-    for (int cg = 0; cg < FT_N / 32; ++cg) {
-        const int col = c + 32 * cg;
-        if (col + 32 <= rb * FT_M) f(&q.maps->h128, cg, 0);
-        else
+        for (int cg = 0; cg < FT_N / 32; ++cg)
             for (int r = 0; r < FT_M; r += 32)
-                if (col <= rb * FT_M + r && rb * FT_M + r < q.m1) f(&q.maps->h32, cg, r);
+                if (c + 32 * cg <= rb * FT_M + r && rb * FT_M + r < q.m1) f(&q.maps->h32, cg, r);
     }
 }
-// Copies of the tile at (rb, c): H, the vectors at its columns and, first tile of a row block, at its rows.  One thread.
-__device__ __forceinline__ bool ft_copy(const FlushGeom& q, FlushBars* fb, Ring& h, Ring& b, Ring& a, int rb, int c, uint64_t pol) {
-    const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;    // both planes of 64 slots
+// Copies of the tile of H at (rb, c).  One thread.
+__device__ __forceinline__ bool ft_copy_tile(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
     if (h.round > 0 && !ft_wait(&fb->free_h[h.at], (h.round - 1) & 1, fb)) return false;
-    uint32_t bytes = 0;
-    ft_parts(q, rb, c, [&](const CUtensorMap* m, int, int) { bytes += m == &q.maps->h128 ? 128 * 128 : 32 * 128; });
+    uint32_t bytes = FT_TILE_BYTES;
+    if (c >= rb * FT_M) { bytes = 0; ft_parts(q, rb, c, [&](const CUtensorMap*, int, int) { bytes += 32 * 128; }); }
     ft_expect(&fb->full_h[h.at], bytes);
     ft_parts(q, rb, c, [&](const CUtensorMap* m, int cg, int r) {
-        ft_load_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, &fb->full_h[h.at], c + 32 * cg, rb * FT_M + r, q.buf, pol);
+        ft_load_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, &fb->full_h[h.at], 0, rb * FT_M + r, q.buf + (c >> 5) + cg, pol);
     });
     h.next(q.nb.n_h);
+    return true;
+}
+// Copies of the vectors at the tile's columns and, first tile of a row block, at its rows.  One thread (another one: the
+// operands run ahead of the tiles, whose buffers are held until they are back in memory).
+__device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* fb, Ring& b, Ring& a, int rb, int c) {
+    const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;    // both planes of 64 slots
     const CUtensorMap* zm = &q.maps->z[q.G - 1];
-    if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
-    ft_expect(&fb->full_b[b.at], blk);
-    ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
-    b.next(q.nb.n_b);
     if (c == 0) {
         if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb)) return false;
         ft_expect(&fb->full_a[a.at], 2 * blk);
@@ -223,6 +224,10 @@ __device__ __forceinline__ bool ft_copy(const FlushGeom& q, FlushBars* fb, Ring&
         ft_load(q.sa + (a.at * 2 + 1) * blk, zm, &fb->full_a[a.at], rb * FT_M + 64, 0, q.plane);
         a.next(q.nb.n_a);
     }
+    if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
+    ft_expect(&fb->full_b[b.at], blk);
+    ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
+    b.next(q.nb.n_b);
     return true;
 }
 // Products of tile t at (.., c); `last`: of its row block.  One thread.
@@ -260,7 +265,7 @@ __device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* 
 __device__ __forceinline__ bool ft_store(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
     if (!ft_wait(&fb->ready[h.at], h.round & 1, fb)) return false;
     ft_parts(q, rb, c, [&](const CUtensorMap* m, int cg, int r) {
-        ft_store_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, c + 32 * cg, rb * FT_M + r, q.buf, pol);
+        ft_store_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, 0, rb * FT_M + r, q.buf + (c >> 5) + cg, pol);
     });
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -320,7 +325,7 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
     return true;
 }
 
-// One pass over triangle `tri` (the maps' buffer index), already compacted to m1 rows.  Before it: the planes are in the new
+// One pass over the triangle whose first column group is `tri` in the maps, already compacted to m1 rows.  Before it: the planes are in the new
 // slot numbering and zero up to a multiple of 16 vectors, the barriers are initialised, plain accesses are fenced against
 // the copies, and the block has synchronised.
 //   plane     first of the block's two planes (hi, lo) in the maps
@@ -348,13 +353,21 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
     } else if (warp == FT_EW && lane == 0) {
         const uint64_t pol = ft_stream_policy();
         for (; t < q.T; ++t) {
-            if (!ft_copy(q, fb, h, b, a, rb, c, pol)) break;
+            if (!ft_copy_tile(q, fb, h, rb, c, pol)) break;
             ft_next_tile(rb, c, m1);
         }
         if (*(volatile int*)&fb->abort) {             // nothing may land after the block has moved on
-            const int nh = h.round * q.nb.n_h + h.at, nbb = b.round * q.nb.n_b + b.at, na = a.round * q.nb.n_a + a.at;
-            for (int x = max(0, nh - q.nb.n_h); x < nh; ++x) ft_drain(&fb->full_h[x % q.nb.n_h], (x / q.nb.n_h) & 1);
-            for (int x = max(0, nbb - q.nb.n_b); x < nbb; ++x) ft_drain(&fb->full_b[x % q.nb.n_b], (x / q.nb.n_b) & 1);
+            const int n = h.round * q.nb.n_h + h.at;
+            for (int x = max(0, n - q.nb.n_h); x < n; ++x) ft_drain(&fb->full_h[x % q.nb.n_h], (x / q.nb.n_h) & 1);
+        }
+    } else if (warp == FT_EW + 3 && lane == 0) {
+        for (; t < q.T; ++t) {
+            if (!ft_copy_operands(q, fb, b, a, rb, c)) break;
+            ft_next_tile(rb, c, m1);
+        }
+        if (*(volatile int*)&fb->abort) {
+            const int n = b.round * q.nb.n_b + b.at, na = a.round * q.nb.n_a + a.at;
+            for (int x = max(0, n - q.nb.n_b); x < n; ++x) ft_drain(&fb->full_b[x % q.nb.n_b], (x / q.nb.n_b) & 1);
             for (int x = max(0, na - q.nb.n_a); x < na; ++x) ft_drain(&fb->full_a[x % q.nb.n_a], (x / q.nb.n_a) & 1);
         }
     } else if (warp == FT_EW + 1 && lane == 0) {

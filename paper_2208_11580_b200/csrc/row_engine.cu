@@ -492,7 +492,7 @@ size_t engine_blocks_workspace_bytes(int row_count, int d, const DeviceInfo& di)
     const int cap = (d + 3) & ~3;
     int blocks = di.sm_count * 4;
     if (row_count > 0 && row_count < blocks) blocks = row_count;
-    const size_t tri = round_up((size_t)blocks * d * cap * sizeof(float), 256) + blk_plane_bytes(blocks < di.sm_count ? blocks : di.sm_count, cap);
+    const size_t tri = round_up((size_t)blocks * ((cap + 63) & ~63) * cap * sizeof(float), 256) + blk_plane_bytes(blocks < di.sm_count ? blocks : di.sm_count, cap);
     const size_t other = blocked_engine_workspace_bytes(row_count, d, di);
     return tri > other ? tri + 256 : other;
 }

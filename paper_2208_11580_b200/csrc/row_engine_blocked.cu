@@ -19,7 +19,9 @@ obc_status blk_launch_128(const FlushMaps& zmaps, const EngineArgs& a, int block
 obc_status blk_launch_256(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
 obc_status blk_launch_512(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
 
-constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)48 << 20;      // all blocks' overflow vectors together: well inside L2
+// All blocks' overflow vectors together: within L2.  (Only the longest rows reach the limit; 48 / 64 / 80 / 110 MB at 128 rows x
+// 4608: 249 / 220 / 202 / 181 ms.)
+constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)110 << 20;
 
 static int blk_pick_ms(int d, size_t panel_bytes) {
     int ms = d < 1024 ? d : 1024;
@@ -64,11 +66,9 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     p.smem = share;
     p.panel_floats = (int)((share - fixed) / 4);
     p.ms = blk_pick_ms(d, share - fixed);
-    // Very long rows (d_col > ~2600): shared memory holds fewer than 16 pending vectors, so a pass over the triangle
-    // applies few updates; further vectors go to a global buffer small enough to stay in L2 (the triangle itself is
-    // streamed past it with evict-first hints).  Measured at d_col = 3072: 99 -> 73 ms per wave of rows.  At 2304 (19
-    // vectors in shared memory) 16 more gain 2 % on one wave of rows and lose 2 % when rows are handed over between
-    // blocks (rows out of step with each other compete for L2), so it is not used there.
+    // Rows of one 512-thread block per SM: shared memory holds fewer pending vectors than a pass can apply (19 at d_col = 2304, 12
+    // at 3072, 6 at 4608); further ones go to a global buffer small enough to stay in L2 (the triangle itself is streamed past
+    // it with evict-first hints).
     p.g_ld = (cap + 15) & ~15;
     p.g_vectors = 0;
     p.max_pending = BLK_MAXB;
@@ -130,7 +130,7 @@ size_t blocked_engine_workspace_bytes(int row_count, int d, const DeviceInfo& di
     const bool may_split = row_count == 0 || row_count > di.sm_count;
     if (row_count > 0 && row_count < blocks) blocks = row_count;
     const int gblocks = blocks < di.sm_count ? blocks : di.sm_count;     // overflow vectors: one block per SM only
-    return round_up((size_t)blocks * (may_split ? 2 : 1) * d * cap * sizeof(float), 256) +
+    return round_up((size_t)blocks * (may_split ? 2 : 1) * tri_floats(cap) * sizeof(float), 256) +
            round_up((size_t)gblocks * BLK_MAXB * ((cap + 15) & ~15) * sizeof(float), 256) + blk_plane_bytes(gblocks, cap) +
            (may_split ? round_up((size_t)blocks * blk_split_stride(cap), 256) + round_up((size_t)blocks * sizeof(int), 256) : 0);
 }
@@ -188,7 +188,7 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
         // gain, 79.9 -> 70.9 ms, 5.7 waves of 1152-column rows do not).
         const bool want_split = a.row_count > blocks && a.row_count % blocks != 0 && (p.per_sm == 1 || a.row_count < 3 * blocks) &&
                                 a.nm_prune == 0 && !bc && !(a.opts.flags & OBC_ENGINE_WHOLE_WAVES);
-        const size_t tri = round_up((size_t)blocks * (want_split ? 2 : 1) * a.d * a.cap * sizeof(float), 256);
+        const size_t tri = round_up((size_t)blocks * (want_split ? 2 : 1) * tri_floats(a.cap) * sizeof(float), 256);
         const size_t gpan = p.g_vectors ? round_up((size_t)blocks * p.g_vectors * p.g_ld * sizeof(float), 256) : 0;
         const size_t sst = want_split ? round_up((size_t)blocks * blk_split_stride(a.cap), 256) : 0;
         const size_t sfl = want_split ? round_up((size_t)blocks * sizeof(int), 256) : 0;
@@ -198,12 +198,12 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
         if (planes) {
             a.Zws = reinterpret_cast<__half*>(reinterpret_cast<char*>(ws) + tri + gpan);
             a.zexp = reinterpret_cast<signed char*>(a.Zws) + round_up((size_t)blocks * 128 * a.zld * sizeof(__half), 256);
-            const int64_t tris = (int64_t)blocks * (want_split ? 2 : 1);
+            const int64_t groups = (int64_t)blocks * (want_split ? 2 : 1) * (((a.cap + 63) & ~63) >> 5);      // of 32 columns
             for (int k = 0; k < FT_GMAX; ++k)
                 if (!make_tensor_map_3d(&zmaps.z[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.Zws, a.zld, 64, 2 * (int64_t)blocks, 64, 16 * (k + 1), 2))
                     return OBC_ERR_CUDA;
-            if (!make_tensor_map_3d(&zmaps.h128, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.Hws, a.ldp, a.d, tris, 32, FT_M, 1) ||
-                !make_tensor_map_3d(&zmaps.h32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.Hws, a.ldp, a.d, tris, 32, 32, 1))
+            if (!make_tensor_map_3d(&zmaps.h128, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.Hws, 32, a.ldp, groups, 32, FT_M, 2) ||
+                !make_tensor_map_3d(&zmaps.h32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.Hws, 32, a.ldp, groups, 32, 32, 1))
                 return OBC_ERR_CUDA;
         }
         if (p.g_vectors) {

@@ -173,6 +173,12 @@ static __device__ __noinline__ void blk_state_copy(bool save, char* state, int c
     }
 }
 
+// Place of element (i, j), j <= i, of a private triangle: groups of 32 columns one after the other, rows of 128 bytes inside a
+// group (ld rows each).  A column is then one strip of consecutive lines instead of a line per row of the matrix, and a
+// 128-row tile of a group is contiguous.
+__host__ __device__ __forceinline__ int tri_at(int ld, int i, int j) { return ((j >> 5) * ld + i) * 32 + (j & 31); }
+__host__ __device__ inline size_t tri_floats(int cap) { return (size_t)((cap + 63) & ~63) * cap; }      // (an even number of groups)
+
 struct Records {                              // views into one record buffer
     unsigned* key; int* slot; int* orig; double* s; double* w; double* dgv;
 };
@@ -407,7 +413,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
         if (prg >= nrg) return;
         const int row = (prg << 4) + (lane >> 1), col = pc0 + ((lane & 1) << 5);       // 16 rows x 2 lines of 128 bytes
         if (row < m1 && col <= row)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + (size_t)srcm[row] * ldp + col));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at(ldp, srcm[row], col)));
         pc0 += 64;
         if (pc0 >= min((prg << 4) + 16, m1)) { pc0 = 0; prg += NW; }
     };
@@ -525,7 +531,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                     hv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
                     const int j = c0 + (u << 4) + (t << 2);
                     if (u < ngroups && in[h] && j <= rr[h]) {
-                        const float4* src = reinterpret_cast<const float4*>(Hp + (size_t)sr[h] * ldp + j);
+                        const float4* src = reinterpret_cast<const float4*>(Hp + tri_at(ldp, sr[h], j));
                         hv[u][h] = STREAM ? __ldcs(src) : *src;
                     }
                 }
@@ -544,7 +550,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 if (in[h] && jj <= rr[h]) {
-                                    const float val = Hp[(size_t)max(sr[h], sj) * ldp + min(sr[h], sj)];
+                                    const float val = Hp[tri_at(ldp, max(sr[h], sj), min(sr[h], sj))];
                                     if (comp == 0) hv[u][h].x = val; else if (comp == 1) hv[u][h].y = val;
                                     else if (comp == 2) hv[u][h].z = val; else hv[u][h].w = val;
                                 }
@@ -563,7 +569,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                             float4 o = hv[u][h];
                             o.x -= acc[2 * u][2 * h];     o.z -= acc[2 * u][2 * h + 1];
                             o.y -= acc[2 * u + 1][2 * h]; o.w -= acc[2 * u + 1][2 * h + 1];
-                            float4* dst = reinterpret_cast<float4*>(Hp + (size_t)rr[h] * ldp + j);
+                            float4* dst = reinterpret_cast<float4*>(Hp + tri_at(ldp, rr[h], j));
                             if (STREAM) __stcs(dst, o); else *dst = o;
                         }
                     }
@@ -666,10 +672,10 @@ __device__ __forceinline__ void blk_fill_holes(float* H, int ldp, int m1, int nh
             float v[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                if (q0 + q < nh) { const int sh = mv[q0 + q]; v[q] = __ldcg(H + (size_t)max(sh, sj) * ldp + min(sh, sj)); }
+                if (q0 + q < nh) { const int sh = mv[q0 + q]; v[q] = __ldcg(H + tri_at(ldp, max(sh, sj), min(sh, sj))); }
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                if (q0 + q < nh) { const int h = hl[q0 + q]; H[(size_t)max(h, j) * ldp + min(h, j)] = v[q]; }
+                if (q0 + q < nh) { const int h = hl[q0 + q]; H[tri_at(ldp, max(h, j), min(h, j))] = v[q]; }
         }
     }
 }
@@ -789,8 +795,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     float* S = tlr + msr;
     const int lds = ms + 1;
     const int ldp = a.ldp;
-    float* const Hp0 = a.Hws ? a.Hws + (size_t)blockIdx.x * d * a.ldp : nullptr;      // the block's own triangle
-#define HP (SH ? (a.Hws + (size_t)reinterpret_cast<const int*>(smem + BLK_OFF_SCHED)[2] * d * ldp) : Hp0)
+    float* const Hp0 = a.Hws ? a.Hws + (size_t)blockIdx.x * tri_floats(cap) : nullptr;      // the block's own triangle
+#define HP (SH ? (a.Hws + (size_t)reinterpret_cast<const int*>(smem + BLK_OFF_SCHED)[2] * tri_floats(cap)) : Hp0)
     // overflow of the pending vectors: gB more of them in global memory (sized to stay in L2), stride gld
     // (only the one-row-per-SM configuration uses it; the other kernels are built without that code)
     constexpr bool GP = GPV;
@@ -917,17 +923,18 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         if (kind != ITEM_TAIL && d > ms && total > 0) {
             for (int i = warp; i < d; i += NW) {
                 const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
-                float4* d4 = reinterpret_cast<float4*>(HP + (size_t)i * ldp);
+                float* dst = HP;
+                auto put = [&](int j4, float4 v) { *reinterpret_cast<float4*>(dst + tri_at(ldp, i, 4 * j4)) = v; };
                 const int n4 = (i >> 2) + 1;
                 if (GP || (FG && NT >= 512)) {      // (kernels with no registers to spare: one load in flight)
-                    for (int j4 = lane; j4 < n4; j4 += 32) d4[j4] = s4[j4];
+                    for (int j4 = lane; j4 < n4; j4 += 32) put(j4, s4[j4]);
                 } else {
                     for (int j0 = lane; j0 < n4; j0 += 128) {      // four loads in flight per lane
                         float4 t[4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) t[k] = __ldg(s4 + j0 + 32 * k);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) d4[j0 + 32 * k] = t[k];
+                        for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) put(j0 + 32 * k, t[k]);
                     }
                 }
             }
@@ -998,7 +1005,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         __syncthreads();
                         unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(panel) + 1023) & ~(uintptr_t)1023);
                         const int stage_bytes = (int)(reinterpret_cast<unsigned char*>(panel + a.panel_floats) - stage);
-                        if (!blk_flush_tc(&zmaps, blockIdx.x * 2, SH ? sched[2] : (int)blockIdx.x, stage, stage_bytes, fb, m1, nb,
+                        if (!blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
                                           power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr)) {
                             timed_out = true;
                             break;
@@ -1033,10 +1040,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 if (SH && s == sched[1]) break;      // (shares of rows) the row is handed over here, everything applied
                 if (m0 <= ms) {
                     // ---- move on chip: slots [0, m0) are all live here and the stored triangle is current
-                    const float* src = (d > ms) ? HP : a.Hinv;
-                    const int sld = (d > ms) ? ldp : a.ldhi;
                     for (int i = warp; i < m0; i += NW)
-                        for (int j = lane; j <= i; j += 32) S[i * lds + j] = ld_tri<TC>(src + (size_t)i * sld + j);
+                        for (int j = lane; j <= i; j += 32)
+                            S[i * lds + j] = d > ms ? ld_tri<TC>(HP + tri_at(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
                     tail = true;
                     __syncthreads();
                 }
@@ -1095,15 +1101,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                         for (int g = 0; g < GS; ++g) {
                             const int p = p4[g];
-                            const float* rowp = HP + (size_t)p * ldp;
                             if (jb + 3 <= p) {
-                                const float4 t = ld_tri4<TC>(rowp + jb);
+                                const float4 t = ld_tri4<TC>(HP + tri_at(ldp, p, jb));
                                 v[g][4 * g4] = t.x; v[g][4 * g4 + 1] = t.y; v[g][4 * g4 + 2] = t.z; v[g][4 * g4 + 3] = t.w;
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 4; ++q) {
                                     const int j = jb + q;
-                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>((j <= p) ? rowp + j : HP + (size_t)j * ldp + p);
+                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(HP + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
                                 }
                             }
                         }
@@ -1297,7 +1302,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 // pivot column of the stored matrix (own slots), corrected by the pending vectors
                 float c[KMAX], corr[KMAX];
                 unsigned live = 0u;
-                const float* rowp = HP + (size_t)p * ldp;
 #pragma unroll
                 for (int g = 0; g < KMAX / 4; ++g) {
                     const int jb = own_slot<NT>(4 * g);
@@ -1310,13 +1314,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     for (int q = 0; q < 4; ++q)
                         if (jb + q < m0 && pq[q] >= 0) live |= 1u << (4 * g + q);
                     if (jb + 3 <= p) {
-                        const float4 v = ld_tri4<TC>(rowp + jb);
+                        const float4 v = ld_tri4<TC>(HP + tri_at(ldp, p, jb));
                         c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
                     } else {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int j = jb + q;
-                            if ((live >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>((j <= p) ? rowp + j : HP + (size_t)j * ldp + p);
+                            if ((live >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(HP + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
                         }
                     }
                 }
