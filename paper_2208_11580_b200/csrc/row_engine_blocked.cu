@@ -77,7 +77,7 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
         int g = (int)(BLK_L2_PANEL_BUDGET / ((size_t)di.sm_count * p.g_ld * 4));
         if (bc == 8) {
             // (passes by mma.sync: their overflow vectors come 8 at a time and need staging space)
-            if (g > 32) g = 32;
+            if (g > 24) g = 24;
             g &= ~7;
             const size_t stage = (size_t)(p.nt / 32) * g * 16 * 4;
             if (in_smem < 16 && g >= 8 && share - fixed >= stage + 4 * min_panel) {
@@ -90,7 +90,9 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
             while (groups > 1 && (size_t)ft_stage_bytes(groups, FlushBufs{1, 1, 2}) + 1024 > share - fixed) --groups;
             if (d > p.ms && (size_t)ft_stage_bytes(1, FlushBufs{1, 1, 1}) + 1024 > share - fixed) return false;
             p.max_pending = 16 * groups;
-            if (g > p.max_pending - in_smem) g = p.max_pending - in_smem;
+            g &= ~7;                                               // (whole multiples of 8, as the plan reports them)
+            const int want = (p.max_pending - in_smem + 7) & ~7;
+            if (g > want) g = want;
             if (g >= 8) p.g_vectors = g;
         }
     }
