@@ -67,33 +67,57 @@ __global__ void __launch_bounds__(F32<TILE>::THREADS, F32<TILE>::BLOCKS) syrk_fp
 // H[i][j] = H[j][i] = (accumulate ? H[i][j] : 0) + 2 * sum_z partial[z][i][j]     for j <= i
 // err (nullable): a non-zero flag from the producing kernel (a bounded wait that expired) turns the whole result
 // into NaN; info (nullable) receives 0 or OBC_ERR_TIMEOUT accordingly.
+// A block takes a 32 x 32 tile on or below the diagonal; the mirror image goes through shared memory, so that both copies are
+// written along rows (column writes of single values took as long as the partial sums of 32 slices).
 __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __restrict__ partial, int splits, int d,
                                                                float* __restrict__ H, int ldh, int accumulate,
                                                                const int* __restrict__ err, int32_t* __restrict__ info) {
-    const int i = blockIdx.y;
-    const int j = blockIdx.x * 256 + threadIdx.x;
-    if (info && i == 0 && j == 0) info[0] = (err && *err != 0) ? (int32_t)OBC_ERR_TIMEOUT : 0;
-    if (j > i || j >= d) return;
-    float s = 0.f;
-    const float* P = partial + (size_t)i * d + j;
-    for (int z0 = 0; z0 < splits; z0 += 16) {             // sixteen loads in flight, added in order
-        float v[16];
+    __shared__ float tile[32][33];
+    const int bi = blockIdx.y, bj = blockIdx.x;
+    const bool failed = err && *err != 0;
+    if (info && bi == 0 && bj == 0 && threadIdx.x == 0) info[0] = failed ? (int32_t)OBC_ERR_TIMEOUT : 0;
+    if (bj > bi) return;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int j = bj * 32 + tx;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int z0 = 0; z0 < splits; z0 += 4) {              // sixteen loads in flight, added in order
+        float v[4][4];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = z0 + q < splits ? P[(size_t)(z0 + q) * d * d] : 0.f;
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int q = 0; q < 16; ++q) s += v[q];
+            for (int r = 0; r < 4; ++r) {
+                const int i = bi * 32 + ty + 8 * r;
+                v[q][r] = z0 + q < splits && i < d && j <= i ? __ldcs(partial + (size_t)(z0 + q) * d * d + (size_t)i * d + j) : 0.f;
+            }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) s[r] += v[q][r];
     }
-    float v = 2.f * s;
-    if (accumulate) v += H[(size_t)i * ldh + j];
-    if (err && *err != 0) v = __int_as_float(0x7fc00000);
-    H[(size_t)i * ldh + j] = v;
-    H[(size_t)j * ldh + i] = v;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = bi * 32 + ty + 8 * r;
+        if (i < d && j <= i) {
+            float v = 2.f * s[r];
+            if (accumulate) v += H[(size_t)i * ldh + j];
+            if (failed) v = __int_as_float(0x7fc00000);
+            H[(size_t)i * ldh + j] = v;
+            s[r] = v;
+        }
+        tile[ty + 8 * r][tx] = s[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {                         // (row, column) of the mirror image: j0 + .., i0 + ..
+        const int mi = bj * 32 + ty + 8 * r, mj = bi * 32 + tx;
+        if (mj < d && mi < mj) H[(size_t)mi * ldh + mj] = tile[tx][ty + 8 * r];
+    }
 }
 
 obc_status hessian_finalize_launch(const float* partial, int splits, int d, float* H, int ldh, int accumulate,
                                    const int* err, int32_t* info, cudaStream_t stream) {
-    dim3 grid((d + 255) / 256, d);
-    hessian_finalize_kernel<<<grid, 256, 0, stream>>>(partial, splits, d, H, ldh, accumulate, err, info);
+    const int T = (d + 31) / 32;
+    hessian_finalize_kernel<<<dim3(T, T), 256, 0, stream>>>(partial, splits, d, H, ldh, accumulate, err, info);
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
     return OBC_OK;
