@@ -255,6 +255,169 @@ __global__ void __launch_bounds__(TC_THREADS) syrk_tc_kernel(const __grid_consta
     }
 }
 
+// ---- 256 x 256 tiles ---------------------------------------------------------------------------------------------------
+// BF16X3 at large widths.  With 128 x 128 tiles every byte copied into shared memory feeds 48 multiply-adds and the kernel is
+// bound by L2 (3072 x 65536: 20 TB at 7.3 TB/s, 2.7 ms).  A 256 x 256 tile -- two accumulators of 128 x 256, all 512 columns of
+// tensor memory -- halves that traffic; a stage then holds 32 k of 512 rows in two parts (64 KB, 64B-swizzled rows of 64 bytes),
+// three stages fit.  On the diagonal both operands are the same rows and are copied once.
+constexpr int TL_TILE = 256;
+constexpr int TL_THREADS = 256;
+constexpr int TL_K = 32;
+constexpr int TL_STAGES = 3;
+constexpr uint32_t TL_OPERAND_BYTES = TL_TILE * TL_K * 2;      // 16 KiB: one part of one operand
+constexpr uint32_t TL_STAGE_BYTES = 4 * TL_OPERAND_BYTES;
+
+// K-major operand with rows of 64 bytes, 64B swizzle: 8-row groups 512 bytes apart
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
+    uint64_t dsc = (uint64_t)((addr >> 4) & 0x3fffu);
+    dsc |= (uint64_t)1 << 16;
+    dsc |= (uint64_t)(512 >> 4) << 32;
+    dsc |= (uint64_t)1 << 46;
+    dsc |= (uint64_t)4 << 61;
+    return dsc;
+}
+
+template <bool CROSS>
+__global__ void __launch_bounds__(TL_THREADS, 1) syrk_tc256_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_alo,
+                                                                   const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_blo,
+                                                                   int rows_a, int rows_b, int64_t n_elems, int64_t slice, float* __restrict__ partial,
+                                                                   int* __restrict__ err, int wait_limit) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ __align__(8) unsigned long long bars[2 * TL_STAGES + 1];      // full, empty, accumulators ready
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_s;
+    __shared__ int mma_issued_s;
+    int bi = 0, bj = 0;
+    if (CROSS) {
+        const int tj = (rows_b + TL_TILE - 1) / TL_TILE;
+        bi = blockIdx.x / tj; bj = blockIdx.x - bi * tj;
+    } else {
+        int t = blockIdx.x;
+        while (t > bi) { t -= bi + 1; ++bi; }
+        bj = t;
+    }
+    const bool same = !CROSS && bi == bj;
+    const int64_t kb0 = (int64_t)blockIdx.y * slice;
+    const int64_t ke = kb0 + slice < n_elems ? kb0 + slice : n_elems;
+    const int nkb = ke > kb0 ? (int)((ke - kb0 + TL_K - 1) / TL_K) : 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[TL_STAGES]), accbar = smem_u32(&bars[2 * TL_STAGES]);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < TL_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        mbar_init(accbar, 1);
+        abort_s = 0;
+        mma_issued_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_d = tmem_base_s;
+    int issued = 0;
+    if (warp == 0 && lane == 0) {
+        for (int kb = 0; kb < nkb; ++kb) {
+            const int s = kb % TL_STAGES;
+            if (kb >= TL_STAGES && !mbar_wait(empty0 + 8 * s, ((kb / TL_STAGES) - 1) & 1, wait_limit)) { atomicExch(err, 1); abort_s = 1; break; }
+            if (*(volatile int*)&abort_s) break;
+            const uint32_t dst = smem_u32(tiles) + s * TL_STAGE_BYTES;
+            const int x = (int)(kb0 + (int64_t)kb * TL_K);
+            mbar_expect_tx(full0 + 8 * s, same ? TL_STAGE_BYTES / 2 : TL_STAGE_BYTES);
+            tma_load_2d(dst, &map_a, full0 + 8 * s, x, bi * TL_TILE);
+            tma_load_2d(dst + TL_OPERAND_BYTES, &map_alo, full0 + 8 * s, x, bi * TL_TILE);
+            if (!same) {
+                tma_load_2d(dst + 2 * TL_OPERAND_BYTES, &map_b, full0 + 8 * s, x, bj * TL_TILE);
+                tma_load_2d(dst + 3 * TL_OPERAND_BYTES, &map_blo, full0 + 8 * s, x, bj * TL_TILE);
+            }
+            issued = kb + 1;
+        }
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TL_TILE >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        for (int kb = 0; kb < nkb; ++kb) {
+            const int s = kb % TL_STAGES;
+            if (!mbar_wait(full0 + 8 * s, (kb / TL_STAGES) & 1, wait_limit)) { atomicExch(err, 2); abort_s = 1; break; }
+            if (*(volatile int*)&abort_s) break;
+            tc_fence_after();
+            mma_issued_s = 1;
+            const uint32_t base = smem_u32(tiles) + s * TL_STAGE_BYTES;
+            const uint64_t ah = smem_desc_sw64(base), al = smem_desc_sw64(base + TL_OPERAND_BYTES);
+            const uint64_t bh = same ? ah : smem_desc_sw64(base + 2 * TL_OPERAND_BYTES), bl = same ? al : smem_desc_sw64(base + 3 * TL_OPERAND_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < TL_K / 16; ++kk) {
+                const uint64_t adv = (uint64_t)(kk * 32 >> 4);
+                const uint32_t acc = (kb > 0 || kk > 0) ? 1u : 0u;
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {             // rows 0 .. 127 and 128 .. 255 of the tile
+                    const uint64_t h = adv + (uint64_t)(half * 128 * 64 >> 4);
+                    const uint32_t d = tmem_d + half * 256;
+                    tc_mma<1>(d, ah + h, bh + adv, idesc, acc);     // hi * hi^T
+                    tc_mma<1>(d, ah + h, bl + adv, idesc, 1u);      // hi * lo^T
+                    tc_mma<1>(d, al + h, bh + adv, idesc, 1u);      // lo * hi^T
+                }
+            }
+            tc_commit(empty0 + 8 * s);
+        }
+        if (nkb > 0 && *(volatile int*)&mma_issued_s) tc_commit(accbar);
+    }
+    __syncwarp();
+    // ---- epilogue: warp w owns accumulator lanes 32 (w % 4) .. + 31 of half w / 4 ------------------------------------------
+    bool ok = true;
+    if (nkb > 0) {
+        if (lane == 0) ok = mbar_wait(accbar, 0, wait_limit);
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        if (!ok && lane == 0) { atomicExch(err, 3); abort_s = 1; }
+    }
+    tc_fence_after();
+    int ab = lane == 0 ? *(volatile int*)&abort_s : 0;
+    ab = __shfl_sync(0xffffffffu, ab, 0);
+    if (ok && ab == 0) {
+        float* P = partial + (size_t)blockIdx.y * rows_a * rows_b;
+        const int half = warp >> 2;
+        const int gi = bi * TL_TILE + half * 128 + (warp & 3) * 32 + lane;
+        const bool vec = (rows_b & 3) == 0;
+        for (int c = 0; c < TL_TILE / 32; ++c) {
+            const int gj0 = bj * TL_TILE + c * 32;
+            if (gj0 >= rows_b) break;
+            uint32_t r[32];
+            if (nkb > 0) tmem_ld32(tmem_d + half * 256 + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(c * 32), r);
+            else {
+#pragma unroll
+                for (int q = 0; q < 32; ++q) r[q] = 0u;
+            }
+            if (gi < rows_a) {
+                float* dst = P + (size_t)gi * rows_b + gj0;
+                if (vec && gj0 + 32 <= rows_b) {
+#pragma unroll
+                    for (int q = 0; q < 32; q += 4)
+                        __stcs(reinterpret_cast<float4*>(dst + q), make_float4(__uint_as_float(r[q]), __uint_as_float(r[q + 1]),
+                                                                               __uint_as_float(r[q + 2]), __uint_as_float(r[q + 3])));
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 32; ++q)
+                        if (gj0 + q < rows_b) dst[q] = __uint_as_float(r[q]);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (*(volatile int*)&abort_s && warp == 0 && lane == 0) {
+        // (as in syrk_tc_kernel: own copies in flight and issued products are over before anything is released)
+        for (int kb = issued > TL_STAGES ? issued - TL_STAGES : 0; kb < issued; ++kb)
+            mbar_wait(full0 + 8 * (kb % TL_STAGES), (kb / TL_STAGES) & 1, TC_WAIT_LIMIT);
+        if (*(volatile int*)&mma_issued_s) mbar_wait(accbar, 0, TC_WAIT_LIMIT);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(512));
+    }
+}
+
 // hi = bf16(x), lo = bf16(x - hi); outputs are d x n_pad (n_pad multiple of 64, padding written as zero)
 __global__ void __launch_bounds__(256) split_bf16_kernel(const float* __restrict__ X, int d, int64_t n, int64_t ldx,
                                                          int64_t n_pad, __nv_bfloat16* __restrict__ hi,
@@ -298,16 +461,42 @@ static PFN_cuTensorMapEncodeTiled encode_fn() {
     return fn;
 }
 
+// boxes of rows x row_bytes (128 or 64: the swizzle follows)
 static bool make_map(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, int64_t inner,
-                     int64_t rows, int64_t row_stride_elems) {
+                     int64_t rows, int64_t row_stride_elems, int box_rows = TC_TILE, int row_bytes = TC_KBYTES) {
     PFN_cuTensorMapEncodeTiled fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)row_stride_elems * elem_bytes};
-    cuuint32_t box[2] = {(cuuint32_t)(TC_KBYTES / elem_bytes), (cuuint32_t)TC_TILE};
+    cuuint32_t box[2] = {(cuuint32_t)(row_bytes / elem_bytes), (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+              row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 256 x 256 tiles where they cost little padding (a quarter of the products at most) and at least about fill the chip
+static bool large_tiles(int rows_a, int rows_b, bool cross, int splits) {
+    const int64_t a = (rows_a + TL_TILE - 1) / TL_TILE, b = (rows_b + TL_TILE - 1) / TL_TILE;
+    const int64_t a1 = (rows_a + TC_TILE - 1) / TC_TILE, b1 = (rows_b + TC_TILE - 1) / TC_TILE;
+    const int64_t big = cross ? a * b : a * (a + 1) / 2, small = cross ? a1 * b1 : a1 * (a1 + 1) / 2;
+    return 16 * big <= 5 * small && big * splits >= 120;
+}
+static bool bf16_maps(CUtensorMap* hi_map, CUtensorMap* lo_map, const __nv_bfloat16* hi, const __nv_bfloat16* lo, int64_t n_pad, int rows, bool large) {
+    const int box = large ? TL_TILE : TC_TILE, bytes = large ? TL_K * 2 : TC_KBYTES;
+    return make_map(hi_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hi, n_pad, rows, n_pad, box, bytes) &&
+           make_map(lo_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lo, n_pad, rows, n_pad, box, bytes);
+}
+template <bool CROSS>
+static obc_status launch_large(const CUtensorMap& a, const CUtensorMap& al, const CUtensorMap& b, const CUtensorMap& bl, int rows_a, int rows_b,
+                               int64_t n_pad, int64_t slice, int splits, float* partial, int* err, int wl, cudaStream_t stream) {
+    const int ta = (rows_a + TL_TILE - 1) / TL_TILE, tb = (rows_b + TL_TILE - 1) / TL_TILE;
+    const size_t smem = (size_t)TL_STAGES * TL_STAGE_BYTES + 1024;
+    OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc256_kernel<CROSS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    syrk_tc256_kernel<CROSS><<<dim3(CROSS ? ta * tb : ta * (ta + 1) / 2, splits), TL_THREADS, smem, stream>>>(a, al, b, bl, rows_a, rows_b, n_pad, slice,
+                                                                                                              partial, err, wl);
+    count_launch();
+    return OBC_OK;
 }
 
 bool make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, int64_t inner, int64_t rows,
@@ -357,13 +546,18 @@ obc_status hessian_tc_launch(const float* X, int d, int64_t n, int64_t ldx, floa
     } else {
         split_bf16_kernel<<<1184, 256, 0, stream>>>(X, d, n, ldx, n_pad, hi, lo);
         count_launch();
-        if (!make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hi, n_pad, d, n_pad)) return OBC_ERR_CUDA;
-        if (!make_map(&ml, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lo, n_pad, d, n_pad)) return OBC_ERR_CUDA;
+        const bool large = large_tiles(d, d, false, splits);
+        if (!bf16_maps(&ma, &ml, hi, lo, n_pad, d, large)) return OBC_ERR_CUDA;
+        if (large) {
+            const obc_status st = launch_large<false>(ma, ml, ma, ml, d, d, n_pad, slice, splits, partial, err, wl, stream);
+            if (st != OBC_OK) return st;
+        } else {
         const int stages = 3;
         const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
         OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         syrk_tc_kernel<1, false><<<grid, TC_THREADS, smem, stream>>>(ma, ml, ma, ml, d, d, n_pad, slice, stages, partial, err, wl);
         count_launch();
+        }
     }
     OBC_CUDA_TRY(cudaGetLastError());
     return hessian_finalize_launch(partial, splits, d, H, ldh, accumulate, err, info, stream);
@@ -437,15 +631,18 @@ obc_status cross_tc_launch(const float* Y, int rows_a, int64_t ldy, const float*
         split_bf16_kernel<<<1184, 256, 0, stream>>>(Y, rows_a, n, ldy, n_pad, yhi, ylo);
         split_bf16_kernel<<<1184, 256, 0, stream>>>(X, rows_b, n, ldx, n_pad, xhi, xlo);
         count_launch(2);
-        if (!make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, yhi, n_pad, rows_a, n_pad)) return OBC_ERR_CUDA;
-        if (!make_map(&mal, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ylo, n_pad, rows_a, n_pad)) return OBC_ERR_CUDA;
-        if (!make_map(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xhi, n_pad, rows_b, n_pad)) return OBC_ERR_CUDA;
-        if (!make_map(&mbl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xlo, n_pad, rows_b, n_pad)) return OBC_ERR_CUDA;
+        const bool large = large_tiles(rows_a, rows_b, true, splits);
+        if (!bf16_maps(&ma, &mal, yhi, ylo, n_pad, rows_a, large) || !bf16_maps(&mb, &mbl, xhi, xlo, n_pad, rows_b, large)) return OBC_ERR_CUDA;
+        if (large) {
+            const obc_status st = launch_large<true>(ma, mal, mb, mbl, rows_a, rows_b, n_pad, slice, splits, partial, err, wl, stream);
+            if (st != OBC_OK) return st;
+        } else {
         const int stages = 3;
         const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
         OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         syrk_tc_kernel<1, true><<<grid, TC_THREADS, smem, stream>>>(ma, mal, mb, mbl, rows_a, rows_b, n_pad, slice, stages, partial, err, wl);
         count_launch();
+        }
     }
     OBC_CUDA_TRY(cudaGetLastError());
     dim3 fgrid((rows_b + 255) / 256, rows_a);
