@@ -15,9 +15,11 @@ struct BlkPlan {
     int max_pending;   // limit on deferred updates
 };
 
-obc_status blk_launch_128(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
-obc_status blk_launch_256(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
-obc_status blk_launch_512(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
+obc_status blk_launch_128_8(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
+obc_status blk_launch_256_8(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
+obc_status blk_launch_512_4(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
+obc_status blk_launch_512_8(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
+obc_status blk_launch_512_12(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
 
 // All blocks' overflow vectors together: within L2.  (Only the longest rows reach the limit; 48 / 64 / 80 / 110 MB at 128 rows x
 // 4608: 249 / 220 / 202 / 181 ms.)
@@ -38,12 +40,14 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     const int cap = (d + 3) & ~3;
     int nt = threads;
     if (nt != 128 && nt != 256 && nt != 512) {
-        // measured on full waves of rows: 128 threads win up to d_col ~ 700, 256 up to ~ 1400, 512 above
-        nt = d <= 704 ? 128 : (d <= 1408 ? 256 : 512);
+        // measured on many rows: 128 threads win up to d_col ~ 700, 256 up to ~ 1200 (1152: 34.3 against 35.2 ms with 512 threads,
+        // 1408: 55.5 against 48.7 ms), 512 above
+        nt = d <= 704 ? 128 : (d <= 1216 ? 256 : 512);
         // few rows (one per SM pair at most): nothing to share an SM with, the larger block is faster per row
         if (nt == 128 && row_count > 0 && row_count <= 2 * di.sm_count) nt = 256;
-        // at most one row per SM: from d_col ~ 1000 the whole SM on one row wins (1024: 7 %, 1280: 20 %)
-        if (nt == 256 && row_count > 0 && row_count <= di.sm_count && d > 960) nt = 512;
+        // at most one row per SM: the whole SM on one row wins from d_col ~ 700 (640: 3.0 against 3.1 ms, 768: 4.0 against 3.9, 960: 6.0
+        // against 5.3)
+        if (nt == 256 && row_count > 0 && row_count <= di.sm_count && d > 704) nt = 512;
     }
     if (nt == 128 && cap > 1024) nt = 256;
     if (nt == 256 && cap > 2048) nt = 512;
@@ -219,9 +223,11 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
             a.split_flags = reinterpret_cast<int*>(reinterpret_cast<char*>(ws) + tri + gpan + planes + sst);
         }
     }
-    if (p.nt == 128) return blk_launch_128(zmaps, a, blocks, p.smem, di.sm_count, stream);
-    if (p.nt == 256) return blk_launch_256(zmaps, a, blocks, p.smem, di.sm_count, stream);
-    return blk_launch_512(zmaps, a, blocks, p.smem, di.sm_count, stream);
+    // Slots per thread of the 512-thread kernels: every one costs instructions in every step (4 against 12: 960 columns, one row per
+    // SM, 7.7 -> 5.3 ms; 8 against 12: 256 x 2304 54 -> 48 ms).  (4 instead of 8 with 128 or 256 threads measured no faster.)
+    auto launch = p.nt == 128 ? blk_launch_128_8 : p.nt == 256 ? blk_launch_256_8
+                : (a.cap <= 2048 ? blk_launch_512_4 : (a.cap <= 4096 ? blk_launch_512_8 : blk_launch_512_12));
+    return launch(zmaps, a, blocks, p.smem, di.sm_count, stream);
 }
 
 }  // namespace obc
