@@ -32,6 +32,7 @@ struct EngineArgs {
     uint8_t* mask;                        // blocked engine, nullable: d_row x d mask, 0 at eliminated columns
     int block_c;                          // blocked engine: 4 = block pruning in blocks of 4 columns (Eq. 5), 0 = off
     __half* Zws; int zld;                 // blocked engine: FP16 planes of the pending vectors, 128 rows of zld per block
+    double2* park;                        // blocked engine: cap per block, a row's FP64 state during a pass
     signed char* zexp;                    // blocked engine: powers of two of the slots (cap per block; wide diagonals)
     float* Gpan; int g_vectors; int g_ld; // blocked engine: overflow pending vectors in global memory (per block
                                           // g_vectors rows of g_ld floats), nullptr = none

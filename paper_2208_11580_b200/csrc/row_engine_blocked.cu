@@ -91,8 +91,8 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
         } else {
             // as many updates per pass as it has accumulators and operand space for
             int groups = FT_GMAX;
-            while (groups > 1 && (size_t)ft_stage_bytes(groups, FlushBufs{1, 1, 2}) + 1024 > share - fixed) --groups;
-            if (d > p.ms && (size_t)ft_stage_bytes(1, FlushBufs{1, 1, 1}) + 1024 > share - fixed) return false;
+            while (groups > 1 && (size_t)ft_stage_bytes(groups, FlushBufs{1, 1, 2}) + 1024 > share - fixed + 16 * (size_t)cap) --groups;
+            if (d > p.ms && (size_t)ft_stage_bytes(1, FlushBufs{1, 1, 1}) + 1024 > share - fixed + 16 * (size_t)cap) return false;
             p.max_pending = 16 * groups;
             g &= ~7;                                               // (whole multiples of 8, as the plan reports them)
             const int want = (p.max_pending - in_smem + 7) & ~7;
@@ -111,10 +111,11 @@ static int blk_max_blocks(int d, const DeviceInfo& di) {
     return di.sm_count * (cap > 2048 ? 1 : (cap > 1024 ? 2 : 4));
 }
 
-// FP16 planes of the pending vectors of every 512-thread block (64 hi, 64 lo rows) and the slots' powers of two
+// FP16 planes of the pending vectors of every 512-thread block (64 hi, 64 lo rows), the parked FP64 state of its row, and the
+// slots' powers of two
 static int blk_zld(int cap) { return (cap + 127) & ~127; }
 size_t blk_plane_bytes(int blocks, int cap) {
-    return round_up((size_t)blocks * 128 * blk_zld(cap) * sizeof(__half), 256) + round_up((size_t)blocks * cap, 256);
+    return round_up((size_t)blocks * 128 * blk_zld(cap) * sizeof(__half), 256) + round_up((size_t)blocks * cap * sizeof(double2), 256) + round_up((size_t)blocks * cap, 256);
 }
 
 size_t blocked_engine_workspace_bytes(int row_count, int d, const DeviceInfo& di) {
@@ -181,7 +182,7 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
     a.ldp = a.cap;
     a.split = 0;
     a.split_state = nullptr; a.split_flags = nullptr; a.split_stride = 0;
-    a.Zws = nullptr; a.zexp = nullptr; a.zld = blk_zld(a.cap);
+    a.Zws = nullptr; a.park = nullptr; a.zexp = nullptr; a.zld = blk_zld(a.cap);
     FlushMaps zmaps = {};
     if (a.d > a.ms) {
         // Shares of rows (equal work per block instead of whole waves): when there are more rows than blocks and they
@@ -203,7 +204,8 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
         a.Hws = reinterpret_cast<float*>(ws);
         if (planes) {
             a.Zws = reinterpret_cast<__half*>(reinterpret_cast<char*>(ws) + tri + gpan);
-            a.zexp = reinterpret_cast<signed char*>(a.Zws) + round_up((size_t)blocks * 128 * a.zld * sizeof(__half), 256);
+            a.park = reinterpret_cast<double2*>(reinterpret_cast<char*>(a.Zws) + round_up((size_t)blocks * 128 * a.zld * sizeof(__half), 256));
+            a.zexp = reinterpret_cast<signed char*>(a.park) + round_up((size_t)blocks * a.cap * sizeof(double2), 256);
             const int64_t groups = (int64_t)blocks * (want_split ? 2 : 1) * (((a.cap + 63) & ~63) >> 5);      // of 32 columns
             for (int k = 0; k < FT_GMAX; ++k)
                 if (!make_tensor_map_3d(&zmaps.z[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.Zws, a.zld, 64, 2 * (int64_t)blocks, 64, 16 * (k + 1), 2))

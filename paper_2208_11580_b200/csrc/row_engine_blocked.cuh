@@ -55,8 +55,9 @@ constexpr int BLK_FIXED = 3584;
 static_assert(BLK_OFF_FB + sizeof(FlushBars) <= BLK_FIXED, "");
 constexpr int BLK_GS = 4;                     // forced eliminations taken together
 
-// Per-row state in shared memory: wd, dg (FP64), perm (int32), srcm (uint16); optional: the row in original
-// order (weight trace), one byte per block of the N:M pattern.
+// Per-row state in shared memory: perm (int32), srcm (uint16); optional: the row in original order (weight trace), one byte
+// per block of the N:M pattern, off-diagonals of block pruning; last, next to the pending vectors, wd and dg (FP64): a pass on
+// tcgen05 parks them in global memory and uses their space too.
 // (block pruning, bc = block size 4 or 8: the 6 or 28 off-diagonal entries of every block's c x c diagonal block, FP64)
 __host__ __device__ inline size_t blk_state_bytes(int cap, bool wfull, bool nm = false, int bc = 0) {
     return (size_t)20 * cap + (((size_t)2 * cap + 15) & ~(size_t)15) + (wfull ? (size_t)4 * cap : 0) +
@@ -776,17 +777,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     int* mv = reinterpret_cast<int*>(smem + BLK_OFF_MV);
     float* rf = reinterpret_cast<float*>(smem + BLK_OFF_RF);
     uint32_t* colmask = reinterpret_cast<uint32_t*>(smem + BLK_OFF_CM);
-    double* wd = reinterpret_cast<double*>(smem + BLK_FIXED);
-    double* dg = wd + cap;
-    int* perm = reinterpret_cast<int*>(dg + cap);
+    int* perm = reinterpret_cast<int*>(smem + BLK_FIXED);
     unsigned short* srcm = reinterpret_cast<unsigned short*>(perm + cap);
     const bool has_wfull = a.w_trace != nullptr;
-    float* wfull = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, false));
+    float* wfull = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, false) - 16 * cap);
     const bool has_nm = a.nm_prune > 0;                         // N:M pattern: at most nm_prune eliminations per block
     const int nm_lg = a.nm_lg, nm_prune = a.nm_prune;
-    unsigned char* blkcnt = reinterpret_cast<unsigned char*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull));
-    double* boff = reinterpret_cast<double*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm));
+    unsigned char* blkcnt = reinterpret_cast<unsigned char*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull) - 16 * cap);
+    double* boff = reinterpret_cast<double*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm) - 16 * cap);
     float* panel = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm, BC));
+    double* wd = reinterpret_cast<double*>(panel) - 2 * cap;
+    double* dg = wd + cap;
     // tail views (step-by-step phase in shared memory) share the panel's space
     const int msr = (ms + 3) & ~3;
     float* tv = panel;
@@ -1001,15 +1002,18 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         signed char* zexp = a.zexp + (size_t)blockIdx.x * cap;
                         const int power = blk_make_planes<NT, KMAX>(panel, ldz, GP ? scap : nb, GP ? GVEC : nullptr, gld, nb, m0, m1, dg, perm, rf,
                                                                     a.Zws + (size_t)blockIdx.x * 128 * a.zld, a.zld, zexp);
+                        // the FP64 state gives its space to the pass (d_col = 4608: three tile buffers instead of two)
+                        double2* park = a.park + (size_t)blockIdx.x * cap;
+                        for (int j = tid; j < cap; j += NT) park[j] = reinterpret_cast<const double2*>(wd)[j];      // (wd and dg: 2 cap doubles)
                         asm volatile("fence.proxy.async;" ::: "memory");            // plain accesses before the copies
                         __syncthreads();
-                        unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(panel) + 1023) & ~(uintptr_t)1023);
+                        unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wd) + 1023) & ~(uintptr_t)1023);
                         const int stage_bytes = (int)(reinterpret_cast<unsigned char*>(panel + a.panel_floats) - stage);
-                        if (!blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
-                                          power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr)) {
-                            timed_out = true;
-                            break;
-                        }
+                        const bool fine = blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
+                                          power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr);
+                        for (int j = tid; j < cap; j += NT) reinterpret_cast<double2*>(wd)[j] = __ldcg(park + j);
+                        __syncthreads();
+                        if (!fine) { timed_out = true; break; }
                     } else if (!GP)
                         blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);      // evict-first at every row length (~1 %)
                     else
