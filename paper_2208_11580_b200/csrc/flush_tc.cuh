@@ -52,9 +52,10 @@ struct FlushBufs { int n_a, n_b, n_h; };
 __host__ __device__ inline int ft_stage_bytes(int g, FlushBufs f) { return 2 * g * FT_GROUP_BYTES * (2 * f.n_a + f.n_b) + f.n_h * FT_TILE_BYTES; }
 __host__ __device__ inline FlushBufs ft_bufs(int g, int bytes) {
     FlushBufs f{2, 2, 4};
-    while (f.n_h > 3 && ft_stage_bytes(g, f) > bytes) --f.n_h;
-    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{1, 2, 3};
-    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{1, 2, 2};
+    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{2, 1, 4};
+    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{2, 2, 3};
+    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{2, 1, 3};
+    if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{2, 1, 2};
     if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{1, 1, 2};
     if (ft_stage_bytes(g, f) > bytes) f = FlushBufs{1, 1, 1};
     return f;
@@ -175,10 +176,10 @@ __device__ __forceinline__ void ft_inval_bars(FlushBars* fb) {
     for (int q = 0; q < (int)(offsetof(FlushBars, tmem) / 8); ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(ft_smem(b + q)) : "memory");
 }
 
-// Tile sequence of a pass: row blocks in order, columns [0, min(128 (rb + 1), m1)) of each in steps of 64.
+// Tile sequence of a pass: column blocks of 64 in order, down the rows from the diagonal -- the order of memory (along the rows
+// instead, every tile is in other pages: 128 x 4608 153 against 149 ms).
 __device__ __forceinline__ void ft_next_tile(int& rb, int& c, int m1) {
-    c += FT_N;
-    if (c >= min((rb + 1) * FT_M, m1)) { c = 0; ++rb; }
+    if (++rb * FT_M >= m1) { c += FT_N; rb = c / FT_M; }
 }
 // A position in a ring of n buffers and how often it has gone round.
 struct Ring {
@@ -212,30 +213,30 @@ __device__ __forceinline__ bool ft_copy_tile(const FlushGeom& q, FlushBars* fb, 
     h.next(q.nb.n_h);
     return true;
 }
-// Copies of the vectors at the tile's columns and, first tile of a row block, at its rows.  One thread (another one: the
+// Copies of the vectors at the tile's rows and, first tile of a column block, at its columns.  One thread (another one: the
 // operands run ahead of the tiles, whose buffers are held until they are back in memory).
 __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* fb, Ring& b, Ring& a, int rb, int c) {
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;    // both planes of 64 slots
     const CUtensorMap* zm = &q.maps->z[q.G - 1];
-    if (c == 0) {
-        if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb)) return false;
-        ft_expect(&fb->full_a[a.at], 2 * blk);
-        ft_load(q.sa + a.at * 2 * blk, zm, &fb->full_a[a.at], rb * FT_M, 0, q.plane);
-        ft_load(q.sa + (a.at * 2 + 1) * blk, zm, &fb->full_a[a.at], rb * FT_M + 64, 0, q.plane);
-        a.next(q.nb.n_a);
+    if (rb == c / FT_M) {
+        if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
+        ft_expect(&fb->full_b[b.at], blk);
+        ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
+        b.next(q.nb.n_b);
     }
-    if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
-    ft_expect(&fb->full_b[b.at], blk);
-    ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
-    b.next(q.nb.n_b);
+    if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb)) return false;
+    ft_expect(&fb->full_a[a.at], 2 * blk);
+    ft_load(q.sa + a.at * 2 * blk, zm, &fb->full_a[a.at], rb * FT_M, 0, q.plane);
+    ft_load(q.sa + (a.at * 2 + 1) * blk, zm, &fb->full_a[a.at], rb * FT_M + 64, 0, q.plane);
+    a.next(q.nb.n_a);
     return true;
 }
-// Products of tile t at (.., c); `last`: of its row block.  One thread.
-__device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, int t, Ring& b, Ring& a, int c, bool last) {
+// Products of tile t; first / last: of its column block.  One thread.
+__device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, int t, Ring& b, Ring& a, bool first, bool last) {
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;
     const int buf = t & 1;
-    if (c == 0 && !ft_wait(&fb->full_a[a.at], a.round & 1, fb)) return false;
-    if (!ft_wait(&fb->full_b[b.at], b.round & 1, fb)) return false;
+    if (first && !ft_wait(&fb->full_b[b.at], b.round & 1, fb)) return false;
+    if (!ft_wait(&fb->full_a[a.at], a.round & 1, fb)) return false;
     if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint64_t da = ft_desc(q.sa + a.at * 2 * blk, blk), db = ft_desc(q.sb + b.at * blk, blk);
@@ -249,17 +250,17 @@ __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, i
 #pragma unroll
     for (int k = 0; k < FT_GMAX; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + k * STEP, db + k * STEP, 1u);
     ft_commit(&fb->done[buf]);
-    ft_commit(&fb->free_b[b.at]);
-    b.next(q.nb.n_b);
-    if (last) { ft_commit(&fb->free_a[a.at]); a.next(q.nb.n_a); }
+    ft_commit(&fb->free_a[a.at]);
+    a.next(q.nb.n_a);
+    if (last) { ft_commit(&fb->free_b[b.at]); b.next(q.nb.n_b); }
     return true;
 }
-// The products of `tiles` tiles in `rbs` row blocks and all that they signal are over.
-__device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* fb, int tiles, int rbs) {
+// The products of `tiles` tiles (of all, if it is q.T: then in `blocks` column blocks) and all that they signal are over.
+__device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* fb, int tiles, int blocks) {
     if (tiles <= 0) return;
     ft_drain(&fb->done[(tiles - 1) & 1], ((tiles - 1) >> 1) & 1);
-    ft_drain(&fb->free_b[(tiles - 1) % q.nb.n_b], ((tiles - 1) / q.nb.n_b) & 1);
-    if (tiles == q.T) ft_drain(&fb->free_a[(rbs - 1) % q.nb.n_a], ((rbs - 1) / q.nb.n_a) & 1);
+    ft_drain(&fb->free_a[(tiles - 1) % q.nb.n_a], ((tiles - 1) / q.nb.n_a) & 1);
+    if (tiles == q.T) ft_drain(&fb->free_b[(blocks - 1) % q.nb.n_b], ((blocks - 1) / q.nb.n_b) & 1);
 }
 // Takes the tile at (rb, c) back to memory once every warp has finished its part.  One thread (of all tiles).
 __device__ __forceinline__ bool ft_store(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
@@ -374,10 +375,10 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
         for (; t < q.T; ++t) {
             int nrb = rb, nc = c;
             ft_next_tile(nrb, nc, m1);
-            if (!ft_multiply(q, fb, t, b, a, c, nc == 0)) break;
+            if (!ft_multiply(q, fb, t, b, a, rb == c / FT_M, nc != c)) break;
             rb = nrb; c = nc;
         }
-        ft_products_over(q, fb, t, n_rb);
+        ft_products_over(q, fb, t, (m1 + FT_N - 1) / FT_N);
     } else if (warp == FT_EW + 2 && lane == 0) {
         const uint64_t pol = ft_stream_policy();
         for (; t < q.T; ++t) {
