@@ -47,10 +47,10 @@ FALLBACK_BF16_SUSTAINED_TFLOPS = 1400.0
 # traffic of a full-size launch is scaled from it by the algorithmic bytes (traffic grows with them).
 ENGINE_TRAFFIC_PER_ALGORITHMIC_BYTE = 291.0 / 603.3
 # The same for the blocked engine, relative to ITS algorithmic bytes (blocked_bytes_flops), per captured row length:
-# profiles/blocked_engine_d2304_rows148_ncu_full.txt: 120.04 GB moved for 98.13 GB;
-# profiles/blocked_engine_d3072_rows148_ncu_full.txt: 201.79 GB for 147.73 GB.  Other row lengths run other
-# configurations of the kernel (threads per row, pending vectors in L2) and have no capture: traffic is null there.
-BLOCKED_TRAFFIC_PER_ALGORITHMIC_BYTE = {2304: 120.04 / 98.13, 3072: 201.79 / 147.73}
+# profiles/blocked_engine_d2304_d3072_ncu.txt: 93.92 GB moved for 50.31 GB at 2304, 219.24 GB for 119.24 GB at 3072.  Other row
+# lengths run other configurations of the kernel (threads per row, pending vectors in L2) and have no capture: traffic is
+# null there.
+BLOCKED_TRAFFIC_PER_ALGORITHMIC_BYTE = {2304: 93.92 / 50.31, 3072: 219.24 / 119.24}
 
 
 def model_bytes_full(d: int, first: int | None = None, steps: int | None = None) -> int:
@@ -443,11 +443,11 @@ def measure(args, name, steps, warmup, rank, world, dev, with_cpu=True, with_e2e
               "unit": "TFLOP/s", "frac": round(tflops / tpeak, 4), "frac_executed": round(3.0 * tflops / tpeak, 4),
               "flops_per_launch": int(flops // n_eng),
               "flops_model": "2 flops per element of the active lower triangle and deferred update (rank-B update on the tensor "
-                             "cores, TF32 m16n8k8); executed = 3 x that: every FP32 operand is split into two TF32 parts and "
-                             "three of the four partial products are formed"}
+                             "cores: FP16 tcgen05 with 512 threads per row, else TF32 m16n8k8); executed = 3 x that: every FP32 "
+                             "operand is split into two parts and three of the four partial products are formed"}
     if blocked and plan.get("l2_vectors", 0) > 0:
-        tensor["note"] = ("rows this long keep %d of their deferred updates per pass in global memory (resident in L2); the rank-B "
-                          "update reads their operands from there in the MMA fragment layout" % plan["l2_vectors"])
+        tensor["note"] = ("rows this long keep up to %d of their deferred updates per pass in global memory (resident in L2); the "
+                          "rank-B update copies all operands from there with TMA" % plan["l2_vectors"])
     # Both engines are reported against HBM.  The streaming engine moves the active triangle once per step.  The blocked
     # engine moves it once per block of deferred updates and applies the block as one rank-B update on the tensor cores;
     # the per-step phase (argmin, pivot column, correction) moves no matrix bytes and is inside the same time.
