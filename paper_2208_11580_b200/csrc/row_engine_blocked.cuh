@@ -15,11 +15,12 @@
 // vectors and compacts at the same time: a dead slot h below the new size m1 is taken over by a live slot
 // s >= m1, i.e. element (i, j) of the new triangle is read from (max(si, sj), min(si, sj)) of the old one.
 // All such foreign reads come from rows >= m1, which the flush never writes, so it runs in place.
-// The flush is a rank-B update and runs on the tensor cores (warp tiles of 16 rows x 64 columns, TF32 split
-// products, see blk_flush_mma); the pending vectors stay in shared memory (at very long rows further ones sit in a
-// global buffer that stays in L2; the flush reads their operands from there).  The O(m) selection state (weights, diagonal) is FP64, as in
-// the streaming engine.  Once the live triangle fits into the shared memory of the pending vectors, the row
-// finishes on chip with step-by-step updates.
+// The flush is a rank-B update and runs on the tensor cores: with 512 threads per row on tcgen05 with the triangle moved by TMA
+// (flush_tc.cuh; pending vectors beyond shared memory wait in a global buffer that stays in L2), with several rows per SM by
+// mma.sync (warp tiles of 16 rows x 64 columns, TF32 split products, see blk_flush_mma): there the passes of one row
+// overlap the steps of another, and tensor memory and tile buffers would have to be shared.  The O(m) selection state (weights,
+// diagonal) is FP64, as in the streaming engine.  Once the live triangle fits into the shared memory of the pending
+// vectors, the row finishes on chip with step-by-step updates.
 //
 // Shares of rows.  When a launch has more rows than resident blocks and the rows do not divide evenly, whole waves
 // would leave most SMs idle through the last one.  Instead every block gets the same amount of work: the rows
