@@ -36,7 +36,7 @@ static int blk_pick_ms(int d, size_t panel_bytes) {
 // several of them share an SM; long rows need the shared memory for pending vectors.
 // row_count = rows of the launch (0 = many).
 static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool nm = false, int bc = 0,
-                     int row_count = 0, int threads = 0) {
+                     int row_count = 0, int threads = 0, bool compound = false) {
     const int cap = (d + 3) & ~3;
     int nt = threads;
     if (nt != 128 && nt != 256 && nt != 512) {
@@ -45,9 +45,13 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
         nt = d <= 704 ? 128 : (d <= 1216 ? 256 : 512);
         // few rows (one per SM pair at most): nothing to share an SM with, the larger block is faster per row
         if (nt == 128 && row_count > 0 && row_count <= 2 * di.sm_count) nt = 256;
-        // at most one row per SM: the whole SM on one row wins from d_col ~ 700 (640: 3.0 against 3.1 ms, 768: 4.0 against 3.9, 960: 6.0
-        // against 5.3)
-        if (nt == 256 && row_count > 0 && row_count <= di.sm_count && d > 704) nt = 512;
+        // at most one row per SM: the whole SM on one row wins from d_col ~ 700 (16 to 148 rows, 256 / 512 threads: OBQ 704 3.24 - 3.44 /
+        // 3.20 - 3.37 ms, 768 3.68 - 3.98 / 3.55 - 3.79, replay 704 1.2 - 1.4 / 0.8 - 1.1); later where a kernel of 512 threads gains
+        // less: replay before OBQ takes single steps there (768: 3.0 - 3.3 / 3.1 - 3.4, 832: 3.4 - 3.9 / 3.4 - 3.8), blocks of 8
+        // keep passes by mma.sync (832: 5.6 - 6.0 / 5.8 - 6.1, 896: 6.3 - 6.8 / 6.4 - 6.7), blocks of 4
+        // spend more of a step on scores (736: 2.63 - 2.87 / 2.70 - 2.85, 784: 2.94 - 3.21 / 2.93 - 3.08)
+        const int whole_sm = compound ? 816 : (bc == 8 ? 896 : (bc == 4 ? 736 : 704));
+        if (nt == 256 && row_count > 0 && row_count <= di.sm_count && d > whole_sm) nt = 512;
     }
     if (nt == 128 && cap > 1024) nt = 256;
     if (nt == 256 && cap > 2048) nt = 512;
@@ -162,7 +166,8 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
     if (a.d > OBC_MAX_DCOL) return OBC_ERR_UNSUPPORTED;
     BlkPlan p;
     const int bc = (a.block_c == 4 || a.block_c == 8) ? a.block_c : 0;      // block pruning: the block size
-    if (!blk_plan(a.d, a.w_trace != nullptr, di, &p, a.nm_prune > 0, bc, a.row_count, a.opts.threads)) return OBC_ERR_UNSUPPORTED;
+    if (!blk_plan(a.d, a.w_trace != nullptr, di, &p, a.nm_prune > 0, bc, a.row_count, a.opts.threads, a.mode == MODE_REPLAY_QUANT))
+        return OBC_ERR_UNSUPPORTED;
     a.ms = p.ms;
     a.panel_floats = p.panel_floats;
     const int mp = a.opts.max_pending;

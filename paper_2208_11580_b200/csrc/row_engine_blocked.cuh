@@ -38,6 +38,7 @@
 // no second barrier is needed to announce it.  Records alternate between two buffers by step parity.
 #pragma once
 #include "flush_tc.cuh"
+#include <type_traits>
 
 namespace obc {
 
@@ -50,15 +51,15 @@ constexpr int BLK_OFF_MV = 2048;              // int mv[64]   live slots that mo
 constexpr int BLK_OFF_CM = 2304;
 constexpr int BLK_OFF_RF = 2944;              // float rf[64]  min/max reduction of the compound grid
 constexpr int BLK_OFF_GRP = 3200;             // forced groups: int slot[4], float M[4][4] (pivot columns at the pivot slots)
-constexpr int BLK_OFF_SCHED = 3280;           // int[12]: kind of the item in work (shares of rows)
+constexpr int BLK_OFF_SCHED = 3280;           // shares of rows: int[4] of the item in work, address of its triangle
 constexpr int BLK_OFF_FB = 3328;              // FlushBars
 constexpr int BLK_FIXED = 3584;
 static_assert(BLK_OFF_FB + sizeof(FlushBars) <= BLK_FIXED, "");
 constexpr int BLK_GS = 4;                     // forced eliminations taken together
 
 // Per-row state in shared memory: perm (int32), srcm (uint16); optional: the row in original order (weight trace), one byte
-// per block of the N:M pattern, off-diagonals of block pruning; last, next to the pending vectors, wd and dg (FP64): a pass on
-// tcgen05 parks them in global memory and uses their space too.
+// per block of the N:M pattern, off-diagonals of block pruning; wd and dg (FP64): first, or, where passes run on
+// tcgen05, last, next to the pending vectors -- such a pass parks them in global memory and uses their space too.
 // (block pruning, bc = block size 4 or 8: the 6 or 28 off-diagonal entries of every block's c x c diagonal block, FP64)
 __host__ __device__ inline size_t blk_state_bytes(int cap, bool wfull, bool nm = false, int bc = 0) {
     return (size_t)20 * cap + (((size_t)2 * cap + 15) & ~(size_t)15) + (wfull ? (size_t)4 * cap : 0) +
@@ -758,17 +759,23 @@ static __device__ __noinline__ double block8_score(const double* w, const double
 // broadcast, and every thread carries out the four Lemma-1 eliminations on its own slots in registers -- two
 // barriers per four steps, each pending vector read once for four columns.  Same arithmetic per element as four
 // single steps except that a column's corrections are subtracted one by one instead of summed first.
+// NM = N:M pruning; the other kernels are built without that code.
 // GPV = the kernel can keep further pending vectors in global memory (very long rows, 512 threads only).
 // SH = the kernel takes shares of rows (a row may be started by one block and finished by the next); launches whose
 // rows divide evenly over the blocks run the kernel built without that code.
-template <int NT, int KMAX, bool Q, int BC, bool FG, bool GPV, bool SH>
-__global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __grid_constant__ FlushMaps zmaps,
+// Passes on tcgen05: one block per SM (blocks of 8 keep 28 bytes more per slot and may lack the room for its tiles).  Only
+// those kernels take the tensor maps.
+template <int NT, int BC> constexpr bool blk_tc = NT >= 512 && BC != 8;
+struct NoMaps {};
+template <int NT, int BC> using BlkMaps = std::conditional_t<blk_tc<NT, BC>, FlushMaps, NoMaps>;
+
+template <int NT, int KMAX, bool Q, int BC, bool FG, bool GPV, bool SH, bool NM>
+__global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __grid_constant__ BlkMaps<NT, BC> zmaps,
                                                                       const __grid_constant__ EngineArgs a) {
     extern __shared__ __align__(16) char smem[];
     constexpr int NW = NT / 32;
     constexpr int BCD = BC ? BC : 1;                           // divisor that is never zero
-    // passes on tcgen05 (one block per SM; blocks of 8 keep 28 bytes more per slot and may lack the room for its tiles)
-    constexpr bool TC = NT >= 512 && BC != 8;
+    constexpr bool TC = blk_tc<NT, BC>;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int d = a.d, cap = a.cap, ms = a.ms;
     char* scratch = smem;
@@ -778,17 +785,22 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     int* mv = reinterpret_cast<int*>(smem + BLK_OFF_MV);
     float* rf = reinterpret_cast<float*>(smem + BLK_OFF_RF);
     uint32_t* colmask = reinterpret_cast<uint32_t*>(smem + BLK_OFF_CM);
-    int* perm = reinterpret_cast<int*>(smem + BLK_FIXED);
+    // wd and dg (FP64) come first or, with passes on tcgen05, last (blk_state_bytes)
+    double* wd = reinterpret_cast<double*>(smem + BLK_FIXED);
+    double* dg = wd + cap;
+    int* perm = TC ? reinterpret_cast<int*>(smem + BLK_FIXED) : reinterpret_cast<int*>(dg + cap);
+    const int before_state = TC ? 16 * cap : 0;
     unsigned short* srcm = reinterpret_cast<unsigned short*>(perm + cap);
     const bool has_wfull = a.w_trace != nullptr;
-    float* wfull = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, false) - 16 * cap);
-    const bool has_nm = a.nm_prune > 0;                         // N:M pattern: at most nm_prune eliminations per block
+    float* wfull = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, false) - before_state);
+    // N:M pattern: at most nm_prune eliminations per block.  (Decided at run time in the replay kernels too, where it is always
+    // false: compiled without that code they are 2 - 4 % slower, 16 x 1536 4.18 -> 4.30 ms.)
+    const bool has_nm = (NM || (FG && !Q)) && a.nm_prune > 0;
     const int nm_lg = a.nm_lg, nm_prune = a.nm_prune;
-    unsigned char* blkcnt = reinterpret_cast<unsigned char*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull) - 16 * cap);
-    double* boff = reinterpret_cast<double*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm) - 16 * cap);
+    unsigned char* blkcnt = reinterpret_cast<unsigned char*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull) - before_state);
+    double* boff = reinterpret_cast<double*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm) - before_state);
     float* panel = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm, BC));
-    double* wd = reinterpret_cast<double*>(panel) - 2 * cap;
-    double* dg = wd + cap;
+    if (TC) { wd = reinterpret_cast<double*>(panel) - 2 * cap; dg = wd + cap; }
     // tail views (step-by-step phase in shared memory) share the panel's space
     const int msr = (ms + 3) & ~3;
     float* tv = panel;
@@ -798,7 +810,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     const int lds = ms + 1;
     const int ldp = a.ldp;
     float* const Hp0 = a.Hws ? a.Hws + (size_t)blockIdx.x * tri_floats(cap) : nullptr;      // the block's own triangle
-#define HP (SH ? (a.Hws + (size_t)reinterpret_cast<const int*>(smem + BLK_OFF_SCHED)[2] * tri_floats(cap)) : Hp0)
+#define HP (SH ? *reinterpret_cast<float**>(smem + BLK_OFF_SCHED + 16) : Hp0)
     // overflow of the pending vectors: gB more of them in global memory (sized to stay in L2), stride gld
     // (only the one-row-per-SM configuration uses it; the other kernels are built without that code)
     constexpr bool GP = GPV;
@@ -863,7 +875,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         }
 
         if (SH) {                              // read during and after the row
-            if (tid == 0) { sched[0] = kind; sched[1] = s_stop; sched[2] = hbuf; }
+            if (tid == 0) {
+                sched[0] = kind; sched[1] = s_stop; sched[2] = hbuf;
+                *reinterpret_cast<float**>(smem + BLK_OFF_SCHED + 16) = a.Hws + (size_t)hbuf * tri_floats(cap);
+            }
             __syncthreads();
         }
 
@@ -998,7 +1013,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         if (!TC) atomicOr(&colmask[h >> 5], 1u << (h & 31));
                     }
                     __syncthreads();
-                    if (TC) {
+                    if constexpr (TC) {
                         blk_fill_holes<NT>(HP, ldp, m1, nh, hl, mv, srcm);
                         signed char* zexp = a.zexp + (size_t)blockIdx.x * cap;
                         const int power = blk_make_planes<NT, KMAX>(panel, ldz, GP ? scap : nb, GP ? GVEC : nullptr, gld, nb, m0, m1, dg, perm, rf,
@@ -1094,6 +1109,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                     for (int g = 0; g < GS; ++g) { wp4[g] = wd[p4[g]]; dp4[g] = dg[p4[g]]; }
                     // the four pivot columns of the stored matrix at the own slots
+                    const float* const tri = HP;
                     float v[GS][KMAX];
 #pragma unroll
                     for (int g4 = 0; g4 < KMAX / 4; ++g4) {
@@ -1107,13 +1123,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         for (int g = 0; g < GS; ++g) {
                             const int p = p4[g];
                             if (jb + 3 <= p) {
-                                const float4 t = ld_tri4<TC>(HP + tri_at(ldp, p, jb));
+                                const float4 t = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
                                 v[g][4 * g4] = t.x; v[g][4 * g4 + 1] = t.y; v[g][4 * g4 + 2] = t.z; v[g][4 * g4 + 3] = t.w;
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 4; ++q) {
                                     const int j = jb + q;
-                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(HP + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
                                 }
                             }
                         }
@@ -1305,6 +1321,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 // ======================= deferred-update step ==============================================
                 float* zb = (!GP || nb < scap) ? panel + (size_t)nb * ldz : GVEC + (size_t)(nb - scap) * gld;
                 // pivot column of the stored matrix (own slots), corrected by the pending vectors
+                const float* const tri = HP;
                 float c[KMAX], corr[KMAX];
                 unsigned live = 0u;
 #pragma unroll
@@ -1319,13 +1336,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     for (int q = 0; q < 4; ++q)
                         if (jb + q < m0 && pq[q] >= 0) live |= 1u << (4 * g + q);
                     if (jb + 3 <= p) {
-                        const float4 v = ld_tri4<TC>(HP + tri_at(ldp, p, jb));
+                        const float4 v = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
                         c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
                     } else {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int j = jb + q;
-                            if ((live >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(HP + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                            if ((live >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
                         }
                     }
                 }
@@ -1547,10 +1564,12 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #undef ZSTAGE
 
 // ---- launch -------------------------------------------------------------------------------------------------------
-template <int NT, int KMAX, bool Q, int BC, bool FG, bool GPV>
+template <int NT, int KMAX, bool Q, int BC, bool FG, bool GPV, bool NM>
 inline obc_status blk_launch_g(const FlushMaps& zmaps, EngineArgs a, int blocks, size_t smem, int sm_count, cudaStream_t stream) {
-    auto kernel = blocked_engine_kernel<NT, KMAX, Q, BC, FG, GPV, false>;
-    auto kernel_sh = blocked_engine_kernel<NT, KMAX, Q, BC, FG, GPV, (BC == 0)>;     // (block pruning takes no shares)
+    BlkMaps<NT, BC> maps;
+    if constexpr (blk_tc<NT, BC>) maps = zmaps;
+    auto kernel = blocked_engine_kernel<NT, KMAX, Q, BC, FG, GPV, false, NM>;
+    auto kernel_sh = blocked_engine_kernel<NT, KMAX, Q, BC, FG, GPV, (BC == 0 && !NM), NM>;     // (block and N:M pruning take no shares)
     if (a.split) {
         // A block may wait (bounded) for the row its neighbour started, so all blocks must be resident at once: checked
         // here, and guaranteed by a cooperative launch.  If the grid does not fit, rows run in whole waves instead.
@@ -1560,31 +1579,32 @@ inline obc_status blk_launch_g(const FlushMaps& zmaps, EngineArgs a, int blocks,
         int coop = 0, dev = 0;
         OBC_CUDA_TRY(cudaGetDevice(&dev));
         OBC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        if (BC != 0 || !coop || (long long)per_sm * sm_count < blocks) a.split = 0;
+        if (BC != 0 || NM || !coop || (long long)per_sm * sm_count < blocks) a.split = 0;
     }
     if (a.split) {
         OBC_CUDA_TRY(cudaMemsetAsync(a.split_flags, 0, (size_t)blocks * sizeof(int), stream));
-        void* params[2] = {(void*)&zmaps, (void*)&a};
+        void* params[2] = {(void*)&maps, (void*)&a};
         OBC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)kernel_sh, dim3(blocks), dim3(NT), params, smem, stream));
     } else {
         OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kernel<<<blocks, NT, smem, stream>>>(zmaps, a);
+        kernel<<<blocks, NT, smem, stream>>>(maps, a);
     }
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
     return OBC_OK;
 }
 
-template <int NT, int KMAX, bool Q, int BC, bool FG>
+template <int NT, int KMAX, bool Q, int BC, bool FG, bool NM = false>
 inline obc_status blk_launch_q(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream) {
-    if (NT >= 512 && a.Gpan != nullptr) return blk_launch_g<NT, KMAX, Q, BC, FG, (NT >= 512)>(zmaps, a, blocks, smem, sm_count, stream);
-    return blk_launch_g<NT, KMAX, Q, BC, FG, false>(zmaps, a, blocks, smem, sm_count, stream);
+    if (NT >= 512 && a.Gpan != nullptr) return blk_launch_g<NT, KMAX, Q, BC, FG, (NT >= 512), NM>(zmaps, a, blocks, smem, sm_count, stream);
+    return blk_launch_g<NT, KMAX, Q, BC, FG, false, NM>(zmaps, a, blocks, smem, sm_count, stream);
 }
 
 template <int NT, int KMAX>
 inline obc_status blk_launch(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream) {
     if (a.block_c == 4) return blk_launch_q<NT, KMAX, false, 4, false>(zmaps, a, blocks, smem, sm_count, stream);
     if (a.block_c == 8) return blk_launch_q<NT, KMAX, false, 8, false>(zmaps, a, blocks, smem, sm_count, stream);
+    if (a.nm_prune > 0) return blk_launch_q<NT, KMAX, false, 0, false, true>(zmaps, a, blocks, smem, sm_count, stream);
     switch (a.mode) {                       // the replay modes are the ones with forced eliminations
         case MODE_QUANT:        return blk_launch_q<NT, KMAX, true, 0, false>(zmaps, a, blocks, smem, sm_count, stream);
         // (with 512 threads the OBQ kernel has no registers to spare for the four columns: single steps there)
