@@ -57,7 +57,10 @@ __host__ __device__ inline void grid_from_range(float lo, float hi, int bits, in
 }
 
 // The per-call engine options of obc_engine_opts after validation (all zero = defaults).
-struct EngineOpts { int engine; int threads; int max_pending; int flags; };
+struct EngineOpts {
+    int engine; int threads; int max_pending; int flags;
+    int wait_limit = 0;      // polls of the waits inside a pass: 0 = the built-in limit, < 0 = they expire at once (tests; not in the C ABI)
+};
 
 // ---- launchers implemented in the kernel files --------------------------------------------------------------
 size_t engine_workspace_bytes(int row_count, int d, const DeviceInfo& di);

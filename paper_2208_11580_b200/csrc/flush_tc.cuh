@@ -21,8 +21,8 @@
 // small products are added first, and the groups are added in FP32 round-to-nearest with the last mantissa bit of each
 // set, which turns "truncated" into "right on average" (+0.07; +0.15 after three chained products).
 //
-// Every wait is bounded.  When one expires the block abandons the pass -- the issuing threads wait for their copies and
-// products in flight -- and the row is reported with -OBC_ERR_TIMEOUT.
+// Every wait is bounded.  When one expires the block abandons the pass: once all its threads have stopped, the issuing ones wait
+// (with the built-in limit) for their copies and products in flight, and the row is reported with -OBC_ERR_TIMEOUT.
 #pragma once
 #include "engine.cuh"
 #include "tensor_map.cuh"
@@ -78,8 +78,8 @@ __device__ __forceinline__ bool ft_test(unsigned long long* b, int parity) {
     return ok != 0;
 }
 // false when the limit is reached or another thread of the block has given up
-__device__ __forceinline__ bool ft_wait(unsigned long long* b, int parity, FlushBars* fb) {
-    for (int i = 0; i < FT_WAIT_LIMIT; ++i) {
+__device__ __forceinline__ bool ft_wait(unsigned long long* b, int parity, FlushBars* fb, int limit) {
+    for (int i = 0; i < limit; ++i) {
         if (ft_test(b, parity)) return true;
         if ((i & 15) == 15) {
             if (*(volatile int*)&fb->abort) return false;
@@ -187,7 +187,7 @@ struct Ring {
     __device__ __forceinline__ void next(int n) { if (++at == n) { at = 0; ++round; } }
 };
 struct FlushGeom {                                // of a pass
-    const FlushMaps* maps; int plane, buf, G, T, m1; FlushBufs nb; uint32_t sa, sb, sh, tmem;
+    const FlushMaps* maps; int plane, buf, G, T, m1, limit; FlushBufs nb; uint32_t sa, sb, sh, tmem;
 };
 // The parts of tile (rb, c) that hold data, each as f(map, 32-column group, first row inside the tile): the whole tile
 // below the diagonal, on it the 32 x 32 parts that reach it.
@@ -203,7 +203,7 @@ __device__ __forceinline__ void ft_parts(const FlushGeom& q, int rb, int c, F f)
 }
 // Copies of the tile of H at (rb, c).  One thread.
 __device__ __forceinline__ bool ft_copy_tile(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
-    if (h.round > 0 && !ft_wait(&fb->free_h[h.at], (h.round - 1) & 1, fb)) return false;
+    if (h.round > 0 && !ft_wait(&fb->free_h[h.at], (h.round - 1) & 1, fb, q.limit)) return false;
     uint32_t bytes = FT_TILE_BYTES;
     if (c >= rb * FT_M) { bytes = 0; ft_parts(q, rb, c, [&](const CUtensorMap*, int, int) { bytes += 32 * 128; }); }
     ft_expect(&fb->full_h[h.at], bytes);
@@ -219,12 +219,12 @@ __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* 
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;    // both planes of 64 slots
     const CUtensorMap* zm = &q.maps->z[q.G - 1];
     if (rb == c / FT_M) {
-        if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
+        if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb, q.limit)) return false;
         ft_expect(&fb->full_b[b.at], blk);
         ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
         b.next(q.nb.n_b);
     }
-    if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb)) return false;
+    if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb, q.limit)) return false;
     ft_expect(&fb->full_a[a.at], 2 * blk);
     ft_load(q.sa + a.at * 2 * blk, zm, &fb->full_a[a.at], rb * FT_M, 0, q.plane);
     ft_load(q.sa + (a.at * 2 + 1) * blk, zm, &fb->full_a[a.at], rb * FT_M + 64, 0, q.plane);
@@ -235,9 +235,9 @@ __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* 
 __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, int t, Ring& b, Ring& a, bool first, bool last) {
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;
     const int buf = t & 1;
-    if (first && !ft_wait(&fb->full_b[b.at], b.round & 1, fb)) return false;
-    if (!ft_wait(&fb->full_a[a.at], a.round & 1, fb)) return false;
-    if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb)) return false;
+    if (first && !ft_wait(&fb->full_b[b.at], b.round & 1, fb, q.limit)) return false;
+    if (!ft_wait(&fb->full_a[a.at], a.round & 1, fb, q.limit)) return false;
+    if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb, q.limit)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint64_t da = ft_desc(q.sa + a.at * 2 * blk, blk), db = ft_desc(q.sb + b.at * blk, blk);
     const uint32_t d = q.tmem + buf * (FT_GMAX * FT_N);
@@ -255,16 +255,20 @@ __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, i
     if (last) { ft_commit(&fb->free_b[b.at]); b.next(q.nb.n_b); }
     return true;
 }
-// The products of `tiles` tiles (of all, if it is q.T: then in `blocks` column blocks) and all that they signal are over.
-__device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* fb, int tiles, int blocks) {
-    if (tiles <= 0) return;
-    ft_drain(&fb->done[(tiles - 1) & 1], ((tiles - 1) >> 1) & 1);
-    ft_drain(&fb->free_a[(tiles - 1) % q.nb.n_a], ((tiles - 1) / q.nb.n_a) & 1);
-    if (tiles == q.T) ft_drain(&fb->free_b[(blocks - 1) % q.nb.n_b], ((blocks - 1) / q.nb.n_b) & 1);
+// The last n uses of a ring of `len` barriers are over (all of them, if there were fewer).
+__device__ __forceinline__ void ft_ring_over(unsigned long long* bars, Ring r, int len, int n) {
+    const int used = r.round * len + r.at;
+    for (int x = max(0, used - n); x < used; ++x) ft_drain(&bars[x % len], (x / len) & 1);
+}
+// The products of `tiles` tiles and all that they signal are over; b, a: the operand rings as ft_multiply left them.
+__device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* fb, int tiles, Ring b, Ring a) {
+    if (tiles > 0) ft_drain(&fb->done[(tiles - 1) & 1], ((tiles - 1) >> 1) & 1);
+    ft_ring_over(fb->free_a, a, q.nb.n_a, 1);
+    ft_ring_over(fb->free_b, b, q.nb.n_b, 1);
 }
 // Takes the tile at (rb, c) back to memory once every warp has finished its part.  One thread (of all tiles).
 __device__ __forceinline__ bool ft_store(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
-    if (!ft_wait(&fb->ready[h.at], h.round & 1, fb)) return false;
+    if (!ft_wait(&fb->ready[h.at], h.round & 1, fb, q.limit)) return false;
     ft_parts(q, rb, c, [&](const CUtensorMap* m, int cg, int r) {
         ft_store_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, 0, rb * FT_M + r, q.buf + (c >> 5) + cg, pol);
     });
@@ -279,8 +283,8 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = hq.at, buf = t & 1;
     const int cg = warp >> 2, r0 = rb * FT_M + 32 * (warp & 3), col = c + 32 * cg;
-    bool ok = ft_wait(&fb->full_h[h], hq.round & 1, fb);
-    ok = ok && ft_wait(&fb->done[buf], (t >> 1) & 1, fb);
+    bool ok = ft_wait(&fb->full_h[h], hq.round & 1, fb, q.limit);
+    ok = ok && ft_wait(&fb->done[buf], (t >> 1) & 1, fb, q.limit);
     if (!__all_sync(0xffffffffu, ok)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool any = r0 < q.m1 && col <= r0;
@@ -331,11 +335,12 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
 // the copies, and the block has synchronised.
 //   plane     first of the block's two planes (hi, lo) in the maps
 //   unscale   2^-2e of the planes' power, or zexp: the slots' own powers
+//   limit     polls of a wait
 __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, int tri, unsigned char* stage, int stage_bytes, FlushBars* fb, int m1,
-                                             int nb, float unscale, const signed char* zexp) {
+                                             int nb, float unscale, const signed char* zexp, int limit) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FlushGeom q;
-    q.maps = maps; q.plane = plane; q.buf = tri; q.m1 = m1;
+    q.maps = maps; q.plane = plane; q.buf = tri; q.m1 = m1; q.limit = limit;
     q.G = (nb + 15) >> 4;
     q.nb = ft_bufs(q.G, stage_bytes);
     q.sh = ft_smem(stage);
@@ -357,19 +362,10 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
             if (!ft_copy_tile(q, fb, h, rb, c, pol)) break;
             ft_next_tile(rb, c, m1);
         }
-        if (*(volatile int*)&fb->abort) {             // nothing may land after the block has moved on
-            const int n = h.round * q.nb.n_h + h.at;
-            for (int x = max(0, n - q.nb.n_h); x < n; ++x) ft_drain(&fb->full_h[x % q.nb.n_h], (x / q.nb.n_h) & 1);
-        }
     } else if (warp == FT_EW + 3 && lane == 0) {
         for (; t < q.T; ++t) {
             if (!ft_copy_operands(q, fb, b, a, rb, c)) break;
             ft_next_tile(rb, c, m1);
-        }
-        if (*(volatile int*)&fb->abort) {
-            const int n = b.round * q.nb.n_b + b.at, na = a.round * q.nb.n_a + a.at;
-            for (int x = max(0, n - q.nb.n_b); x < n; ++x) ft_drain(&fb->full_b[x % q.nb.n_b], (x / q.nb.n_b) & 1);
-            for (int x = max(0, na - q.nb.n_a); x < na; ++x) ft_drain(&fb->full_a[x % q.nb.n_a], (x / q.nb.n_a) & 1);
         }
     } else if (warp == FT_EW + 1 && lane == 0) {
         for (; t < q.T; ++t) {
@@ -378,7 +374,6 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
             if (!ft_multiply(q, fb, t, b, a, rb == c / FT_M, nc != c)) break;
             rb = nrb; c = nc;
         }
-        ft_products_over(q, fb, t, (m1 + FT_N - 1) / FT_N);
     } else if (warp == FT_EW + 2 && lane == 0) {
         const uint64_t pol = ft_stream_policy();
         for (; t < q.T; ++t) {
@@ -389,7 +384,18 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
     }
     __syncwarp();
     __syncthreads();
+    // Nothing may land or be signalled after the block has moved on.  The products' last signals may be under way in any case; copies
+    // are all consumed unless the pass was abandoned, which is only certain now: another thread's wait may have expired
+    // after this one's last copy.
     const bool aborted = *(volatile int*)&fb->abort != 0;
+    if (warp == FT_EW + 1 && lane == 0) ft_products_over(q, fb, t, b, a);
+    if (aborted && warp == FT_EW && lane == 0) ft_ring_over(fb->full_h, h, q.nb.n_h, q.nb.n_h);
+    if (aborted && warp == FT_EW + 3 && lane == 0) {
+        ft_ring_over(fb->full_b, b, q.nb.n_b, q.nb.n_b);
+        ft_ring_over(fb->full_a, a, q.nb.n_a, q.nb.n_a);
+    }
+    __syncwarp();
+    __syncthreads();
     asm volatile("fence.proxy.async;" ::: "memory");  // the copies' writes before the plain accesses that follow
     if (threadIdx.x == 0) ft_inval_bars(fb);
     __syncthreads();

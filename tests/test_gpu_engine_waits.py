@@ -1,0 +1,98 @@
+"""Bounded waits that run out on purpose: the pipeline of a pass on tcgen05, the 256 x 256 tiles of the Hessian and the cross product.
+Nothing hangs and nothing faults: a limit of -1 lets every wait expire at once, a few polls let some of them expire at any point of
+a pass.  The call returns, the failure is reported, and the next ordinary call is right."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+OBC_ERR_TIMEOUT = 6
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def shim(tmp_path_factory):
+    import paper_2208_11580_b200 as m
+    m.load_library()
+    out = str(tmp_path_factory.mktemp("shim") / "wait_limit_shim.so")
+    pkg = os.path.dirname(m.library_path())
+    subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", "-O1", "-o", out, os.path.join(HERE, "wait_limit_shim.cpp"), "-I", os.path.join(pkg, "csrc"),
+                           "-I", os.path.join(os.path.dirname(pkg), "include"), "-I", "/usr/local/cuda/include", m.library_path()])
+    return m, ctypes.CDLL(out)
+
+
+def pointer(t):
+    return ctypes.c_void_p(t.data_ptr())
+
+
+def spd(d, g):
+    X = torch.randn(d, 2 * d, device="cuda", generator=g, dtype=torch.float64)
+    H = X @ X.T
+    H.diagonal().add_(0.01 * H.diagonal().mean())
+    return torch.cholesky_inverse(torch.linalg.cholesky(H))
+
+
+# a few tiles / rows handed over between blocks / pending vectors in global memory, the smallest rings
+@pytest.mark.parametrize("rows,d", [(5, 600), (1, 261), (161, 520), (3, 4200)])
+def test_pass_that_runs_out_of_time(shim, rows, d):
+    m, lib = shim
+    g = torch.Generator(device="cuda").manual_seed(d)
+    inv = spd(d, g)
+    Hinv, W = ((inv + inv.T) / 2).float().contiguous(), torch.randn(rows, (d + 3) // 4 * 4, device="cuda", generator=g)
+    if d % 4:
+        pad = torch.zeros(d, W.shape[1], device="cuda")
+        pad[:, :d] = Hinv
+        Hinv = pad
+    ws = torch.empty(m.obc_workspace_bytes(m.OP_PRUNE_TRACE, rows, d), dtype=torch.uint8, device="cuda")
+
+    def call(limit):
+        order = torch.full((rows, d), -7, dtype=torch.int32, device="cuda")
+        loss, st = torch.zeros(rows, d, device="cuda"), torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+        rc = lib.shim_prune_trace(pointer(W), W.shape[1], rows, d, pointer(Hinv), Hinv.shape[1], pointer(order), pointer(loss), pointer(st), pointer(ws),
+                                  ctypes.c_size_t(ws.numel()), 512, limit, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+        torch.cuda.synchronize()
+        return order, loss, st
+
+    want = call(0)
+    assert int(want[2].abs().sum()) == 0
+    for limit in (-1, 1, 2, 5, 20, 100, 400):
+        order, loss, st = call(limit)
+        late = st == -OBC_ERR_TIMEOUT
+        assert bool((late | (st == 0)).all())
+        if limit < 0:
+            assert bool(late.all())
+        assert torch.equal(order[~late], want[0][~late]) and torch.equal(loss[~late], want[1][~late])
+        assert bool((order[late][:, -1] == -1).all()) and bool(torch.isinf(loss[late][:, -1]).all())      # what was not produced
+        assert torch.equal(torch.where(order[late] == -1, want[0][late], order[late]), want[0][late])         # what was, before
+        again = call(0)
+        assert all(torch.equal(a, b) for a, b in zip(again, want))
+
+
+def test_large_hessian_tiles_that_run_out_of_time():
+    import paper_2208_11580_b200 as m
+    d, n = 2304, 1500
+    X = torch.randn(d, n, device="cuda")
+    H, info = torch.zeros(d, d, device="cuda"), torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    want = 2 * X.double() @ X.double().T
+    for limit in (-1, 0, 3, 0):
+        m.obc_hessian(X, H, prec=m.PREC_BF16X3, info=info, wait_limit=limit)
+        late = int(info.item())
+        assert late == {-1: OBC_ERR_TIMEOUT, 0: 0}.get(limit, late)
+        assert bool(torch.isnan(H).all()) if late else float((H.double() - want).abs().max() / want.abs().max()) <= 3e-5
+
+
+def test_large_cross_product_tiles_that_run_out_of_time():
+    import paper_2208_11580_b200 as m
+    r, d, n = 1536, 2048, 1500
+    Y, X = torch.randn(r, n, device="cuda"), torch.randn(d, n, device="cuda")
+    G, info = torch.zeros(r, d, device="cuda"), torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    want = Y.double() @ X.double().T
+    for limit in (-1, 0, 3, 0):
+        m.obc_cross_gram(Y, X, G, prec=m.PREC_BF16X3, info=info, wait_limit=limit)
+        late = int(info.item())
+        assert late == {-1: OBC_ERR_TIMEOUT, 0: 0}.get(limit, late)
+        assert bool(torch.isnan(G).all()) if late else float((G.double() - want).abs().max() / want.abs().max()) <= 3e-5
