@@ -11,8 +11,9 @@
 //
 // Operands.  Before the pass every pending vector is written as two FP16 planes, z * 2^e = hi + lo (hi rounded to 11 bits, lo
 // the rounded rest: 22 significant bits), to global memory (they stay in L2).  The power of two takes the largest entry to
-// [2^13, 2^14); lo then has an absolute error of 2^-39 of that entry.  Where the live diagonal spans more than 2^24 every slot has
-// a power of its own (zexp), so that small rows of the matrix keep their own precision.  lo*hi + hi*lo + hi*hi is formed; the
+// [2^13, 2^14); an entry's error is then 2^-23 of itself or, where lo is subnormal, 2^-39 of the largest entry.  Where the diagonal
+// (the live one, or the squares of the largest entries) spans more than 2^24 every slot has a power of its own (zexp), so that
+// small rows of the matrix keep their own precision.  lo*hi + hi*lo + hi*hi is formed; the
 // missing lo*lo is below 2^-22 of a product.  Boxes of 16 G vectors x 64 slots go into 128B-swizzled shared memory as
 // MN-major operands.
 //

@@ -626,7 +626,9 @@ __device__ __forceinline__ int blk_make_planes(const float* panel, int ldz, int 
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NW; ++w) { zmax = fmaxf(zmax, rf[w]); dmax = fmaxf(dmax, rf[NW + w]); dmin = fminf(dmin, rf[2 * NW + w]); }
-    const bool wide = dmin < dmax * 5.9604645e-8f;             // 2^-24
+    // the planes hold vectors of the diagonal before the pending eliminations: zmax^2 is what it had been (at least) where it has
+    // collapsed since
+    const bool wide = dmin < fmaxf(dmax, zmax * zmax) * 5.9604645e-8f;             // 2^-24
     const int power = plane_power(zmax);
     const int nb16 = (nb + 15) & ~15;
 #pragma unroll

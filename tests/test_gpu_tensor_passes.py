@@ -33,3 +33,33 @@ def test_passes_against_oracle(d, pending, wide):
     torch.cuda.synchronize()
     assert int(status.abs().sum()) == 0
     check_rows(Hd.cpu().numpy(), Wd.cpu().numpy(), order.cpu().numpy(), loss.cpu().numpy())
+
+
+def test_diagonal_that_collapses_before_the_pass():
+    """Two slots with diagonal 2^41 and correlation 1 - 2^-20: once the first is eliminated the other has 2^22 left, within 2^24 of the
+    rest (about 1), but its entry of the pending vector is still 2^20.5.  A common power of two for that entry would lose the
+    others' (about 2^-21); the products of the two are what the survivor's column is made of."""
+    import paper_2208_11580_b200 as obc
+    d, T, eps = 300, 2.0 ** 41, 2.0 ** -20
+    rng = np.random.default_rng(3)
+    _, X = obc_synth.make_small(1, d - 2, 3 * d, 9, "relu")
+    A, info = oracle.inverse(oracle.hessian(X), obc_synth.DAMP_REL)
+    assert info == 0
+    Hinv = np.zeros((d, d))
+    Hinv[2:, 2:] = A / np.diag(A).mean()
+    Hinv[:2, :2] = T * np.array([[1, 1 - eps], [1 - eps, 1]])
+    u = rng.standard_normal(d - 2)
+    u *= 0.2 * np.sqrt(T * eps * np.linalg.eigvalsh(Hinv[2:, 2:])[0]) / np.linalg.norm(u)
+    Hinv[0, 2:] = Hinv[2:, 0] = u
+    Hinv[1, 2:] = Hinv[2:, 1] = -u
+    W = rng.standard_normal((2, d))
+    W[:, 0], W[:, 1] = 0.0, 1400.0                  # the first goes at once, the second in the middle of the row
+    Hd, Wd = torch.from_numpy(Hinv.astype(np.float32)).cuda(), torch.from_numpy(W.astype(np.float32)).cuda()
+    order = torch.full((2, d), -7, dtype=torch.int32, device="cuda")
+    loss, status = torch.zeros(2, d, device="cuda"), torch.full((2,), -7, dtype=torch.int32, device="cuda")
+    obc.obc_prune_trace(Wd, Hd, order, loss, status, opts=obc.engine_opts(obc.ENGINE_BLOCKED, 512, 0))
+    torch.cuda.synchronize()
+    assert int(status.abs().sum()) == 0
+    P = order.cpu().numpy()
+    assert (P[:, 0] == 0).all() and (np.argwhere(P == 1)[:, 1] > 48).all()
+    check_rows(Hd.cpu().numpy(), Wd.cpu().numpy(), P, loss.cpu().numpy())
