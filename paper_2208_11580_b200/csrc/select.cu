@@ -193,6 +193,32 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                         }
                     }
                 }
+            } else if (!IN_SMEM) {
+                // What is left of a row may be long here (rows of equal or almost equal losses).  Its keys do not decrease, so of 32 keys
+                // in a row only the ends are read unless their digits differ.
+                for (int u = warp; u < units; u += SEL_WARPS) {
+                    const int r = u / segs, g = u - r * segs;
+                    const unsigned int* K = keys + (size_t)r * ldk;
+                    const int b = row_lt[r], e = row_le[r];
+                    auto digit = [&](int t) { return t < e ? (int)((K[t] >> shift) & dmask) : -1; };
+                    for (int64_t p0 = (int64_t)b + (int64_t)g * 1024; p0 < e; p0 += (int64_t)segs * 1024) {
+                        const int x = (int)min(p0 + 32 * lane, (int64_t)e), y = min(e - x, 32) + x;      // this lane's piece
+                        const int f = digit(x), last = x < e ? digit(y - 1) : -1, fn = digit(y);
+                        if (x == b && b > 0) atomicAdd(&sh.hist[f], 0u - (unsigned int)b);
+                        if (x < e && f == last && last != fn) {
+                            atomicAdd(&sh.hist[f], (unsigned int)y);
+                            if (fn >= 0) atomicAdd(&sh.hist[fn], 0u - (unsigned int)y);
+                        }
+                        for (unsigned int todo = __ballot_sync(0xffffffffu, f != last); todo; todo &= todo - 1) {
+                            const int at = __shfl_sync(0xffffffffu, x, __ffs(todo) - 1), end = __shfl_sync(0xffffffffu, y, __ffs(todo) - 1);
+                            const int t = at + lane, h = t < end ? digit(t) : -1, hn = digit(t + 1);
+                            if (h >= 0 && h != hn) {
+                                atomicAdd(&sh.hist[h], (unsigned int)(t + 1));
+                                if (hn >= 0) atomicAdd(&sh.hist[hn], 0u - (unsigned int)(t + 1));
+                            }
+                        }
+                    }
+                }
             } else {
                 for (int u = warp; u < nr; u += SEL_WARPS) {      // what is left of a row is short: one warp per row
                     const unsigned int* K = keys + (size_t)u * ldk;
