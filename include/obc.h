@@ -207,7 +207,11 @@ obc_status obc_prune_blocks(const float *W, int ldw, int d_row, int d_col, int r
 /* Algorithm 2 (appendix, "ExactOBS Global Step"): repeatedly prune, across all rows, the weight whose
  * next recorded loss is smallest (ties: lowest row), k times.  k is a count, 0 <= k <= d_row*d_col.
  *   counts: d_row int32, weights pruned per row;  mask: d_row x d_col uint8, 0 at order[r][t], t < counts[r].
- * The result is exactly the sequential procedure's (computed as a selection over prefix-maximum keys). */
+ * The result is exactly the sequential procedure's (computed as a selection over prefix-maximum keys).
+ * One launch whose blocks wait for one another (bounded, about a second; they are resident together).  Should a wait expire
+ * all the same, rows of the blocks that gave up get counts[r] = -OBC_ERR_TIMEOUT and their mask is not written;
+ * obc_prune_apply and obc_quantize report rows with such a count in row_status[r] = -OBC_ERR_TIMEOUT (and prune
+ * nothing of them). */
 obc_status obc_select_global_mask(const float *loss, const int32_t *order, int d_row, int d_col, int64_t k,
                                   int32_t *counts, uint8_t *mask,
                                   void *ws, size_t ws_bytes, obc_stream stream);
@@ -236,7 +240,8 @@ obc_status obc_select_global_mask_static(const float *loss, const int32_t *order
 
 /* Section 3 / Figure 1: the weights of each row after its first counts[r] eliminations.
  * w_trace != NULL (layout of obc_prune_trace with this `trace_steps`): rows are gathered from the trace.
- * w_trace == NULL: the eliminations order[r][0..counts[r]) are replayed on W (no argmin). */
+ * w_trace == NULL: the eliminations order[r][0..counts[r]) are replayed on W (no argmin).
+ * counts[r] = -OBC_ERR_TIMEOUT (a global selection that gave up): the row's dense weights, row_status[r] = that value. */
 obc_status obc_prune_apply(const float *W, int ldw, int d_row, int d_col, int row_begin, int row_count,
                            const float *Hinv, int ldhi, const int32_t *order, const int32_t *counts,
                            const float *w_trace, int trace_steps,

@@ -215,7 +215,7 @@ obc_status obc_prune_apply(const float* W, int ldw, int d_row, int d_col, int ro
         return OBC_ERR_INVALID_ARG;
     if (w_trace) {
         if (trace_steps < 1 || trace_steps > d_col) return OBC_ERR_INVALID_ARG;
-        return trace_gather_launch(w_trace, trace_steps, counts, d_col, row_begin, row_count, W_out, ldwo,
+        return trace_gather_launch(w_trace, trace_steps, counts, d_col, row_begin, row_count, W_out, ldwo, row_status,
                                    (cudaStream_t)stream);
     }
     if (!mat_ok(W, ldw, d_col) || !mat_ok(Hinv, ldhi, d_col) || !order || !row_status) return OBC_ERR_INVALID_ARG;

@@ -62,13 +62,16 @@ struct EngineOpts {
     int wait_limit = 0;      // polls of the waits inside a pass: 0 = the built-in limit, < 0 = they expire at once (tests; not in the C ABI)
 };
 
+// What the global selection leaves in counts[] when its blocks could not meet: the calls that take counts report such rows.
+constexpr int COUNT_TIMED_OUT = -(int)OBC_ERR_TIMEOUT;
+
 // ---- launchers implemented in the kernel files --------------------------------------------------------------
 size_t engine_workspace_bytes(int row_count, int d, const DeviceInfo& di);
 size_t select_workspace_bytes(int rows, int d);
 size_t inverse_workspace_bytes(int d);
 size_t hessian_workspace_bytes(int d, int64_t n);
 obc_status select_launch(const float* loss, const int32_t* order, int rows, int d, int64_t k, int32_t* counts,
-                         uint8_t* mask, void* ws, cudaStream_t stream);
+                         uint8_t* mask, void* ws, cudaStream_t stream, int wait_limit = 0);      // (limit as in EngineOpts)
 obc_status inverse_launch(const float* H, int d, int ldh, float damp_rel, float* Hinv, int ldhi, int32_t* info,
                           void* ws, cudaStream_t s);
 obc_status hessian_fp32_launch(const float* X, int d, int64_t n, int64_t ldx, float* H, int ldh, int accumulate,
@@ -84,7 +87,7 @@ obc_status sgemm_nt_launch(int M, int N, int64_t K, float alpha, const float* A,
 obc_status minmax_grid_launch(const float* W, int ldw, int rows, int d, const uint8_t* mask, int bits, int symmetric,
                               float* scale, float* zero, cudaStream_t stream);
 obc_status trace_gather_launch(const float* w_trace, int trace_steps, const int32_t* counts, int d, int row_begin,
-                               int row_count, float* W_out, int ldwo, cudaStream_t stream);
+                               int row_count, float* W_out, int ldwo, int32_t* row_status, cudaStream_t stream);
 obc_status engine_prune_trace(const float* W, int ldw, int d_row, int d_col, int row_begin, int row_count,
                               const float* Hinv, int ldhi, int steps, int32_t* order, float* loss, float* w_trace,
                               int32_t* row_status, void* ws, size_t ws_bytes, const EngineOpts& eo, cudaStream_t stream);

@@ -54,6 +54,11 @@ __device__ __forceinline__ bool key_less(double s, int o, double s2, int o2) {
     return s < s2 || (s == s2 && o < o2);
 }
 
+// A row's status before its first step: a replay without a count (the global selection gave up) is reported.
+__device__ __forceinline__ int first_status(const EngineArgs& a, int r) {
+    return a.forced_counts && a.forced_counts[r] == COUNT_TIMED_OUT ? COUNT_TIMED_OUT : 0;
+}
+
 // q(x) on the uniform grid; all FP64 so that the integer code is decided in the same precision as the
 // FP64 reference decides it.
 __device__ __forceinline__ double grid_q(double x, double sc, double ze, double mq, double* code) {

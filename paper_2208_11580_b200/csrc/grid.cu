@@ -31,12 +31,14 @@ __global__ void __launch_bounds__(GRID_THREADS) minmax_grid_kernel(const float* 
     if (threadIdx.x == 0) grid_from_range(slo[0], shi[0], bits, symmetric, &scale[r], &zero[r]);
 }
 
-// W_out[r][:] = w_trace[r][counts[r]][:]      one block per row
+// W_out[r][:] = w_trace[r][counts[r]][:]      one block per row; row_status (nullable): written for rows without a count
 __global__ void __launch_bounds__(GRID_THREADS) trace_gather_kernel(const float* __restrict__ w_trace, int trace_steps,
                                                                     const int32_t* __restrict__ counts, int d,
-                                                                    int row_begin, float* __restrict__ W_out, int ldwo) {
+                                                                    int row_begin, float* __restrict__ W_out, int ldwo,
+                                                                    int32_t* __restrict__ row_status) {
     const int r = row_begin + blockIdx.x;
     int c = counts[r];
+    if (row_status && c == COUNT_TIMED_OUT && threadIdx.x == 0) row_status[r] = c;
     c = c < 0 ? 0 : (c > trace_steps ? trace_steps : c);
     const float* src = w_trace + ((size_t)r * (trace_steps + 1) + c) * d;
     for (int j = threadIdx.x; j < d; j += GRID_THREADS) W_out[(size_t)r * ldwo + j] = src[j];
@@ -51,8 +53,8 @@ obc_status minmax_grid_launch(const float* W, int ldw, int rows, int d, const ui
 }
 
 obc_status trace_gather_launch(const float* w_trace, int trace_steps, const int32_t* counts, int d, int row_begin,
-                               int row_count, float* W_out, int ldwo, cudaStream_t stream) {
-    trace_gather_kernel<<<row_count, GRID_THREADS, 0, stream>>>(w_trace, trace_steps, counts, d, row_begin, W_out, ldwo);
+                               int row_count, float* W_out, int ldwo, int32_t* row_status, cudaStream_t stream) {
+    trace_gather_kernel<<<row_count, GRID_THREADS, 0, stream>>>(w_trace, trace_steps, counts, d, row_begin, W_out, ldwo, row_status);
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
     return OBC_OK;

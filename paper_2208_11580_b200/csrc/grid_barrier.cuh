@@ -8,14 +8,15 @@ constexpr int GRID_BARRIER_LIMIT = 1 << 22;       // polls before a block gives 
 
 // `arrived` counts arrivals since the launch (zero before it); `target` = gridDim.x times the number of this barrier,
 // counted from 1.  Called by every thread of every block; false, for the whole block, when the others did not come in time.
-__device__ __forceinline__ bool grid_barrier(unsigned int* arrived, unsigned int target) {
+// `limit`: polls (GRID_BARRIER_LIMIT unless a test wants the wait to expire).
+__device__ __forceinline__ bool grid_barrier(unsigned int* arrived, unsigned int target, int limit) {
     __syncthreads();
     bool ok = true;
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(arrived, 1u);
         ok = false;
-        for (int i = 0; i < GRID_BARRIER_LIMIT && !ok; ++i) {
+        for (int i = 0; i < limit && !ok; ++i) {
             unsigned int v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
             ok = v >= target;

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(ENGINE_THREADS, 1) row_engine_kernel(const Eng
                 bc->sc = (double)a.scale[r]; bc->ze = (double)a.zero[r];
                 bc->mq = (double)grid_maxq(a.bits, a.symmetric);
             }
-            a.row_status[r] = 0;
+            a.row_status[r] = first_status(a, r);
         }
         if (a.w_trace)
             for (int j = tid; j < d; j += ENGINE_THREADS)

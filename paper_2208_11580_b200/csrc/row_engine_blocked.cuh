@@ -932,7 +932,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 bc->sc = (double)a.scale[r]; bc->ze = (double)a.zero[r];
                 bc->mq = (double)grid_maxq(a.bits, a.symmetric);
             }
-            a.row_status[r] = 0;
+            a.row_status[r] = first_status(a, r);
         }
         if (a.w_trace)
             for (int j = tid; j < d; j += NT)

@@ -92,7 +92,7 @@ template <bool IN_SMEM, typename Count>
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ loss, const int32_t* __restrict__ order, int rows, int d,
                                                              unsigned long long k, int rpb, int segs, unsigned int* __restrict__ gkeys,
                                                              int* __restrict__ glt, int* __restrict__ gle, SelectState* __restrict__ st,
-                                                             int* __restrict__ counts, uint8_t* __restrict__ mask) {
+                                                             int* __restrict__ counts, uint8_t* __restrict__ mask, int wait_limit) {
     extern __shared__ __align__(16) unsigned int skeys[];
     __shared__ SelectShared<Count> sh;
     __shared__ int slt[SEL_THREADS], sle[SEL_THREADS];
@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
             if (G > 1) {
                 if (a) atomicAdd(&st->hist[pass][2 * tid], a);
                 if (b) atomicAdd(&st->hist[pass][2 * tid + 1], b);
-                if (!grid_barrier(&st->arrived, G * ++barrier_no)) {      // cannot happen in a cooperative launch; reported, not hidden
-                    for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = -1;
+                if (!grid_barrier(&st->arrived, G * ++barrier_no, wait_limit)) {      // (all blocks of a cooperative launch are resident)
+                    for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = COUNT_TIMED_OUT;
                     return;
                 }
                 const uint2 v = __ldcg(reinterpret_cast<const uint2*>(st->hist[pass]) + tid);
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
         for (int r = tid; r < nr; r += SEL_THREADS) mine += (Count)(row_le[r] - row_lt[r]);
         const Count total = block_scan(mine, sh);
         if (tid == SEL_THREADS - 1) st->ties[blockIdx.x] = total;
-        if (!grid_barrier(&st->arrived, G * ++barrier_no)) {
-            for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = -1;
+        if (!grid_barrier(&st->arrived, G * ++barrier_no, wait_limit)) {
+            for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = COUNT_TIMED_OUT;
             return;
         }
         Count b = 0;
@@ -350,7 +350,7 @@ size_t select_workspace_bytes(int rows, int d) {
 }
 
 obc_status select_launch(const float* loss, const int32_t* order, int rows, int d, int64_t k, int32_t* counts,
-                         uint8_t* mask, void* ws, cudaStream_t stream) {
+                         uint8_t* mask, void* ws, cudaStream_t stream, int wait_limit) {
     DeviceInfo di;
     const obc_status ds = device_info(&di);
     if (ds != OBC_OK) return ds;
@@ -374,8 +374,9 @@ obc_status select_launch(const float* loss, const int32_t* order, int rows, int 
     const size_t key_bytes = (size_t)rpb * ((d + 3) & ~3) * 4 + 32;        // (the mask is built in the same space, shifted by up to 15 bytes)
     const bool in_smem = key_bytes <= (size_t)SEL_SMEM && n < (1ll << 32);
     unsigned long long kk = (unsigned long long)k;
+    int limit = wait_limit == 0 ? GRID_BARRIER_LIMIT : (wait_limit < 0 ? 0 : wait_limit);
     if (grid > 1) OBC_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(SelectState), stream));
-    void* args[] = {&loss, &order, &rows, &d, &kk, &rpb, &segs, &gkeys, &glt, &gle, &st, &counts, &mask};
+    void* args[] = {&loss, &order, &rows, &d, &kk, &rpb, &segs, &gkeys, &glt, &gle, &st, &counts, &mask, &limit};
     const void* kernel = in_smem ? (const void*)select_kernel<true, unsigned int>
                                  : (n < (1ll << 32) ? (const void*)select_kernel<false, unsigned int> : (const void*)select_kernel<false, unsigned long long>);
     const size_t smem = in_smem ? key_bytes : 0;

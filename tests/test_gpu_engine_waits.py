@@ -96,3 +96,43 @@ def test_large_cross_product_tiles_that_run_out_of_time():
         late = int(info.item())
         assert late == {-1: OBC_ERR_TIMEOUT, 0: 0}.get(limit, late)
         assert bool(torch.isnan(G).all()) if late else float((G.double() - want).abs().max() / want.abs().max()) <= 3e-5
+
+
+def test_selection_that_runs_out_of_time_is_reported_downstream(shim):
+    m, lib = shim
+    rows, d = 300, 96
+    g = torch.Generator(device="cuda").manual_seed(4)
+    inv = spd(d, g)
+    Hinv, W = ((inv + inv.T) / 2).float().contiguous(), torch.randn(rows, d, device="cuda", generator=g)
+    order, loss = torch.zeros(rows, d, dtype=torch.int32, device="cuda"), torch.zeros(rows, d, device="cuda")
+    st = torch.zeros(rows, dtype=torch.int32, device="cuda")
+    trace = torch.zeros(rows, d + 1, d, device="cuda")
+    m.obc_prune_trace(W, Hinv, order, loss, st, w_trace=trace)
+    counts, mask = torch.zeros(rows, dtype=torch.int32, device="cuda"), torch.full((rows, d), 7, dtype=torch.uint8, device="cuda")
+    ws = torch.empty(m.obc_workspace_bytes(m.OP_SELECT, rows, d), dtype=torch.uint8, device="cuda")
+
+    def select(limit):
+        rc = lib.shim_select(pointer(loss), pointer(order), rows, d, ctypes.c_longlong(rows * d // 2), pointer(counts), pointer(mask), pointer(ws), limit,
+                             ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+
+    select(-1)
+    assert bool((counts == -OBC_ERR_TIMEOUT).all())
+    counts[::3] = 5                                 # the other rows are ordinary ones
+    late = counts == -OBC_ERR_TIMEOUT
+    out = torch.zeros(rows, d, device="cuda")
+    for kw in (dict(), dict(w_trace=trace, trace_steps=d), dict(opts=m.engine_opts(m.ENGINE_STREAMING))):
+        st.zero_()
+        m.obc_prune_apply(W, Hinv, order, counts, out, st, **kw)
+        assert torch.equal(st, torch.where(late, -OBC_ERR_TIMEOUT, 0).int())
+        assert torch.equal(out[late], W[late]) and bool(((out == 0).sum(1)[~late] == 5).all())
+    scale, zero, codes = torch.zeros(rows, device="cuda"), torch.zeros(rows, device="cuda"), torch.zeros(rows, d, dtype=torch.int32, device="cuda")
+    m.obc_quantize(W, Hinv, scale, zero, 4, True, out, codes, st, prune_order=order, prune_counts=counts)
+    assert torch.equal(st, torch.where(late, -OBC_ERR_TIMEOUT, 0).int())
+    counts.fill_(-3)                                # any other negative count prunes nothing, as ever
+    m.obc_prune_apply(W, Hinv, order, counts, out, st)
+    assert int(st.abs().sum()) == 0 and torch.equal(out, W)
+    select(0)                                       # and the next selection is right
+    want = (torch.zeros_like(counts), torch.zeros_like(mask))
+    m.obc_select_global_mask(loss, order, rows * d // 2, *want)
+    assert torch.equal(counts, want[0]) and torch.equal(mask, want[1]) and int(counts.sum()) == rows * d // 2

@@ -8,3 +8,8 @@ extern "C" int shim_prune_trace(const float* W, int ldw, int rows, int d, const 
     eo.wait_limit = wait_limit;
     return obc::engine_prune_trace(W, ldw, rows, d, 0, rows, Hinv, ldhi, d, order, loss, nullptr, row_status, ws, ws_bytes, eo, (cudaStream_t)stream);
 }
+
+extern "C" int shim_select(const float* loss, const int32_t* order, int rows, int d, long long k, int32_t* counts, uint8_t* mask, void* ws,
+                           int wait_limit, void* stream) {
+    return obc::select_launch(loss, order, rows, d, k, counts, mask, ws, (cudaStream_t)stream, wait_limit);
+}
