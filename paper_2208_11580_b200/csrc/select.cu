@@ -25,10 +25,12 @@ constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr int SEL_MAX_BLOCKS = 512;
 constexpr int SEL_MAX_UNITS = 128;                // row segments of a block, when rows are cut into segments
 constexpr int SEL_BINS = 2048;
+constexpr int64_t SEL_WIDE = 1ll << 32;           // from this many keys on, counts and bins have 64 bits
+constexpr size_t SEL_WIDE_BYTES = 3 * SEL_BINS * 8;
 constexpr int SEL_SMEM = 200 * 1024;              // keys of a block's rows, if they fit
 
 struct SelectState {            // in the workspace, zero before the launch
-    unsigned int hist[3][SEL_BINS];
+    unsigned int hist[3][SEL_BINS];               // (from 2^32 keys on: 64-bit bins behind the other arrays)
     unsigned int arrived;       // blocks at the grid barriers
     unsigned int pad[63];
     unsigned long long ties[SEL_MAX_BLOCKS];      // keys equal to the k-th one, per block
@@ -42,11 +44,12 @@ __device__ __forceinline__ unsigned int loss_key(float x) {
 }
 
 template <typename Count> struct SelectShared {
-    unsigned int hist[SEL_BINS];
+    Count hist[SEL_BINS];
     unsigned int segmax[SEL_MAX_UNITS];
     Count scan[SEL_WARPS];
     Count rem, before;
-    unsigned int digit, digit_count;
+    unsigned int digit;
+    Count digit_count;
 };
 
 // Inclusive scan over the block of one value per thread; sh.scan[w] = total of warps 0 .. w afterwards.
@@ -73,8 +76,8 @@ __device__ __forceinline__ Count block_scan(Count v, SelectShared<Count>& sh) {
 
 // Thread t owns bins 2t, 2t + 1 (counts a, b): the bin that holds rank sh.rem becomes sh.digit, sh.rem the rank inside it.
 template <typename Count>
-__device__ __forceinline__ void pick_digit(unsigned int a, unsigned int b, SelectShared<Count>& sh) {
-    const Count incl = block_scan((Count)a + b, sh);
+__device__ __forceinline__ void pick_digit(Count a, Count b, SelectShared<Count>& sh) {
+    const Count incl = block_scan((Count)(a + b), sh);
     const Count rem = sh.rem, before = incl - a - b;
     __syncthreads();
     if (before < rem && rem <= incl) {
@@ -91,7 +94,7 @@ __device__ __forceinline__ void pick_digit(unsigned int a, unsigned int b, Selec
 template <bool IN_SMEM, typename Count>
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ loss, const int32_t* __restrict__ order, int rows, int d,
                                                              unsigned long long k, int rpb, int segs, unsigned int* __restrict__ gkeys,
-                                                             int* __restrict__ glt, int* __restrict__ gle, SelectState* __restrict__ st,
+                                                             int* __restrict__ glt, int* __restrict__ gle, SelectState* __restrict__ st, Count* __restrict__ ghist,
                                                              int* __restrict__ counts, uint8_t* __restrict__ mask, int wait_limit) {
     extern __shared__ __align__(16) unsigned int skeys[];
     __shared__ SelectShared<Count> sh;
@@ -108,7 +111,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     int* row_le = rpb <= SEL_THREADS ? sle : gle + r0;
     unsigned int barrier_no = 0;
 
-    for (int b = tid; b < SEL_BINS; b += SEL_THREADS) sh.hist[b] = 0u;
+    for (int b = tid; b < SEL_BINS; b += SEL_THREADS) sh.hist[b] = 0;
     if (tid == 0) sh.rem = (Count)k;
     // keys [row_lt, row_le) of a row share the digits decided so far (in the end: are equal to the k-th key)
     for (int r = tid; r < nr; r += SEL_THREADS) { row_lt[r] = 0; row_le[r] = k > 0 ? d : 0; }
@@ -161,10 +164,10 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                     const int e = min(d, (g + 1) * seg_len);
                     auto change = [&](unsigned int key, unsigned int next, int t) {      // t < d
                         const unsigned int f = key >> 22, fn = next >> 22;
-                        if (t + 1 == d) atomicAdd(&sh.hist[f], (unsigned int)d);
+                        if (t + 1 == d) atomicAdd(&sh.hist[f], (Count)d);
                         else if (f != fn) {
-                            atomicAdd(&sh.hist[f], (unsigned int)(t + 1));
-                            atomicAdd(&sh.hist[fn], 0u - (unsigned int)(t + 1));
+                            atomicAdd(&sh.hist[f], (Count)(t + 1));
+                            atomicAdd(&sh.hist[fn], (Count)0 - (Count)(t + 1));
                         }
                     };
                     if (IN_SMEM) {
@@ -204,17 +207,17 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                     for (int64_t p0 = (int64_t)b + (int64_t)g * 1024; p0 < e; p0 += (int64_t)segs * 1024) {
                         const int x = (int)min(p0 + 32 * lane, (int64_t)e), y = min(e - x, 32) + x;      // this lane's piece
                         const int f = digit(x), last = x < e ? digit(y - 1) : -1, fn = digit(y);
-                        if (x == b && b > 0) atomicAdd(&sh.hist[f], 0u - (unsigned int)b);
+                        if (x == b && b > 0) atomicAdd(&sh.hist[f], (Count)0 - (Count)b);
                         if (x < e && f == last && last != fn) {
-                            atomicAdd(&sh.hist[f], (unsigned int)y);
-                            if (fn >= 0) atomicAdd(&sh.hist[fn], 0u - (unsigned int)y);
+                            atomicAdd(&sh.hist[f], (Count)y);
+                            if (fn >= 0) atomicAdd(&sh.hist[fn], (Count)0 - (Count)y);
                         }
                         for (unsigned int todo = __ballot_sync(0xffffffffu, f != last); todo; todo &= todo - 1) {
                             const int at = __shfl_sync(0xffffffffu, x, __ffs(todo) - 1), end = __shfl_sync(0xffffffffu, y, __ffs(todo) - 1);
                             const int t = at + lane, h = t < end ? digit(t) : -1, hn = digit(t + 1);
                             if (h >= 0 && h != hn) {
-                                atomicAdd(&sh.hist[h], (unsigned int)(t + 1));
-                                if (hn >= 0) atomicAdd(&sh.hist[hn], 0u - (unsigned int)(t + 1));
+                                atomicAdd(&sh.hist[h], (Count)(t + 1));
+                                if (hn >= 0) atomicAdd(&sh.hist[hn], (Count)0 - (Count)(t + 1));
                             }
                         }
                     }
@@ -226,27 +229,27 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                     for (int t = b + lane; t < e; t += 32) {
                         const int f = (int)((K[t] >> shift) & dmask);
                         const int fn = t + 1 < e ? (int)((K[t + 1] >> shift) & dmask) : -1;
-                        if (t == b && b > 0) atomicAdd(&sh.hist[f], 0u - (unsigned int)b);
+                        if (t == b && b > 0) atomicAdd(&sh.hist[f], (Count)0 - (Count)b);
                         if (f != fn) {
-                            atomicAdd(&sh.hist[f], (unsigned int)(t + 1));
-                            if (fn >= 0) atomicAdd(&sh.hist[fn], 0u - (unsigned int)(t + 1));
+                            atomicAdd(&sh.hist[f], (Count)(t + 1));
+                            if (fn >= 0) atomicAdd(&sh.hist[fn], (Count)0 - (Count)(t + 1));
                         }
                     }
                 }
             }
             __syncthreads();
-            unsigned int a = sh.hist[2 * tid], b = sh.hist[2 * tid + 1];
+            Count a = sh.hist[2 * tid], b = sh.hist[2 * tid + 1];
             if (G > 1) {
-                if (a) atomicAdd(&st->hist[pass][2 * tid], a);
-                if (b) atomicAdd(&st->hist[pass][2 * tid + 1], b);
+                Count* bins = ghist + pass * SEL_BINS + 2 * tid;
+                if (a) atomicAdd(bins, a);
+                if (b) atomicAdd(bins + 1, b);
                 if (!grid_barrier(&st->arrived, G * ++barrier_no, wait_limit)) {      // (all blocks of a cooperative launch are resident)
                     for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = COUNT_TIMED_OUT;
                     return;
                 }
-                const uint2 v = __ldcg(reinterpret_cast<const uint2*>(st->hist[pass]) + tid);
-                a = v.x; b = v.y;
+                a = __ldcg(bins); b = __ldcg(bins + 1);
             }
-            sh.hist[2 * tid] = 0u; sh.hist[2 * tid + 1] = 0u;
+            sh.hist[2 * tid] = 0; sh.hist[2 * tid + 1] = 0;
             pick_digit(a, b, sh);
             prefix |= sh.digit << shift;
             // narrow every row to the keys that share the prefix: one thread per row, both ends in one loop
@@ -346,7 +349,8 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 }
 
 size_t select_workspace_bytes(int rows, int d) {
-    return round_up((size_t)rows * d * 4, 256) + round_up(sizeof(SelectState), 256) + 2 * round_up((size_t)rows * 4, 256);
+    return round_up((size_t)rows * d * 4, 256) + round_up(sizeof(SelectState), 256) + 2 * round_up((size_t)rows * 4, 256) +
+           ((int64_t)rows * d < SEL_WIDE ? 0 : SEL_WIDE_BYTES);
 }
 
 obc_status select_launch(const float* loss, const int32_t* order, int rows, int d, int64_t k, int32_t* counts,
@@ -358,7 +362,7 @@ obc_status select_launch(const float* loss, const int32_t* order, int rows, int 
     unsigned int* gkeys = reinterpret_cast<unsigned int*>(p); p += round_up((size_t)rows * d * 4, 256);
     SelectState* st = reinterpret_cast<SelectState*>(p); p += round_up(sizeof(SelectState), 256);
     int* glt = reinterpret_cast<int*>(p); p += round_up((size_t)rows * 4, 256);
-    int* gle = reinterpret_cast<int*>(p);
+    int* gle = reinterpret_cast<int*>(p); p += round_up((size_t)rows * 4, 256);
     // Blocks: one SM each, at least SEL_BLOCK_KEYS keys a block -- below that the barriers of a further block cost more than
     // its share of the scans saves -- and a single block (no barriers at all) up to SEL_ONE_BLOCK_KEYS.
     constexpr int64_t SEL_BLOCK_KEYS = 4096, SEL_ONE_BLOCK_KEYS = 12288;
@@ -372,13 +376,15 @@ obc_status select_launch(const float* loss, const int32_t* order, int rows, int 
     int segs = rpb >= 2 * SEL_WARPS ? 1 : 2 * SEL_WARPS / rpb;       // about two segments per warp, of 256 keys or more
     while (segs > 1 && d / segs < 256) --segs;
     const size_t key_bytes = (size_t)rpb * ((d + 3) & ~3) * 4 + 32;        // (the mask is built in the same space, shifted by up to 15 bytes)
-    const bool in_smem = key_bytes <= (size_t)SEL_SMEM && n < (1ll << 32);
+    const bool wide = n >= SEL_WIDE, in_smem = key_bytes <= (size_t)SEL_SMEM && !wide;
+    void* ghist = wide ? (void*)p : (void*)st->hist;
     unsigned long long kk = (unsigned long long)k;
     int limit = wait_limit == 0 ? GRID_BARRIER_LIMIT : (wait_limit < 0 ? 0 : wait_limit);
     if (grid > 1) OBC_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(SelectState), stream));
-    void* args[] = {&loss, &order, &rows, &d, &kk, &rpb, &segs, &gkeys, &glt, &gle, &st, &counts, &mask, &limit};
+    if (wide && grid > 1) OBC_CUDA_TRY(cudaMemsetAsync(ghist, 0, SEL_WIDE_BYTES, stream));
+    void* args[] = {&loss, &order, &rows, &d, &kk, &rpb, &segs, &gkeys, &glt, &gle, &st, &ghist, &counts, &mask, &limit};
     const void* kernel = in_smem ? (const void*)select_kernel<true, unsigned int>
-                                 : (n < (1ll << 32) ? (const void*)select_kernel<false, unsigned int> : (const void*)select_kernel<false, unsigned long long>);
+                                 : (!wide ? (const void*)select_kernel<false, unsigned int> : (const void*)select_kernel<false, unsigned long long>);
     const size_t smem = in_smem ? key_bytes : 0;
     if (in_smem) OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
     if (grid > 1) OBC_CUDA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(SEL_THREADS), args, smem, stream));

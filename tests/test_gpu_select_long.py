@@ -27,3 +27,24 @@ def test_long_runs_of_equal_digits(R, d, kind):
         want = reference(key, order, k)
         assert np.array_equal(counts.cpu().numpy(), want[0])
         assert np.array_equal(mask.cpu().numpy(), want[1])
+
+
+def test_more_keys_than_32_bits_count():
+    """All losses equal: one bin of the histograms holds all 2^32 + 2^20 keys."""
+    import paper_2208_11580_b200 as m
+    R, d = 4097, 1 << 20
+    loss = torch.full((R, d), 0.5, device="cuda")
+    order = torch.arange(d, dtype=torch.int32, device="cuda").repeat(R, 1)
+    counts = torch.full((R,), -7, dtype=torch.int32, device="cuda")
+    mask = torch.full((R, d), 7, dtype=torch.uint8, device="cuda")
+    for k in (R * d - 5, (1 << 32) + 3, 12345):
+        m.obc_select_global_mask(loss, order, k, counts, mask)
+        full, rest = divmod(k, d)
+        want = torch.zeros(R, dtype=torch.int32, device="cuda")
+        want[:full] = d
+        want[full] = rest
+        assert torch.equal(counts, want)
+        assert bool((mask[:full] == 0).all()) and bool((mask[full + 1:] == 1).all())
+        assert bool((mask[full, :rest] == 0).all()) and bool((mask[full, rest:] == 1).all())
+    del loss, order, mask
+    torch.cuda.empty_cache()
