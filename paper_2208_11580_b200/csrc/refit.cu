@@ -21,7 +21,9 @@ __global__ void __launch_bounds__(F32<TILE>::THREADS, F32<TILE>::BLOCKS) sgemm_n
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
-    const int i0 = blockIdx.y * TILE, j0 = blockIdx.z * TILE;
+    // (clusters are numbered along x alone: the other grid dimensions end at 65535 tiles)
+    const int tile = blockIdx.x / parts, rows = (M + TILE - 1) / TILE;
+    const int i0 = tile % rows * TILE, j0 = tile / rows * TILE;
     const int64_t kb = (int64_t)part * slice, ke = kb + slice < K ? kb + slice : K;
     static_assert(F32<TILE>::SMEM >= TILE * TILE * 4 || TILE == 64, "the partial tile takes the place of the stages");
     f32_tile_product<TILE, VEC>(fsm, A, lda, M, i0, B, ldb, N, j0, kb, ke, [&](int i, int j, float v) { fsm[i * TILE + j] = v; });
@@ -50,7 +52,7 @@ static obc_status sgemm_nt_tiles(int M, int N, int64_t K, float alpha, const flo
     auto kernel = sgemm_nt_kernel<TILE, VEC>;
     OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, F32<TILE>::SMEM));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(parts, (M + TILE - 1) / TILE, (N + TILE - 1) / TILE);
+    cfg.gridDim = dim3((unsigned)(tiles * parts));
     cfg.blockDim = dim3(F32<TILE>::THREADS);
     cfg.dynamicSmemBytes = F32<TILE>::SMEM;
     cfg.stream = stream;

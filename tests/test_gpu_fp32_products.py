@@ -20,3 +20,15 @@ def test_hessian_rounding(kind, d, n, bound):
     m.obc_hessian(X, H, prec=m.PREC_FP32)
     want = 2 * X.double() @ X.double().T
     assert float((H.double() - want).norm() / want.norm()) <= 1.1 * bound
+
+
+def test_cross_product_of_more_columns_than_a_grid_dimension_has_tiles():
+    import paper_2208_11580_b200 as m
+    r, d, n = 2, 65535 * 128 + 130, 4
+    g = torch.Generator(device="cuda").manual_seed(1)
+    Y, X = torch.randn(r, n, device="cuda", generator=g), torch.randn(d, n, device="cuda", generator=g)
+    G = torch.zeros(r, (d + 3) // 4 * 4, device="cuda")[:, :d]
+    m.obc_cross_gram(Y, X, G, prec=m.PREC_FP32)
+    want = Y.double() @ X.double().T
+    # four products and their sum, each rounded once, of the size of the row norms' product
+    assert float((G - want).abs().max()) <= 8 * 2.0 ** -24 * float(Y.double().norm(dim=1).max() * X.double().norm(dim=1).max())
