@@ -20,6 +20,10 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 inline bool aligned256(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// SMs of a B200.  Where the number of slices of a sum follows from it, it is this constant and not the current device's count: a
+// slice count is part of a result's rounding and of the workspace size, which is also asked for without a device.
+constexpr int B200_SMS = 148;
+
 // Properties of the current device, queried once per device and cached (host side only).
 struct DeviceInfo {
     int sm_count;

@@ -33,7 +33,7 @@ static bool fp32_small_tile(int d) { return d <= 640; }
 static int fp32_splits(int d, int64_t n) {
     const int tile = fp32_small_tile(d) ? 64 : 128;
     const int64_t T = (d + tile - 1) / tile, ntiles = T * (T + 1) / 2;
-    const int64_t resident = 148 * (tile == 64 ? F32<64>::BLOCKS : F32<128>::BLOCKS);
+    const int64_t resident = B200_SMS * (tile == 64 ? F32<64>::BLOCKS : F32<128>::BLOCKS);
     int64_t s = resident / ntiles;                                      // one full wave ...
     const int64_t by_len = (n + 2047) / 2048;                           // ... or chains of at most 2048 products
     const int64_t least = tile == 128 && hessian_splits(d, n) > by_len ? hessian_splits(d, n) : by_len;

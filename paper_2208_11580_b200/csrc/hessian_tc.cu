@@ -552,11 +552,11 @@ obc_status hessian_tc_launch(const float* X, int d, int64_t n, int64_t ldx, floa
             const obc_status st = launch_large<false>(ma, ml, ma, ml, d, d, n_pad, slice, splits, partial, err, wl, stream);
             if (st != OBC_OK) return st;
         } else {
-        const int stages = 3;
-        const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
-        OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        syrk_tc_kernel<1, false><<<grid, TC_THREADS, smem, stream>>>(ma, ml, ma, ml, d, d, n_pad, slice, stages, partial, err, wl);
-        count_launch();
+            const int stages = 3;
+            const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
+            OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            syrk_tc_kernel<1, false><<<grid, TC_THREADS, smem, stream>>>(ma, ml, ma, ml, d, d, n_pad, slice, stages, partial, err, wl);
+            count_launch();
         }
     }
     OBC_CUDA_TRY(cudaGetLastError());
@@ -637,11 +637,11 @@ obc_status cross_tc_launch(const float* Y, int rows_a, int64_t ldy, const float*
             const obc_status st = launch_large<true>(ma, mal, mb, mbl, rows_a, rows_b, n_pad, slice, splits, partial, err, wl, stream);
             if (st != OBC_OK) return st;
         } else {
-        const int stages = 3;
-        const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
-        OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        syrk_tc_kernel<1, true><<<grid, TC_THREADS, smem, stream>>>(ma, mal, mb, mbl, rows_a, rows_b, n_pad, slice, stages, partial, err, wl);
-        count_launch();
+            const int stages = 3;
+            const size_t smem = (size_t)stages * 4 * TC_TILE_BYTES + 1024;
+            OBC_CUDA_TRY(cudaFuncSetAttribute(syrk_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            syrk_tc_kernel<1, true><<<grid, TC_THREADS, smem, stream>>>(ma, mal, mb, mbl, rows_a, rows_b, n_pad, slice, stages, partial, err, wl);
+            count_launch();
         }
     }
     OBC_CUDA_TRY(cudaGetLastError());

@@ -46,7 +46,7 @@ static obc_status sgemm_nt_tiles(int M, int N, int64_t K, float alpha, const flo
     const int64_t tiles = (int64_t)((M + TILE - 1) / TILE) * ((N + TILE - 1) / TILE);
     // parts of K: as long as all blocks still fit at once, slices of 256 or more
     int parts = 1;
-    while (parts < 8 && tiles * parts * 2 <= 148 * F32<TILE>::BLOCKS && K / (parts * 2) >= 256) parts *= 2;
+    while (parts < 8 && tiles * parts * 2 <= B200_SMS * F32<TILE>::BLOCKS && K / (parts * 2) >= 256) parts *= 2;
     int64_t slice = (K + parts - 1) / parts;
     slice = (slice + 31) / 32 * 32;
     auto kernel = sgemm_nt_kernel<TILE, VEC>;

@@ -898,45 +898,45 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 }
             }
         } else {
-        for (int j = tid; j < d; j += NT) {
-            const float w = a.W[(size_t)r * a.ldw + j];
-            wd[j] = (double)w;
-            dg[j] = (double)a.Hinv[(size_t)j * a.ldhi + j];
-            perm[j] = j;
-            srcm[j] = (unsigned short)j;
-            if (has_wfull) wfull[j] = w;
-            if (a.codes) a.codes[(size_t)r * d + j] = -1;
-            if (a.mask) a.mask[(size_t)r * d + j] = 1;
-        }
-        if (has_nm) for (int b = tid; b < (d >> nm_lg); b += NT) blkcnt[b] = 0;
-        if (BC == 8) {
-            for (int e = tid; e < (d >> 3) * 28; e += NT) {
-                const int g = e / 28, k = e - g * 28;
-                int ia = 0, rest = k;
-                while (rest >= 7 - ia) { rest -= 7 - ia; ++ia; }
-                const int ib = ia + 1 + rest;
-                boff[e] = (double)a.Hinv[(size_t)(8 * g + ia) * a.ldhi + 8 * g + ib];
+            for (int j = tid; j < d; j += NT) {
+                const float w = a.W[(size_t)r * a.ldw + j];
+                wd[j] = (double)w;
+                dg[j] = (double)a.Hinv[(size_t)j * a.ldhi + j];
+                perm[j] = j;
+                srcm[j] = (unsigned short)j;
+                if (has_wfull) wfull[j] = w;
+                if (a.codes) a.codes[(size_t)r * d + j] = -1;
+                if (a.mask) a.mask[(size_t)r * d + j] = 1;
             }
-        } else if (BC) {
-            for (int e = tid; e < (d >> 2) * 6; e += NT) {
-                const int g = e / 6, k = e - g * 6;
-                const int ia = k < 3 ? 0 : (k < 5 ? 1 : 2), ib = k < 3 ? k + 1 : (k < 5 ? k - 1 : 3);
-                boff[e] = (double)a.Hinv[(size_t)(4 * g + ia) * a.ldhi + 4 * g + ib];
+            if (has_nm) for (int b = tid; b < (d >> nm_lg); b += NT) blkcnt[b] = 0;
+            if (BC == 8) {
+                for (int e = tid; e < (d >> 3) * 28; e += NT) {
+                    const int g = e / 28, k = e - g * 28;
+                    int ia = 0, rest = k;
+                    while (rest >= 7 - ia) { rest -= 7 - ia; ++ia; }
+                    const int ib = ia + 1 + rest;
+                    boff[e] = (double)a.Hinv[(size_t)(8 * g + ia) * a.ldhi + 8 * g + ib];
+                }
+            } else if (BC) {
+                for (int e = tid; e < (d >> 2) * 6; e += NT) {
+                    const int g = e / 6, k = e - g * 6;
+                    const int ia = k < 3 ? 0 : (k < 5 ? 1 : 2), ib = k < 3 ? k + 1 : (k < 5 ? k - 1 : 3);
+                    boff[e] = (double)a.Hinv[(size_t)(4 * g + ia) * a.ldhi + 4 * g + ib];
+                }
             }
-        }
-        for (int k = tid; k < 160; k += NT) colmask[k] = 0u;
-        for (int j = d + tid; j < cap; j += NT) perm[j] = -1;
-        if (tid == 0) {
-            bc->sc = 1.0; bc->ze = 0.0; bc->mq = 0.0;
-            if (a.mode == MODE_QUANT) {
-                bc->sc = (double)a.scale[r]; bc->ze = (double)a.zero[r];
-                bc->mq = (double)grid_maxq(a.bits, a.symmetric);
+            for (int k = tid; k < 160; k += NT) colmask[k] = 0u;
+            for (int j = d + tid; j < cap; j += NT) perm[j] = -1;
+            if (tid == 0) {
+                bc->sc = 1.0; bc->ze = 0.0; bc->mq = 0.0;
+                if (a.mode == MODE_QUANT) {
+                    bc->sc = (double)a.scale[r]; bc->ze = (double)a.zero[r];
+                    bc->mq = (double)grid_maxq(a.bits, a.symmetric);
+                }
+                a.row_status[r] = first_status(a, r);
             }
-            a.row_status[r] = first_status(a, r);
-        }
-        if (a.w_trace)
-            for (int j = tid; j < d; j += NT)
-                a.w_trace[((size_t)r * (a.trace_steps + 1)) * d + j] = a.W[(size_t)r * a.ldw + j];
+            if (a.w_trace)
+                for (int j = tid; j < d; j += NT)
+                    a.w_trace[((size_t)r * (a.trace_steps + 1)) * d + j] = a.W[(size_t)r * a.ldw + j];
         }
         bool tail = false;
         if (kind != ITEM_TAIL && d > ms && total > 0) {
