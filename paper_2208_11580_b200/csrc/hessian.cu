@@ -27,8 +27,9 @@ int hessian_splits(int d, int64_t n) {
 // FP32 path: tile and slices.  64 x 64 tiles (four blocks per SM) waste less on the diagonal and on ragged edges;
 // 128 x 128 tiles (two blocks per SM) halve the traffic from L2, which matters once the padding no longer does.
 // Slices bound the rounding: a chain of L products and s slices err by about sqrt(L / s) roundings of the result (64 x 64 tiles
-// add even and odd k apart, which halves their chains; the finalize kernel adds the slices in FP64).  So 128 x 128 tiles take at
-// least as many slices as the tensor-core paths: 1024 x 8192 with 8 slices in FP32 erred by 2.5e-7, with 13 by 1.9e-7.
+// add even and odd k apart, which halves their chains; the finalize kernel adds the slices in four chains).  So 128 x 128 tiles
+// take at least as many slices as the tensor-core paths, 64 x 64 tiles half as many: 1024 x 8192 with 8 slices erred by 2.5e-7,
+// with 13 by 1.9e-7.
 static bool fp32_small_tile(int d) { return d <= 640; }
 static int fp32_splits(int d, int64_t n) {
     const int tile = fp32_small_tile(d) ? 64 : 128;
@@ -36,9 +37,12 @@ static int fp32_splits(int d, int64_t n) {
     const int64_t resident = B200_SMS * (tile == 64 ? F32<64>::BLOCKS : F32<128>::BLOCKS);
     int64_t s = resident / ntiles;                                      // one full wave ...
     const int64_t by_len = (n + 2047) / 2048;                           // ... or chains of at most 2048 products
-    const int64_t least = tile == 128 && hessian_splits(d, n) > by_len ? hessian_splits(d, n) : by_len;
+    const int64_t tc = hessian_splits(d, n);
+    const int64_t least = tile == 128 && tc > by_len ? tc : by_len;
     if (least > s) s = (least * ntiles + resident - 1) / resident * resident / ntiles;        // (whole waves)
-    if (s * 128 > n) s = n / 128;                                       // slices of 128 or more
+    const int64_t shortest = tile == 64 ? 128 : 64;
+    if (s * shortest > n) s = n / shortest;
+    if (tile == 64 && s < (tc + 1) / 2) s = (tc + 1) / 2;
     if (s > 512) s = 512;
     return s < 1 ? 1 : (int)s;
 }
@@ -73,8 +77,9 @@ __global__ void __launch_bounds__(F32<TILE>::THREADS, F32<TILE>::BLOCKS) syrk_fp
 // into NaN; info (nullable) receives 0 or OBC_ERR_TIMEOUT accordingly.
 // A block takes a 32 x 32 tile on or below the diagonal; the mirror image goes through shared memory, so that both copies are
 // written along rows (column writes of single values took as long as the partial sums of 32 slices).
-// Sum: FP64 for the many slices of the FP32 path (512 slices added in FP32 are 512 more roundings of the result).
-template <typename Sum>
+// CHAINS = 4: every fourth slice in a sum of its own, for the many slices of the FP32 path (512 slices in one chain are 512 more
+// roundings of the result; in FP64 the additions took longer than the loads, 64 x 65536 133 -> 567 us).
+template <int CHAINS>
 __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __restrict__ partial, int splits, int d,
                                                                float* __restrict__ H, int ldh, int accumulate,
                                                                const int* __restrict__ err, int32_t* __restrict__ info) {
@@ -85,7 +90,7 @@ __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __re
     if (bj > bi) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = bj * 32 + tx;
-    Sum s[4] = {};
+    float s[CHAINS][4] = {};
     for (int z0 = 0; z0 < splits; z0 += 4) {              // sixteen loads in flight, added in order
         float v[4][4];
 #pragma unroll
@@ -98,19 +103,23 @@ __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __re
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) s[r] += v[q][r];
+            for (int r = 0; r < 4; ++r) s[q % CHAINS][r] += v[q][r];
+    }
+    if (CHAINS == 4) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[0][r] = (s[0][r] + s[1 % CHAINS][r]) + (s[2 % CHAINS][r] + s[3 % CHAINS][r]);
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int i = bi * 32 + ty + 8 * r;
         if (i < d && j <= i) {
-            float v = (float)(2 * s[r]);
+            float v = 2.f * s[0][r];
             if (accumulate) v += H[(size_t)i * ldh + j];
             if (failed) v = __int_as_float(0x7fc00000);
             H[(size_t)i * ldh + j] = v;
-            s[r] = v;
+            s[0][r] = v;
         }
-        tile[ty + 8 * r][tx] = (float)s[r];
+        tile[ty + 8 * r][tx] = s[0][r];
     }
     __syncthreads();
 #pragma unroll
@@ -120,11 +129,11 @@ __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __re
     }
 }
 
-template <typename Sum>
+template <int CHAINS>
 static obc_status finalize_launch(const float* partial, int splits, int d, float* H, int ldh, int accumulate, const int* err,
                                   int32_t* info, cudaStream_t stream) {
     const int T = (d + 31) / 32;
-    hessian_finalize_kernel<Sum><<<dim3(T, T), 256, 0, stream>>>(partial, splits, d, H, ldh, accumulate, err, info);
+    hessian_finalize_kernel<CHAINS><<<dim3(T, T), 256, 0, stream>>>(partial, splits, d, H, ldh, accumulate, err, info);
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
     return OBC_OK;
@@ -132,7 +141,7 @@ static obc_status finalize_launch(const float* partial, int splits, int d, float
 
 obc_status hessian_finalize_launch(const float* partial, int splits, int d, float* H, int ldh, int accumulate,
                                    const int* err, int32_t* info, cudaStream_t stream) {
-    return finalize_launch<float>(partial, splits, d, H, ldh, accumulate, err, info, stream);
+    return finalize_launch<1>(partial, splits, d, H, ldh, accumulate, err, info, stream);
 }
 
 obc_status hessian_fp32_launch(const float* X, int d, int64_t n, int64_t ldx, float* H, int ldh, int accumulate,
@@ -153,7 +162,7 @@ obc_status hessian_fp32_launch(const float* X, int d, int64_t n, int64_t ldx, fl
     }
     count_launch();
     OBC_CUDA_TRY(cudaGetLastError());
-    return finalize_launch<double>(partial, splits, d, H, ldh, accumulate, nullptr, info, stream);
+    return finalize_launch<4>(partial, splits, d, H, ldh, accumulate, nullptr, info, stream);
 }
 
 }  // namespace obc
