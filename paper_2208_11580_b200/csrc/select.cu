@@ -92,7 +92,7 @@ __device__ __forceinline__ void pick_digit(Count a, Count b, SelectShared<Count>
 // keys: the block's rows in shared memory (IN_SMEM) or this call's rows in the workspace.  A block takes rows
 // [rpb * blockIdx.x, + rpb), cut into `segs` segments each for the scans (one warp per segment).
 template <bool IN_SMEM, typename Count>
-__global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ loss, const int32_t* __restrict__ order, int rows, int d,
+__global__ void __launch_bounds__(SEL_THREADS, 1) select_kernel(const float* __restrict__ loss, const int32_t* __restrict__ order, int rows, int d,
                                                              unsigned long long k, int rpb, int segs, unsigned int* __restrict__ gkeys,
                                                              int* __restrict__ glt, int* __restrict__ gle, SelectState* __restrict__ st, Count* __restrict__ ghist,
                                                              int* __restrict__ counts, uint8_t* __restrict__ mask, int wait_limit) {
@@ -197,27 +197,45 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                     }
                 }
             } else if (!IN_SMEM) {
-                // What is left of a row may be long here (rows of equal or almost equal losses).  Its keys do not decrease, so of 32 keys
-                // in a row only the ends are read unless their digits differ.
+                // What is left of a row may be long here (rows of equal or almost equal losses).  Its keys do not decrease, so between two
+                // keys of the same digit nothing is read: first 1024 keys at a time, then 32.
                 for (int u = warp; u < units; u += SEL_WARPS) {
-                    const int r = u / segs, g = u - r * segs;
+                    const int r = segs == 1 ? u : u / segs, g = u - r * segs;
                     const unsigned int* K = keys + (size_t)r * ldk;
                     const int b = row_lt[r], e = row_le[r];
                     auto digit = [&](int t) { return t < e ? (int)((K[t] >> shift) & dmask) : -1; };
+                    auto change = [&](int t, int f, int fn) {      // key t ends a run of digit f
+                        if (f == fn) return;
+                        atomicAdd(&sh.hist[f], (Count)(t + 1));
+                        if (fn >= 0) atomicAdd(&sh.hist[fn], (Count)0 - (Count)(t + 1));
+                    };
+                    auto scan = [&](int from, int to) {
+                        for (int t = from + lane; t < to; t += 32) change(t, digit(t), digit(t + 1));
+                    };
+                    if (g == 0 && b > 0 && b < e && lane == 0) atomicAdd(&sh.hist[digit(b)], (Count)0 - (Count)b);
+                    if (e - b <= 256) {
+                        if (g == 0) scan(b, e);
+                        continue;
+                    }
                     for (int64_t p0 = (int64_t)b + (int64_t)g * 1024; p0 < e; p0 += (int64_t)segs * 1024) {
-                        const int x = (int)min(p0 + 32 * lane, (int64_t)e), y = min(e - x, 32) + x;      // this lane's piece
-                        const int f = digit(x), last = x < e ? digit(y - 1) : -1, fn = digit(y);
-                        if (x == b && b > 0) atomicAdd(&sh.hist[f], (Count)0 - (Count)b);
-                        if (x < e && f == last && last != fn) {
-                            atomicAdd(&sh.hist[f], (Count)y);
-                            if (fn >= 0) atomicAdd(&sh.hist[fn], (Count)0 - (Count)y);
+                        const int from = (int)p0, to = (int)min(p0 + 1024, (int64_t)e);
+                        const int whole = digit(to - 1);
+                        if (digit(from) == whole) {
+                            if (lane == 0) change(to - 1, whole, digit(to));
+                            continue;
                         }
-                        for (unsigned int todo = __ballot_sync(0xffffffffu, f != last); todo; todo &= todo - 1) {
-                            const int at = __shfl_sync(0xffffffffu, x, __ffs(todo) - 1), end = __shfl_sync(0xffffffffu, y, __ffs(todo) - 1);
-                            const int t = at + lane, h = t < end ? digit(t) : -1, hn = digit(t + 1);
-                            if (h >= 0 && h != hn) {
-                                atomicAdd(&sh.hist[h], (Count)(t + 1));
-                                if (hn >= 0) atomicAdd(&sh.hist[hn], (Count)0 - (Count)(t + 1));
+                        const int x = min(from + 32 * lane, to), y = min(x + 32, to);      // this lane's piece
+                        const int last = x < to ? digit(y - 1) : -1;
+                        const bool same = x == to || digit(x) == last;
+                        if (same && x < to) change(y - 1, last, digit(y));
+                        unsigned int todo = __ballot_sync(0xffffffffu, !same);
+                        if (__popc(todo) > 8) {                    // (pieces one after the other would cost more than reading all)
+                            for (int t = from + lane; t < to; t += 32)
+                                if (todo >> ((t - from) >> 5) & 1u) change(t, digit(t), digit(t + 1));
+                        } else {
+                            for (; todo; todo &= todo - 1) {
+                                const int at = from + 32 * (__ffs(todo) - 1);
+                                scan(at, min(at + 32, to));
                             }
                         }
                     }
@@ -335,7 +353,11 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
                 for (int x = max(lo, skew); x < hi && (size_t)x < bytes + skew; ++x) base[x] = reinterpret_cast<uint8_t*>(skeys)[x];
         }
     } else {
-        for (size_t x = tid; x < bytes; x += SEL_THREADS) M[x] = 1;
+        const size_t head = min((size_t)((0 - reinterpret_cast<uintptr_t>(M)) & 15u), bytes), n16 = (bytes - head) >> 4;
+        for (size_t x = tid; x < n16; x += SEL_THREADS)
+            reinterpret_cast<uint4*>(M + head)[x] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
+        if (tid < head) M[tid] = 1;
+        for (size_t x = head + 16 * n16 + tid; x < bytes; x += SEL_THREADS) M[x] = 1;
         __syncthreads();
         for (int u = warp; u < units; u += SEL_WARPS) {
             const int r = u / segs, g = u - r * segs;
