@@ -446,7 +446,7 @@ def measure(args, name, steps, warmup, rank, world, dev, with_cpu=True, with_e2e
                              "cores: FP16 tcgen05 with 512 threads per row, else TF32 m16n8k8); executed = 3 x that: every FP32 "
                              "operand is split into two parts and three of the four partial products are formed"}
     if blocked and plan.get("l2_vectors", 0) > 0:
-        tensor["note"] = ("rows this long keep up to %d of their deferred updates per pass in global memory (resident in L2); the "
+        tensor["note"] = ("rows this long keep up to %d of their deferred updates per pass in global memory (sized to L2); the "
                           "rank-B update copies all operands from there with TMA" % plan["l2_vectors"])
     # Both engines are reported against HBM.  The streaming engine moves the active triangle once per step.  The blocked
     # engine moves it once per block of deferred updates and applies the block as one rank-B update on the tensor cores;

@@ -1,13 +1,15 @@
 // The rank-B update of the blocked row engine for long rows on the 5th-generation tensor cores: H -= sum_b z_b z_b^T over the
 // compacted lower triangle of one row's private inverse Hessian (B <= 48 pending vectors), one 512-thread block per SM.
 //
-// A pass reads and writes every element of the triangle once (8 bytes) and is bound by HBM, so everything but that traffic
-// is kept off the warps: TMA brings tiles of 128 rows x 64 columns of H into shared memory and takes them back,
+// A pass reads and writes every element of the triangle once (8 bytes); a tile takes about 2600 cycles of its SM's pipeline of copy,
+// products, subtraction and store, which is the copy rate of HBM when all SMs pass at once (16 rows of 4608 alone: 51 ms of passes,
+// 128 rows: 56 ms).  Everything but that traffic is kept off the warps: TMA brings tiles of 128 rows x 64 columns of H into shared memory and takes them back,
 // tcgen05.mma (kind::f16) forms the tile's increment in tensor memory, and eight warps only subtract one from the other.
 // The products cost nothing beside the traffic, so a pass takes as many pending vectors as tensor memory holds partial sums
 // for; most of them wait in L2 (the mma.sync form spent half of a warp's time multiplying, so more vectors per pass bought it
 // little).  48 of them, not the 64 that four groups would allow: the steps between two passes read them all, and from
-// there on that costs as much as the rarer passes save (768 x 3072: 285 against 300 ms; 128 x 4608: 156 against 161 ms).  During a pass the space of the FP32 pending vectors is free and holds the tiles and operands.
+// there on that costs about as much as the rarer passes save (64 / 48: 128 x 4608 161 / 156 ms, 256 x 2304 46.9 / 47.0, 768 x 3072
+// 260 / 269).  During a pass the space of the FP32 pending vectors is free and holds the tiles and operands.
 //
 // Operands.  Before the pass every pending vector is written as two FP16 planes, z * 2^e = hi + lo (hi rounded to 11 bits, lo
 // the rounded rest: 22 significant bits), to global memory (they stay in L2).  The power of two takes the largest entry to

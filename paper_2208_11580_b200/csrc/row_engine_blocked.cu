@@ -21,8 +21,9 @@ obc_status blk_launch_512_4(const FlushMaps& zmaps, const EngineArgs& a, int blo
 obc_status blk_launch_512_8(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
 obc_status blk_launch_512_12(const FlushMaps& zmaps, const EngineArgs& a, int blocks, size_t smem, int sm_count, cudaStream_t stream);
 
-// All blocks' overflow vectors together: within L2.  (Only the longest rows reach the limit; 48 / 64 / 80 / 110 MB at 128 rows x
-// 4608: 249 / 220 / 202 / 181 ms.)
+// All blocks' overflow vectors together: the size of L2, which they share with the planes and the streamed triangles.  (Only the
+// longest rows reach the limit; when it was chosen, 48 / 64 / 80 / 110 MB at 128 rows x 4608 took 249 / 220 / 202 / 181 ms; the case
+// takes 149 ms since the layout and the tile order changed.)
 constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)110 << 20;
 
 static int blk_pick_ms(int d, size_t panel_bytes) {

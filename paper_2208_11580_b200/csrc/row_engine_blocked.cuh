@@ -82,8 +82,9 @@ struct SplitHeader {                          // what the block that started a r
 __host__ __device__ inline size_t blk_split_stride(int cap) { return sizeof(SplitHeader) + (size_t)28 * cap + 256; }
 
 // Work model of a row, in units of "half a matrix element moved by a flush": a pass over the compacted triangle of m
-// slots costs m^2 / 2, a deferred-update step costs as much as BLK_STEP_COST of those (measured on B200: a pass takes
-// 1.1 - 1.3e-10 s per m^2; a step 7 us with one 512-thread row per SM, 3.4 us with several smaller blocks per SM).
+// slots costs m^2 / 2, a deferred-update step costs as much as blk_step_cost of those.  Fitted when every pass ran by mma.sync (1.1 -
+// 1.3e-10 s per m^2; a step 7 us with one 512-thread row per SM, 3.4 us with several smaller blocks per SM); with passes on
+// tcgen05 a step takes 7 us at d = 2304, 8 at 3072, 17 at 4608, and the values were not fitted again.
 __host__ __device__ inline double blk_step_cost(int nt) { return nt >= 512 ? 30000.0 : 14000.0; }
 
 // The flush boundary of a row's schedule at which about num/den of the row's work is done (0: before the first
@@ -762,7 +763,7 @@ static __device__ __noinline__ double block8_score(const double* w, const double
 // barriers per four steps, each pending vector read once for four columns.  Same arithmetic per element as four
 // single steps except that a column's corrections are subtracted one by one instead of summed first.
 // NM = N:M pruning; the other kernels are built without that code.
-// GPV = the kernel can keep further pending vectors in global memory (very long rows, 512 threads only).
+// GPV = the kernel can keep further pending vectors in global memory (long rows, 512 threads only).
 // SH = the kernel takes shares of rows (a row may be started by one block and finished by the next); launches whose
 // rows divide evenly over the blocks run the kernel built without that code.
 // Passes on tcgen05: one block per SM (blocks of 8 keep 28 bytes more per slot and may lack the room for its tiles).  Only
