@@ -26,10 +26,10 @@ int hessian_splits(int d, int64_t n) {
 
 // FP32 path: tile and slices.  64 x 64 tiles (four blocks per SM) waste less on the diagonal and on ragged edges;
 // 128 x 128 tiles (two blocks per SM) halve the traffic from L2, which matters once the padding no longer does.
-// Slices bound the rounding: a chain of L products and s slices err by about sqrt(L / s) roundings of the result (64 x 64 tiles
-// add even and odd k apart, which halves their chains; the finalize kernel adds the slices in four chains).  So 128 x 128 tiles
-// take at least as many slices as the tensor-core paths, 64 x 64 tiles half as many: 1024 x 8192 with 8 slices erred by 2.5e-7,
-// with 13 by 1.9e-7.
+// Slices bound the rounding: s chains of n / s products, added in c chains, err by about sqrt(n / s^2 + s / c) roundings of the result
+// (64 x 64 tiles add even and odd k apart: 2 s chains; the finalize kernel adds this path's slices in four).  Where that is more
+// than one chain of the tensor-core paths' slices would give, more slices are taken: 1024 x 8192 with 8 slices erred by 2.5e-7, with
+// 13 by 1.9e-7.
 static bool fp32_small_tile(int d) { return d <= 640; }
 static int fp32_splits(int d, int64_t n) {
     const int tile = fp32_small_tile(d) ? 64 : 128;
@@ -37,14 +37,16 @@ static int fp32_splits(int d, int64_t n) {
     const int64_t resident = B200_SMS * (tile == 64 ? F32<64>::BLOCKS : F32<128>::BLOCKS);
     int64_t s = resident / ntiles;                                      // one full wave ...
     const int64_t by_len = (n + 2047) / 2048;                           // ... or chains of at most 2048 products
-    const int64_t tc = hessian_splits(d, n);
-    const int64_t least = tile == 128 && tc > by_len ? tc : by_len;
-    if (least > s) s = (least * ntiles + resident - 1) / resident * resident / ntiles;        // (whole waves)
-    const int64_t shortest = tile == 64 ? 128 : 64;
-    if (s * shortest > n) s = n / shortest;
-    if (tile == 64 && s < (tc + 1) / 2) s = (tc + 1) / 2;
+    if (by_len > s) s = (by_len * ntiles + resident - 1) / resident * resident / ntiles;      // (whole waves)
+    if (s * 128 > n) s = n / 128;                                       // slices of 128 or more
+    if (s < 1) s = 1;
+    const double tc = hessian_splits(d, n), chains = (tile == 64 ? 2.0 : 1.0) * s;
+    if (n / (chains * chains) + s / 4.0 > n / (tc * tc) + tc) {
+        s = (int64_t)(tile == 64 ? (tc + 1) / 2 : tc);
+        if (s * ntiles > resident) s = (s * ntiles + resident - 1) / resident * resident / ntiles;
+    }
     if (s > 512) s = 512;
-    return s < 1 ? 1 : (int)s;
+    return (int)s;
 }
 
 size_t hessian_tc_extra_bytes(int d, int64_t n);
@@ -91,17 +93,18 @@ __global__ void __launch_bounds__(256) hessian_finalize_kernel(const float* __re
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = bj * 32 + tx;
     float s[CHAINS][4] = {};
-    for (int z0 = 0; z0 < splits; z0 += 4) {              // sixteen loads in flight, added in order
-        float v[4][4];
+    constexpr int AHEAD = CHAINS == 4 ? 8 : 4;            // slices read together: 16 or 32 loads in flight, added in order
+    for (int z0 = 0; z0 < splits; z0 += AHEAD) {
+        float v[AHEAD][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < AHEAD; ++q)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int i = bi * 32 + ty + 8 * r;
                 v[q][r] = z0 + q < splits && i < d && j <= i ? __ldcs(partial + (size_t)(z0 + q) * d * d + (size_t)i * d + j) : 0.f;
             }
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < AHEAD; ++q)
 #pragma unroll
             for (int r = 0; r < 4; ++r) s[q % CHAINS][r] += v[q][r];
     }
