@@ -63,7 +63,8 @@ __host__ __device__ inline void grid_from_range(float lo, float hi, int bits, in
 // The per-call engine options of obc_engine_opts after validation (all zero = defaults).
 struct EngineOpts {
     int engine; int threads; int max_pending; int flags;
-    int wait_limit = 0;      // polls of the waits inside a pass: 0 = the built-in limit, < 0 = they expire at once (tests; not in the C ABI)
+    int stop_tile = 0;       // > 0: passes on tcgen05 are abandoned at that tile (counted from 1) as if a wait had expired there (for tests;
+                             // not in the C ABI)
 };
 
 // What the global selection leaves in counts[] when its blocks could not meet: the calls that take counts report such rows.
@@ -75,7 +76,7 @@ size_t select_workspace_bytes(int rows, int d);
 size_t inverse_workspace_bytes(int d);
 size_t hessian_workspace_bytes(int d, int64_t n);
 obc_status select_launch(const float* loss, const int32_t* order, int rows, int d, int64_t k, int32_t* counts,
-                         uint8_t* mask, void* ws, cudaStream_t stream, int wait_limit = 0);      // (limit as in EngineOpts)
+                         uint8_t* mask, void* ws, cudaStream_t stream, int wait_limit = 0);      // polls at the grid barriers: 0 = the built-in limit, < 0 = none (tests)
 obc_status inverse_launch(const float* H, int d, int ldh, float damp_rel, float* Hinv, int ldhi, int32_t* info,
                           void* ws, cudaStream_t s);
 obc_status hessian_fp32_launch(const float* X, int d, int64_t n, int64_t ldx, float* H, int ldh, int accumulate,

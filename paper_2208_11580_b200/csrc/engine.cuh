@@ -34,7 +34,7 @@ struct EngineArgs {
     __half* Zws; int zld;                 // blocked engine: FP16 planes of the pending vectors, 128 rows of zld per block
     double2* park;                        // blocked engine: cap per block, a row's FP64 state during a pass
     signed char* zexp;                    // blocked engine: powers of two of the slots (cap per block; wide diagonals)
-    int wait_limit;                       // blocked engine: polls before a wait inside a pass on tcgen05 gives up
+    int stop_tile;                        // blocked engine: see EngineOpts
     float* Gpan; int g_vectors; int g_ld; // blocked engine: overflow pending vectors in global memory (per block
                                           // g_vectors rows of g_ld floats), nullptr = none
     int split;                            // blocked engine: rows are shared out in equal work per block, a row may be

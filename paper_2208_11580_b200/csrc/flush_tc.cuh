@@ -81,8 +81,8 @@ __device__ __forceinline__ bool ft_test(unsigned long long* b, int parity) {
     return ok != 0;
 }
 // false when the limit is reached or another thread of the block has given up
-__device__ __forceinline__ bool ft_wait(unsigned long long* b, int parity, FlushBars* fb, int limit) {
-    for (int i = 0; i < limit; ++i) {
+__device__ __forceinline__ bool ft_wait(unsigned long long* b, int parity, FlushBars* fb) {
+    for (int i = 0; i < FT_WAIT_LIMIT; ++i) {
         if (ft_test(b, parity)) return true;
         if ((i & 15) == 15) {
             if (*(volatile int*)&fb->abort) return false;
@@ -190,7 +190,7 @@ struct Ring {
     __device__ __forceinline__ void next(int n) { if (++at == n) { at = 0; ++round; } }
 };
 struct FlushGeom {                                // of a pass
-    const FlushMaps* maps; int plane, buf, G, T, m1, limit; FlushBufs nb; uint32_t sa, sb, sh, tmem;
+    const FlushMaps* maps; int plane, buf, G, T, m1; FlushBufs nb; uint32_t sa, sb, sh, tmem;
 };
 // The parts of tile (rb, c) that hold data, each as f(map, 32-column group, first row inside the tile): the whole tile
 // below the diagonal, on it the 32 x 32 parts that reach it.
@@ -206,7 +206,7 @@ __device__ __forceinline__ void ft_parts(const FlushGeom& q, int rb, int c, F f)
 }
 // Copies of the tile of H at (rb, c).  One thread.
 __device__ __forceinline__ bool ft_copy_tile(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
-    if (h.round > 0 && !ft_wait(&fb->free_h[h.at], (h.round - 1) & 1, fb, q.limit)) return false;
+    if (h.round > 0 && !ft_wait(&fb->free_h[h.at], (h.round - 1) & 1, fb)) return false;
     uint32_t bytes = FT_TILE_BYTES;
     if (c >= rb * FT_M) { bytes = 0; ft_parts(q, rb, c, [&](const CUtensorMap*, int, int) { bytes += 32 * 128; }); }
     ft_expect(&fb->full_h[h.at], bytes);
@@ -222,12 +222,12 @@ __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* 
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;    // both planes of 64 slots
     const CUtensorMap* zm = &q.maps->z[q.G - 1];
     if (rb == c / FT_M) {
-        if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb, q.limit)) return false;
+        if (b.round > 0 && !ft_wait(&fb->free_b[b.at], (b.round - 1) & 1, fb)) return false;
         ft_expect(&fb->full_b[b.at], blk);
         ft_load(q.sb + b.at * blk, zm, &fb->full_b[b.at], c, 0, q.plane);
         b.next(q.nb.n_b);
     }
-    if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb, q.limit)) return false;
+    if (a.round > 0 && !ft_wait(&fb->free_a[a.at], (a.round - 1) & 1, fb)) return false;
     ft_expect(&fb->full_a[a.at], 2 * blk);
     ft_load(q.sa + a.at * 2 * blk, zm, &fb->full_a[a.at], rb * FT_M, 0, q.plane);
     ft_load(q.sa + (a.at * 2 + 1) * blk, zm, &fb->full_a[a.at], rb * FT_M + 64, 0, q.plane);
@@ -238,9 +238,9 @@ __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* 
 __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, int t, Ring& b, Ring& a, bool first, bool last) {
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;
     const int buf = t & 1;
-    if (first && !ft_wait(&fb->full_b[b.at], b.round & 1, fb, q.limit)) return false;
-    if (!ft_wait(&fb->full_a[a.at], a.round & 1, fb, q.limit)) return false;
-    if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb, q.limit)) return false;
+    if (first && !ft_wait(&fb->full_b[b.at], b.round & 1, fb)) return false;
+    if (!ft_wait(&fb->full_a[a.at], a.round & 1, fb)) return false;
+    if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint64_t da = ft_desc(q.sa + a.at * 2 * blk, blk), db = ft_desc(q.sb + b.at * blk, blk);
     const uint32_t d = q.tmem + buf * (FT_GMAX * FT_N);
@@ -271,7 +271,7 @@ __device__ __forceinline__ void ft_products_over(const FlushGeom& q, FlushBars* 
 }
 // Takes the tile at (rb, c) back to memory once every warp has finished its part.  One thread (of all tiles).
 __device__ __forceinline__ bool ft_store(const FlushGeom& q, FlushBars* fb, Ring& h, int rb, int c, uint64_t pol) {
-    if (!ft_wait(&fb->ready[h.at], h.round & 1, fb, q.limit)) return false;
+    if (!ft_wait(&fb->ready[h.at], h.round & 1, fb)) return false;
     ft_parts(q, rb, c, [&](const CUtensorMap* m, int cg, int r) {
         ft_store_stream(q.sh + h.at * FT_TILE_BYTES + cg * (FT_M * 128) + r * 128, m, 0, rb * FT_M + r, q.buf + (c >> 5) + cg, pol);
     });
@@ -286,8 +286,8 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = hq.at, buf = t & 1;
     const int cg = warp >> 2, r0 = rb * FT_M + 32 * (warp & 3), col = c + 32 * cg;
-    bool ok = ft_wait(&fb->full_h[h], hq.round & 1, fb, q.limit);
-    ok = ok && ft_wait(&fb->done[buf], (t >> 1) & 1, fb, q.limit);
+    bool ok = ft_wait(&fb->full_h[h], hq.round & 1, fb);
+    ok = ok && ft_wait(&fb->done[buf], (t >> 1) & 1, fb);
     if (!__all_sync(0xffffffffu, ok)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool any = r0 < q.m1 && col <= r0;
@@ -338,12 +338,12 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
 // the copies, and the block has synchronised.
 //   plane     first of the block's two planes (hi, lo) in the maps
 //   unscale   2^-2e of the planes' power, or zexp: the slots' own powers
-//   limit     polls of a wait
+//   stop      tile (from 1) at which the products give up, for tests; 0: never
 __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, int tri, unsigned char* stage, int stage_bytes, FlushBars* fb, int m1,
-                                             int nb, float unscale, const signed char* zexp, int limit) {
+                                             int nb, float unscale, const signed char* zexp, int stop) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FlushGeom q;
-    q.maps = maps; q.plane = plane; q.buf = tri; q.m1 = m1; q.limit = limit;
+    q.maps = maps; q.plane = plane; q.buf = tri; q.m1 = m1;
     q.G = (nb + 15) >> 4;
     q.nb = ft_bufs(q.G, stage_bytes);
     q.sh = ft_smem(stage);
@@ -372,6 +372,10 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
         }
     } else if (warp == FT_EW + 1 && lane == 0) {
         for (; t < q.T; ++t) {
+            if (t + 1 == stop) {                      // (as if a wait had expired: constant limits keep the waits short)
+                *(volatile int*)&fb->abort = 1;
+                break;
+            }
             int nrb = rb, nc = c;
             ft_next_tile(nrb, nc, m1);
             if (!ft_multiply(q, fb, t, b, a, rb == c / FT_M, nc != c)) break;

@@ -188,7 +188,7 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
     a.ldp = a.cap;
     a.split = 0;
     a.split_state = nullptr; a.split_flags = nullptr; a.split_stride = 0;
-    a.wait_limit = a.opts.wait_limit == 0 ? FT_WAIT_LIMIT : (a.opts.wait_limit < 0 ? 0 : a.opts.wait_limit);
+    a.stop_tile = a.opts.stop_tile;
     a.Zws = nullptr; a.park = nullptr; a.zexp = nullptr; a.zld = blk_zld(a.cap);
     FlushMaps zmaps = {};
     if (a.d > a.ms) {

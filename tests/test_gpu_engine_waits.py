@@ -1,6 +1,6 @@
 """Bounded waits that run out on purpose: the pipeline of a pass on tcgen05, the 256 x 256 tiles of the Hessian and the cross product.
-Nothing hangs and nothing faults: a limit of -1 lets every wait expire at once, a few polls let some of them expire at any point of
-a pass.  The call returns, the failure is reported, and the next ordinary call is right."""
+Nothing hangs and nothing faults: the products of a pass give up at a given tile, as after a wait that expired, and the block abandons
+the pass; the other kernels take a limit of -1 (every wait expires at once) or a few polls.  The call returns, the failure is reported, and the next ordinary call is right."""
 import ctypes
 import os
 import subprocess
@@ -48,23 +48,26 @@ def test_pass_that_runs_out_of_time(shim, rows, d):
         Hinv = pad
     ws = torch.empty(m.obc_workspace_bytes(m.OP_PRUNE_TRACE, rows, d), dtype=torch.uint8, device="cuda")
 
-    def call(limit):
+    def call(stop):
         order = torch.full((rows, d), -7, dtype=torch.int32, device="cuda")
         loss, st = torch.zeros(rows, d, device="cuda"), torch.full((rows,), -7, dtype=torch.int32, device="cuda")
         rc = lib.shim_prune_trace(pointer(W), W.shape[1], rows, d, pointer(Hinv), Hinv.shape[1], pointer(order), pointer(loss), pointer(st), pointer(ws),
-                                  ctypes.c_size_t(ws.numel()), 512, limit, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+                                  ctypes.c_size_t(ws.numel()), 512, stop, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
         assert rc == 0
         torch.cuda.synchronize()
         return order, loss, st
 
     want = call(0)
     assert int(want[2].abs().sum()) == 0
-    for limit in (-1, 1, 2, 5, 20, 100, 400):
-        order, loss, st = call(limit)
+    tiles = sum(-(-(d - 48 - 64 * c) // 128) for c in range(d // 64))      # about those of the first pass
+    for stop in (1, 2, 3, 4, 5, 6, 8, 11, tiles // 2, tiles - 2, tiles - 1, tiles, 10 ** 6):
+        order, loss, st = call(max(stop, 1))
         late = st == -OBC_ERR_TIMEOUT
         assert bool((late | (st == 0)).all())
-        if limit < 0:
+        if stop == 1:
             assert bool(late.all())
+        if stop == 10 ** 6:
+            assert not bool(late.any())
         assert torch.equal(order[~late], want[0][~late]) and torch.equal(loss[~late], want[1][~late])
         assert bool((order[late][:, -1] == -1).all()) and bool(torch.isinf(loss[late][:, -1]).all())      # what was not produced
         assert torch.equal(torch.where(order[late] == -1, want[0][late], order[late]), want[0][late])         # what was, before
