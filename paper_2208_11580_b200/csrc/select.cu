@@ -265,7 +265,12 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) select_kernel(const float* __r
                     for (int r = tid; r < nr; r += SEL_THREADS) counts[r0 + r] = COUNT_TIMED_OUT;
                     return;
                 }
-                a = __ldcg(bins); b = __ldcg(bins + 1);
+                if constexpr (sizeof(Count) == 4) {
+                    const uint2 v = __ldcg(reinterpret_cast<const uint2*>(bins));
+                    a = v.x; b = v.y;
+                } else {
+                    a = __ldcg(bins); b = __ldcg(bins + 1);
+                }
             }
             sh.hist[2 * tid] = 0; sh.hist[2 * tid + 1] = 0;
             pick_digit(a, b, sh);
