@@ -32,10 +32,12 @@
 //
 // Step protocol.  Between two flushes every slot belongs to one thread (groups of 4 consecutive slots per
 // thread), which is the only one to touch wd[j], dg[j], perm[j] and its entries of the pending vectors; the
-// update phase also leaves an FP32 estimate of each own slot's next score in registers.  Each thread proposes its best slot, the
-// warps combine the proposals and publish one record per warp (with the candidate's weight and diagonal),
-// and after the single barrier of the step every warp reads the records and derives the same winner, so
-// no second barrier is needed to announce it.  Records alternate between two buffers by step parity.
+// update phase also leaves an FP32 estimate of each own slot's next score in registers.  The warps publish one record each
+// (their smallest estimate, and whether another one is near it), and after the single barrier of the step every warp reads the
+// records and derives the same winner (fast_pick).  Only where another slot's estimate is within 1e-4 of the smallest is the
+// choice made on FP64 scores, with a second barrier (thread_best, block_pick): ties to the last bit go by original index.
+// Records alternate between two buffers by step parity.
+// What bounds a step is the latency of this chain (scores, pick, pivot column, corrections, state), not its arithmetic.
 #pragma once
 #include "flush_tc.cuh"
 #include <type_traits>
@@ -43,7 +45,7 @@
 namespace obc {
 
 constexpr int BLK_MAXB = 64;
-constexpr int BLK_REC_BYTES = 640;            // one record buffer: 16 warps x (key, slot, orig, s, w, dg)
+constexpr int BLK_REC_BYTES = 640;            // one record buffer: 16 warps x fast record, 16 warps x (s, key, slot, orig)
 constexpr int BLK_OFF_BC = 1280;              // Bcast (grid parameters, flush bookkeeping)
 constexpr int BLK_OFF_PV = 1536;              // int pv[64]   slots eliminated since the last flush
 constexpr int BLK_OFF_HL = 1792;              // int hl[64]   holes (dead slots below the new size)
@@ -184,15 +186,14 @@ __host__ __device__ __forceinline__ int tri_at(int ld, int i, int j) { return ((
 __host__ __device__ inline size_t tri_floats(int cap) { return (size_t)((cap + 63) & ~63) * cap; }      // (an even number of groups)
 
 struct Records {                              // views into one record buffer
-    unsigned* key; int* slot; int* orig; double* s; double* w; double* dgv;
+    uint4* fast; unsigned* key; int* slot; int* orig; double* s;
 };
 __device__ __forceinline__ Records rec_view(char* scratch, int parity) {
     char* b = scratch + parity * BLK_REC_BYTES;
     Records r;
-    r.s = reinterpret_cast<double*>(b);       // [16]
-    r.w = r.s + 16;                           // [16]
-    r.dgv = r.w + 16;                         // [16]
-    r.key = reinterpret_cast<unsigned*>(r.dgv + 16);
+    r.fast = reinterpret_cast<uint4*>(b);     // [16]
+    r.s = reinterpret_cast<double*>(b + 256); // [16]
+    r.key = reinterpret_cast<unsigned*>(r.s + 16);
     r.slot = reinterpret_cast<int*>(r.key + 16);
     r.orig = r.slot + 16;
     return r;
@@ -203,9 +204,52 @@ __device__ __forceinline__ unsigned float_key(float x) {
     const unsigned u = __float_as_uint(x);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+__device__ __forceinline__ float key_float(unsigned k) { return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k); }
 constexpr unsigned KEY_NONE = 0xFFFFFFFFu;
+constexpr float NEAR = 1e-4f;                 // estimates this close (relative) are told apart by their FP64 scores
 
-struct Pick { int slot; int orig; double w; double dgv; double s; };
+struct Pick { int slot; int orig; double s; };
+
+// The block's smallest estimate.  m1: the thread's smallest (slot, orig: its slot; slot < 0: none), m2: its second smallest.
+// `sure`: no other estimate of the block is near it and it is well inside the FP32 range, so its slot has the smallest FP64
+// score too (an estimate is off by a few 1e-7).  One barrier.
+template <int NT>
+__device__ __forceinline__ Pick fast_pick(float m1, float m2, int slot, int orig, const Records& rec, bool* sure) {
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned key = slot >= 0 ? float_key(m1) : KEY_NONE;
+    const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
+    const float v = key_float(kmin), t = v + NEAR * fabsf(v);
+    const unsigned near = __ballot_sync(0xffffffffu, slot >= 0 && m1 <= t), two = __ballot_sync(0xffffffffu, m2 <= t);
+    const bool many = kmin == KEY_NONE || two != 0u || __popc(near) != 1;
+    if (many ? lane == 0 : m1 <= t && slot >= 0) rec.fast[warp] = make_uint4(kmin, (unsigned)slot, (unsigned)orig, many ? 1u : 0u);
+    __syncthreads();
+    uint4 q = make_uint4(KEY_NONE, 0u, 0u, 0u);
+    if (lane < NW) q = rec.fast[lane];
+    const unsigned kg = __reduce_min_sync(0xffffffffu, q.x);
+    const float vg = key_float(kg), tg = vg + NEAR * fabsf(vg);
+    const unsigned at = __ballot_sync(0xffffffffu, q.x == kg);
+    const unsigned others = __ballot_sync(0xffffffffu, q.x != kg && q.x <= float_key(tg));
+    const uint4 w = rec.fast[(__ffs(at) - 1) & (NW - 1)];
+    *sure = others == 0u && __popc(at) == 1 && w.w == 0u && vg >= 1e-30f && vg <= 1e30f;
+    Pick p;
+    p.slot = kg == KEY_NONE ? -1 : (int)w.y; p.orig = (int)w.z; p.s = 0.0;
+    return p;
+}
+// A slot that is known: its owner names it, the others have slot < 0.  One barrier.
+template <int NT>
+__device__ __forceinline__ Pick known_pick(int slot, int orig, const Records& rec) {
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned has = __ballot_sync(0xffffffffu, slot >= 0);
+    if (has ? slot >= 0 : lane == 0) rec.fast[warp] = make_uint4(has ? 0u : KEY_NONE, (unsigned)slot, (unsigned)orig, 0u);
+    __syncthreads();
+    const unsigned at = __ballot_sync(0xffffffffu, lane < NW && rec.fast[lane & (NW - 1)].x == 0u);
+    const uint4 w = rec.fast[at ? __ffs(at) - 1 : 0];
+    Pick p;
+    p.slot = at ? (int)w.y : -1; p.orig = (int)w.z; p.s = 0.0;
+    return p;
+}
 
 // Combines one candidate per lane into the lane holding the smallest (s, orig); key = float_key((float)s)
 // orders all but near-equal candidates, which are then compared exactly.  Returns the winning lane or -1.
@@ -230,8 +274,7 @@ __device__ __forceinline__ int warp_winner(unsigned key, double s, int orig) {
 // Every thread holds at most one candidate (slot < 0: none).  Publishes the warp's best in the record buffer,
 // then, after the barrier, every warp derives the block's best from the records.
 template <int NT>
-__device__ __forceinline__ Pick block_pick(unsigned key, double s, int slot, int orig, double w, double dgv,
-                                           const Records& rec) {
+__device__ __forceinline__ Pick block_pick(unsigned key, double s, int slot, int orig, const Records& rec) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (slot < 0) key = KEY_NONE;
@@ -239,7 +282,7 @@ __device__ __forceinline__ Pick block_pick(unsigned key, double s, int slot, int
     if (wl < 0) { if (lane == 0) rec.key[warp] = KEY_NONE; }
     else if (lane == wl) {
         rec.key[warp] = key; rec.slot[warp] = slot; rec.orig[warp] = orig;
-        rec.s[warp] = s; rec.w[warp] = w; rec.dgv[warp] = dgv;
+        rec.s[warp] = s;
     }
     __syncthreads();
     const bool in = lane < NW;
@@ -248,8 +291,8 @@ __device__ __forceinline__ Pick block_pick(unsigned key, double s, int slot, int
     const int o2 = (in && k2 != KEY_NONE) ? rec.orig[lane] : 0x7fffffff;
     const int ww = warp_winner(k2, s2, o2);
     Pick p;
-    p.slot = -1; p.orig = -1; p.w = 0.0; p.dgv = 0.0; p.s = 0.0;
-    if (ww >= 0) { p.slot = rec.slot[ww]; p.orig = rec.orig[ww]; p.w = rec.w[ww]; p.dgv = rec.dgv[ww]; p.s = rec.s[ww]; }
+    p.slot = -1; p.orig = -1; p.s = 0.0;
+    if (ww >= 0) { p.slot = rec.slot[ww]; p.orig = rec.orig[ww]; p.s = rec.s[ww]; }
     return p;
 }
 
@@ -267,20 +310,42 @@ static __device__ __noinline__ double grid_error(double w, double sc, double isc
     return grid_q_fast(w, sc, isc, ze, mq, &code) - w;
 }
 
-// FP32 estimate of the score of a slot (relative error of a few 1e-7): it only screens candidates, the slots
-// within 1e-4 of the thread's best estimate are scored again with the FP64 division.
+// The grid of a row as the estimates use it: the codes' integer range without the zero point.  sc = 0: a grid whose zero point
+// is no integer, or a scale far outside the range of ordinary weights; there every estimate is 0, which leaves the choice
+// to the FP64 scores of all slots.
+struct GridRange { float sc; int lo, hi; };
+__device__ __forceinline__ GridRange grid_range(double sc, double ze, double mq) {
+    GridRange g;
+    g.sc = __double2float_rn(sc);
+    const bool plain = fabs(ze) < 1e9 && ze == rint(ze) && fabs(sc) > 1e-30 && fabs(sc) < 1e30;      // (false for NaN)
+    if (!plain) g.sc = 0.f;
+    g.lo = plain ? -(int)ze : 0;
+    g.hi = plain ? (int)(mq - ze) : 0;
+    return g;
+}
+
+// FP32 estimate of the score of a slot (relative error of a few 1e-7): it only screens candidates, slots that are near the best
+// estimate are told apart by FP64 scores.  On a grid the distance to the nearest integer is taken in FP64 (w / scale has up to 8
+// bits before the point and a small distance is what wins); x + 1.5 * 2^52 - 1.5 * 2^52 rounds x to an integer whose low 32
+// bits are the sum's (three FP64 additions; rint, the clamps and the conversions take four times as many slots of the
+// FP64 and conversion pipes).
 template <bool Q>
-__device__ __forceinline__ float score_estimate(double w, double dgv, bool quant, double sc, double isc, double ze,
-                                                double mq) {
+__device__ __forceinline__ float score_estimate(double w, double dgv, bool quant, double isc, double ze, double mq,
+                                                const GridRange& gr) {
+    float ef;
     if (Q && quant) {
-        // plain product and rounding: next to a rounding boundary the two possible codes give the same |err| to
-        // ~1e-16, which is all an estimate needs (the exact scoring goes through grid_error)
-        const double c = fmin(fmax(rint(w * isc) + ze, 0.0), mq);
-        const double err = sc * (c - ze) - w;
-        return __fdividef(__double2float_rn(err * err), __double2float_rn(dgv));
+        constexpr double M = 6755399441055744.0;
+        const double t = w * isc, u = t + M;
+        const int r = __double2loint(u);
+        // (the high word says whether the integer fits 32 bits.)  Next to a rounding boundary the two possible codes give
+        // the same |err| to ~1e-16, which is all an estimate needs
+        double c = u - M;
+        if ((unsigned)__double2hiint(u) - 0x4337FFFFu > 1u || r < gr.lo || r > gr.hi) c = t < -ze ? -ze : mq - ze;
+        ef = gr.sc == 0.f ? 0.f : __double2float_rn(c - t) * gr.sc;
+    } else {
+        ef = __double2float_rn(w);
     }
-    const float wf = __double2float_rn(w);
-    return __fdividef(wf * wf, __double2float_rn(dgv));
+    return ef * __fdividef(ef, __double2float_rn(dgv));
 }
 
 // Estimates of all own slots from the state arrays (NaN for dead or unused slots).
@@ -289,7 +354,7 @@ __device__ __forceinline__ float score_estimate(double w, double dgv, bool quant
 // own slots' blocks, one byte per slot, which the update phase then keeps current in registers.
 template <int NT, int KMAX, bool Q>
 __device__ __forceinline__ void estimate_own(float (&sa)[KMAX], const double* wd, const double* dg, const int* perm,
-                                             int m0, bool quant, double sc, double isc, double ze, double mq,
+                                             int m0, bool quant, double isc, double ze, double mq, const GridRange& gr,
                                              const unsigned char* blkcnt, int nm_lg, int nm_prune,
                                              unsigned (&cntw)[KMAX / 4]) {
 #pragma unroll
@@ -301,9 +366,24 @@ __device__ __forceinline__ void estimate_own(float (&sa)[KMAX], const double* wd
         if (j < m0 && perm[j] >= 0) {
             unsigned c = 0u;
             if (blkcnt) { c = blkcnt[perm[j] >> nm_lg]; cntw[k >> 2] |= c << (8 * (k & 3)); }
-            if (!blkcnt || (int)c < nm_prune) sa[k] = score_estimate<Q>(wd[j], dg[j], quant, sc, isc, ze, mq);
+            if (!blkcnt || (int)c < nm_prune) sa[k] = score_estimate<Q>(wd[j], dg[j], quant, isc, ze, mq, gr);
         }
     }
+}
+
+// The thread's two smallest estimates and the slot of the first (-1: none); NaN estimates are no candidates.
+template <int NT, int KMAX>
+__device__ __forceinline__ void smallest_own(const float (&sa)[KMAX], float* m1, float* m2, int* slot) {
+    float a = CUDART_INF_F, b = CUDART_INF_F;
+    int ka = -1;
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) {
+        const bool lt = sa[k] < a;
+        b = lt ? a : fminf(b, sa[k]);                                   // (fminf ignores NaN)
+        a = lt ? sa[k] : a;
+        ka = lt ? k : ka;
+    }
+    *m1 = a; *m2 = b; *slot = ka < 0 ? -1 : own_slot<NT>(ka);
 }
 
 // The thread's best live slot among its own by (score, original index), given the estimates: only the slots
@@ -319,7 +399,7 @@ __device__ __forceinline__ void thread_best(const float (&sa)[KMAX], const doubl
     float smin = CUDART_INF_F;
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) smin = fminf(smin, sa[k]);           // fminf ignores NaN estimates
-    const float thr = smin + 1e-4f * fabsf(smin);
+    const float thr = smin + NEAR * fabsf(smin);
     unsigned cand = 0u, valid = 0u;
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) {
@@ -961,6 +1041,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         }
         __syncthreads();
         double gsc = bc->sc, gze = bc->ze, gmq = bc->mq;       // grid parameters of the row (registers)
+        GridRange gr = grid_range(gsc, gze, gmq);
 
         int m0 = m_begin;                // slots in use (tail phase: number of live slots)
         int nb = 0;                      // pending vectors
@@ -970,13 +1051,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         if (BC) bcur &= ~(BC - 1);           // whole blocks between two flushes, so that 4-slot groups stay together
         int s = s_begin;
         bool failed = false, timed_out = false;
-        int blk_base = 0;                // block pruning: first slot and score of the block being eliminated
+        int blk_base = 0, blk_orig = 0;  // block pruning: first slot, its column and the score of the block being eliminated
         double blk_score = 0.0;
         float sa[KMAX];                  // score estimates of the own slots, kept up to date by the update phase
         unsigned cntw[KMAX / 4];         // N:M: eliminations so far in the block of each own slot (one byte per slot)
 #pragma unroll
         for (int g = 0; g < KMAX / 4; ++g) cntw[g] = 0u;
         bool sa_valid = false;
+        unsigned alive = 0u;             // own slots that are live
+        bool alive_valid = false;
         double gisc = 1.0 / gsc;
         for (; s < total; ++s) {
             if (!tail) {
@@ -1049,7 +1132,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         if (!TC) colmask[h >> 5] = 0u;
                     }
                     m0 = m1; nb = 0;
-                    sa_valid = false;
+                    sa_valid = false; alive_valid = false;
 #pragma unroll
                     for (int k = 0; k < KMAX; ++k) sa[k] = CUDART_NAN_F;      // slots changed hands: not carried over
 #pragma unroll
@@ -1239,7 +1322,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         }
                         nb += GS;
                         s += GS - 1;
-                        sa_valid = false;
+                        sa_valid = false; alive_valid = false;
 #pragma unroll
                         for (int k = 0; k < KMAX; ++k) sa[k] = CUDART_NAN_F;
                         continue;
@@ -1269,28 +1352,31 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 if (tid == 0) { a.scale[r] = sc; a.zero[r] = ze; }
                 gsc = (double)sc; gze = (double)ze; gmq = (double)grid_maxq(a.bits, a.symmetric);
                 gisc = 1.0 / gsc;
+                gr = grid_range(gsc, gze, gmq);
                 sa_valid = false;
                 __syncthreads();                               // rf is reused by the next row's grid
             }
-            // ---- pick the slot: one candidate per thread, combined through the record buffer ------------
-            unsigned key = KEY_NONE;
-            double cs = 0.0;
-            int cslot = -1;
+            // ---- pick the slot ---------------------------------------------------------------------------
+            const Records rec = rec_view(scratch, s & 1);
+            Pick pk;
+            bool sure = true;
             if (forced) {
                 const int f = a.forced_order[(size_t)r * d + s];
+                int cslot = -1;
 #pragma unroll
                 for (int k = 0; k < KMAX; ++k) {
                     const int j = own_slot<NT>(k);
-                    if (j < m0 && perm[j] == f) { cslot = j; key = 0x80000000u; }
+                    if (j < m0 && perm[j] == f) cslot = j;
                 }
+                pk = known_pick<NT>(cslot, f, rec);
             } else if (BC && (s - n_forced) % BCD != 0) {
-                // the next member of the block chosen at the last block boundary
-                const int j = blk_base + (s - n_forced) % BCD;
-                if (j >= (tid << 2) && ((j - (tid << 2)) % (4 * NT)) < 4) { cslot = j; key = 0x80000000u; }
+                // the next member of the block chosen at the last block boundary: a block's slots hold consecutive columns
+                __syncthreads();
+                pk.slot = blk_base + (s - n_forced) % BCD; pk.orig = blk_orig + (s - n_forced) % BCD; pk.s = 0.0;
             } else if (BC) {
                 // block boundary: exact FP64 score of every own live group (its four slots are all live here)
                 double bs = CUDART_INF;
-                int bo = 0x7fffffff;
+                int bo = 0x7fffffff, cslot = -1;
 #pragma unroll
                 for (int g = 0; g < KMAX / 4; ++g) {
                     const int jb = own_slot<NT>(4 * g);
@@ -1302,23 +1388,33 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         if (key_less(sc4, o, bs, bo)) { bs = sc4; bo = o; cslot = jb; }
                     }
                 }
-                cs = bs;
-                if (cslot >= 0) key = float_key(__double2float_rn(bs));
+                pk = block_pick<NT>(cslot >= 0 ? float_key(__double2float_rn(bs)) : KEY_NONE, bs, cslot, cslot >= 0 ? perm[cslot] : -1, rec);
+                blk_base = pk.slot; blk_orig = pk.orig; blk_score = pk.s;
             } else {
                 if (!sa_valid || tail || outliers)
-                    estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gsc, gisc, gze, gmq, has_nm ? blkcnt : nullptr,
+                    estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gisc, gze, gmq, gr, has_nm ? blkcnt : nullptr,
                                            nm_lg, nm_prune, cntw);
-                thread_best<NT, KMAX, Q>(sa, wd, dg, perm, q_now, outliers, gsc, gisc, gze, gmq, &key, &cs, &cslot);
+                if (!(Q && outliers)) {
+                    float e1, e2;
+                    int cslot;
+                    smallest_own<NT, KMAX>(sa, &e1, &e2, &cslot);
+                    pk = fast_pick<NT>(e1, e2, cslot, cslot >= 0 ? perm[cslot] : -1, rec, &sure);
+                } else {
+                    sure = false;
+                }
+                if (!sure) {                                   // (the same for every thread of the block)
+                    unsigned key = KEY_NONE;
+                    double cs = 0.0;
+                    int cslot = -1;
+                    thread_best<NT, KMAX, Q>(sa, wd, dg, perm, q_now, outliers, gsc, gisc, gze, gmq, &key, &cs, &cslot);
+                    pk = block_pick<NT>(key, cs, cslot, cslot >= 0 ? perm[cslot] : -1, rec);
+                }
             }
-            const Records rec = rec_view(scratch, s & 1);
-            const Pick pk = block_pick<NT>(key, cs, cslot, cslot >= 0 ? perm[cslot] : -1,
-                                           cslot >= 0 ? wd[cslot] : 0.0, cslot >= 0 ? dg[cslot] : 0.0, rec);
             const int p = pk.slot, op = pk.orig;
-            const double dpp = pk.dgv, wp = pk.w;
-            if (BC && !forced && (s - n_forced) % BCD == 0) { blk_base = p; blk_score = pk.s; }
+            const double dpp = p < 0 ? 0.0 : dg[p], wp = p < 0 ? 0.0 : wd[p];      // (a pivot's state is not written again)
             if (p < 0 || !(dpp > 0.0) || !isfinite(dpp) || !isfinite(wp)) { failed = true; break; }
             double qp = 0.0, code = -1.0;
-            if (Q && q_now) qp = grid_q(wp, gsc, gze, gmq, &code);
+            if (Q && q_now) qp = grid_q_fast(wp, gsc, gisc, gze, gmq, &code);
             const double e = wp - qp;
             if (!tail) {
                 // ======================= deferred-update step ==============================================
@@ -1326,18 +1422,28 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 // pivot column of the stored matrix (own slots), corrected by the pending vectors
                 const float* const tri = HP;
                 float c[KMAX], corr[KMAX];
-                unsigned live = 0u;
+                if (!alive_valid) {
+                    alive = 0u;
+#pragma unroll
+                    for (int g = 0; g < KMAX / 4; ++g) {
+                        const int jb = own_slot<NT>(4 * g);
+                        if (jb >= m0) continue;
+                        const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
+                        const int pq[4] = {pm.x, pm.y, pm.z, pm.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (jb + q < m0 && pq[q] >= 0) alive |= 1u << (4 * g + q);
+                    }
+                    alive_valid = true;
+                }
+                const bool owner = ((p >> 2) & (NT - 1)) == tid;
+                if (owner) alive &= ~(1u << ((p >> 2) / NT * 4 + (p & 3)));
 #pragma unroll
                 for (int g = 0; g < KMAX / 4; ++g) {
                     const int jb = own_slot<NT>(4 * g);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) { c[4 * g + q] = 0.f; corr[4 * g + q] = 0.f; }
                     if (jb >= m0) continue;
-                    const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
-                    const int pq[4] = {pm.x, pm.y, pm.z, pm.w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (jb + q < m0 && pq[q] >= 0) live |= 1u << (4 * g + q);
                     if (jb + 3 <= p) {
                         const float4 v = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
                         c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
@@ -1345,7 +1451,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int j = jb + q;
-                            if ((live >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                            if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
                         }
                     }
                 }
@@ -1358,7 +1464,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     const float zp = zo[p];
 #pragma unroll
                     for (int g = 0; g < KMAX / 4; ++g) {
-                        if ((live >> (4 * g)) & 0xFu) {
+                        if ((alive >> (4 * g)) & 0xFu) {
                             const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
                             corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
                             corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
@@ -1374,7 +1480,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     const float zp = zo[p];
 #pragma unroll
                     for (int g = 0; g < KMAX / 4; ++g) {
-                        if ((live >> (4 * g)) & 0xFu) {
+                        if ((alive >> (4 * g)) & 0xFu) {
                             const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
                             corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
                             corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
@@ -1391,8 +1497,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int g = 0; g < KMAX / 4; ++g) {
                     const int jb = own_slot<NT>(4 * g);
                     if (jb >= m0) continue;
-                    const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
-                    const int pq[4] = {pm.x, pm.y, pm.z, pm.w};
+                    int pq[4] = {0, 0, 0, 0};
+                    if (has_nm || has_wfull) {
+                        const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
+                        pq[0] = pm.x; pq[1] = pm.y; pq[2] = pm.z; pq[3] = pm.w;
+                    }
                     float zv[4];
                     // the group's FP64 state as 128-bit accesses: a warp's 64-bit accesses at this stride (32 bytes
                     // between lanes) would meet four to a bank; dead slots keep the value they had
@@ -1402,21 +1511,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     double wv[4] = {w01.x, w01.y, w23.x, w23.y}, dv[4] = {d01.x, d01.y, d23.x, d23.y};
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const int k = 4 * g + q, j = jb + q;
+                        const int k = 4 * g + q;
                         zv[q] = 0.f;
                         sa[k] = CUDART_NAN_F;
-                        if (!((live >> k) & 1u)) continue;
-                        if (j == p) {
-                            perm[j] = -1;
-                            if (has_nm) blkcnt[op >> nm_lg] += 1;      // read again only behind a barrier
-                            continue;
-                        }
+                        if (!((alive >> k) & 1u)) continue;
                         const float vj = c[k] - corr[k];
                         const double nw = wv[q] - f * (double)vj;
                         const double nd = dv[q] - (double)vj * (double)vj * idpp;
                         wv[q] = nw; dv[q] = nd;
                         zv[q] = vj * rs;
-                        if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gsc, gisc, gze, gmq);
+                        if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gisc, gze, gmq, gr);
                         if (has_nm) {
                             if ((pq[q] >> nm_lg) == (op >> nm_lg)) cntw[g] += 1u << (8 * q);
                             if ((int)((cntw[g] >> (8 * q)) & 0xFFu) >= nm_prune) sa[k] = CUDART_NAN_F;
@@ -1426,7 +1530,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     wq[0] = make_double2(wv[0], wv[1]); wq[1] = make_double2(wv[2], wv[3]);
                     dq[0] = make_double2(dv[0], dv[1]); dq[1] = make_double2(dv[2], dv[3]);
                     *reinterpret_cast<float4*>(zb + jb) = make_float4(zv[0], zv[1], zv[2], zv[3]);
-                    if (BC == 4 && ((live >> (4 * g)) & 0xFu) == 0xFu && jb != (p & ~3)) {
+                    if (BC == 4 && ((alive >> (4 * g)) & 0xFu) == 0xFu) {
                         // Lemma 1 on the group's own 4 x 4 diagonal block (off-diagonal part; dg holds the diagonal)
                         double* o = boff + (jb >> 2) * 6;
                         const double v0 = (double)(c[4 * g] - corr[4 * g]), v1 = (double)(c[4 * g + 1] - corr[4 * g + 1]);
@@ -1447,7 +1551,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         for (int q = 0; q < 4; ++q) mine[q] = c[4 * g + q] - corr[4 * g + q];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) other[q] = __shfl_xor_sync(0xffffffffu, mine[q], 1);
-                        if (jb < m0 && ((live >> (4 * g)) & 0xFu) == 0xFu && (jb & ~7) != (p & ~7)) {
+                        if (jb < m0 && ((alive >> (4 * g)) & 0xFu) == 0xFu && (jb & ~7) != (p & ~7)) {
                             const bool first = (jb & 7) == 0;
                             double v[8];
 #pragma unroll
@@ -1465,7 +1569,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     }
                 }
                 sa_valid = est_next;
-                if (tid == 0) {
+                if (owner) {
+                    perm[p] = -1;
+                    if (has_nm) blkcnt[op >> nm_lg] += 1;              // read again only behind a barrier
+                }
+                if (tid == NT - 32) {                          // (of the warp with the fewest slots)
                     pv[nb] = p;
                     if (has_wfull) wfull[op] = (float)qp;
                     if (a.W_out) a.W_out[(size_t)r * a.ldwo + op] = (float)qp;
@@ -1473,7 +1581,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     if (!forced) {
                         const int t = s - n_forced;
                         if (a.order) a.order[(size_t)r * d + t] = op;
-                        if (a.loss) a.loss[(size_t)r * d + t] = BC ? ((t % BCD) ? 0.f : (float)blk_score) : (float)(e * e / dpp);
+                        if (a.loss) a.loss[(size_t)r * d + t] = BC ? ((t % BCD) ? 0.f : (float)blk_score) : (float)(e * f);
                     }
                     if (q_now && a.codes) a.codes[(size_t)r * d + op] = (int)code;
                 }
