@@ -26,8 +26,9 @@ obc_status blk_launch_512_12(const FlushMaps& zmaps, const EngineArgs& a, int bl
 // takes 149 ms since the layout and the tile order changed.)
 constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)110 << 20;
 
-static int blk_pick_ms(int d, size_t panel_bytes) {
-    int ms = d < 1024 ? d : 1024;
+// (one slot per thread on chip)
+static int blk_pick_ms(int d, size_t panel_bytes, int nt) {
+    int ms = d < nt ? d : nt;
     if (ms < 2) ms = 2;
     while (ms > 2 && blk_tail_bytes(ms) > panel_bytes) --ms;
     return ms;
@@ -74,7 +75,7 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     if (share < fixed + min_panel || share < fixed + blk_tail_bytes(2)) return false;
     p.smem = share;
     p.panel_floats = (int)((share - fixed) / 4);
-    p.ms = blk_pick_ms(d, share - fixed);
+    p.ms = blk_pick_ms(d, share - fixed, nt);
     // Rows of one 512-thread block per SM: shared memory holds fewer pending vectors than a pass can apply (19 at d_col = 2304, 12
     // at 3072, 6 at 4608); further ones go to a global buffer small enough to stay in L2 (the triangle itself is streamed past
     // it with evict-first hints).

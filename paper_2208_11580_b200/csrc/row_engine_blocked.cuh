@@ -20,7 +20,7 @@
 // mma.sync (warp tiles of 16 rows x 64 columns, TF32 split products, see blk_flush_mma): there the passes of one row
 // overlap the steps of another, and tensor memory and tile buffers would have to be shared.  The O(m) selection state (weights,
 // diagonal) is FP64, as in the streaming engine.  Once the live triangle fits into the shared memory of the pending
-// vectors, the row finishes on chip with step-by-step updates.
+// vectors, the row finishes on chip: one slot per thread with its state in registers, eight updates deferred.
 //
 // Shares of rows.  When a launch has more rows than resident blocks and the rows do not divide evenly, whole waves
 // would leave most SMs idle through the last one.  Instead every block gets the same amount of work: the rows
@@ -70,7 +70,12 @@ __host__ __device__ inline size_t blk_state_bytes(int cap, bool wfull, bool nm =
 // Stride of the pending vectors for a row of m slots: = 8 (mod 32), so that the tensor-core fragments of the
 // flush (4 vectors x 8 consecutive slots per load) touch 32 different banks.
 __host__ __device__ inline int blk_ldz(int m) { return ((m + 8 + 31) & ~31) + 8; }     // >= m + 16
-static size_t blk_tail_bytes(int ms) { return (size_t)12 * ((ms + 3) & ~3) + (size_t)4 * ms * (ms + 1); }
+// On chip: TAIL_B deferred updates as two arrays per slot (column entries v, v / [H]_pp; TAIL_LD floats apart: 128-bit accesses
+// of consecutive slots meet no bank twice), then the lower triangle, its rows end to end: column p of 32 rows from a multiple of
+// 32 on touches 32 different banks (triangular numbers mod 32 are a permutation).
+constexpr int TAIL_B = 8, TAIL_LD = 12;
+__host__ __device__ __forceinline__ int tail_at(int i, int j) { return i * (i + 1) / 2 + j; }      // j <= i
+static size_t blk_tail_bytes(int ms) { return (size_t)8 * TAIL_LD * ms + (size_t)4 * tail_at(ms, 0); }
 
 // ---- shares of rows ------------------------------------------------------------------------------------------------
 constexpr int BLK_SPLIT_WAIT_LIMIT = 1 << 22;  // polls (256 ns apart) before a block gives up on a row its neighbour started
@@ -766,21 +771,30 @@ __device__ __forceinline__ void blk_fill_holes(float* H, int ldp, int m1, int nh
     }
 }
 
-// Step-by-step Lemma-1 update on the shared-memory triangle S (leading dimension lds) in the coordinates
-// that hold after slot `last` moved into slot pm (pm < 0: nothing moved); mp = rows left.
+// The deferred updates of the on-chip triangle S (m slots): S[i][j] -= sum_b v_b[i] u_b[j].  A warp takes 8 rows and 32 columns at a
+// time; rows of eliminated slots are left out.
 template <int NT>
-__device__ __forceinline__ void blk_pass_shared(float* S, int lds, int mp, int pm, const float* v, const float* u,
-                                                const float* lr) {
+__device__ __forceinline__ void tail_flush(float* S, int m, const float* vt, const float* ut, const int* perm) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = warp; i < mp; i += NW) {
-        float* row = S + i * lds;
-        const float nv = -v[i];
-        for (int j = lane; j <= i; j += 32) {
-            const float base = (i == pm) ? lr[j] : (j == pm ? lr[i] : row[j]);
-            row[j] = fmaf(nv, u[j], base);
+    for (int i0 = 8 * warp; i0 < m; i0 += 8 * NW)
+        for (int c0 = 0; c0 < min(i0 + 8, m); c0 += 32) {
+            const int j = c0 + lane;
+            const float4* uj = reinterpret_cast<const float4*>(ut + min(j, m - 1) * TAIL_LD);
+            const float4 u0 = uj[0], u1 = uj[1];
+#pragma unroll 4
+            for (int i = i0; i < min(i0 + 8, m); ++i) {
+                if (perm[i] < 0) continue;
+                const float4* vi = reinterpret_cast<const float4*>(vt + i * TAIL_LD);
+                const float4 v0 = vi[0], v1 = vi[1];
+                if (j <= i) {
+                    float x = v0.x * u0.x;
+                    x = fmaf(v0.y, u0.y, x); x = fmaf(v0.z, u0.z, x); x = fmaf(v0.w, u0.w, x);
+                    x = fmaf(v1.x, u1.x, x); x = fmaf(v1.y, u1.y, x); x = fmaf(v1.z, u1.z, x); x = fmaf(v1.w, u1.w, x);
+                    S[tail_at(i, j)] -= x;
+                }
+            }
         }
-    }
 }
 
 // Block pruning (Section 3, "Block-Sparsity", Eq. 5), blocks of 4: score w_P^T ((Hinv)_P)^-1 w_P of one 4-slot group
@@ -884,13 +898,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     double* boff = reinterpret_cast<double*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm) - before_state);
     float* panel = reinterpret_cast<float*>(smem + BLK_FIXED + blk_state_bytes(cap, has_wfull, has_nm, BC));
     if (TC) { wd = reinterpret_cast<double*>(panel) - 2 * cap; dg = wd + cap; }
-    // tail views (step-by-step phase in shared memory) share the panel's space
-    const int msr = (ms + 3) & ~3;
-    float* tv = panel;
-    float* tu = tv + msr;
-    float* tlr = tu + msr;
-    float* S = tlr + msr;
-    const int lds = ms + 1;
+    // tail views (the end of a row in shared memory) share the panel's space
+    float* vt = panel;
+    float* ut = vt + TAIL_LD * ms;
+    float* S = ut + TAIL_LD * ms;
     const int ldp = a.ldp;
     float* const Hp0 = a.Hws ? a.Hws + (size_t)blockIdx.x * tri_floats(cap) : nullptr;      // the block's own triangle
 #define HP (SH ? *reinterpret_cast<float**>(smem + BLK_OFF_SCHED + 16) : Hp0)
@@ -1019,7 +1030,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int j = tid; j < d; j += NT)
                     a.w_trace[((size_t)r * (a.trace_steps + 1)) * d + j] = a.W[(size_t)r * a.ldw + j];
         }
-        bool tail = false;
         if (kind != ITEM_TAIL && d > ms && total > 0) {
             for (int i = warp; i < d; i += NW) {
                 const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
@@ -1061,101 +1071,110 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         unsigned alive = 0u;             // own slots that are live
         bool alive_valid = false;
         double gisc = 1.0 / gsc;
-        for (; s < total; ++s) {
-            if (!tail) {
-                if (d > ms && nb > 0 && (nb == bcur || m0 - nb <= ms || (SH && s == sched[1]))) {
-                    // ---- flush: apply the pending vectors and compact to m1 slots ------------------------
-                    __syncthreads();                           // the last step's vector and perm updates
-                    const int m1 = m0 - nb;
-                    if (warp == 0) {
-                        // holes (dead slots below the new size) and, as many, live slots above it, paired by rank
-                        int nh = 0, nm = 0;
+        // (every thread: the smallest and largest weight of its survivors)
+        auto survivors_grid = [&](float lo, float hi) {
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int b = lane + 32 * q;
-                            const int h = b < nb ? pv[b] : 0x7fffffff;
-                            const unsigned hm = __ballot_sync(0xffffffffu, h < m1);
-                            if (h < m1) hl[nh + __popc(hm & ((1u << lane) - 1u))] = h;
-                            nh += __popc(hm);
-                            const bool lv = b < nb && perm[m1 + b] >= 0;
-                            const unsigned lm = __ballot_sync(0xffffffffu, lv);
-                            if (lv) mv[nm + __popc(lm & ((1u << lane) - 1u))] = m1 + b;
-                            nm += __popc(lm);
-                        }
-                        if (lane == 0) bc->nh = nh;
-                    } else if (TC && tid == 32) {
-                        ft_init_bars(fb);
-                    }
-                    __syncthreads();
-                    const int nh = bc->nh;
-                    for (int idx = tid; idx < nh * nb; idx += NT) {
-                        const int q = idx / nb, b = idx - q * nb;
-                        float* zr = (!GP || b < scap) ? panel + (size_t)b * ldz : GVEC + (size_t)(b - scap) * gld;
-                        zr[hl[q]] = zr[mv[q]];
-                    }
-                    if (tid < nh) {
-                        const int h = hl[tid];
-                        srcm[h] = (unsigned short)mv[tid];
-                        if (!TC) atomicOr(&colmask[h >> 5], 1u << (h & 31));
-                    }
-                    __syncthreads();
-                    if constexpr (TC) {
-                        blk_fill_holes<NT>(HP, ldp, m1, nh, hl, mv, srcm);
-                        signed char* zexp = a.zexp + (size_t)blockIdx.x * cap;
-                        const int power = blk_make_planes<NT, KMAX>(panel, ldz, GP ? scap : nb, GP ? GVEC : nullptr, gld, nb, m0, m1, dg, perm, rf,
-                                                                    a.Zws + (size_t)blockIdx.x * 128 * a.zld, a.zld, zexp);
-                        // the FP64 state gives its space to the pass (d_col = 4608: three tile buffers instead of two)
-                        double2* park = a.park + (size_t)blockIdx.x * cap;
-                        for (int j = tid; j < cap; j += NT) park[j] = reinterpret_cast<const double2*>(wd)[j];      // (wd and dg: 2 cap doubles)
-                        asm volatile("fence.proxy.async;" ::: "memory");            // plain accesses before the copies
-                        __syncthreads();
-                        unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wd) + 1023) & ~(uintptr_t)1023);
-                        const int stage_bytes = (int)(reinterpret_cast<unsigned char*>(panel + a.panel_floats) - stage);
-                        const bool fine = blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
-                                          power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr, a.stop_tile);
-                        for (int j = tid; j < cap; j += NT) reinterpret_cast<double2*>(wd)[j] = __ldcg(park + j);
-                        __syncthreads();
-                        if (!fine) { timed_out = true; break; }
-                    } else if (!GP)
-                        blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);      // evict-first at every row length (~1 %)
-                    else
-                        blk_flush_mma<NT, true, true>(HP, ldp, m1, nb, min(nb, scap), panel, ldz, GVEC, gld, ZSTAGE, srcm, colmask);
-                    __syncthreads();
-                    if (tid < nh) {
-                        const int h = hl[tid], sv = mv[tid];
-                        wd[h] = wd[sv]; dg[h] = dg[sv]; perm[h] = perm[sv];
-                        if (BC == 4 && (h & 3) == 0)      // holes and movers are whole aligned groups in block mode
-                            for (int k = 0; k < 6; ++k) boff[(h >> 2) * 6 + k] = boff[(sv >> 2) * 6 + k];
-                        if (BC == 8 && (h & 7) == 0)
-                            for (int k = 0; k < 28; ++k) boff[(h >> 3) * 28 + k] = boff[(sv >> 3) * 28 + k];
-                        srcm[h] = (unsigned short)h;
-                        if (!TC) colmask[h >> 5] = 0u;
-                    }
-                    m0 = m1; nb = 0;
-                    sa_valid = false; alive_valid = false;
-#pragma unroll
-                    for (int k = 0; k < KMAX; ++k) sa[k] = CUDART_NAN_F;      // slots changed hands: not carried over
-#pragma unroll
-                    for (int g = 0; g < KMAX / 4; ++g) cntw[g] = 0u;
-                    ldz = blk_ldz(m0);
-                    scap = a.panel_floats / ldz;
-                    bcur = min(a.max_pending, scap + gB);
-                    if (BC) bcur &= ~(BC - 1);
-                    __syncthreads();
-                }
-                if (SH && s == sched[1]) break;      // (shares of rows) the row is handed over here, everything applied
-                if (m0 <= ms) {
-                    // ---- move on chip: slots [0, m0) are all live here and the stored triangle is current
-                    for (int i = warp; i < m0; i += NW)
-                        for (int j = lane; j <= i; j += 32)
-                            S[i * lds + j] = d > ms ? ld_tri<TC>(HP + tri_at(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
-                    tail = true;
-                    __syncthreads();
-                }
+            for (int off = 16; off; off >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
             }
+            if (lane == 0) { rf[warp] = lo; rf[32 + warp] = hi; }
+            __syncthreads();
+            for (int k = 0; k < NW; ++k) { lo = fminf(lo, rf[k]); hi = fmaxf(hi, rf[32 + k]); }
+            float sc, ze;
+            grid_from_range(lo, hi, a.bits, a.symmetric, &sc, &ze);
+            if (tid == 0) { a.scale[r] = sc; a.zero[r] = ze; }
+            gsc = (double)sc; gze = (double)ze; gmq = (double)grid_maxq(a.bits, a.symmetric);
+            gisc = 1.0 / gsc;
+            gr = grid_range(gsc, gze, gmq);
+            __syncthreads();                                   // rf is reused by the next row's grid
+        };
+        for (; s < total; ++s) {
+            if (d > ms && nb > 0 && (nb == bcur || m0 - nb <= ms || (SH && s == sched[1]))) {
+                // ---- flush: apply the pending vectors and compact to m1 slots ------------------------
+                __syncthreads();                           // the last step's vector and perm updates
+                const int m1 = m0 - nb;
+                if (warp == 0) {
+                    // holes (dead slots below the new size) and, as many, live slots above it, paired by rank
+                    int nh = 0, nm = 0;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int b = lane + 32 * q;
+                        const int h = b < nb ? pv[b] : 0x7fffffff;
+                        const unsigned hm = __ballot_sync(0xffffffffu, h < m1);
+                        if (h < m1) hl[nh + __popc(hm & ((1u << lane) - 1u))] = h;
+                        nh += __popc(hm);
+                        const bool lv = b < nb && perm[m1 + b] >= 0;
+                        const unsigned lm = __ballot_sync(0xffffffffu, lv);
+                        if (lv) mv[nm + __popc(lm & ((1u << lane) - 1u))] = m1 + b;
+                        nm += __popc(lm);
+                    }
+                    if (lane == 0) bc->nh = nh;
+                } else if (TC && tid == 32) {
+                    ft_init_bars(fb);
+                }
+                __syncthreads();
+                const int nh = bc->nh;
+                for (int idx = tid; idx < nh * nb; idx += NT) {
+                    const int q = idx / nb, b = idx - q * nb;
+                    float* zr = (!GP || b < scap) ? panel + (size_t)b * ldz : GVEC + (size_t)(b - scap) * gld;
+                    zr[hl[q]] = zr[mv[q]];
+                }
+                if (tid < nh) {
+                    const int h = hl[tid];
+                    srcm[h] = (unsigned short)mv[tid];
+                    if (!TC) atomicOr(&colmask[h >> 5], 1u << (h & 31));
+                }
+                __syncthreads();
+                if constexpr (TC) {
+                    blk_fill_holes<NT>(HP, ldp, m1, nh, hl, mv, srcm);
+                    signed char* zexp = a.zexp + (size_t)blockIdx.x * cap;
+                    const int power = blk_make_planes<NT, KMAX>(panel, ldz, GP ? scap : nb, GP ? GVEC : nullptr, gld, nb, m0, m1, dg, perm, rf,
+                                                                a.Zws + (size_t)blockIdx.x * 128 * a.zld, a.zld, zexp);
+                    // the FP64 state gives its space to the pass (d_col = 4608: three tile buffers instead of two)
+                    double2* park = a.park + (size_t)blockIdx.x * cap;
+                    for (int j = tid; j < cap; j += NT) park[j] = reinterpret_cast<const double2*>(wd)[j];      // (wd and dg: 2 cap doubles)
+                    asm volatile("fence.proxy.async;" ::: "memory");            // plain accesses before the copies
+                    __syncthreads();
+                    unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wd) + 1023) & ~(uintptr_t)1023);
+                    const int stage_bytes = (int)(reinterpret_cast<unsigned char*>(panel + a.panel_floats) - stage);
+                    const bool fine = blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
+                                      power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr, a.stop_tile);
+                    for (int j = tid; j < cap; j += NT) reinterpret_cast<double2*>(wd)[j] = __ldcg(park + j);
+                    __syncthreads();
+                    if (!fine) { timed_out = true; break; }
+                } else if (!GP)
+                    blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);      // evict-first at every row length (~1 %)
+                else
+                    blk_flush_mma<NT, true, true>(HP, ldp, m1, nb, min(nb, scap), panel, ldz, GVEC, gld, ZSTAGE, srcm, colmask);
+                __syncthreads();
+                if (tid < nh) {
+                    const int h = hl[tid], sv = mv[tid];
+                    wd[h] = wd[sv]; dg[h] = dg[sv]; perm[h] = perm[sv];
+                    if (BC == 4 && (h & 3) == 0)      // holes and movers are whole aligned groups in block mode
+                        for (int k = 0; k < 6; ++k) boff[(h >> 2) * 6 + k] = boff[(sv >> 2) * 6 + k];
+                    if (BC == 8 && (h & 7) == 0)
+                        for (int k = 0; k < 28; ++k) boff[(h >> 3) * 28 + k] = boff[(sv >> 3) * 28 + k];
+                    srcm[h] = (unsigned short)h;
+                    if (!TC) colmask[h >> 5] = 0u;
+                }
+                m0 = m1; nb = 0;
+                sa_valid = false; alive_valid = false;
+#pragma unroll
+                for (int k = 0; k < KMAX; ++k) sa[k] = CUDART_NAN_F;      // slots changed hands: not carried over
+#pragma unroll
+                for (int g = 0; g < KMAX / 4; ++g) cntw[g] = 0u;
+                ldz = blk_ldz(m0);
+                scap = a.panel_floats / ldz;
+                bcur = min(a.max_pending, scap + gB);
+                if (BC) bcur &= ~(BC - 1);
+                __syncthreads();
+            }
+            if (SH && s == sched[1]) break;      // (shares of rows) the row is handed over here, everything applied
+            if (m0 <= ms) break;                 // on chip from here
             const bool forced = s < n_forced;
             const bool q_now = Q && quant && !forced;
-            if (FG && forced && !tail && !has_wfull && !has_nm && s + BLK_GS <= (SH ? min(n_forced, sched[1]) : n_forced) && nb + BLK_GS <= bcur &&
+            if (FG && forced && !has_wfull && !has_nm && s + BLK_GS <= (SH ? min(n_forced, sched[1]) : n_forced) && nb + BLK_GS <= bcur &&
                 (!GP || nb + BLK_GS <= scap)) {
                 // ======================= four forced eliminations together ================================
                 constexpr int GS = BLK_GS;
@@ -1339,22 +1358,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     const int j = own_slot<NT>(k);
                     if (j < m0 && perm[j] >= 0) { const float w = (float)wd[j]; lo = fminf(lo, w); hi = fmaxf(hi, w); }
                 }
-#pragma unroll
-                for (int off = 16; off; off >>= 1) {
-                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
-                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
-                }
-                if (lane == 0) { rf[warp] = lo; rf[32 + warp] = hi; }
-                __syncthreads();
-                for (int k = 0; k < NW; ++k) { lo = fminf(lo, rf[k]); hi = fmaxf(hi, rf[32 + k]); }
-                float sc, ze;
-                grid_from_range(lo, hi, a.bits, a.symmetric, &sc, &ze);
-                if (tid == 0) { a.scale[r] = sc; a.zero[r] = ze; }
-                gsc = (double)sc; gze = (double)ze; gmq = (double)grid_maxq(a.bits, a.symmetric);
-                gisc = 1.0 / gsc;
-                gr = grid_range(gsc, gze, gmq);
+                survivors_grid(lo, hi);
                 sa_valid = false;
-                __syncthreads();                               // rf is reused by the next row's grid
             }
             // ---- pick the slot ---------------------------------------------------------------------------
             const Records rec = rec_view(scratch, s & 1);
@@ -1391,7 +1396,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 pk = block_pick<NT>(cslot >= 0 ? float_key(__double2float_rn(bs)) : KEY_NONE, bs, cslot, cslot >= 0 ? perm[cslot] : -1, rec);
                 blk_base = pk.slot; blk_orig = pk.orig; blk_score = pk.s;
             } else {
-                if (!sa_valid || tail || outliers)
+                if (!sa_valid || outliers)
                     estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gisc, gze, gmq, gr, has_nm ? blkcnt : nullptr,
                                            nm_lg, nm_prune, cntw);
                 if (!(Q && outliers)) {
@@ -1416,226 +1421,337 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
             double qp = 0.0, code = -1.0;
             if (Q && q_now) qp = grid_q_fast(wp, gsc, gisc, gze, gmq, &code);
             const double e = wp - qp;
-            if (!tail) {
-                // ======================= deferred-update step ==============================================
-                float* zb = (!GP || nb < scap) ? panel + (size_t)nb * ldz : GVEC + (size_t)(nb - scap) * gld;
-                // pivot column of the stored matrix (own slots), corrected by the pending vectors
-                const float* const tri = HP;
-                float c[KMAX], corr[KMAX];
-                if (!alive_valid) {
-                    alive = 0u;
-#pragma unroll
-                    for (int g = 0; g < KMAX / 4; ++g) {
-                        const int jb = own_slot<NT>(4 * g);
-                        if (jb >= m0) continue;
-                        const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
-                        const int pq[4] = {pm.x, pm.y, pm.z, pm.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (jb + q < m0 && pq[q] >= 0) alive |= 1u << (4 * g + q);
-                    }
-                    alive_valid = true;
-                }
-                const bool owner = ((p >> 2) & (NT - 1)) == tid;
-                if (owner) alive &= ~(1u << ((p >> 2) / NT * 4 + (p & 3)));
-#pragma unroll
-                for (int g = 0; g < KMAX / 4; ++g) {
-                    const int jb = own_slot<NT>(4 * g);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) { c[4 * g + q] = 0.f; corr[4 * g + q] = 0.f; }
-                    if (jb >= m0) continue;
-                    if (jb + 3 <= p) {
-                        const float4 v = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
-                        c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int j = jb + q;
-                            if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
-                        }
-                    }
-                }
-                const double idpp = 1.0 / dpp;
-                const double f = e * idpp;
-                const float rs = __frsqrt_rn((float)dpp);
-                const int nbs = GP ? min(nb, scap) : nb;
-                for (int b = 0; b < nbs; ++b) {
-                    const float* zo = panel + (size_t)b * ldz;
-                    const float zp = zo[p];
-#pragma unroll
-                    for (int g = 0; g < KMAX / 4; ++g) {
-                        if ((alive >> (4 * g)) & 0xFu) {
-                            const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
-                            corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
-                            corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
-                            corr[4 * g + 2] = fmaf(z.z, zp, corr[4 * g + 2]);
-                            corr[4 * g + 3] = fmaf(z.w, zp, corr[4 * g + 3]);
-                        }
-                    }
-                }
-                if (GP)
-#pragma unroll 4
-                for (int b = nbs; b < nb; ++b) {               // the overflow vectors, from L2
-                    const float* zo = GVEC + (size_t)(b - scap) * gld;
-                    const float zp = zo[p];
-#pragma unroll
-                    for (int g = 0; g < KMAX / 4; ++g) {
-                        if ((alive >> (4 * g)) & 0xFu) {
-                            const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
-                            corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
-                            corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
-                            corr[4 * g + 2] = fmaf(z.z, zp, corr[4 * g + 2]);
-                            corr[4 * g + 3] = fmaf(z.w, zp, corr[4 * g + 3]);
-                        }
-                    }
-                }
-                // state update of the own slots (Eq. 3 / Eq. 7), the new pending vector, and the score
-                // estimates the next free step starts from
-                const bool est_next = !BC && (s + 1 >= n_forced) && !outliers;
-                const bool q_next = Q && quant && (s + 1 >= n_forced);
+            // ======================= deferred-update step ==============================================
+            float* zb = (!GP || nb < scap) ? panel + (size_t)nb * ldz : GVEC + (size_t)(nb - scap) * gld;
+            // pivot column of the stored matrix (own slots), corrected by the pending vectors
+            const float* const tri = HP;
+            float c[KMAX], corr[KMAX];
+            if (!alive_valid) {
+                alive = 0u;
 #pragma unroll
                 for (int g = 0; g < KMAX / 4; ++g) {
                     const int jb = own_slot<NT>(4 * g);
                     if (jb >= m0) continue;
-                    int pq[4] = {0, 0, 0, 0};
-                    if (has_nm || has_wfull) {
-                        const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
-                        pq[0] = pm.x; pq[1] = pm.y; pq[2] = pm.z; pq[3] = pm.w;
-                    }
-                    float zv[4];
-                    // the group's FP64 state as 128-bit accesses: a warp's 64-bit accesses at this stride (32 bytes
-                    // between lanes) would meet four to a bank; dead slots keep the value they had
-                    double2* wq = reinterpret_cast<double2*>(wd + jb);
-                    double2* dq = reinterpret_cast<double2*>(dg + jb);
-                    const double2 w01 = wq[0], w23 = wq[1], d01 = dq[0], d23 = dq[1];
-                    double wv[4] = {w01.x, w01.y, w23.x, w23.y}, dv[4] = {d01.x, d01.y, d23.x, d23.y};
+                    const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
+                    const int pq[4] = {pm.x, pm.y, pm.z, pm.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (jb + q < m0 && pq[q] >= 0) alive |= 1u << (4 * g + q);
+                }
+                alive_valid = true;
+            }
+            const bool owner = ((p >> 2) & (NT - 1)) == tid;
+            if (owner) alive &= ~(1u << ((p >> 2) / NT * 4 + (p & 3)));
+#pragma unroll
+            for (int g = 0; g < KMAX / 4; ++g) {
+                const int jb = own_slot<NT>(4 * g);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { c[4 * g + q] = 0.f; corr[4 * g + q] = 0.f; }
+                if (jb >= m0) continue;
+                if (jb + 3 <= p) {
+                    const float4 v = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
+                    c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
+                } else {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const int k = 4 * g + q;
-                        zv[q] = 0.f;
-                        sa[k] = CUDART_NAN_F;
-                        if (!((alive >> k) & 1u)) continue;
-                        const float vj = c[k] - corr[k];
-                        const double nw = wv[q] - f * (double)vj;
-                        const double nd = dv[q] - (double)vj * (double)vj * idpp;
-                        wv[q] = nw; dv[q] = nd;
-                        zv[q] = vj * rs;
-                        if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gisc, gze, gmq, gr);
-                        if (has_nm) {
-                            if ((pq[q] >> nm_lg) == (op >> nm_lg)) cntw[g] += 1u << (8 * q);
-                            if ((int)((cntw[g] >> (8 * q)) & 0xFFu) >= nm_prune) sa[k] = CUDART_NAN_F;
+                        const int j = jb + q;
+                        if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                    }
+                }
+            }
+            const double idpp = 1.0 / dpp;
+            const double f = e * idpp;
+            const float rs = __frsqrt_rn((float)dpp);
+            const int nbs = GP ? min(nb, scap) : nb;
+            for (int b = 0; b < nbs; ++b) {
+                const float* zo = panel + (size_t)b * ldz;
+                const float zp = zo[p];
+#pragma unroll
+                for (int g = 0; g < KMAX / 4; ++g) {
+                    if ((alive >> (4 * g)) & 0xFu) {
+                        const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
+                        corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
+                        corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
+                        corr[4 * g + 2] = fmaf(z.z, zp, corr[4 * g + 2]);
+                        corr[4 * g + 3] = fmaf(z.w, zp, corr[4 * g + 3]);
+                    }
+                }
+            }
+            if (GP)
+#pragma unroll 4
+            for (int b = nbs; b < nb; ++b) {               // the overflow vectors, from L2
+                const float* zo = GVEC + (size_t)(b - scap) * gld;
+                const float zp = zo[p];
+#pragma unroll
+                for (int g = 0; g < KMAX / 4; ++g) {
+                    if ((alive >> (4 * g)) & 0xFu) {
+                        const float4 z = *reinterpret_cast<const float4*>(zo + own_slot<NT>(4 * g));
+                        corr[4 * g] = fmaf(z.x, zp, corr[4 * g]);
+                        corr[4 * g + 1] = fmaf(z.y, zp, corr[4 * g + 1]);
+                        corr[4 * g + 2] = fmaf(z.z, zp, corr[4 * g + 2]);
+                        corr[4 * g + 3] = fmaf(z.w, zp, corr[4 * g + 3]);
+                    }
+                }
+            }
+            // state update of the own slots (Eq. 3 / Eq. 7), the new pending vector, and the score
+            // estimates the next free step starts from
+            const bool est_next = !BC && (s + 1 >= n_forced) && !outliers;
+            const bool q_next = Q && quant && (s + 1 >= n_forced);
+#pragma unroll
+            for (int g = 0; g < KMAX / 4; ++g) {
+                const int jb = own_slot<NT>(4 * g);
+                if (jb >= m0) continue;
+                int pq[4] = {0, 0, 0, 0};
+                if (has_nm || has_wfull) {
+                    const int4 pm = *reinterpret_cast<const int4*>(perm + jb);
+                    pq[0] = pm.x; pq[1] = pm.y; pq[2] = pm.z; pq[3] = pm.w;
+                }
+                float zv[4];
+                // the group's FP64 state as 128-bit accesses: a warp's 64-bit accesses at this stride (32 bytes
+                // between lanes) would meet four to a bank; dead slots keep the value they had
+                double2* wq = reinterpret_cast<double2*>(wd + jb);
+                double2* dq = reinterpret_cast<double2*>(dg + jb);
+                const double2 w01 = wq[0], w23 = wq[1], d01 = dq[0], d23 = dq[1];
+                double wv[4] = {w01.x, w01.y, w23.x, w23.y}, dv[4] = {d01.x, d01.y, d23.x, d23.y};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int k = 4 * g + q;
+                    zv[q] = 0.f;
+                    sa[k] = CUDART_NAN_F;
+                    if (!((alive >> k) & 1u)) continue;
+                    const float vj = c[k] - corr[k];
+                    const double nw = wv[q] - f * (double)vj;
+                    const double nd = dv[q] - (double)vj * (double)vj * idpp;
+                    wv[q] = nw; dv[q] = nd;
+                    zv[q] = vj * rs;
+                    if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gisc, gze, gmq, gr);
+                    if (has_nm) {
+                        if ((pq[q] >> nm_lg) == (op >> nm_lg)) cntw[g] += 1u << (8 * q);
+                        if ((int)((cntw[g] >> (8 * q)) & 0xFFu) >= nm_prune) sa[k] = CUDART_NAN_F;
+                    }
+                    if (has_wfull) wfull[pq[q]] = (float)nw;
+                }
+                wq[0] = make_double2(wv[0], wv[1]); wq[1] = make_double2(wv[2], wv[3]);
+                dq[0] = make_double2(dv[0], dv[1]); dq[1] = make_double2(dv[2], dv[3]);
+                *reinterpret_cast<float4*>(zb + jb) = make_float4(zv[0], zv[1], zv[2], zv[3]);
+                if (BC == 4 && ((alive >> (4 * g)) & 0xFu) == 0xFu) {
+                    // Lemma 1 on the group's own 4 x 4 diagonal block (off-diagonal part; dg holds the diagonal)
+                    double* o = boff + (jb >> 2) * 6;
+                    const double v0 = (double)(c[4 * g] - corr[4 * g]), v1 = (double)(c[4 * g + 1] - corr[4 * g + 1]);
+                    const double v2 = (double)(c[4 * g + 2] - corr[4 * g + 2]), v3 = (double)(c[4 * g + 3] - corr[4 * g + 3]);
+                    o[0] -= v0 * v1 * idpp; o[1] -= v0 * v2 * idpp; o[2] -= v0 * v3 * idpp;
+                    o[3] -= v1 * v2 * idpp; o[4] -= v1 * v3 * idpp; o[5] -= v2 * v3 * idpp;
+                }
+            }
+            if (BC == 8) {
+                // Lemma 1 on the 8 x 8 diagonal block of every other whole block: its two halves belong to
+                // neighbouring lanes, which exchange their four column entries; the lane of the first half takes
+                // the pairs whose smaller index is 0 or 1, the other lane the rest
+#pragma unroll
+                for (int g = 0; g < KMAX / 4; ++g) {
+                    const int jb = own_slot<NT>(4 * g);
+                    float mine[4], other[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) mine[q] = c[4 * g + q] - corr[4 * g + q];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) other[q] = __shfl_xor_sync(0xffffffffu, mine[q], 1);
+                    if (jb < m0 && ((alive >> (4 * g)) & 0xFu) == 0xFu && (jb & ~7) != (p & ~7)) {
+                        const bool first = (jb & 7) == 0;
+                        double v[8];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            v[q] = (double)(first ? mine[q] : other[q]);
+                            v[4 + q] = (double)(first ? other[q] : mine[q]);
                         }
-                        if (has_wfull) wfull[pq[q]] = (float)nw;
-                    }
-                    wq[0] = make_double2(wv[0], wv[1]); wq[1] = make_double2(wv[2], wv[3]);
-                    dq[0] = make_double2(dv[0], dv[1]); dq[1] = make_double2(dv[2], dv[3]);
-                    *reinterpret_cast<float4*>(zb + jb) = make_float4(zv[0], zv[1], zv[2], zv[3]);
-                    if (BC == 4 && ((alive >> (4 * g)) & 0xFu) == 0xFu) {
-                        // Lemma 1 on the group's own 4 x 4 diagonal block (off-diagonal part; dg holds the diagonal)
-                        double* o = boff + (jb >> 2) * 6;
-                        const double v0 = (double)(c[4 * g] - corr[4 * g]), v1 = (double)(c[4 * g + 1] - corr[4 * g + 1]);
-                        const double v2 = (double)(c[4 * g + 2] - corr[4 * g + 2]), v3 = (double)(c[4 * g + 3] - corr[4 * g + 3]);
-                        o[0] -= v0 * v1 * idpp; o[1] -= v0 * v2 * idpp; o[2] -= v0 * v3 * idpp;
-                        o[3] -= v1 * v2 * idpp; o[4] -= v1 * v3 * idpp; o[5] -= v2 * v3 * idpp;
+                        double* o = boff + (jb >> 3) * 28;
+#pragma unroll
+                        for (int i = 0; i < 7; ++i)
+#pragma unroll
+                            for (int j = i + 1; j < 8; ++j)
+                                if ((i < 2) == first) o[block8_index(i, j)] -= v[i] * v[j] * idpp;
                     }
                 }
-                if (BC == 8) {
-                    // Lemma 1 on the 8 x 8 diagonal block of every other whole block: its two halves belong to
-                    // neighbouring lanes, which exchange their four column entries; the lane of the first half takes
-                    // the pairs whose smaller index is 0 or 1, the other lane the rest
-#pragma unroll
-                    for (int g = 0; g < KMAX / 4; ++g) {
-                        const int jb = own_slot<NT>(4 * g);
-                        float mine[4], other[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) mine[q] = c[4 * g + q] - corr[4 * g + q];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) other[q] = __shfl_xor_sync(0xffffffffu, mine[q], 1);
-                        if (jb < m0 && ((alive >> (4 * g)) & 0xFu) == 0xFu && (jb & ~7) != (p & ~7)) {
-                            const bool first = (jb & 7) == 0;
-                            double v[8];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                v[q] = (double)(first ? mine[q] : other[q]);
-                                v[4 + q] = (double)(first ? other[q] : mine[q]);
-                            }
-                            double* o = boff + (jb >> 3) * 28;
-#pragma unroll
-                            for (int i = 0; i < 7; ++i)
-#pragma unroll
-                                for (int j = i + 1; j < 8; ++j)
-                                    if ((i < 2) == first) o[block8_index(i, j)] -= v[i] * v[j] * idpp;
+            }
+            sa_valid = est_next;
+            if (owner) {
+                perm[p] = -1;
+                if (has_nm) blkcnt[op >> nm_lg] += 1;              // read again only behind a barrier
+            }
+            if (tid == NT - 32) {                          // (of the warp with the fewest slots)
+                pv[nb] = p;
+                if (has_wfull) wfull[op] = (float)qp;
+                if (a.W_out) a.W_out[(size_t)r * a.ldwo + op] = (float)qp;
+                if (a.mask) a.mask[(size_t)r * d + op] = 0;
+                if (!forced) {
+                    const int t = s - n_forced;
+                    if (a.order) a.order[(size_t)r * d + t] = op;
+                    if (a.loss) a.loss[(size_t)r * d + t] = BC ? ((t % BCD) ? 0.f : (float)blk_score) : (float)(e * f);
+                }
+                if (q_now && a.codes) a.codes[(size_t)r * d + op] = (int)code;
+            }
+            ++nb;
+            if (a.w_trace && s < a.trace_steps) {
+                __syncthreads();
+                for (int j = tid; j < d; j += NT)
+                    a.w_trace[((size_t)r * (a.trace_steps + 1) + s + 1) * d + j] = wfull[j];
+                // wfull is next written in the update phase of the following step, i.e. behind that step's
+                // barrier, which every thread reaches only after these reads
+            }
+        }
+        // ======================= the end of a row on chip ==========================================================
+        // At most ms <= NT slots: one per thread, its weight, diagonal and score estimate in registers (the state arrays are kept
+        // current for the pivot's readers).  A step is the pick's barrier, one entry of the pivot's column, its corrections by the
+        // deferred updates (all TAIL_B of them, zero where there are none yet) and the state; every TAIL_B steps the triangle is
+        // updated, and compacted when 32 slots or a quarter of them are gone.  What bounds it is the latency of that chain: about
+        // 1500 cycles a step, where KMAX slots per thread, four barriers and a pass over the triangle in every step took 8000.
+        if (s < total && m0 <= ms && !failed && !timed_out) {
+            __syncthreads();                                   // (pending vectors' space changes hands)
+            for (int i = warp; i < m0; i += NW)
+                for (int j = lane; j <= i; j += 32)
+                    S[tail_at(i, j)] = d > ms ? ld_tri<TC>(HP + tri_at(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
+            const int j = tid;
+            double w = 0.0, g = 0.0;
+            int o = -1, cnt = 0;
+            float est = CUDART_NAN_F;
+            auto take_slot = [&](int from) {                   // this thread's slot holds what slot `from` held
+                w = wd[from]; g = dg[from]; o = perm[from];
+                if (has_nm && o >= 0) cnt = blkcnt[o >> nm_lg];
+            };
+            auto clear_updates = [&]() {
+                if (j < ms) {
+                    float4* z = reinterpret_cast<float4*>(vt + j * TAIL_LD);
+                    float4* u = reinterpret_cast<float4*>(ut + j * TAIL_LD);
+                    z[0] = z[1] = u[0] = u[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            };
+            if (j < m0) take_slot(j);
+            clear_updates();
+            bool est_valid = false;
+            int left = m0;                                     // live slots among the m0
+            nb = 0;
+            __syncthreads();
+            for (; s < total; ++s) {
+                const bool forced = s < n_forced;
+                const bool q_now = Q && quant && !forced;
+                if (Q && a.mode == MODE_REPLAY_QUANT && s == n_forced) {
+                    survivors_grid(o >= 0 ? fminf(0.f, (float)w) : 0.f, o >= 0 ? fmaxf(0.f, (float)w) : 0.f);
+                    est_valid = false;
+                }
+                const Records rec = rec_view(scratch, s & 1);
+                Pick pk;
+                if (forced) {
+                    const int f = a.forced_order[(size_t)r * d + s];
+                    pk = known_pick<NT>(o == f ? j : -1, f, rec);
+                } else {
+                    if (!est_valid) {
+                        est = CUDART_NAN_F;
+                        if (o >= 0 && !(has_nm && cnt >= nm_prune)) est = score_estimate<Q>(w, g, q_now, gisc, gze, gmq, gr);
+                    }
+                    bool sure = false;
+                    if (!(Q && outliers)) pk = fast_pick<NT>(est, CUDART_INF_F, est == est ? j : -1, o, rec, &sure);
+                    if (!sure) {                               // FP64 scores of all slots; the outlier rule as in thread_best
+                        unsigned key = KEY_NONE;
+                        double cs = CUDART_INF;
+                        if (est == est) {
+                            const double err = q_now ? grid_error(w, gsc, gisc, gze, gmq) : -w;
+                            cs = err * err / g;
+                            if (Q && outliers && fabs(err) > 0.5 * gsc) cs = -fabs(err);
+                            if (cs == cs) key = float_key(__double2float_rn(cs));
                         }
+                        pk = block_pick<NT>(key, cs, key != KEY_NONE ? j : -1, o, rec);
                     }
                 }
-                sa_valid = est_next;
-                if (owner) {
-                    perm[p] = -1;
-                    if (has_nm) blkcnt[op >> nm_lg] += 1;              // read again only behind a barrier
+                const int p = pk.slot, op = pk.orig;
+                const double dpp = p < 0 ? 0.0 : dg[p], wp = p < 0 ? 0.0 : wd[p];      // (a pivot's state is not written again)
+                if (p < 0 || !(dpp > 0.0) || !isfinite(dpp) || !isfinite(wp)) { failed = true; break; }
+                double qp = 0.0, code = -1.0;
+                if (Q && q_now) qp = grid_q_fast(wp, gsc, gisc, gze, gmq, &code);
+                const double e = wp - qp, idpp = 1.0 / dpp, f = e * idpp;
+                if (j == p) {
+                    if (has_nm) blkcnt[op >> nm_lg] += 1;      // read again only behind a barrier
+                    perm[p] = -1; o = -1;
+                    est = CUDART_NAN_F;
                 }
-                if (tid == NT - 32) {                          // (of the warp with the fewest slots)
-                    pv[nb] = p;
+                const bool est_next = s + 1 >= n_forced && !outliers;
+                if (o >= 0) {
+                    float* vj = vt + j * TAIL_LD;
+                    float* uj = ut + j * TAIL_LD;
+                    const float4* up = reinterpret_cast<const float4*>(ut + p * TAIL_LD);
+                    const float4 a0 = *reinterpret_cast<const float4*>(vj), a1 = *reinterpret_cast<const float4*>(vj + 4), b0 = up[0], b1 = up[1];
+                    float x = a0.x * b0.x;
+                    x = fmaf(a0.y, b0.y, x); x = fmaf(a0.z, b0.z, x); x = fmaf(a0.w, b0.w, x);
+                    x = fmaf(a1.x, b1.x, x); x = fmaf(a1.y, b1.y, x); x = fmaf(a1.z, b1.z, x); x = fmaf(a1.w, b1.w, x);
+                    const float v = S[j > p ? tail_at(j, p) : tail_at(p, j)] - x;
+                    const double vd = (double)v, ud = vd * idpp;
+                    w -= f * vd;
+                    g -= vd * ud;
+                    vj[nb] = v; uj[nb] = (float)ud;
+                    wd[j] = w; dg[j] = g;
+                    if (has_wfull) wfull[o] = (float)w;
+                    if (has_nm && (o >> nm_lg) == (op >> nm_lg)) ++cnt;
+                    if (est_next) {
+                        est = score_estimate<Q>(w, g, Q && quant, gisc, gze, gmq, gr);
+                        if (has_nm && cnt >= nm_prune) est = CUDART_NAN_F;
+                    }
+                }
+                est_valid = est_next;
+                if (tid == NT - 32) {
                     if (has_wfull) wfull[op] = (float)qp;
                     if (a.W_out) a.W_out[(size_t)r * a.ldwo + op] = (float)qp;
                     if (a.mask) a.mask[(size_t)r * d + op] = 0;
                     if (!forced) {
                         const int t = s - n_forced;
                         if (a.order) a.order[(size_t)r * d + t] = op;
-                        if (a.loss) a.loss[(size_t)r * d + t] = BC ? ((t % BCD) ? 0.f : (float)blk_score) : (float)(e * f);
+                        if (a.loss) a.loss[(size_t)r * d + t] = (float)(e * f);
                     }
                     if (q_now && a.codes) a.codes[(size_t)r * d + op] = (int)code;
                 }
-                ++nb;
+                --left;
                 if (a.w_trace && s < a.trace_steps) {
                     __syncthreads();
-                    for (int j = tid; j < d; j += NT)
-                        a.w_trace[((size_t)r * (a.trace_steps + 1) + s + 1) * d + j] = wfull[j];
-                    // wfull is next written in the update phase of the following step, i.e. behind that step's
-                    // barrier, which every thread reaches only after these reads
+                    for (int i = tid; i < d; i += NT)
+                        a.w_trace[((size_t)r * (a.trace_steps + 1) + s + 1) * d + i] = wfull[i];
                 }
-            } else {
-                // ======================= on-chip step (compaction at every step) ===========================
-                const int m = m0, last = m0 - 1;
-                for (int j = tid; j < m; j += NT) {
-                    tv[j] = (j <= p) ? S[p * lds + j] : S[j * lds + p];
-                    tlr[j] = S[last * lds + j];
-                }
-                __syncthreads();
-                {
-                    const double f = e / dpp;
-                    for (int j = tid; j < m; j += NT) {
-                        if (j == p) continue;
-                        const float vj = tv[j];
-                        const double nw = wd[j] - f * (double)vj;
-                        const double nd = dg[j] - (double)vj * (double)vj / dpp;
-                        const float uj = (float)((double)vj / dpp);
-                        const int oj = perm[j];
-                        if (has_wfull) wfull[oj] = (float)nw;
-                        const int dst = (j == last) ? p : j;       // p != last here
-                        wd[dst] = nw; dg[dst] = nd; tu[dst] = uj;
-                        if (j == last) { perm[p] = oj; tv[p] = vj; tlr[p] = tlr[last]; }
-                    }
-                    if (tid == 0) {
-                        if (has_nm) blkcnt[op >> nm_lg] += 1;
-                        if (a.mask) a.mask[(size_t)r * d + op] = 0;
-                        if (has_wfull) wfull[op] = (float)qp;
-                        if (a.W_out) a.W_out[(size_t)r * a.ldwo + op] = (float)qp;
-                        if (!forced) {
-                            const int t = s - n_forced;
-                            if (a.order) a.order[(size_t)r * d + t] = op;
-                            if (a.loss) a.loss[(size_t)r * d + t] = (float)(e * e / dpp);
+                if (++nb == TAIL_B && s + 1 < total) {
+                    __syncthreads();
+                    tail_flush<NT>(S, m0, vt, ut, perm);
+                    const bool compact = m0 - left >= min(32, m0 >> 2);      // (at most 39 slots are gone: hl and mv hold 64)
+                    if (compact && warp == NW - 1) {           // holes and, as many, live slots above the new size
+                        int nh = 0, nm = 0;
+                        for (int i0 = 0; i0 < m0; i0 += 32) {
+                            const int i = i0 + lane;
+                            const bool lv = i < m0 && perm[i] >= 0;
+                            const unsigned hm = __ballot_sync(0xffffffffu, i < left && !lv), lm = __ballot_sync(0xffffffffu, i >= left && lv);
+                            const unsigned below = (1u << lane) - 1u;
+                            if (i < left && !lv) hl[nh + __popc(hm & below)] = i;
+                            if (i >= left && lv) mv[nm + __popc(lm & below)] = i;
+                            nh += __popc(hm); nm += __popc(lm);
                         }
-                        if (q_now && a.codes) a.codes[(size_t)r * d + op] = (int)code;
+                        if (lane == 0) bc->nh = nh;
+                        __syncwarp();
+                        for (int q = lane; q < nh; q += 32) srcm[hl[q]] = (unsigned short)mv[q];
                     }
+                    __syncthreads();
+                    clear_updates();
+                    nb = 0;
+                    if (compact) {
+                        const int nh = bc->nh;
+                        for (int q = warp; q < nh; q += NW) {  // read from rows >= left, which nothing here writes
+                            const int h = hl[q], from = mv[q];
+                            for (int i = lane; i < left; i += 32) {
+                                const int si = srcm[i];
+                                S[tail_at(max(h, i), min(h, i))] = S[tail_at(max(from, si), min(from, si))];
+                            }
+                        }
+                        const int from = j < left ? (int)srcm[j] : j;
+                        __syncthreads();
+                        if (j >= left) o = -1;
+                        else if (from != j) { take_slot(from); wd[j] = w; dg[j] = g; perm[j] = o; srcm[j] = (unsigned short)j; }
+                        m0 = left;
+                        est_valid = false;
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
-                if (a.w_trace && s < a.trace_steps)
-                    for (int j = tid; j < d; j += NT)
-                        a.w_trace[((size_t)r * (a.trace_steps + 1) + s + 1) * d + j] = wfull[j];
-                const int pm = (p == last) ? -1 : p;
-                if (s + 1 < total) blk_pass_shared<NT>(S, lds, m - 1, pm, tv, tu, tlr);
-                --m0;
-                __syncthreads();
             }
         }
         // ---- row epilogue ---------------------------------------------------------------------------------
