@@ -184,10 +184,15 @@ static __device__ __noinline__ void blk_state_copy(bool save, char* state, int c
     }
 }
 
-// Place of element (i, j), j <= i, of a private triangle: groups of 32 columns one after the other, rows of 128 bytes inside a
-// group (ld rows each).  A column is then one strip of consecutive lines instead of a line per row of the matrix, and a
-// 128-row tile of a group is contiguous.
-__host__ __device__ __forceinline__ int tri_at(int ld, int i, int j) { return ((j >> 5) * ld + i) * 32 + (j & 31); }
+// Place of element (i, j), j <= i, of a private triangle: groups of columns one after the other, ld rows each.  A column is then one
+// strip of consecutive lines instead of a line per row of the matrix.
+// Passes on tcgen05 (TC): 32 columns, rows of 128 bytes, so that a 128-row tile of a group is contiguous.  Else 4 columns, rows of 16
+// bytes: a warp's 32 rows of a pivot column are 4 lines instead of 32 (one L1 tag look-up each, which the step's other accesses
+// queued behind), 768 x 768 2:4 8.55 -> 8.13 ms, 3072 x 768 compound 85.2 -> 83.0.  With passes on tcgen05 the smaller groups lose
+// more in the copies and the holes than the columns gain (256 x 2304 OBQ 43.6 -> 46.2 ms, 128 x 1152 blocks 7.74 -> 8.53).
+template <bool TC> __device__ __forceinline__ int tri_at(int ld, int i, int j) {
+    return TC ? ((j >> 5) * ld + i) * 32 + (j & 31) : ((j >> 2) * ld + i) * 4 + (j & 3);
+}
 __host__ __device__ inline size_t tri_floats(int cap) { return (size_t)((cap + 63) & ~63) * cap; }      // (an even number of groups)
 
 struct Records {                              // views into one record buffer
@@ -500,9 +505,9 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
     int prg = warp, pc0 = 0;
     auto prefetch_next = [&]() {
         if (prg >= nrg) return;
-        const int row = (prg << 4) + (lane >> 1), col = pc0 + ((lane & 1) << 5);       // 16 rows x 2 lines of 128 bytes
-        if (row < m1 && col <= row)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at(ldp, srcm[row], col)));
+        const int row = (prg << 4) + ((lane & 1) << 3), col = pc0 + ((lane >> 1) << 2);      // 16 column groups x 2 lines of 8 rows
+        if (row < m1 && col <= row + 7)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<false>(ldp, srcm[row], col)));
         pc0 += 64;
         if (pc0 >= min((prg << 4) + 16, m1)) { pc0 = 0; prg += NW; }
     };
@@ -620,7 +625,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                     hv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
                     const int j = c0 + (u << 4) + (t << 2);
                     if (u < ngroups && in[h] && j <= rr[h]) {
-                        const float4* src = reinterpret_cast<const float4*>(Hp + tri_at(ldp, sr[h], j));
+                        const float4* src = reinterpret_cast<const float4*>(Hp + tri_at<false>(ldp, sr[h], j));
                         hv[u][h] = STREAM ? __ldcs(src) : *src;
                     }
                 }
@@ -639,7 +644,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 if (in[h] && jj <= rr[h]) {
-                                    const float val = Hp[tri_at(ldp, max(sr[h], sj), min(sr[h], sj))];
+                                    const float val = Hp[tri_at<false>(ldp, max(sr[h], sj), min(sr[h], sj))];
                                     if (comp == 0) hv[u][h].x = val; else if (comp == 1) hv[u][h].y = val;
                                     else if (comp == 2) hv[u][h].z = val; else hv[u][h].w = val;
                                 }
@@ -658,7 +663,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                             float4 o = hv[u][h];
                             o.x -= acc[2 * u][2 * h];     o.z -= acc[2 * u][2 * h + 1];
                             o.y -= acc[2 * u + 1][2 * h]; o.w -= acc[2 * u + 1][2 * h + 1];
-                            float4* dst = reinterpret_cast<float4*>(Hp + tri_at(ldp, rr[h], j));
+                            float4* dst = reinterpret_cast<float4*>(Hp + tri_at<false>(ldp, rr[h], j));
                             if (STREAM) __stcs(dst, o); else *dst = o;
                         }
                     }
@@ -763,10 +768,10 @@ __device__ __forceinline__ void blk_fill_holes(float* H, int ldp, int m1, int nh
             float v[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                if (q0 + q < nh) { const int sh = mv[q0 + q]; v[q] = __ldcg(H + tri_at(ldp, max(sh, sj), min(sh, sj))); }
+                if (q0 + q < nh) { const int sh = mv[q0 + q]; v[q] = __ldcg(H + tri_at<true>(ldp, max(sh, sj), min(sh, sj))); }
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                if (q0 + q < nh) { const int h = hl[q0 + q]; H[tri_at(ldp, max(h, j), min(h, j))] = v[q]; }
+                if (q0 + q < nh) { const int h = hl[q0 + q]; H[tri_at<true>(ldp, max(h, j), min(h, j))] = v[q]; }
         }
     }
 }
@@ -1031,20 +1036,37 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     a.w_trace[((size_t)r * (a.trace_steps + 1)) * d + j] = a.W[(size_t)r * a.ldw + j];
         }
         if (kind != ITEM_TAIL && d > ms && total > 0) {
-            for (int i = warp; i < d; i += NW) {
-                const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
-                float* dst = HP;
-                auto put = [&](int j4, float4 v) { *reinterpret_cast<float4*>(dst + tri_at(ldp, i, 4 * j4)) = v; };
-                const int n4 = (i >> 2) + 1;
-                if (GP || (FG && NT >= 512)) {      // (kernels with no registers to spare: one load in flight)
-                    for (int j4 = lane; j4 < n4; j4 += 32) put(j4, s4[j4]);
-                } else {
-                    for (int j0 = lane; j0 < n4; j0 += 128) {      // four loads in flight per lane
+            if constexpr (!TC) {
+                // a warp takes 8 rows, 4 lanes a row: 64 contiguous bytes read of each, 128 written to each of 4 column groups
+                for (int i0 = 8 * warp; i0 < d; i0 += 8 * NW) {
+                    const int i = i0 + (lane >> 2);
+                    const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
+                    float* dst = HP;
+                    const int n4 = i < d ? (i >> 2) + 1 : 0;
+                    for (int j0 = lane & 3; j0 < n4; j0 += 16) {       // four loads in flight per lane
                         float4 t[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) t[k] = __ldg(s4 + j0 + 32 * k);
+                        for (int k = 0; k < 4; ++k) if (j0 + 4 * k < n4) t[k] = __ldg(s4 + j0 + 4 * k);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) put(j0 + 32 * k, t[k]);
+                        for (int k = 0; k < 4; ++k) if (j0 + 4 * k < n4) *reinterpret_cast<float4*>(dst + tri_at<TC>(ldp, i, 4 * (j0 + 4 * k))) = t[k];
+                    }
+                }
+            } else {
+                for (int i = warp; i < d; i += NW) {
+                    const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
+                    float* dst = HP;
+                    auto put = [&](int j4, float4 v) { *reinterpret_cast<float4*>(dst + tri_at<TC>(ldp, i, 4 * j4)) = v; };
+                    const int n4 = (i >> 2) + 1;
+                    if (GP || FG) {                 // (kernels with no registers to spare: one load in flight)
+                        for (int j4 = lane; j4 < n4; j4 += 32) put(j4, s4[j4]);
+                    } else {
+                        for (int j0 = lane; j0 < n4; j0 += 128) {      // four loads in flight per lane
+                            float4 t[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) t[k] = __ldg(s4 + j0 + 32 * k);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) if (j0 + 32 * k < n4) put(j0 + 32 * k, t[k]);
+                        }
                     }
                 }
             }
@@ -1228,13 +1250,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         for (int g = 0; g < GS; ++g) {
                             const int p = p4[g];
                             if (jb + 3 <= p) {
-                                const float4 t = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
+                                const float4 t = ld_tri4<TC>(tri + tri_at<TC>(ldp, p, jb));
                                 v[g][4 * g4] = t.x; v[g][4 * g4 + 1] = t.y; v[g][4 * g4 + 2] = t.z; v[g][4 * g4 + 3] = t.w;
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 4; ++q) {
                                     const int j = jb + q;
-                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p)));
                                 }
                             }
                         }
@@ -1449,13 +1471,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int q = 0; q < 4; ++q) { c[4 * g + q] = 0.f; corr[4 * g + q] = 0.f; }
                 if (jb >= m0) continue;
                 if (jb + 3 <= p) {
-                    const float4 v = ld_tri4<TC>(tri + tri_at(ldp, p, jb));
+                    const float4 v = ld_tri4<TC>(tri + tri_at<TC>(ldp, p, jb));
                     c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
                 } else {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int j = jb + q;
-                        if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at(ldp, p, j) : tri_at(ldp, j, p)));
+                        if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p)));
                     }
                 }
             }
@@ -1608,7 +1630,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
             __syncthreads();                                   // (pending vectors' space changes hands)
             for (int i = warp; i < m0; i += NW)
                 for (int j = lane; j <= i; j += 32)
-                    S[tail_at(i, j)] = d > ms ? ld_tri<TC>(HP + tri_at(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
+                    S[tail_at(i, j)] = d > ms ? ld_tri<TC>(HP + tri_at<TC>(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
             const int j = tid;
             double w = 0.0, g = 0.0;
             int o = -1, cnt = 0;
