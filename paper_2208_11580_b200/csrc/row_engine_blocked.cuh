@@ -67,9 +67,9 @@ __host__ __device__ inline size_t blk_state_bytes(int cap, bool wfull, bool nm =
     return (size_t)20 * cap + (((size_t)2 * cap + 15) & ~(size_t)15) + (wfull ? (size_t)4 * cap : 0) +
            (nm ? (((size_t)(cap >> 1) + 15) & ~(size_t)15) : 0) + (bc == 8 ? (size_t)28 * cap : (bc ? (size_t)12 * cap : 0));
 }
-// Stride of the pending vectors for a row of m slots: = 8 (mod 32), so that the tensor-core fragments of the
-// flush (4 vectors x 8 consecutive slots per load) touch 32 different banks.
-__host__ __device__ inline int blk_ldz(int m) { return ((m + 8 + 31) & ~31) + 8; }     // >= m + 16
+// Stride of the pending vectors for a row of m slots: = 4 (mod 32), so that the tensor-core fragments of the flush (every second
+// row of 4 pairs of vectors x 8 consecutive slots per load) touch 32 different banks.
+__host__ __device__ inline int blk_ldz(int m) { return ((m + 12 + 31) & ~31) + 4; }     // >= m + 16
 // On chip: TAIL_B deferred updates as two arrays per slot (column entries v, v / [H]_pp; TAIL_LD floats apart: 128-bit accesses
 // of consecutive slots meet no bank twice), then the lower triangle, its rows end to end: column p of 32 rows from a multiple of
 // 32 on touches 32 different banks (triangular numbers mod 32 are a permutation).
@@ -487,6 +487,66 @@ __device__ __forceinline__ void tf32_split2(float2 x, uint32_t& hi0, uint32_t& h
     lo0 = __float_as_uint(l.x); lo1 = __float_as_uint(l.y);
 }
 
+// A tile of H (16 rows x 64 columns from c0; in L2 by now: the cursor passed it two tiles ago) minus the increment acc * unscale.
+template <bool STREAM>
+__device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp, int c0, int ngroups, const int (&rr)[2], const bool (&in)[2],
+                                                const int (&sr)[2], int t, const float (&acc)[8][4], float unscale,
+                                                const unsigned short* srcm, const uint32_t* colmask) {
+    // ---- the tile of H (in L2 by now: the cursor passed it two tiles ago), minus the increment -----------
+    float4 hv[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            hv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int j = c0 + (u << 4) + (t << 2);
+            if (u < ngroups && in[h] && j <= rr[h]) {
+                const float4* src = reinterpret_cast<const float4*>(Hp + tri_at<false>(ldp, sr[h], j));
+                hv[u][h] = STREAM ? __ldcs(src) : *src;
+            }
+        }
+    // columns of this lane that are holes: their data sits in the mover's row
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        if (u < ngroups) {
+            const int j = c0 + (u << 4) + (t << 2);
+            const uint32_t my4 = (colmask[j >> 5] >> (j & 31)) & 0xFu;
+            if (my4) {
+#pragma unroll
+                for (int comp = 0; comp < 4; ++comp) {
+                    if (!((my4 >> comp) & 1u)) continue;
+                    const int jj = j + comp;
+                    const int sj = (int)srcm[jj];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (in[h] && jj <= rr[h]) {
+                            const float val = Hp[tri_at<false>(ldp, max(sr[h], sj), min(sr[h], sj))];
+                            if (comp == 0) hv[u][h].x = val; else if (comp == 1) hv[u][h].y = val;
+                            else if (comp == 2) hv[u][h].z = val; else hv[u][h].w = val;
+                        }
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        if (u < ngroups) {
+            const int j = c0 + (u << 4) + (t << 2);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (in[h] && j <= rr[h]) {
+                    float4 o = hv[u][h];
+                    o.x = fmaf(-unscale, acc[2 * u][2 * h], o.x);     o.z = fmaf(-unscale, acc[2 * u][2 * h + 1], o.z);
+                    o.y = fmaf(-unscale, acc[2 * u + 1][2 * h], o.y); o.w = fmaf(-unscale, acc[2 * u + 1][2 * h + 1], o.w);
+                    float4* dst = reinterpret_cast<float4*>(Hp + tri_at<false>(ldp, rr[h], j));
+                    if (STREAM) __stcs(dst, o); else *dst = o;
+                }
+            }
+        }
+    }
+}
+
 template <int NT, bool STREAM, bool GP>
 __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, int m1, int nb, int nbs, const float* Z, int ldz,
                                               const float* __restrict__ G, int gld, float* zstage,
@@ -616,59 +676,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                 if (kg + 1 < ksteps_g) load_g(kg + 1);
                 kstep(av, b0, b1);
             }
-            // ---- the tile of H (in L2 by now: the cursor passed it two tiles ago), minus the increment -----------
-            float4 hv[4][2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    hv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const int j = c0 + (u << 4) + (t << 2);
-                    if (u < ngroups && in[h] && j <= rr[h]) {
-                        const float4* src = reinterpret_cast<const float4*>(Hp + tri_at<false>(ldp, sr[h], j));
-                        hv[u][h] = STREAM ? __ldcs(src) : *src;
-                    }
-                }
-            // columns of this lane that are holes: their data sits in the mover's row
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (u < ngroups) {
-                    const int j = c0 + (u << 4) + (t << 2);
-                    const uint32_t my4 = (colmask[j >> 5] >> (j & 31)) & 0xFu;
-                    if (my4) {
-#pragma unroll
-                        for (int comp = 0; comp < 4; ++comp) {
-                            if (!((my4 >> comp) & 1u)) continue;
-                            const int jj = j + comp;
-                            const int sj = (int)srcm[jj];
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                if (in[h] && jj <= rr[h]) {
-                                    const float val = Hp[tri_at<false>(ldp, max(sr[h], sj), min(sr[h], sj))];
-                                    if (comp == 0) hv[u][h].x = val; else if (comp == 1) hv[u][h].y = val;
-                                    else if (comp == 2) hv[u][h].z = val; else hv[u][h].w = val;
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (u < ngroups) {
-                    const int j = c0 + (u << 4) + (t << 2);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if (in[h] && j <= rr[h]) {
-                            float4 o = hv[u][h];
-                            o.x -= acc[2 * u][2 * h];     o.z -= acc[2 * u][2 * h + 1];
-                            o.y -= acc[2 * u + 1][2 * h]; o.w -= acc[2 * u + 1][2 * h + 1];
-                            float4* dst = reinterpret_cast<float4*>(Hp + tri_at<false>(ldp, rr[h], j));
-                            if (STREAM) __stcs(dst, o); else *dst = o;
-                        }
-                    }
-                }
-            }
+            blk_flush_store<STREAM>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, 1.f, srcm, colmask);
         }
     }
 }
@@ -683,12 +691,10 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) 
 // the power of two that takes v (> 0, finite) to [2^13, 2^14), within what a float power of two and its square hold
 __device__ __forceinline__ int plane_power(float v) { return min(60, max(-50, 13 - ((int)(__float_as_uint(v) >> 23) - 127))); }
 
-// The pending vectors (b < scap in shared memory, the rest in G), already in the new slot numbering, as FP16 planes hi, lo
-// (64 rows each); rows nb .. of the last group of 16 become zero.  Returns the planes' power of two, or 99 where every slot has
-// its own (zexp).  Every thread of the block calls it; the caller synchronises before the planes are read.
+// The power of two that takes the pending vectors' largest entry to [2^13, 2^14), and whether the diagonal spans more than 2^24.
 template <int NT, int KMAX>
-__device__ __forceinline__ int blk_make_planes(const float* panel, int ldz, int scap, const float* G, int gld, int nb, int m0, int m1,
-                                               const double* dg, const int* perm, float* rf, __half* planes, int zld, signed char* zexp) {
+__device__ __forceinline__ int blk_plane_range(const float* panel, int ldz, int scap, const float* G, int gld, int nb, int m0, int m1,
+                                               const double* dg, const int* perm, float* rf, bool* wide) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto vec = [&](int b) { return b < scap ? panel + (size_t)b * ldz : G + (size_t)(b - scap) * gld; };
@@ -719,8 +725,19 @@ __device__ __forceinline__ int blk_make_planes(const float* panel, int ldz, int 
     for (int w = 0; w < NW; ++w) { zmax = fmaxf(zmax, rf[w]); dmax = fmaxf(dmax, rf[NW + w]); dmin = fminf(dmin, rf[2 * NW + w]); }
     // the planes hold vectors of the diagonal before the pending eliminations: zmax^2 is what it had been (at least) where it has
     // collapsed since
-    const bool wide = dmin < fmaxf(dmax, zmax * zmax) * 5.9604645e-8f;             // 2^-24
-    const int power = plane_power(zmax);
+    *wide = dmin < fmaxf(dmax, zmax * zmax) * 5.9604645e-8f;             // 2^-24
+    return plane_power(zmax);
+}
+
+// The pending vectors (b < scap in shared memory, the rest in G), already in the new slot numbering, as FP16 planes hi, lo
+// (64 rows each); rows nb .. of the last group of 16 become zero.  Returns the planes' power of two, or 99 where every slot has
+// its own (zexp).  Every thread of the block calls it; the caller synchronises before the planes are read.
+template <int NT, int KMAX>
+__device__ __forceinline__ int blk_make_planes(const float* panel, int ldz, int scap, const float* G, int gld, int nb, int m0, int m1,
+                                               const double* dg, const int* perm, float* rf, __half* planes, int zld, signed char* zexp) {
+    auto vec = [&](int b) { return b < scap ? panel + (size_t)b * ldz : G + (size_t)(b - scap) * gld; };
+    bool wide;
+    const int power = blk_plane_range<NT, KMAX>(panel, ldz, scap, G, gld, nb, m0, m1, dg, perm, rf, &wide);
     const int nb16 = (nb + 15) & ~15;
 #pragma unroll
     for (int g = 0; g < KMAX / 4; ++g) {
@@ -756,6 +773,126 @@ __device__ __forceinline__ int blk_make_planes(const float* panel, int ldz, int 
         }
     }
     return wide ? 99 : power;
+}
+
+// The same planes in the vectors' own place in shared memory, for the flush by mma.sync: rows 2b and 2b + 1 become the hi and the lo
+// halves of vectors 2b and 2b + 1, two FP16 to a word (a fragment register of m16n8k16).  Row nb is there when nb is odd.
+template <int NT, int KMAX>
+__device__ __forceinline__ void blk_pack_planes(float* panel, int ldz, int nb, int m1, float scale) {
+#pragma unroll
+    for (int g = 0; g < KMAX / 4; ++g) {
+        const int jb = own_slot<NT>(4 * g);
+        if (jb >= m1) continue;
+#pragma unroll 4
+        for (int b = 0; b < nb; b += 2) {
+            float* z = panel + (size_t)b * ldz + jb;
+            const float4 u = *reinterpret_cast<const float4*>(z);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (b + 1 < nb) v = *reinterpret_cast<const float4*>(z + ldz);
+            const float x0[4] = {u.x * scale, u.y * scale, u.z * scale, u.w * scale}, x1[4] = {v.x * scale, v.y * scale, v.z * scale, v.w * scale};
+            unsigned hi[4], lo[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const __half2 h = __floats2half2_rn(x0[q], x1[q]);
+                const float2 f = __half22float2(h);
+                const __half2 l = __floats2half2_rn(x0[q] - f.x, x1[q] - f.y);
+                hi[q] = *reinterpret_cast<const unsigned*>(&h); lo[q] = *reinterpret_cast<const unsigned*>(&l);
+            }
+            *reinterpret_cast<uint4*>(z) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(z + ldz) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+    }
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16_z(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// The flush by mma.sync on packed planes (blk_pack_planes): tiles, register layout, compaction and the treatment of the partial sums as
+// in blk_flush_mma, with m16n8k16 on FP16 planes instead of m16n8k8 on TF32 parts: half the products per vector, and the operands
+// are split once per flush instead of in every tile.  Partial sums are over 16 vectors, scaled by `unscale` = 2^-2e of the planes.
+template <int NT>
+__device__ __forceinline__ void blk_flush_f16(float* __restrict__ Hp, int ldp, int m1, int nb, const float* Z, int ldz, float unscale,
+                                              const unsigned short* srcm, const uint32_t* colmask) {
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const int nrg = (m1 + 15) >> 4;
+    const int pairs = (nb + 1) >> 1, ksteps = (pairs + 7) >> 3;
+    const uint32_t* W = reinterpret_cast<const uint32_t*>(Z);
+    constexpr int FLUSH_AHEAD = 2;                             // as in blk_flush_mma
+    int prg = warp, pc0 = 0;
+    auto prefetch_next = [&]() {
+        if (prg >= nrg) return;
+        const int row = (prg << 4) + ((lane & 1) << 3), col = pc0 + ((lane >> 1) << 2);      // 16 column groups x 2 lines of 8 rows
+        if (row < m1 && col <= row + 7)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<false>(ldp, srcm[row], col)));
+        pc0 += 64;
+        if (pc0 >= min((prg << 4) + 16, m1)) { pc0 = 0; prg += NW; }
+    };
+#pragma unroll
+    for (int a = 0; a < FLUSH_AHEAD; ++a) prefetch_next();
+    for (int rg = warp; rg < nrg; rg += NW) {
+        const int i0 = rg << 4;
+        const int jend = min(i0 + 16, m1);                     // columns [0, jend) hold data of this row group
+        const int rr[2] = {i0 + g, i0 + g + 8};                // the lane's two rows
+        const bool in[2] = {rr[0] < m1, rr[1] < m1};
+        const int sr[2] = {in[0] ? (int)srcm[rr[0]] : 0, in[1] ? (int)srcm[rr[1]] : 0};
+        for (int c0 = 0; c0 < jend; c0 += 64) {
+            const int ngroups = min(4, (jend - c0 + 15) >> 4);
+            prefetch_next();
+            float acc[8][4];
+#pragma unroll
+            for (int n = 0; n < 8; ++n) { acc[n][0] = 0.f; acc[n][1] = 0.f; acc[n][2] = 0.f; acc[n][3] = 0.f; }
+            for (int ks = 0; ks < ksteps; ++ks) {
+                // this lane: pairs 8 ks + t and + 4; past the last pair zeros
+                const int p0 = (ks << 3) + t, p1 = p0 + 4;
+                const bool v0 = p0 < pairs, v1 = p1 < pairs;
+                const uint32_t* z0 = W + (size_t)(2 * p0) * ldz;
+                const uint32_t* z1 = W + (size_t)(2 * p1) * ldz;
+                uint32_t ah[4], al[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    ah[h] = v0 && in[h] ? z0[rr[h]] : 0u;     al[h] = v0 && in[h] ? z0[ldz + rr[h]] : 0u;
+                    ah[2 + h] = v1 && in[h] ? z1[rr[h]] : 0u; al[2 + h] = v1 && in[h] ? z1[ldz + rr[h]] : 0u;
+                }
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {         // two column groups at a time
+                    if (2 * half >= ngroups) break;
+                    uint2 bh0[2], bl0[2], bh1[2], bl1[2];
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const int u = 2 * half + x, c = c0 + (u << 4) + (g << 1);      // < m1 + 16 <= ldz
+                        bh0[x] = bl0[x] = bh1[x] = bl1[x] = make_uint2(0u, 0u);
+                        if (u < ngroups && v0) { bh0[x] = *reinterpret_cast<const uint2*>(z0 + c); bl0[x] = *reinterpret_cast<const uint2*>(z0 + ldz + c); }
+                        if (u < ngroups && v1) { bh1[x] = *reinterpret_cast<const uint2*>(z1 + c); bl1[x] = *reinterpret_cast<const uint2*>(z1 + ldz + c); }
+                    }
+                    float dk[4][4];
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) { mma_f16_z(dk[2 * x], al, bh0[x].x, bh1[x].x); mma_f16_z(dk[2 * x + 1], al, bh0[x].y, bh1[x].y); }
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) { mma_f16(dk[2 * x], ah, bl0[x].x, bl1[x].x); mma_f16(dk[2 * x + 1], ah, bl0[x].y, bl1[x].y); }
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) { mma_f16(dk[2 * x], ah, bh0[x].x, bh1[x].x); mma_f16(dk[2 * x + 1], ah, bh0[x].y, bh1[x].y); }
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int e = 0; e < 4; e += 2) {
+                            const float2 r = __fadd2_rn(make_float2(acc[4 * half + n][e], acc[4 * half + n][e + 1]),
+                                                        make_float2(__uint_as_float(__float_as_uint(dk[n][e]) | 1u),
+                                                                    __uint_as_float(__float_as_uint(dk[n][e + 1]) | 1u)));
+                            acc[4 * half + n][e] = r.x; acc[4 * half + n][e + 1] = r.y;
+                        }
+                }
+            }
+            blk_flush_store<true>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, unscale, srcm, colmask);
+        }
+    }
 }
 
 // The triangle's part of the compaction: the movers' rows and columns into the holes.  They come from rows >= m1, which
@@ -1079,7 +1216,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         int nb = 0;                      // pending vectors
         int ldz = blk_ldz(m0);
         int scap = a.panel_floats / ldz;     // pending vectors that fit into shared memory at this row length
-        int bcur = min(a.max_pending, scap + gB);
+        int bcur = min(a.max_pending, GP || TC ? scap + gB : max(2, scap & ~1));      // (packed planes: vectors in pairs)
         if (BC) bcur &= ~(BC - 1);           // whole blocks between two flushes, so that 4-slot groups stay together
         int s = s_begin;
         bool failed = false, timed_out = false;
@@ -1165,8 +1302,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     for (int j = tid; j < cap; j += NT) reinterpret_cast<double2*>(wd)[j] = __ldcg(park + j);
                     __syncthreads();
                     if (!fine) { timed_out = true; break; }
-                } else if (!GP)
-                    blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);      // evict-first at every row length (~1 %)
+                } else if (!GP) {                              // (evict-first at every row length: ~1 %)
+                    bool wide;
+                    const int power = blk_plane_range<NT, KMAX>(panel, ldz, nb, nullptr, 0, nb, m0, m1, dg, perm, rf, &wide);
+                    if (!wide) {
+                        blk_pack_planes<NT, KMAX>(panel, ldz, nb, m1, pow2f(power));
+                        __syncthreads();
+                        blk_flush_f16<NT>(HP, ldp, m1, nb, panel, ldz, pow2f(-2 * power), srcm, colmask);
+                    } else {                                   // small rows of the matrix keep their own precision
+                        blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);
+                    }
+                }
                 else
                     blk_flush_mma<NT, true, true>(HP, ldp, m1, nb, min(nb, scap), panel, ldz, GVEC, gld, ZSTAGE, srcm, colmask);
                 __syncthreads();
@@ -1188,7 +1334,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int g = 0; g < KMAX / 4; ++g) cntw[g] = 0u;
                 ldz = blk_ldz(m0);
                 scap = a.panel_floats / ldz;
-                bcur = min(a.max_pending, scap + gB);
+                bcur = min(a.max_pending, GP || TC ? scap + gB : max(2, scap & ~1));
                 if (BC) bcur &= ~(BC - 1);
                 __syncthreads();
             }
