@@ -60,6 +60,8 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     BlkPlan p;
     p.nt = nt;
     p.per_sm = 512 / nt;
+    // at most one row per SM: all of its shared memory (more updates per pass, more slots on chip: 64 x 576 layer 2283 -> 2180 us)
+    if (row_count > 0 && row_count <= di.sm_count) p.per_sm = 1;
     // 1 KB per resident block is reserved by the hardware; keep every block's share 128-byte aligned
     const size_t sm_total = (size_t)di.smem_optin + 1024;
     size_t share = (sm_total / p.per_sm - 1024) & ~(size_t)127;
