@@ -26,9 +26,10 @@ obc_status blk_launch_512_12(const FlushMaps& zmaps, const EngineArgs& a, int bl
 // takes 149 ms since the layout and the tile order changed.)
 constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)110 << 20;
 
-// (one slot per thread on chip)
+// One slot per thread on chip, at most 256 of them.
 static int blk_pick_ms(int d, size_t panel_bytes, int nt) {
-    int ms = d < nt ? d : nt;
+    const int most = nt < 256 ? nt : 256;
+    int ms = d < most ? d : most;
     if (ms < 2) ms = 2;
     while (ms > 2 && blk_tail_bytes(ms) > panel_bytes) --ms;
     return ms;
