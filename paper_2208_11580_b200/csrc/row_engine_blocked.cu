@@ -39,21 +39,21 @@ static int blk_pick_ms(int d, size_t panel_bytes, int nt) {
 // several of them share an SM; long rows need the shared memory for pending vectors.
 // row_count = rows of the launch (0 = many).
 static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool nm = false, int bc = 0,
-                     int row_count = 0, int threads = 0, bool compound = false) {
+                     int row_count = 0, int threads = 0, int mode = MODE_PRUNE) {
     const int cap = (d + 3) & ~3;
     int nt = threads;
     if (nt != 128 && nt != 256 && nt != 512) {
-        // measured on many rows: 128 threads win up to d_col ~ 700, 256 up to ~ 1200 (1152: 34.3 against 35.2 ms with 512 threads,
-        // 1408: 55.5 against 48.7 ms), 512 above
-        nt = d <= 704 ? 128 : (d <= 1216 ? 256 : 512);
-        // few rows (one per SM pair at most): nothing to share an SM with, the larger block is faster per row
+        // measured on 1184 rows (ms with 128 / 256 / 512 threads): pruning 560 6.72 / 7.45 / 12.1, 640 9.65 / 9.61 / 14.7, 704 12.4 / 11.5 /
+        // 17.2, 1152 - / 38.5 / 43.3, 1280 - / 53.8 / 52.8; OBQ 640 11.0 / 11.2, 1280 57.1 / 57.1; replay before OBQ 560 7.25 / 7.24
+        nt = d <= 624 ? 128 : (d <= 1216 ? 256 : 512);
+        // few rows (one per SM pair at most): nothing to share an SM with, the larger block is faster per row (260 rows, 128 / 256
+        // threads: 320 0.75 / 0.73, 576 2.42 / 1.98)
         if (nt == 128 && row_count > 0 && row_count <= 2 * di.sm_count) nt = 256;
-        // at most one row per SM: the whole SM on one row wins from d_col ~ 700 (16 to 148 rows, 256 / 512 threads: OBQ 704 3.24 - 3.44 /
-        // 3.20 - 3.37 ms, 768 3.68 - 3.98 / 3.55 - 3.79, replay 704 1.2 - 1.4 / 0.8 - 1.1); later where a kernel of 512 threads gains
-        // less: replay before OBQ takes single steps there (768: 3.0 - 3.3 / 3.1 - 3.4, 832: 3.4 - 3.9 / 3.4 - 3.8), blocks of 8
-        // keep passes by mma.sync (832: 5.6 - 6.0 / 5.8 - 6.1, 896: 6.3 - 6.8 / 6.4 - 6.7), blocks of 4
-        // spend more of a step on scores (736: 2.63 - 2.87 / 2.70 - 2.85, 784: 2.94 - 3.21 / 2.93 - 3.08)
-        const int whole_sm = compound ? 816 : (bc == 8 ? 896 : (bc == 4 ? 736 : 704));
+        // at most one row per SM, which then has all its shared memory: 512 threads (passes on tcgen05) win from d_col ~ 1050 on (64
+        // rows, 256 / 512: pruning 960 3.46 / 3.55, 1152 5.08 / 4.85, OBQ 960 3.88 / 3.95, 1152 5.65 / 5.33, replay before OBQ 960 3.49 /
+        // 3.63, 1152 5.16 / 4.96), blocks of 4 at 736, blocks of 8 at 896, a replay alone, which is all passes, from 450 on (64
+        // rows: 320 0.36 / 0.35, 480 0.59 / 0.52, 704 1.04 / 0.85)
+        const int whole_sm = mode == MODE_REPLAY ? 448 : (bc == 4 ? 736 : bc == 8 ? 896 : 1056);
         if (nt == 256 && row_count > 0 && row_count <= di.sm_count && d > whole_sm) nt = 512;
     }
     if (nt == 128 && cap > 1024) nt = 256;
@@ -171,7 +171,7 @@ obc_status blocked_engine_launch(EngineArgs a, void* ws, size_t ws_bytes, cudaSt
     if (a.d > OBC_MAX_DCOL) return OBC_ERR_UNSUPPORTED;
     BlkPlan p;
     const int bc = (a.block_c == 4 || a.block_c == 8) ? a.block_c : 0;      // block pruning: the block size
-    if (!blk_plan(a.d, a.w_trace != nullptr, di, &p, a.nm_prune > 0, bc, a.row_count, a.opts.threads, a.mode == MODE_REPLAY_QUANT))
+    if (!blk_plan(a.d, a.w_trace != nullptr, di, &p, a.nm_prune > 0, bc, a.row_count, a.opts.threads, a.mode))
         return OBC_ERR_UNSUPPORTED;
     a.ms = p.ms;
     a.panel_floats = p.panel_floats;
