@@ -1,5 +1,5 @@
 // The rank-B update of the blocked row engine for long rows on the 5th-generation tensor cores: H -= sum_b z_b z_b^T over the
-// compacted lower triangle of one row's private inverse Hessian (B <= 48 pending vectors), one 512-thread block per SM.
+// compacted lower triangle of one row's private inverse Hessian (B <= 64 pending vectors), one 512-thread block per SM.
 //
 // A pass reads and writes every element of the triangle once (8 bytes); a tile takes about 2600 cycles of its SM's pipeline of copy,
 // products, subtraction and store, which is the copy rate of HBM when all SMs pass at once (16 rows of 4608 alone: 51 ms of passes,
@@ -7,9 +7,8 @@
 // tcgen05.mma (kind::f16) forms the tile's increment in tensor memory, and eight warps only subtract one from the other.
 // The products cost nothing beside the traffic, so a pass takes as many pending vectors as tensor memory holds partial sums
 // for; most of them wait in L2 (the mma.sync form spent half of a warp's time multiplying, so more vectors per pass bought it
-// little).  48 of them, not the 64 that four groups would allow: the steps between two passes read them all, and from
-// there on that costs about as much as the rarer passes save (64 / 48: 128 x 4608 161 / 156 ms, 256 x 2304 46.9 / 47.0, 768 x 3072
-// 260 / 269).  During a pass the space of the FP32 pending vectors is free and holds the tiles and operands.
+// little).  48 or 64 of them by the row's length (blk_plan): the steps between two passes read them all.  During a pass the space of the FP32
+// pending vectors is free and holds the tiles and operands.
 //
 // Operands.  Before the pass every pending vector is written as two FP16 planes, z * 2^e = hi + lo (hi rounded to 11 bits, lo
 // the rounded rest: 22 significant bits), to global memory (they stay in L2).  The power of two takes the largest entry to
@@ -34,7 +33,7 @@
 namespace obc {
 
 constexpr int FT_M = 128, FT_N = 64;              // tile
-constexpr int FT_GMAX = 3;                        // groups of 16 pending vectors (two tiles' accumulators in tensor memory)
+constexpr int FT_GMAX = 4;                        // groups of 16 pending vectors (two tiles' accumulators in tensor memory)
 constexpr int FT_COLS = 512;
 constexpr int FT_EW = 8;                          // warps that subtract: 32 rows x 32 columns each; four more issue
 constexpr int FT_WAIT_LIMIT = 1 << 22;            // polls before a wait gives up
@@ -235,6 +234,7 @@ __device__ __forceinline__ bool ft_copy_operands(const FlushGeom& q, FlushBars* 
     return true;
 }
 // Products of tile t; first / last: of its column block.  One thread.
+template <int GM>
 __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, int t, Ring& b, Ring& a, bool first, bool last) {
     const uint32_t blk = q.G * 2 * FT_GROUP_BYTES;
     const int buf = t & 1;
@@ -243,15 +243,15 @@ __device__ __forceinline__ bool ft_multiply(const FlushGeom& q, FlushBars* fb, i
     if (t > 1 && !ft_wait(&fb->free_d[buf], ((t >> 1) - 1) & 1, fb)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint64_t da = ft_desc(q.sa + a.at * 2 * blk, blk), db = ft_desc(q.sb + b.at * blk, blk);
-    const uint32_t d = q.tmem + buf * (FT_GMAX * FT_N);
+    const uint32_t d = q.tmem + buf * (GM * FT_N);
     constexpr uint64_t STEP = FT_GROUP_BYTES >> 4;
     const uint64_t LO = q.G * STEP;
 #pragma unroll
-    for (int k = 0; k < FT_GMAX; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + LO + k * STEP, db + k * STEP, 0u);
+    for (int k = 0; k < GM; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + LO + k * STEP, db + k * STEP, 0u);
 #pragma unroll
-    for (int k = 0; k < FT_GMAX; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + k * STEP, db + LO + k * STEP, 1u);
+    for (int k = 0; k < GM; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + k * STEP, db + LO + k * STEP, 1u);
 #pragma unroll
-    for (int k = 0; k < FT_GMAX; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + k * STEP, db + k * STEP, 1u);
+    for (int k = 0; k < GM; ++k) if (k < q.G) ft_mma(d + k * FT_N, da + k * STEP, db + k * STEP, 1u);
     ft_commit(&fb->done[buf]);
     ft_commit(&fb->free_a[a.at]);
     a.next(q.nb.n_a);
@@ -282,6 +282,7 @@ __device__ __forceinline__ bool ft_store(const FlushGeom& q, FlushBars* fb, Ring
     return true;
 }
 // A warp's 32 x 32 part of tile t: H minus the increment, in shared memory.
+template <int GM>
 __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, int t, Ring& hq, int rb, int c, float unscale, const signed char* zexp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = hq.at, buf = t & 1;
@@ -292,7 +293,7 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool any = r0 < q.m1 && col <= r0;
     const uint32_t row = q.sh + h * FT_TILE_BYTES + cg * (FT_M * 128) + (32 * (warp & 3) + lane) * 128;
-    const uint32_t d = q.tmem + buf * (FT_GMAX * FT_N) + 32 * cg + ((uint32_t)(32 * (warp & 3)) << 16);
+    const uint32_t d = q.tmem + buf * (GM * FT_N) + 32 * cg + ((uint32_t)(32 * (warp & 3)) << 16);
     const float rs = zexp && any && r0 + lane < q.m1 ? -ft_unscale(zexp, r0 + lane) : -unscale;
 #pragma unroll
     for (int v = 0; v < 2; ++v) {                     // 16 columns at a time
@@ -338,7 +339,9 @@ __device__ __forceinline__ bool ft_subtract(const FlushGeom& q, FlushBars* fb, i
 // the copies, and the block has synchronised.
 //   plane     first of the block's two planes (hi, lo) in the maps
 //   unscale   2^-2e of the planes' power, or zexp: the slots' own powers
+//   GM        most groups of 16 vectors that the kernel takes
 //   stop      tile (from 1) at which the products give up, for tests; 0: never
+template <int GM>
 __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, int tri, unsigned char* stage, int stage_bytes, FlushBars* fb, int m1,
                                              int nb, float unscale, const signed char* zexp, int stop) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -356,7 +359,7 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
     int rb = 0, c = 0, t = 0;
     if (warp < FT_EW) {
         for (; t < q.T; ++t) {
-            if (!ft_subtract(q, fb, t, h, rb, c, unscale, zexp)) break;
+            if (!ft_subtract<GM>(q, fb, t, h, rb, c, unscale, zexp)) break;
             ft_next_tile(rb, c, m1);
         }
     } else if (warp == FT_EW && lane == 0) {
@@ -378,7 +381,7 @@ __device__ __forceinline__ bool blk_flush_tc(const FlushMaps* maps, int plane, i
             }
             int nrb = rb, nc = c;
             ft_next_tile(nrb, nc, m1);
-            if (!ft_multiply(q, fb, t, b, a, rb == c / FT_M, nc != c)) break;
+            if (!ft_multiply<GM>(q, fb, t, b, a, rb == c / FT_M, nc != c)) break;
             rb = nrb; c = nc;
         }
     } else if (warp == FT_EW + 2 && lane == 0) {

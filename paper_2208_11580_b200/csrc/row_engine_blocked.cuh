@@ -1297,7 +1297,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     __syncthreads();
                     unsigned char* stage = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wd) + 1023) & ~(uintptr_t)1023);
                     const int stage_bytes = (int)(reinterpret_cast<unsigned char*>(panel + a.panel_floats) - stage);
-                    const bool fine = blk_flush_tc(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
+                    const bool fine = blk_flush_tc<(KMAX > 8 ? 3 : FT_GMAX)>(&zmaps, blockIdx.x * 2, (SH ? sched[2] : (int)blockIdx.x) * (((cap + 63) & ~63) >> 5), stage, stage_bytes, fb, m1, nb,
                                       power == 99 ? 1.f : pow2f(-2 * power), power == 99 ? zexp : nullptr, a.stop_tile);
                     for (int j = tid; j < cap; j += NT) reinterpret_cast<double2*>(wd)[j] = __ldcg(park + j);
                     __syncthreads();
