@@ -998,6 +998,7 @@ static __device__ __noinline__ double block8_score(const double* w, const double
 // broadcast, and every thread carries out the four Lemma-1 eliminations on its own slots in registers -- two
 // barriers per four steps, each pending vector read once for four columns.  Same arithmetic per element as four
 // single steps except that a column's corrections are subtracted one by one instead of summed first.
+// Block pruning in blocks of 4 does the same with the four members of the block it has picked (BG).
 // NM = N:M pruning; the other kernels are built without that code.
 // GPV = the kernel can keep further pending vectors in global memory (long rows, 512 threads only).
 // SH = the kernel takes shares of rows (a row may be started by one block and finished by the next); launches whose
@@ -1050,6 +1051,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     // overflow of the pending vectors: gB more of them in global memory (sized to stay in L2), stride gld
     // (only the one-row-per-SM configuration uses it; the other kernels are built without that code)
     constexpr bool GP = GPV;
+    constexpr bool BG = BC == 4 && KMAX == 4;                  // (the kernels with more slots per thread have no registers for it)
     const int gB = (GP && a.Gpan) ? a.g_vectors : 0, gld = a.g_ld;
     // (recomputed at every use instead of held in registers: the kernels with the overflow code have none to spare)
 #define GVEC (a.Gpan + (size_t)blockIdx.x * a.g_vectors * a.g_ld)
@@ -1230,6 +1232,26 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         unsigned alive = 0u;             // own slots that are live
         bool alive_valid = false;
         double gisc = 1.0 / gsc;
+        // The block of columns to go next (block pruning).
+        auto pick_block = [&](const Records& rec) {
+            // block boundary: exact FP64 score of every own live group (its four slots are all live here)
+            double bs = CUDART_INF;
+            int bo = 0x7fffffff, cslot = -1;
+#pragma unroll
+            for (int g = 0; g < KMAX / 4; ++g) {
+                const int jb = own_slot<NT>(4 * g);
+                if (BC == 8 && (jb & 7) != 0) continue;      // a block of 8 is scored by the owner of its first half
+                if (jb < m0 && perm[jb] >= 0) {
+                    const double sc4 = BC == 8 ? block8_score(wd + jb, dg + jb, boff + (jb >> 3) * 28)
+                                               : block4_score(wd + jb, dg + jb, boff + (jb >> 2) * 6);
+                    const int o = perm[jb];
+                    if (key_less(sc4, o, bs, bo)) { bs = sc4; bo = o; cslot = jb; }
+                }
+            }
+            const Pick pk = block_pick<NT>(cslot >= 0 ? float_key(__double2float_rn(bs)) : KEY_NONE, bs, cslot, cslot >= 0 ? perm[cslot] : -1, rec);
+            blk_base = pk.slot; blk_orig = pk.orig; blk_score = pk.s;
+            return pk;
+        };
         // (every thread: the smallest and largest weight of its survivors)
         auto survivors_grid = [&](float lo, float hi) {
 #pragma unroll
@@ -1342,15 +1364,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
             if (m0 <= ms) break;                 // on chip from here
             const bool forced = s < n_forced;
             const bool q_now = Q && quant && !forced;
-            if (FG && forced && !has_wfull && !has_nm && s + BLK_GS <= (SH ? min(n_forced, sched[1]) : n_forced) && nb + BLK_GS <= bcur &&
-                (!GP || nb + BLK_GS <= scap)) {
+            if ((BG && !has_wfull && (s - n_forced) % BCD == 0 && (!GP || nb + BLK_GS <= scap)) ||
+                (FG && forced && !has_wfull && !has_nm && s + BLK_GS <= (SH ? min(n_forced, sched[1]) : n_forced) && nb + BLK_GS <= bcur &&
+                 (!GP || nb + BLK_GS <= scap))) {
                 // ======================= four forced eliminations together ================================
                 constexpr int GS = BLK_GS;
+                if (BG) pick_block(rec_view(scratch, s & 1));
                 int* gslot = reinterpret_cast<int*>(smem + BLK_OFF_GRP);
                 float* gM = reinterpret_cast<float*>(smem + BLK_OFF_GRP + 16);
                 int fo[GS];
 #pragma unroll
-                for (int g = 0; g < GS; ++g) fo[g] = a.forced_order[(size_t)r * d + s + g];
+                for (int g = 0; g < GS; ++g) fo[g] = BG ? blk_orig + g : a.forced_order[(size_t)r * d + s + g];
                 unsigned live = 0u;
 #pragma unroll
                 for (int g4 = 0; g4 < KMAX / 4; ++g4) {
@@ -1364,15 +1388,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                             live |= 1u << (4 * g4 + q);
 #pragma unroll
                             for (int g = 0; g < GS; ++g)
-                                if (pq[q] == fo[g]) gslot[g] = jb + q;
+                                if (!BG && pq[q] == fo[g]) gslot[g] = jb + q;
                         }
                 }
-                __syncthreads();
+                if (!BG) __syncthreads();
                 int p4[GS];
                 bool ok = true;
 #pragma unroll
                 for (int g = 0; g < GS; ++g) {
-                    p4[g] = gslot[g];
+                    p4[g] = BG ? blk_base + g : gslot[g];
                     ok = ok && p4[g] >= 0 && p4[g] < m0 && perm[p4[g]] == fo[g];     // a stale entry never matches
                 }
                 ok = ok && p4[0] != p4[1] && p4[0] != p4[2] && p4[0] != p4[3] && p4[1] != p4[2] && p4[1] != p4[3] &&
@@ -1472,7 +1496,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         for (int g4 = 0; g4 < KMAX / 4; ++g4) {
                             const int jb = own_slot<NT>(4 * g4);
                             if (jb >= m0) continue;
-                            float zv[GS][4];
+                            float zv[GS][4], vv[BG ? GS : 1][4];
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 const int k = 4 * g4 + q, j = jb + q;
@@ -1492,6 +1516,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                                         nw -= fg[g] * (double)vj;
                                         nd -= (double)vj * (double)vj * idp[g];
                                         zv[g][q] = vj * rsq[g];
+                                        if (BG) vv[BG ? g : 0][q] = vj;
                                     }
                                 }
                                 if (gm < GS) perm[j] = -1;
@@ -1501,8 +1526,28 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                             for (int g = 0; g < GS; ++g)
                                 *reinterpret_cast<float4*>(panel + (size_t)(nb + g) * ldz + jb) =
                                     make_float4(zv[g][0], zv[g][1], zv[g][2], zv[g][3]);
+                            if (BG && ((live >> (4 * g4)) & 0xFu) == 0xFu && jb != p4[0]) {
+                                // Lemma 1 on the group's own 4 x 4 diagonal block, member by member (off-diagonal part)
+                                double* o = boff + (jb >> 2) * 6;
+#pragma unroll
+                                for (int g = 0; g < GS; ++g) {
+                                    const double v0 = (double)vv[BG ? g : 0][0], v1 = (double)vv[BG ? g : 0][1];
+                                    const double v2 = (double)vv[BG ? g : 0][2], v3 = (double)vv[BG ? g : 0][3];
+                                    o[0] -= v0 * v1 * idp[g]; o[1] -= v0 * v2 * idp[g]; o[2] -= v0 * v3 * idp[g];
+                                    o[3] -= v1 * v2 * idp[g]; o[4] -= v1 * v3 * idp[g]; o[5] -= v2 * v3 * idp[g];
+                                }
+                            }
                         }
-                        if (tid < GS) {
+                        if (BG) {
+                            if (tid < GS) {
+                                pv[nb + tid] = blk_base + tid;
+                                const int t = s - n_forced + tid;
+                                if (a.W_out) a.W_out[(size_t)r * a.ldwo + blk_orig + tid] = 0.f;
+                                if (a.mask) a.mask[(size_t)r * d + blk_orig + tid] = 0;
+                                if (a.order) a.order[(size_t)r * d + t] = blk_orig + tid;
+                                if (a.loss) a.loss[(size_t)r * d + t] = tid ? 0.f : (float)blk_score;
+                            }
+                        } else if (tid < GS) {
                             pv[nb + tid] = p4[tid];
                             if (a.W_out) a.W_out[(size_t)r * a.ldwo + fo[tid]] = 0.f;
                             if (a.mask) a.mask[(size_t)r * d + fo[tid]] = 0;
@@ -1547,22 +1592,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 __syncthreads();
                 pk.slot = blk_base + (s - n_forced) % BCD; pk.orig = blk_orig + (s - n_forced) % BCD; pk.s = 0.0;
             } else if (BC) {
-                // block boundary: exact FP64 score of every own live group (its four slots are all live here)
-                double bs = CUDART_INF;
-                int bo = 0x7fffffff, cslot = -1;
-#pragma unroll
-                for (int g = 0; g < KMAX / 4; ++g) {
-                    const int jb = own_slot<NT>(4 * g);
-                    if (BC == 8 && (jb & 7) != 0) continue;      // a block of 8 is scored by the owner of its first half
-                    if (jb < m0 && perm[jb] >= 0) {
-                        const double sc4 = BC == 8 ? block8_score(wd + jb, dg + jb, boff + (jb >> 3) * 28)
-                                                   : block4_score(wd + jb, dg + jb, boff + (jb >> 2) * 6);
-                        const int o = perm[jb];
-                        if (key_less(sc4, o, bs, bo)) { bs = sc4; bo = o; cslot = jb; }
-                    }
-                }
-                pk = block_pick<NT>(cslot >= 0 ? float_key(__double2float_rn(bs)) : KEY_NONE, bs, cslot, cslot >= 0 ? perm[cslot] : -1, rec);
-                blk_base = pk.slot; blk_orig = pk.orig; blk_score = pk.s;
+                pk = pick_block(rec);
             } else {
                 if (!sa_valid || outliers)
                     estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gisc, gze, gmq, gr, has_nm ? blkcnt : nullptr,
