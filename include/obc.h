@@ -241,6 +241,8 @@ obc_status obc_select_global_mask_static(const float *loss, const int32_t *order
 /* Section 3 / Figure 1: the weights of each row after its first counts[r] eliminations.
  * w_trace != NULL (layout of obc_prune_trace with this `trace_steps`): rows are gathered from the trace.
  * w_trace == NULL: the eliminations order[r][0..counts[r]) are replayed on W (no argmin).
+ * A replay stops at an entry of the order that names no remaining column (-1, beyond the row, named before): row_status[r] =
+ * 1 + its step, and W_out holds the row as it was before that step (obc_quantize replays by the same rule).
  * counts[r] = -OBC_ERR_TIMEOUT (a global selection that gave up): the row's dense weights, row_status[r] = that value. */
 obc_status obc_prune_apply(const float *W, int ldw, int d_row, int d_col, int row_begin, int row_count,
                            const float *Hinv, int ldhi, const int32_t *order, const int32_t *counts,

@@ -1400,7 +1400,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                 for (int g = 0; g < GS; ++g) {
                     p4[g] = BG ? blk_base + g : gslot[g];
-                    ok = ok && p4[g] >= 0 && p4[g] < m0 && perm[p4[g]] == fo[g];     // a stale entry never matches
+                    // (a stale slot is dead, perm = -1, or holds another column)
+                    ok = ok && fo[g] >= 0 && p4[g] >= 0 && p4[g] < m0 && perm[p4[g]] == fo[g];
                 }
                 ok = ok && p4[0] != p4[1] && p4[0] != p4[2] && p4[0] != p4[3] && p4[1] != p4[2] && p4[1] != p4[3] &&
                      p4[2] != p4[3];
@@ -1563,7 +1564,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         continue;
                     }
                 }
-                // an entry of the order that is not live, or a pivot that is not positive: the single steps below
+                // an entry of the order that names no live column, or a pivot that is not positive: the single steps below
                 // meet it again and report it
             }
             // ---- grid of the compound path: built from the survivors when the replay is over -----------
@@ -1587,7 +1588,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                 for (int k = 0; k < KMAX; ++k) {
                     const int j = own_slot<NT>(k);
-                    if (j < m0 && perm[j] == f) cslot = j;
+                    if (j < m0 && f >= 0 && perm[j] == f) cslot = j;      // (perm = -1: a dead slot)
                 }
                 pk = known_pick<NT>(cslot, f, rec);
             } else if (BC && (s - n_forced) % BCD != 0) {
@@ -1842,7 +1843,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 Pick pk;
                 if (forced) {
                     const int f = a.forced_order[(size_t)r * d + s];
-                    pk = known_pick<NT>(o == f ? j : -1, f, rec);
+                    pk = known_pick<NT>(o >= 0 && o == f ? j : -1, f, rec);      // (o = -1: a dead slot, or none)
                 } else {
                     if (!est_valid) {
                         est = CUDART_NAN_F;
