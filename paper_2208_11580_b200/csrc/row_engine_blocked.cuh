@@ -1238,6 +1238,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         // The block of columns to go next (block pruning).
         auto pick_block = [&](const Records& rec) {
             // block boundary: exact FP64 score of every own live group (its four slots are all live here)
+            if (BC == 8) __syncwarp();       // the second half's state and some off-diagonals were written by the neighbouring lane
             double bs = CUDART_INF;
             int bo = 0x7fffffff, cslot = -1;
 #pragma unroll
