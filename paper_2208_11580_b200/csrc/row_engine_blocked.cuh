@@ -687,6 +687,9 @@ template <bool TC> __device__ __forceinline__ float ld_tri(const float* p) { ret
 template <bool TC> __device__ __forceinline__ float4 ld_tri4(const float* p) {
     return TC ? __ldcg(reinterpret_cast<const float4*>(p)) : *reinterpret_cast<const float4*>(p);
 }
+template <int BYTES> __device__ __forceinline__ void copy_async(float* to, const float* from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "n"(BYTES) : "memory");
+}
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
 // the power of two that takes v (> 0, finite) to [2^13, 2^14), within what a float power of two and its square hold
 __device__ __forceinline__ int plane_power(float v) { return min(60, max(-50, 13 - ((int)(__float_as_uint(v) >> 23) - 127))); }
@@ -1000,7 +1003,7 @@ static __device__ __noinline__ double block8_score(const double* w, const double
 // four pivot columns are fetched and corrected together, the 4 x 4 block of the columns at the pivot slots is
 // broadcast, and every thread carries out the four Lemma-1 eliminations on its own slots in registers -- two
 // barriers per four steps, each pending vector read once for four columns.  Same arithmetic per element as four
-// single steps except that a column's corrections are subtracted one by one instead of summed first.
+// single steps, but for the order in which the four members' own corrections are added.
 // Block pruning in blocks of 4 does the same with the four members of the block it has picked (BG).
 // NM = N:M pruning; the other kernels are built without that code.
 // GPV = the kernel can keep further pending vectors in global memory (long rows, 512 threads only).
@@ -1055,6 +1058,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     // (only the one-row-per-SM configuration uses it; the other kernels are built without that code)
     constexpr bool GP = GPV;
     constexpr bool BG = BC == 4 && KMAX == 4;                  // (the kernels with more slots per thread have no registers for it)
+    enum { COLS_REGS, COLS_SMEM, COLS_SUBTRACT };              // where the columns of four eliminations wait for their corrections
+    constexpr int COLS = KMAX == 4 ? COLS_REGS : (TC ? COLS_SUBTRACT : COLS_SMEM);
     const int gB = (GP && a.Gpan) ? a.g_vectors : 0, gld = a.g_ld;
     // (recomputed at every use instead of held in registers: the kernels with the overflow code have none to spare)
 #define GVEC (a.Gpan + (size_t)blockIdx.x * a.g_vectors * a.g_ld)
@@ -1410,33 +1415,47 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     double wp4[GS], dp4[GS];
 #pragma unroll
                     for (int g = 0; g < GS; ++g) { wp4[g] = wd[p4[g]]; dp4[g] = dg[p4[g]]; }
-                    // the four pivot columns of the stored matrix at the own slots
+                    // the four pivot columns of the stored matrix at the own slots, minus the pending vectors' part (all of them
+                    // in shared memory here).  The part is summed first and subtracted once, as a single step does: taken
+                    // from the column product by product, every product is rounded at the size of the column's entry (rms error
+                    // of the loss 1.2 times as large for blocks of 4, 1.7 times for a replay before OBQ at 960 columns).  The
+                    // columns wait in registers of their own or, where there are none, in shared memory at the place of the
+                    // vectors to come; only the kernels with more slots and passes on tcgen05, whose stores a copy by way of L1
+                    // might miss, subtract product by product.
                     const float* const tri = HP;
-                    float v[GS][KMAX];
+                    float v[GS][KMAX], cols[COLS == COLS_REGS ? GS : 1][COLS == COLS_REGS ? KMAX : 1];
+                    float* const wait = panel + (size_t)nb * ldz;
 #pragma unroll
                     for (int g4 = 0; g4 < KMAX / 4; ++g4) {
                         const int jb = own_slot<NT>(4 * g4);
+                        auto stored = [&](int g, int k) -> float& { return COLS == COLS_REGS ? cols[COLS == COLS_REGS ? g : 0][COLS == COLS_REGS ? k : 0] : v[g][k]; };
 #pragma unroll
                         for (int g = 0; g < GS; ++g)
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) v[g][4 * g4 + q] = 0.f;
+                            for (int q = 0; q < 4; ++q) { v[g][4 * g4 + q] = 0.f; stored(g, 4 * g4 + q) = 0.f; }
                         if (jb >= m0) continue;
 #pragma unroll
                         for (int g = 0; g < GS; ++g) {
                             const int p = p4[g];
                             if (jb + 3 <= p) {
-                                const float4 t = ld_tri4<TC>(tri + tri_at<TC>(ldp, p, jb));
-                                v[g][4 * g4] = t.x; v[g][4 * g4 + 1] = t.y; v[g][4 * g4 + 2] = t.z; v[g][4 * g4 + 3] = t.w;
+                                const float* from = tri + tri_at<TC>(ldp, p, jb);
+                                if (COLS == COLS_SMEM) copy_async<16>(wait + (size_t)g * ldz + jb, from);
+                                else {
+                                    const float4 t = ld_tri4<TC>(from);
+                                    stored(g, 4 * g4) = t.x; stored(g, 4 * g4 + 1) = t.y; stored(g, 4 * g4 + 2) = t.z; stored(g, 4 * g4 + 3) = t.w;
+                                }
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 4; ++q) {
                                     const int j = jb + q;
-                                    if ((live >> (4 * g4 + q)) & 1u) v[g][4 * g4 + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p)));
+                                    if (!((live >> (4 * g4 + q)) & 1u)) continue;
+                                    const float* from = tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p));
+                                    if (COLS == COLS_SMEM) copy_async<4>(wait + (size_t)g * ldz + j, from);
+                                    else stored(g, 4 * g4 + q) = ld_tri<TC>(from);
                                 }
                             }
                         }
                     }
-                    // corrected by the pending vectors (all of them in shared memory here)
                     for (int b = 0; b < nb; ++b) {
                         const float* zo = panel + (size_t)b * ldz;
                         float zp[GS];
@@ -1453,6 +1472,23 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                                     v[g][4 * g4 + 2] = fmaf(-z.z, zp[g], v[g][4 * g4 + 2]);
                                     v[g][4 * g4 + 3] = fmaf(-z.w, zp[g], v[g][4 * g4 + 3]);
                                 }
+                            }
+                        }
+                    }
+                    if (COLS == COLS_REGS) {
+#pragma unroll
+                        for (int g = 0; g < GS; ++g)
+#pragma unroll
+                            for (int k = 0; k < KMAX; ++k) v[g][k] += cols[COLS == COLS_REGS ? g : 0][COLS == COLS_REGS ? k : 0];
+                    } else if (COLS == COLS_SMEM) {
+                        asm volatile("cp.async.wait_all;" ::: "memory");       // own copies only: no barrier
+#pragma unroll
+                        for (int g4 = 0; g4 < KMAX / 4; ++g4) {
+                            if (!((live >> (4 * g4)) & 0xFu)) continue;
+#pragma unroll
+                            for (int g = 0; g < GS; ++g) {
+                                const float4 t = *reinterpret_cast<const float4*>(wait + (size_t)g * ldz + own_slot<NT>(4 * g4));
+                                v[g][4 * g4] += t.x; v[g][4 * g4 + 1] += t.y; v[g][4 * g4 + 2] += t.z; v[g][4 * g4 + 3] += t.w;
                             }
                         }
                     }

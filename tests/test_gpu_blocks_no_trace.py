@@ -52,3 +52,31 @@ def _check(Wd, Hd, c, threads, pending):
 @pytest.mark.parametrize("threads,d,pending", [(0, 64, 0), (128, 320, 0), (128, 600, 8), (256, 600, 0), (256, 1000, 16), (512, 600, 0), (512, 1000, 24)])
 def test_blocks_of_8(threads, d, pending):
     _check(*_layer(d, 3), 8, threads, pending)
+
+
+@pytest.mark.parametrize("threads,d,pending", [(512, 12, 0), (512, 320, 16), (512, 640, 0), (0, 740, 0), (0, 740, 12), (512, 1000, 20), (0, 1152, 0), (512, 1152, 12),
+                                               (0, 2040, 0), (0, 2060, 0), (128, 600, 0), (256, 1000, 16)])
+def test_blocks_of_4(threads, d, pending):
+    _check(*_layer(d, 2 if d > 1500 else 3), 4, threads, pending)
+
+
+@pytest.mark.parametrize("d", [640, 1152])
+def test_block_that_is_not_positive_definite(d):
+    """such a block is never chosen and is reported when nothing else is left, as in the single steps that a weight trace asks for"""
+    import paper_2208_11580_b200 as obc
+    g = np.random.default_rng(d)
+    H = g.standard_normal((d, d)) * 1e-3
+    H = H + H.T + np.eye(d)
+    at = 4 * (d // 8)
+    H[at:at + 4, :] = H[:, at:at + 4] = 0.0
+    H[at:at + 4, at:at + 4] = np.eye(4)
+    H[at, at + 1] = H[at + 1, at] = 2.0                        # minor 1 - 4 < 0
+    Hd = torch.from_numpy(H.astype(np.float32)).cuda()
+    Wd = torch.from_numpy(g.standard_normal((2, d)).astype(np.float32)).cuda()
+    o, l, st = _run(Wd, Hd, 4, 512, 0)
+    assert np.all(st == 1 + d - 4) and np.all(o[:, -4:] == -1) and np.all(np.isinf(l[:, -4:])) and not np.any(o[:, :-4] // 4 == at // 4)
+    order, loss = torch.zeros(2, d, dtype=torch.int32, device="cuda"), torch.zeros(2, d, device="cuda")
+    status, trace = torch.zeros(2, dtype=torch.int32, device="cuda"), torch.zeros(2, d + 1, d, device="cuda")
+    obc.obc_prune_blocks(Wd, Hd, order, loss, status, block=4, w_trace=trace, opts=obc.engine_opts(obc.ENGINE_BLOCKED, 512, 0))
+    torch.cuda.synchronize()
+    assert np.array_equal(status.cpu().numpy(), st) and (order.cpu().numpy() == o).mean() > 0.99
