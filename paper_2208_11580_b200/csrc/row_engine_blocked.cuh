@@ -347,10 +347,10 @@ __device__ __forceinline__ float score_estimate(double w, double dgv, bool quant
         constexpr double M = 6755399441055744.0;
         const double t = w * isc, u = t + M;
         const int r = __double2loint(u);
-        // (the high word says whether the integer fits 32 bits.)  Next to a rounding boundary the two possible codes give
-        // the same |err| to ~1e-16, which is all an estimate needs
+        // (the high word says whether the integer fits 32 bits: it has to agree with the low word's sign.)  Next to a rounding
+        // boundary the two possible codes give the same |err| to ~1e-16, which is all an estimate needs
         double c = u - M;
-        if ((unsigned)__double2hiint(u) - 0x4337FFFFu > 1u || r < gr.lo || r > gr.hi) c = t < -ze ? -ze : mq - ze;
+        if (__double2hiint(u) != 0x43380000 + (r >> 31) || r < gr.lo || r > gr.hi) c = t < -ze ? -ze : mq - ze;
         ef = gr.sc == 0.f ? 0.f : __double2float_rn(c - t) * gr.sc;
     } else {
         ef = __double2float_rn(w);
