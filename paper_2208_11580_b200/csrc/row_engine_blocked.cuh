@@ -320,27 +320,25 @@ static __device__ __noinline__ double grid_error(double w, double sc, double isc
     return grid_q_fast(w, sc, isc, ze, mq, &code) - w;
 }
 
-// The grid of a row as the estimates use it: the codes' integer range without the zero point.  sc = 0: a grid whose zero point
+// The grid of a row as the estimates use it: the codes' integer range without the zero point.  lo > hi: a grid whose zero point
 // is no integer, or a scale far outside the range of ordinary weights; there every estimate is 0, which leaves the choice
 // to the FP64 scores of all slots.
-struct GridRange { float sc; int lo, hi; };
+struct GridRange { int lo, hi; };
 __device__ __forceinline__ GridRange grid_range(double sc, double ze, double mq) {
-    GridRange g;
-    g.sc = __double2float_rn(sc);
     const bool plain = fabs(ze) < 1e9 && ze == rint(ze) && fabs(sc) > 1e-30 && fabs(sc) < 1e30;      // (false for NaN)
-    if (!plain) g.sc = 0.f;
-    g.lo = plain ? -(int)ze : 0;
+    GridRange g;
+    g.lo = plain ? -(int)ze : 1;
     g.hi = plain ? (int)(mq - ze) : 0;
     return g;
 }
 
 // FP32 estimate of the score of a slot (relative error of a few 1e-7): it only screens candidates, slots that are near the best
-// estimate are told apart by FP64 scores.  On a grid the distance to the nearest integer is taken in FP64 (w / scale has up to 8
-// bits before the point and a small distance is what wins); x + 1.5 * 2^52 - 1.5 * 2^52 rounds x to an integer whose low 32
-// bits are the sum's (three FP64 additions; rint, the clamps and the conversions take four times as many slots of the
-// FP64 and conversion pipes).
+// estimate are told apart by FP64 scores.  On a grid the distance to the nearest code's value is taken in FP64, as the exact score
+// takes it: a small distance is what wins, and weights may lie on the grid already.  x + 1.5 * 2^52 - 1.5 * 2^52 rounds x to an
+// integer whose low 32 bits are the sum's (rint, the clamps and the conversions take four times as many slots of the FP64
+// and conversion pipes).
 template <bool Q>
-__device__ __forceinline__ float score_estimate(double w, double dgv, bool quant, double isc, double ze, double mq,
+__device__ __forceinline__ float score_estimate(double w, double dgv, bool quant, double sc, double isc, double ze, double mq,
                                                 const GridRange& gr) {
     float ef;
     if (Q && quant) {
@@ -351,7 +349,7 @@ __device__ __forceinline__ float score_estimate(double w, double dgv, bool quant
         // boundary the two possible codes give the same |err| to ~1e-16, which is all an estimate needs
         double c = u - M;
         if (__double2hiint(u) != 0x43380000 + (r >> 31) || r < gr.lo || r > gr.hi) c = t < -ze ? -ze : mq - ze;
-        ef = gr.sc == 0.f ? 0.f : __double2float_rn(c - t) * gr.sc;
+        ef = gr.lo > gr.hi ? 0.f : __double2float_rn(fma(c, sc, -w));
     } else {
         ef = __double2float_rn(w);
     }
@@ -364,7 +362,7 @@ __device__ __forceinline__ float score_estimate(double w, double dgv, bool quant
 // own slots' blocks, one byte per slot, which the update phase then keeps current in registers.
 template <int NT, int KMAX, bool Q>
 __device__ __forceinline__ void estimate_own(float (&sa)[KMAX], const double* wd, const double* dg, const int* perm,
-                                             int m0, bool quant, double isc, double ze, double mq, const GridRange& gr,
+                                             int m0, bool quant, double sc, double isc, double ze, double mq, const GridRange& gr,
                                              const unsigned char* blkcnt, int nm_lg, int nm_prune,
                                              unsigned (&cntw)[KMAX / 4]) {
 #pragma unroll
@@ -376,7 +374,7 @@ __device__ __forceinline__ void estimate_own(float (&sa)[KMAX], const double* wd
         if (j < m0 && perm[j] >= 0) {
             unsigned c = 0u;
             if (blkcnt) { c = blkcnt[perm[j] >> nm_lg]; cntw[k >> 2] |= c << (8 * (k & 3)); }
-            if (!blkcnt || (int)c < nm_prune) sa[k] = score_estimate<Q>(wd[j], dg[j], quant, isc, ze, mq, gr);
+            if (!blkcnt || (int)c < nm_prune) sa[k] = score_estimate<Q>(wd[j], dg[j], quant, sc, isc, ze, mq, gr);
         }
     }
 }
@@ -1636,7 +1634,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 pk = pick_block(rec);
             } else {
                 if (!sa_valid || outliers)
-                    estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gisc, gze, gmq, gr, has_nm ? blkcnt : nullptr,
+                    estimate_own<NT, KMAX, Q>(sa, wd, dg, perm, m0, q_now, gsc, gisc, gze, gmq, gr, has_nm ? blkcnt : nullptr,
                                            nm_lg, nm_prune, cntw);
                 if (!(Q && outliers)) {
                     float e1, e2;
@@ -1763,7 +1761,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     const double nd = dv[q] - (double)vj * (double)vj * idpp;
                     wv[q] = nw; dv[q] = nd;
                     zv[q] = vj * rs;
-                    if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gisc, gze, gmq, gr);
+                    if (est_next) sa[k] = score_estimate<Q>(nw, nd, q_next, gsc, gisc, gze, gmq, gr);
                     if (has_nm) {
                         if ((pq[q] >> nm_lg) == (op >> nm_lg)) cntw[g] += 1u << (8 * q);
                         if ((int)((cntw[g] >> (8 * q)) & 0xFFu) >= nm_prune) sa[k] = CUDART_NAN_F;
@@ -1884,7 +1882,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 } else {
                     if (!est_valid) {
                         est = CUDART_NAN_F;
-                        if (o >= 0 && !(has_nm && cnt >= nm_prune)) est = score_estimate<Q>(w, g, q_now, gisc, gze, gmq, gr);
+                        if (o >= 0 && !(has_nm && cnt >= nm_prune)) est = score_estimate<Q>(w, g, q_now, gsc, gisc, gze, gmq, gr);
                     }
                     bool sure = false;
                     if (!(Q && outliers)) pk = fast_pick<NT>(est, CUDART_INF_F, est == est ? j : -1, o, rec, &sure);
@@ -1929,7 +1927,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     if (has_wfull) wfull[o] = (float)w;
                     if (has_nm && (o >> nm_lg) == (op >> nm_lg)) ++cnt;
                     if (est_next) {
-                        est = score_estimate<Q>(w, g, Q && quant, gisc, gze, gmq, gr);
+                        est = score_estimate<Q>(w, g, Q && quant, gsc, gisc, gze, gmq, gr);
                         if (has_nm && cnt >= nm_prune) est = CUDART_NAN_F;
                     }
                 }

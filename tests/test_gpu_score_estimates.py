@@ -1,5 +1,5 @@
 """The FP32 estimates that screen the candidates of a step, where they could lead away from the FP64 scores: weights far beyond the grid (the
-integer nearest to w / scale does not fit 32 bits)."""
+integer nearest to w / scale does not fit 32 bits), weights that lie on the grid exactly (all scores 0: the lowest column goes first)."""
 import numpy as np
 import pytest
 import torch
@@ -51,3 +51,16 @@ def test_weights_far_beyond_the_grid(threads, d, sign):
     at = [int(np.argmax(order[r] == d // 3)) for r in range(2)]
     assert min(at) >= first
     check_rows(_hinv(d), W, order, loss, mode="quant", scale=np.full(2, np.float64(sc)), zero=np.full(2, np.float64(ze)), maxq=maxq, steps=first)
+
+
+@pytest.mark.parametrize("threads,d", [(128, 64), (128, 320), (256, 512), (512, 640)])
+def test_weights_on_the_grid(threads, d):
+    # w = scale * a power of two: the FP64 distance to the grid is 0, w / scale through the reciprocal is not
+    cand = (0.3 + 0.01 * np.arange(200)).astype(np.float32)
+    sc = next(s for s in cand if np.float64(s) * (1.0 / np.float64(s)) != 1.0)
+    g = np.random.default_rng(d)
+    W = (sc * np.array([1, -1, 2, -2, 4, -4], np.float32)[g.integers(0, 6, (2, d))]).astype(np.float32)
+    H = (np.diag(g.uniform(1e-4, 1e-3, d)) + 1e-5).astype(np.float32)
+    order, loss, Wq, codes = _quantize(W, H, np.full(2, sc), np.full(2, np.float32(7)), 4, threads, True)
+    assert np.array_equal(order, np.tile(np.arange(d), (2, 1))) and np.all(loss == 0.0)
+    assert np.array_equal(Wq, W) and np.array_equal(codes, np.rint(W / sc).astype(np.int64) + 7)
