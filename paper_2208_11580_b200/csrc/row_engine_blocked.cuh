@@ -320,15 +320,17 @@ static __device__ __noinline__ double grid_error(double w, double sc, double isc
     return grid_q_fast(w, sc, isc, ze, mq, &code) - w;
 }
 
-// The grid of a row as the estimates use it: the codes' integer range without the zero point.  lo > hi: a grid whose zero point
-// is no integer, or a scale far outside the range of ordinary weights; there every estimate is 0, which leaves the choice
-// to the FP64 scores of all slots.
+// The grid of a row as the estimates use it: the codes' integer range without the zero point.  lo > hi: a zero point whose
+// sum with a code is not exact, or a scale far outside the range of ordinary weights; there every estimate is 0, which leaves the
+// choice to the FP64 scores of all slots.
 struct GridRange { int lo, hi; };
 __device__ __forceinline__ GridRange grid_range(double sc, double ze, double mq) {
-    const bool plain = fabs(ze) < 1e9 && ze == rint(ze) && fabs(sc) > 1e-30 && fabs(sc) < 1e30;      // (false for NaN)
+    const double fine = ze * 1073741824.0;                     // (a multiple of 2^-30 below 1e5 plus a code: 48 bits)
+    const bool exact = (ze == rint(ze) && fabs(ze) < 1e9) || (fine == rint(fine) && fabs(ze) < 1e5);
+    const bool plain = exact && fabs(sc) > 1e-30 && fabs(sc) < 1e30;      // (false for NaN)
     GridRange g;
-    g.lo = plain ? -(int)ze : 1;
-    g.hi = plain ? (int)(mq - ze) : 0;
+    g.lo = plain ? (int)ceil(-ze) : 1;
+    g.hi = plain ? (int)floor(mq - ze) : 0;
     return g;
 }
 

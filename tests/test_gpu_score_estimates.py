@@ -1,5 +1,6 @@
 """The FP32 estimates that screen the candidates of a step, where they could lead away from the FP64 scores: weights far beyond the grid (the
-integer nearest to w / scale does not fit 32 bits), weights that lie on the grid exactly (all scores 0: the lowest column goes first)."""
+integer nearest to w / scale does not fit 32 bits), weights that lie on the grid exactly (all scores 0: the lowest column goes first), grids
+whose zero point is no integer."""
 import numpy as np
 import pytest
 import torch
@@ -64,3 +65,14 @@ def test_weights_on_the_grid(threads, d):
     order, loss, Wq, codes = _quantize(W, H, np.full(2, sc), np.full(2, np.float32(7)), 4, threads, True)
     assert np.array_equal(order, np.tile(np.arange(d), (2, 1))) and np.all(loss == 0.0)
     assert np.array_equal(Wq, W) and np.array_equal(codes, np.rint(W / sc).astype(np.int64) + 7)
+
+
+@pytest.mark.parametrize("zero", [7.25, 7.5, 7.000001, 1e-12])
+@pytest.mark.parametrize("threads,d", [(128, 64), (128, 300), (512, 516)])
+def test_zero_point_that_is_no_integer(threads, d, zero):
+    W, H = obc_synth.make_small(2, d, 2 * d + 40, d, "relu")[0].astype(np.float32), _hinv(d)
+    if zero < 1:                                       # (a grid of positive values)
+        W = np.abs(W)
+    sc, ze = (np.abs(W).max(axis=1) / (7 if zero > 1 else 15)).astype(np.float32), np.full(2, zero, np.float32)
+    order, loss, Wq, codes = _quantize(W, H, sc, ze, 4, threads, False)
+    check_rows(H, W, order, loss, gpu_w=Wq, mode="quant", scale=sc.astype(np.float64), zero=ze.astype(np.float64), maxq=15, gpu_codes=codes)
