@@ -64,19 +64,26 @@ def model_bytes_full(d: int, first: int | None = None, steps: int | None = None)
 
 def pending_stride(m: int) -> int:
     """Floats between two pending update vectors of a row of m slots (the stride obc_engine_plan documents)."""
-    return (m + 8 + 31) // 32 * 32 + 8
+    return (m + 12 + 31) // 32 * 32 + 4
+
+
+def pending_updates(plan: dict, m: int) -> int:
+    """Updates that a row of m slots defers between two passes (as obc_engine_plan documents it)."""
+    fit = plan["panel_floats"] // pending_stride(m)
+    if plan.get("threads", 512) < 512:
+        fit = max(2, fit // 2 * 2)
+    return min(plan["max_pending"], fit + plan.get("l2_vectors", 0))
 
 
 def blocked_schedule(plan: dict, first: int, steps: int):
     """(m_after_flush, updates_applied) for every pass the blocked engine makes over a row's matrix when `steps`
-    eliminations start at active size `first`: it defers min(max_pending, panel_floats // pending_stride(m) + l2_vectors)
-    updates, flushes early when the live size reaches the on-chip threshold, and finishes in shared memory below it."""
-    ms, panel, maxp = plan["on_chip_below"], plan["panel_floats"], plan["max_pending"]
+    eliminations start at active size `first`: it defers pending_updates(plan, m) updates, flushes early when the live size reaches the on-chip threshold, and finishes in shared memory below it."""
+    ms = plan["on_chip_below"]
     out, m0, left = [], first, steps
     if first <= ms:
         return out
     while left > 0 and m0 > ms:
-        b = max(1, min(maxp, panel // pending_stride(m0) + plan.get("l2_vectors", 0)))
+        b = max(1, pending_updates(plan, m0))
         nb = min(b, m0 - ms, left)
         left -= nb
         if left <= 0:

@@ -106,9 +106,11 @@ enum { OBC_ENGINE_WHOLE_WAVES = 1 };
  * [2] rows resident per SM, [3] active size at which a row moves into shared memory, [4] floats of shared memory
  * for deferred update vectors (BLOCKED), [5] limit on deferred updates (BLOCKED), [6] SM count, [7] further
  * deferred update vectors kept in global memory (BLOCKED, long rows; sized to stay in L2).
- * A BLOCKED row of current size m defers min(plan[5], plan[4] / stride(m) + plan[7]) updates between two passes
- * over its matrix, stride(m) = round_up(m + 8, 32) + 8 floats per deferred vector.  Used by the benchmark to state
- * the bytes a launch has to move. */
+ * A BLOCKED row of current size m defers min(plan[5], fit + plan[7]) updates between two passes over its matrix, fit =
+ * plan[4] / stride(m) with stride(m) = round_up(m + 12, 32) + 4 floats per deferred vector; with fewer than 512 threads, fit is
+ * rounded down to an even number (at least 2).  Used by the benchmark to state the bytes a launch has to move.
+ * The plan is that of pruning and OBQ.  A replay alone (obc_prune_apply) and block pruning choose threads, updates per pass and
+ * the move into shared memory by rules of their own. */
 obc_status obc_engine_plan(int d_col, int with_trace, int row_count, const obc_engine_opts *opts, int32_t *plan);
 
 /* Bytes of workspace the given call needs for these sizes on the CURRENT device (host function, no launch).

@@ -70,6 +70,12 @@ __host__ __device__ inline size_t blk_state_bytes(int cap, bool wfull, bool nm =
 // Stride of the pending vectors for a row of m slots: = 4 (mod 32), so that the tensor-core fragments of the flush (every second
 // row of 4 pairs of vectors x 8 consecutive slots per load) touch 32 different banks.
 __host__ __device__ inline int blk_ldz(int m) { return ((m + 12 + 31) & ~31) + 4; }     // >= m + 16
+// Updates that a row of m slots defers between two passes: as many vectors as there is room for.  pairs: passes by mma.sync on packed
+// planes, which hold two vectors each (fewer than 512 threads; no overflow vectors there).
+__host__ __device__ inline int blk_updates(int m, int panel_floats, int max_pending, int g_vectors, bool pairs) {
+    const int fit = panel_floats / blk_ldz(m), n = !pairs ? fit + g_vectors : fit < 2 ? 2 : fit & ~1;
+    return n < max_pending ? n : max_pending;
+}
 // On chip: TAIL_B deferred updates as two arrays per slot (column entries v, v / [H]_pp; TAIL_LD floats apart: 128-bit accesses
 // of consecutive slots meet no bank twice), then the lower triangle, its rows end to end: column p of 32 rows from a multiple of
 // 32 on touches 32 different banks (triangular numbers mod 32 are a permutation).
@@ -98,14 +104,14 @@ __host__ __device__ inline double blk_step_cost(int nt) { return nt >= 512 ? 300
 // boundary; total: the share reaches into the on-chip end of the row, which is then left to the starting block).
 // Every thread of a block computes the same value from the same arguments.
 static __device__ __noinline__ int blk_cut_step(int d, int ms, int total, int panel_floats, int max_pending, int g_vectors,
-                                        int num, int den, double step_cost) {
+                                        bool pairs, int num, int den, double step_cost) {
     double all = 0.0, at = 0.0;
     int cut = 0;
     for (int pass = 0; pass < 2; ++pass) {
         int m = d, s = 0;
         double cost = 0.0;
         while (s < total && m > ms) {
-            int b = min(max_pending, panel_floats / blk_ldz(m) + g_vectors);
+            int b = blk_updates(m, panel_floats, max_pending, g_vectors, pairs);
             b = max(1, min(b, min(m - ms, total - s)));
             cost += step_cost * b;
             s += b; m -= b;
@@ -1099,7 +1105,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         // ---- shares of rows: where this item stops, and what a continued row starts from -----------------
         int s_stop = total;                // steps [s_begin, s_stop) of the row are this item's
         int s_begin = 0, m_begin = d;
-        if (kind == ITEM_HEAD) s_stop = blk_cut_step(d, ms, total, a.panel_floats, a.max_pending, gB, head_num, NG, blk_step_cost(NT));
+        if (kind == ITEM_HEAD) s_stop = blk_cut_step(d, ms, total, a.panel_floats, a.max_pending, gB, !(GP || TC), head_num, NG, blk_step_cost(NT));
         if (kind == ITEM_HEAD && s_stop <= 0) {
             // too small a share to be worth a start: the neighbour takes the whole row
             if (tid == 0) blk_publish(a.split_state + (size_t)blockIdx.x * a.split_stride, a.split_flags + blockIdx.x, 0, d, 0);
@@ -1226,7 +1232,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
         int nb = 0;                      // pending vectors
         int ldz = blk_ldz(m0);
         int scap = a.panel_floats / ldz;     // pending vectors that fit into shared memory at this row length
-        int bcur = min(a.max_pending, GP || TC ? scap + gB : max(2, scap & ~1));      // (packed planes: vectors in pairs)
+        int bcur = blk_updates(m0, a.panel_floats, a.max_pending, gB, !(GP || TC));
         if (BC) bcur &= ~(BC - 1);           // whole blocks between two flushes, so that 4-slot groups stay together
         int s = s_begin;
         bool failed = false, timed_out = false;
@@ -1365,7 +1371,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int g = 0; g < KMAX / 4; ++g) cntw[g] = 0u;
                 ldz = blk_ldz(m0);
                 scap = a.panel_floats / ldz;
-                bcur = min(a.max_pending, GP || TC ? scap + gB : max(2, scap & ~1));
+                bcur = blk_updates(m0, a.panel_floats, a.max_pending, gB, !(GP || TC));
                 if (BC) bcur &= ~(BC - 1);
                 __syncthreads();
             }

@@ -18,6 +18,14 @@ def test_blocked_schedule_accounts_for_every_step():
         assert nbytes > 2.0 * d * (d + 1) and flops > 0
 
 
+def test_updates_of_the_short_row_kernels_come_in_pairs():
+    plan = {"on_chip_below": 128, "panel_floats": 10051, "max_pending": 64, "l2_vectors": 0, "threads": 128}
+    assert bench.pending_stride(576) == 612 and 10051 // 612 == 16 and bench.pending_updates(plan, 576) == 16
+    assert bench.pending_stride(500) == 516 and 10051 // 516 == 19 and bench.pending_updates(plan, 500) == 18
+    assert bench.pending_updates({**plan, "threads": 512}, 500) == 19 and bench.pending_updates({**plan, "panel_floats": 600}, 500) == 2
+    assert all(nb % 2 == 0 for _, nb in bench.blocked_schedule(plan, 576, 400)[:-1])
+
+
 def test_one_update_per_pass_moves_the_triangle_every_step():
     d = 200
     plan = {"on_chip_below": 0, "panel_floats": 10 ** 9, "max_pending": 1, "l2_vectors": 0}
