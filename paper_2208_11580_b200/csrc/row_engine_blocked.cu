@@ -107,7 +107,9 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
             // 64 for rows of middling length: shorter ones hold nearly all of 48 in shared memory, for longer ones the steps between two
             // passes, which read them all from L2, cost more than the rarer passes save (148 rows, pruning, 48 / 64 updates: 1280
             // 6.75 / 6.78, 1536 9.88 / 9.72, 2304 23.9 / 23.1, 3072 49.3 / 47.0, 3584 74.0 / 72.6, 4096 107 / 109, 4608 156 / 157)
-            if (d <= 1408 || d > 3840) groups = 3;
+            // A replay alone reads them for four columns at a time: 64 from 1921 on (64 rows, 48 / 64: 1536 5.00 / 5.20, 1800 7.61 / 7.96, 2048 10.26 /
+            // 10.11, 2304 14.4 / 14.0, 3072 28.9 / 27.6).
+            if (d <= (mode == MODE_REPLAY ? 1920 : 1408) || d > 3840) groups = 3;
             while (groups > 1 && (size_t)ft_stage_bytes(groups, FlushBufs{1, 1, 2}) + 1024 > share - fixed + 16 * (size_t)cap) --groups;
             if (d > p.ms && (size_t)ft_stage_bytes(1, FlushBufs{1, 1, 1}) + 1024 > share - fixed + 16 * (size_t)cap) return false;
             p.max_pending = 16 * groups;
