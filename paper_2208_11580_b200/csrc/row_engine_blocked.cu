@@ -109,7 +109,9 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
             // 6.75 / 6.78, 1536 9.88 / 9.72, 2304 23.9 / 23.1, 3072 49.3 / 47.0, 3584 74.0 / 72.6, 4096 107 / 109, 4608 156 / 157)
             // A replay alone reads them for four columns at a time: 64 from 1921 on (64 rows, 48 / 64: 1536 5.00 / 5.20, 1800 7.61 / 7.96, 2048 10.26 /
             // 10.11, 2304 14.4 / 14.0, 3072 28.9 / 27.6).
-            if (d <= (mode == MODE_REPLAY ? 1920 : 1408) || d > 3840) groups = 3;
+            // Blocks of 4 have less shared memory for them (six FP64 off-diagonals a block): 64 from 2049 to 2752 (32 / 148 rows, 48 : 64: 1536 6.72 :
+            // 6.90 / 7.85 : 8.07, 2304 17.8 : 17.6 / 21.0 : 20.3, 2700 25.4 : 25.6 / 31.2 : 31.0, 2900 30.1 : 32.2 / 37.8 : 39.2, 3584 49.7 : 53.9).
+            if (d <= (bc ? 2048 : mode == MODE_REPLAY ? 1920 : 1408) || d > (bc ? 2752 : 3840)) groups = 3;
             while (groups > 1 && (size_t)ft_stage_bytes(groups, FlushBufs{1, 1, 2}) + 1024 > share - fixed + 16 * (size_t)cap) --groups;
             if (d > p.ms && (size_t)ft_stage_bytes(1, FlushBufs{1, 1, 1}) + 1024 > share - fixed + 16 * (size_t)cap) return false;
             p.max_pending = 16 * groups;
