@@ -192,12 +192,13 @@ static __device__ __noinline__ void blk_state_copy(bool save, char* state, int c
 
 // Place of element (i, j), j <= i, of a private triangle: groups of columns one after the other, ld rows each.  A column is then one
 // strip of consecutive lines instead of a line per row of the matrix.
-// Passes on tcgen05 (TC): 32 columns, rows of 128 bytes, so that a 128-row tile of a group is contiguous.  Else 4 columns, rows of 16
+// One row per SM (WIDE): 32 columns, rows of 128 bytes, so that a 128-row tile of a group is contiguous.  Else 4 columns, rows of 16
 // bytes: a warp's 32 rows of a pivot column are 4 lines instead of 32 (one L1 tag look-up each, which the step's other accesses
-// queued behind), 768 x 768 2:4 8.55 -> 8.13 ms, 3072 x 768 compound 85.2 -> 83.0.  With passes on tcgen05 the smaller groups lose
-// more in the copies and the holes than the columns gain (256 x 2304 OBQ 43.6 -> 46.2 ms, 128 x 1152 blocks 7.74 -> 8.53).
-template <bool TC> __device__ __forceinline__ int tri_at(int ld, int i, int j) {
-    return TC ? ((j >> 5) * ld + i) * 32 + (j & 31) : ((j >> 2) * ld + i) * 4 + (j & 3);
+// queued behind), 768 x 768 2:4 8.55 -> 8.06 ms, 3072 x 768 compound 85.2 -> 82.7.  With one long row per SM the smaller groups lose
+// more in the passes and the holes than the columns gain: with passes on tcgen05 256 x 2304 OBQ 43.6 -> 46.2 ms, 128 x 1152 blocks of 4 7.74 ->
+// 8.53; blocks of 8, whose passes are by mma.sync, 32 x 3072 88.4 -> 92.8, 64 x 2304 40.9 -> 41.8, 64 x 1536 15.0 -> 15.3.
+template <bool WIDE> __device__ __forceinline__ int tri_at(int ld, int i, int j) {
+    return WIDE ? ((j >> 5) * ld + i) * 32 + (j & 31) : ((j >> 2) * ld + i) * 4 + (j & 3);
 }
 __host__ __device__ inline size_t tri_floats(int cap) { return (size_t)((cap + 63) & ~63) * cap; }      // (an even number of groups)
 
@@ -494,7 +495,7 @@ __device__ __forceinline__ void tf32_split2(float2 x, uint32_t& hi0, uint32_t& h
 }
 
 // A tile of H (16 rows x 64 columns from c0; in L2 by now: the cursor passed it two tiles ago) minus the increment acc * unscale.
-template <bool STREAM>
+template <bool STREAM, bool WIDE>
 __device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp, int c0, int ngroups, const int (&rr)[2], const bool (&in)[2],
                                                 const int (&sr)[2], int t, const float (&acc)[8][4], float unscale,
                                                 const unsigned short* srcm, const uint32_t* colmask) {
@@ -507,7 +508,7 @@ __device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp,
             hv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
             const int j = c0 + (u << 4) + (t << 2);
             if (u < ngroups && in[h] && j <= rr[h]) {
-                const float4* src = reinterpret_cast<const float4*>(Hp + tri_at<false>(ldp, sr[h], j));
+                const float4* src = reinterpret_cast<const float4*>(Hp + tri_at<WIDE>(ldp, sr[h], j));
                 hv[u][h] = STREAM ? __ldcs(src) : *src;
             }
         }
@@ -526,7 +527,7 @@ __device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp,
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         if (in[h] && jj <= rr[h]) {
-                            const float val = Hp[tri_at<false>(ldp, max(sr[h], sj), min(sr[h], sj))];
+                            const float val = Hp[tri_at<WIDE>(ldp, max(sr[h], sj), min(sr[h], sj))];
                             if (comp == 0) hv[u][h].x = val; else if (comp == 1) hv[u][h].y = val;
                             else if (comp == 2) hv[u][h].z = val; else hv[u][h].w = val;
                         }
@@ -545,7 +546,7 @@ __device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp,
                     float4 o = hv[u][h];
                     o.x = fmaf(-unscale, acc[2 * u][2 * h], o.x);     o.z = fmaf(-unscale, acc[2 * u][2 * h + 1], o.z);
                     o.y = fmaf(-unscale, acc[2 * u + 1][2 * h], o.y); o.w = fmaf(-unscale, acc[2 * u + 1][2 * h + 1], o.w);
-                    float4* dst = reinterpret_cast<float4*>(Hp + tri_at<false>(ldp, rr[h], j));
+                    float4* dst = reinterpret_cast<float4*>(Hp + tri_at<WIDE>(ldp, rr[h], j));
                     if (STREAM) __stcs(dst, o); else *dst = o;
                 }
             }
@@ -553,7 +554,7 @@ __device__ __forceinline__ void blk_flush_store(float* __restrict__ Hp, int ldp,
     }
 }
 
-template <int NT, bool STREAM, bool GP>
+template <int NT, bool STREAM, bool GP, bool WIDE>
 __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, int m1, int nb, int nbs, const float* Z, int ldz,
                                               const float* __restrict__ G, int gld, float* zstage,
                                               const unsigned short* srcm, const uint32_t* colmask) {
@@ -571,9 +572,10 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
     int prg = warp, pc0 = 0;
     auto prefetch_next = [&]() {
         if (prg >= nrg) return;
-        const int row = (prg << 4) + ((lane & 1) << 3), col = pc0 + ((lane >> 1) << 2);      // 16 column groups x 2 lines of 8 rows
-        if (row < m1 && col <= row + 7)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<false>(ldp, srcm[row], col)));
+        // 16 rows x 2 lines of 128 bytes, or 16 column groups x 2 lines of 8 rows
+        const int row = (prg << 4) + (WIDE ? lane >> 1 : (lane & 1) << 3), col = pc0 + (WIDE ? (lane & 1) << 5 : (lane >> 1) << 2);
+        if (row < m1 && col <= row + (WIDE ? 0 : 7))
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<WIDE>(ldp, srcm[row], col)));
         pc0 += 64;
         if (pc0 >= min((prg << 4) + 16, m1)) { pc0 = 0; prg += NW; }
     };
@@ -682,7 +684,7 @@ __device__ __forceinline__ void blk_flush_mma(float* __restrict__ Hp, int ldp, i
                 if (kg + 1 < ksteps_g) load_g(kg + 1);
                 kstep(av, b0, b1);
             }
-            blk_flush_store<STREAM>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, 1.f, srcm, colmask);
+            blk_flush_store<STREAM, WIDE>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, 1.f, srcm, colmask);
         }
     }
 }
@@ -828,7 +830,7 @@ __device__ __forceinline__ void mma_f16_z(float (&c)[4], const uint32_t (&a)[4],
 // over 16 vectors, scaled by `unscale` = 2^-2e of the planes.  What bounds it is the latency of a warp's one tile in flight: read, products,
 // subtraction, store.  Rows whose diagonal is too wide for a common power of two, and rows with overflow vectors (blocks of 8),
 // take the TF32 form.
-template <int NT>
+template <int NT, bool WIDE>
 __device__ __forceinline__ void blk_flush_f16(float* __restrict__ Hp, int ldp, int m1, int nb, const float* Z, int ldz, float unscale,
                                               const unsigned short* srcm, const uint32_t* colmask) {
     constexpr int NW = NT / 32;
@@ -841,9 +843,10 @@ __device__ __forceinline__ void blk_flush_f16(float* __restrict__ Hp, int ldp, i
     int prg = warp, pc0 = 0;
     auto prefetch_next = [&]() {
         if (prg >= nrg) return;
-        const int row = (prg << 4) + ((lane & 1) << 3), col = pc0 + ((lane >> 1) << 2);      // 16 column groups x 2 lines of 8 rows
-        if (row < m1 && col <= row + 7)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<false>(ldp, srcm[row], col)));
+        // 16 rows x 2 lines of 128 bytes, or 16 column groups x 2 lines of 8 rows
+        const int row = (prg << 4) + (WIDE ? lane >> 1 : (lane & 1) << 3), col = pc0 + (WIDE ? (lane & 1) << 5 : (lane >> 1) << 2);
+        if (row < m1 && col <= row + (WIDE ? 0 : 7))
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Hp + tri_at<WIDE>(ldp, srcm[row], col)));
         pc0 += 64;
         if (pc0 >= min((prg << 4) + 16, m1)) { pc0 = 0; prg += NW; }
     };
@@ -902,7 +905,7 @@ __device__ __forceinline__ void blk_flush_f16(float* __restrict__ Hp, int ldp, i
                         }
                 }
             }
-            blk_flush_store<true>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, unscale, srcm, colmask);
+            blk_flush_store<true, WIDE>(Hp, ldp, c0, ngroups, rr, in, sr, t, acc, unscale, srcm, colmask);
         }
     }
 }
@@ -1027,7 +1030,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
     extern __shared__ __align__(16) char smem[];
     constexpr int NW = NT / 32;
     constexpr int BCD = BC ? BC : 1;                           // divisor that is never zero
-    constexpr bool TC = blk_tc<NT, BC>;
+    constexpr bool TC = blk_tc<NT, BC>, WIDE = NT >= 512;      // (WIDE: the triangle in groups of 32 columns)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int d = a.d, cap = a.cap, ms = a.ms;
     char* scratch = smem;
@@ -1189,7 +1192,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     a.w_trace[((size_t)r * (a.trace_steps + 1)) * d + j] = a.W[(size_t)r * a.ldw + j];
         }
         if (kind != ITEM_TAIL && d > ms && total > 0) {
-            if constexpr (!TC) {
+            if constexpr (!WIDE) {
                 // a warp takes 8 rows, 4 lanes a row: 64 contiguous bytes read of each, 128 written to each of 4 column groups
                 for (int i0 = 8 * warp; i0 < d; i0 += 8 * NW) {
                     const int i = i0 + (lane >> 2);
@@ -1201,14 +1204,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
 #pragma unroll
                         for (int k = 0; k < 4; ++k) if (j0 + 4 * k < n4) t[k] = __ldg(s4 + j0 + 4 * k);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) if (j0 + 4 * k < n4) *reinterpret_cast<float4*>(dst + tri_at<TC>(ldp, i, 4 * (j0 + 4 * k))) = t[k];
+                        for (int k = 0; k < 4; ++k) if (j0 + 4 * k < n4) *reinterpret_cast<float4*>(dst + tri_at<WIDE>(ldp, i, 4 * (j0 + 4 * k))) = t[k];
                     }
                 }
             } else {
                 for (int i = warp; i < d; i += NW) {
                     const float4* s4 = reinterpret_cast<const float4*>(a.Hinv + (size_t)i * a.ldhi);
                     float* dst = HP;
-                    auto put = [&](int j4, float4 v) { *reinterpret_cast<float4*>(dst + tri_at<TC>(ldp, i, 4 * j4)) = v; };
+                    auto put = [&](int j4, float4 v) { *reinterpret_cast<float4*>(dst + tri_at<WIDE>(ldp, i, 4 * j4)) = v; };
                     const int n4 = (i >> 2) + 1;
                     if (GP || FG) {                 // (kernels with no registers to spare: one load in flight)
                         for (int j4 = lane; j4 < n4; j4 += 32) put(j4, s4[j4]);
@@ -1345,13 +1348,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                     if (!wide) {
                         blk_pack_planes<NT, KMAX>(panel, ldz, nb, m1, pow2f(power));
                         __syncthreads();
-                        blk_flush_f16<NT>(HP, ldp, m1, nb, panel, ldz, pow2f(-2 * power), srcm, colmask);
+                        blk_flush_f16<NT, WIDE>(HP, ldp, m1, nb, panel, ldz, pow2f(-2 * power), srcm, colmask);
                     } else {                                   // small rows of the matrix keep their own precision
-                        blk_flush_mma<NT, true, false>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);
+                        blk_flush_mma<NT, true, false, WIDE>(HP, ldp, m1, nb, nb, panel, ldz, nullptr, 0, nullptr, srcm, colmask);
                     }
                 }
                 else
-                    blk_flush_mma<NT, true, true>(HP, ldp, m1, nb, min(nb, scap), panel, ldz, GVEC, gld, ZSTAGE, srcm, colmask);
+                    blk_flush_mma<NT, true, true, WIDE>(HP, ldp, m1, nb, min(nb, scap), panel, ldz, GVEC, gld, ZSTAGE, srcm, colmask);
                 __syncthreads();
                 if (tid < nh) {
                     const int h = hl[tid], sv = mv[tid];
@@ -1444,7 +1447,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                         for (int g = 0; g < GS; ++g) {
                             const int p = p4[g];
                             if (jb + 3 <= p) {
-                                const float* from = tri + tri_at<TC>(ldp, p, jb);
+                                const float* from = tri + tri_at<WIDE>(ldp, p, jb);
                                 if (COLS == COLS_SMEM) copy_async<16>(wait + (size_t)g * ldz + jb, from);
                                 else {
                                     const float4 t = ld_tri4<TC>(from);
@@ -1455,7 +1458,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                                 for (int q = 0; q < 4; ++q) {
                                     const int j = jb + q;
                                     if (!((live >> (4 * g4 + q)) & 1u)) continue;
-                                    const float* from = tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p));
+                                    const float* from = tri + ((j <= p) ? tri_at<WIDE>(ldp, p, j) : tri_at<WIDE>(ldp, j, p));
                                     if (COLS == COLS_SMEM) copy_async<4>(wait + (size_t)g * ldz + j, from);
                                     else stored(g, 4 * g4 + q) = ld_tri<TC>(from);
                                 }
@@ -1694,13 +1697,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
                 for (int q = 0; q < 4; ++q) { c[4 * g + q] = 0.f; corr[4 * g + q] = 0.f; }
                 if (jb >= m0) continue;
                 if (jb + 3 <= p) {
-                    const float4 v = ld_tri4<TC>(tri + tri_at<TC>(ldp, p, jb));
+                    const float4 v = ld_tri4<TC>(tri + tri_at<WIDE>(ldp, p, jb));
                     c[4 * g] = v.x; c[4 * g + 1] = v.y; c[4 * g + 2] = v.z; c[4 * g + 3] = v.w;
                 } else {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int j = jb + q;
-                        if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at<TC>(ldp, p, j) : tri_at<TC>(ldp, j, p)));
+                        if ((alive >> (4 * g + q)) & 1u) c[4 * g + q] = ld_tri<TC>(tri + ((j <= p) ? tri_at<WIDE>(ldp, p, j) : tri_at<WIDE>(ldp, j, p)));
                     }
                 }
             }
@@ -1853,7 +1856,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) blocked_engine_kernel(const __gr
             __syncthreads();                                   // (pending vectors' space changes hands)
             for (int i = warp; i < m0; i += NW)
                 for (int j = lane; j <= i; j += 32)
-                    S[tail_at(i, j)] = d > ms ? ld_tri<TC>(HP + tri_at<TC>(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
+                    S[tail_at(i, j)] = d > ms ? ld_tri<TC>(HP + tri_at<WIDE>(ldp, i, j)) : a.Hinv[(size_t)i * a.ldhi + j];
             const int j = tid;
             double w = 0.0, g = 0.0;
             int o = -1, cnt = 0;
