@@ -79,10 +79,11 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     p.smem = share;
     p.panel_floats = (int)((share - fixed) / 4);
     p.ms = blk_pick_ms(d, share - fixed, nt);
-    // A replay alone that does not fit on chip from its start: four known eliminations off chip take less time than four steps on chip until
-    // few slots are left (30 % / 95 % of a row, ms, on chip as soon as it fits / by this rule: 64 x 320 0.247 / 0.201 and 0.520 / 0.522, 64 x 256
-    // 0.195 / 0.163 and 0.377 / 0.384, 600 x 160 0.216 / 0.173 and 0.455 / 0.400).
-    if (mode == MODE_REPLAY && d > p.ms && p.ms > (nt == 128 ? 64 : 128)) p.ms = nt == 128 ? 64 : 128;
+    // A replay alone that does not fit on chip from its start, or takes more than 224 slots there: four known eliminations off chip take less time
+    // than four steps on chip until few slots are left (30 % / 95 % of a row, ms, on chip as soon as it fits / by this rule: 64 x 320
+    // 0.247 / 0.201 and 0.520 / 0.522, 64 x 256 0.195 / 0.163 and 0.377 / 0.384, 600 x 160 0.216 / 0.173 and 0.455 / 0.400; 64 x 224 the
+    // other way round, 0.151 / 0.155 and 0.300 / 0.311).
+    if (mode == MODE_REPLAY && (d > p.ms || d > 224) && p.ms > (nt == 128 ? 64 : 128)) p.ms = nt == 128 ? 64 : 128;
     // Rows of one 512-thread block per SM: shared memory holds fewer pending vectors than a pass can apply (19 at d_col = 2304, 12
     // at 3072, 6 at 4608); further ones go to a global buffer small enough to stay in L2 (the triangle itself is streamed past
     // it with evict-first hints).
