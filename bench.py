@@ -450,7 +450,8 @@ def measure(args, name, steps, warmup, rank, world, dev, with_cpu=True, with_e2e
               "unit": "TFLOP/s", "frac": round(tflops / tpeak, 4), "frac_executed": round(3.0 * tflops / tpeak, 4),
               "flops_per_launch": int(flops // n_eng),
               "flops_model": "2 flops per element of the active lower triangle and deferred update (rank-B update on the tensor "
-                             "cores: FP16 tcgen05 with 512 threads per row, else FP16 m16n8k16); executed = 3 x that: every FP32 "
+                             "cores: FP16 tcgen05 with 512 threads per row, else FP16 m16n8k16, or TF32 where the diagonal spans "
+                             "more than 2^24); executed = 3 x that: every FP32 "
                              "operand is split into two parts and three of the four partial products are formed"}
     if blocked and plan.get("l2_vectors", 0) > 0:
         tensor["note"] = ("rows this long keep up to %d of their deferred updates per pass in global memory (sized to L2); the "

@@ -90,6 +90,8 @@ unsigned long long obc_kernel_launches(void);
  *                 gives every thread block the same amount of work, so a row may be started by one block and finished
  *                 by another; with OBC_ENGINE_WHOLE_WAVES every row stays on one block and the last wave runs partly
  *                 empty.
+ * A call with at most one row per SM gives a row all shared memory of its SM, so two such calls on two streams run beside each other only
+ * as far as there are SMs for the rows of both.
  * Values outside these sets make the call return OBC_ERR_INVALID_ARG.  Workspace sizes reported by
  * obc_workspace_bytes are valid for every choice. */
 typedef struct {

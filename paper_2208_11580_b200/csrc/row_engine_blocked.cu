@@ -23,10 +23,12 @@ obc_status blk_launch_512_12(const FlushMaps& zmaps, const EngineArgs& a, int bl
 
 // All blocks' overflow vectors together: the size of L2, which they share with the planes and the streamed triangles.  (Only the
 // longest rows reach the limit; when it was chosen, 48 / 64 / 80 / 110 MB at 128 rows x 4608 took 249 / 220 / 202 / 181 ms; the case
-// takes 149 ms since the layout and the tile order changed.)
+// takes 141 ms now.)
 constexpr size_t BLK_L2_PANEL_BUDGET = (size_t)110 << 20;
 
-// One slot per thread on chip, at most 256 of them.
+// One slot per thread on chip, at most 256 of them: 512 threads could hold 309, which measured the same (256 / 309 slots, pruning, OBQ:
+// 64 x 1152 4.71 / 4.70, 5.15 / 5.10 ms, 148 x 2304 23.0 / 23.2, 24.5 / 24.8, 64 x 3072 36.1 / 36.0, 38.9 / 39.0), and so rows from 257
+// columns on have passes with every thread count.
 static int blk_pick_ms(int d, size_t panel_bytes, int nt) {
     const int most = nt < 256 ? nt : 256;
     int ms = d < most ? d : most;
@@ -61,7 +63,10 @@ static bool blk_plan(int d, bool wfull, const DeviceInfo& di, BlkPlan* out, bool
     BlkPlan p;
     p.nt = nt;
     p.per_sm = 512 / nt;
-    // at most one row per SM: all of its shared memory (more updates per pass, more slots on chip: 64 x 576 layer 2283 -> 2180 us)
+    // at most one row per SM: all of its shared memory (more updates per pass, more slots on chip: 64 x 576 layer 2283 -> 2180 us).  Two such
+    // calls on two streams then share no SM.  Half of it from 75 rows on would let them (two calls / one call of 100 rows, all -> half, ms: 576
+    // 2.83 -> 2.07 / 1.41 -> 1.52, 704 3.93 -> 2.97 / 1.97 -> 2.17, 960 7.02 -> 5.86 / 3.58 -> 4.26): layers are solved one call after
+    // another, so the single call decides.
     if (row_count > 0 && row_count <= di.sm_count) p.per_sm = 1;
     // 1 KB per resident block is reserved by the hardware; keep every block's share 128-byte aligned
     const size_t sm_total = (size_t)di.smem_optin + 1024;

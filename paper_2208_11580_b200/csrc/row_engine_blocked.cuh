@@ -95,9 +95,10 @@ struct SplitHeader {                          // what the block that started a r
 __host__ __device__ inline size_t blk_split_stride(int cap) { return sizeof(SplitHeader) + (size_t)28 * cap + 256; }
 
 // Work model of a row, in units of "half a matrix element moved by a flush": a pass over the compacted triangle of m
-// slots costs m^2 / 2, a deferred-update step costs as much as blk_step_cost of those.  Fitted when every pass ran by mma.sync (1.1 -
-// 1.3e-10 s per m^2; a step 7 us with one 512-thread row per SM, 3.4 us with several smaller blocks per SM); with passes on
-// tcgen05 a step takes 7 us at d = 2304, 8 at 3072, 17 at 4608, and the values were not fitted again.
+// slots costs m^2 / 2, a deferred-update step costs as much as blk_step_cost of those, a step on chip 0.6 of that.  Fitted when every pass
+// ran by mma.sync (1.1 - 1.3e-10 s per m^2; a step 7 us with one 512-thread row per SM, 3.4 us with several smaller blocks per SM) and a
+// step on chip took 8000 cycles (1500 now).  Passes and steps have become shorter since and the values were not fitted again: 256 rows x
+// 2304 of 25 ms each on 148 SMs take 43.5 ms, which is 256 / 148 of a row.
 __host__ __device__ inline double blk_step_cost(int nt) { return nt >= 512 ? 30000.0 : 14000.0; }
 
 // The flush boundary of a row's schedule at which about num/den of the row's work is done (0: before the first
