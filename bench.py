@@ -47,10 +47,10 @@ FALLBACK_BF16_SUSTAINED_TFLOPS = 1400.0
 # traffic of a full-size launch is scaled from it by the algorithmic bytes (traffic grows with them).
 ENGINE_TRAFFIC_PER_ALGORITHMIC_BYTE = 291.0 / 603.3
 # The same for the blocked engine, relative to ITS algorithmic bytes (blocked_bytes_flops), per captured row length:
-# profiles/blocked_engine_d2304_d3072_ncu.txt: 93.92 GB moved for 50.31 GB at 2304, 219.24 GB for 119.24 GB at 3072.  Other row
+# profiles/blocked_engine_d2304_d3072_ncu.txt: 82.19 GB moved for 37.72 GB at 2304, 195.92 GB for 89.42 GB at 3072.  Other row
 # lengths run other configurations of the kernel (threads per row, pending vectors in L2) and have no capture: traffic is
 # null there.
-BLOCKED_TRAFFIC_PER_ALGORITHMIC_BYTE = {2304: 93.92 / 50.31, 3072: 219.24 / 119.24}
+BLOCKED_TRAFFIC_PER_ALGORITHMIC_BYTE = {2304: 82.19 / 37.72, 3072: 195.92 / 89.42}
 
 
 def model_bytes_full(d: int, first: int | None = None, steps: int | None = None) -> int:
